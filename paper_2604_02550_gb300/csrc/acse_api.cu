@@ -278,12 +278,12 @@ int acse_gemm_list_f64(acse_ctx* c, GemmF64* g, int* n) {
     int k = 0;
     for (int s = 0; s < 3; ++s) {
         const double f = (s == 1) ? 2.0 : 1.0;   // mixed-spin (rs) sums count both orders
-        g[k++] = GemmF64{w.M[s], c->cur_W[s], w.X[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0, 0};
-        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], w.Y[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0, 0};
+        g[k++] = GemmF64{w.M[s], c->cur_W[s], w.X[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0};
+        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], w.Y[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0};
     }
-    g[k++] = GemmF64{w.Zd, w.Md, w.X5d, R22, R22, R22, R22, R22, R22, 1.0, 0.0, 0, 0, 0};
-    g[k++] = GemmF64{w.Zf1, w.Mf1, w.X5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0, 0};
-    g[k++] = GemmF64{w.Zf2, w.Mf2, w.X5f2, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0, 0};
+    g[k++] = GemmF64{w.Zd, w.Md, w.X5d, R22, R22, R22, R22, R22, R22, 1.0, 0.0, 0, 0};
+    g[k++] = GemmF64{w.Zf1, w.Mf1, w.X5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0};
+    g[k++] = GemmF64{w.Zf2, w.Mf2, w.X5f2, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0};
     *n = k;
     return ACSE_OK;
 }

@@ -26,7 +26,6 @@ struct GemmF64 {
     int M, N, K;
     int lda, ldb, ldc;
     double alpha, beta;
-    int perm_r;   // 0: C row-major; r: particle-hole output stored permuted (see gemm_tc.cu)
     int transA, transB;
 };
 

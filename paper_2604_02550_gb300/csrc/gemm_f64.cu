@@ -1,15 +1,19 @@
 // FP64 grouped "NT" GEMM on the DFMA pipe:  C = alpha * A . B^T (+ beta C), A and B K-major.
 //
-// One launch runs every tile of up to GEMM_F64_MAXP problems (the sector GEMMs of one
-// contraction pass).  GB300's FP64 rate is low (about 2 DFMA per clock per SM), so each
-// 64x64 tile with a 4x4 register block per thread is bound by the DFMA pipe, not by shared
-// memory or HBM; the kernel keeps the loads simple and guarded (any M, N, K, lda, ldb).
+// One launch runs every tile of up to GEMM_F64_MAXP problems (the sector GEMMs of one contraction pass).
+// GB300 issues two DFMA per clock and SM, so the kernel is bound by that pipe at any tile size: a warp's
+// DFMA takes 16 cycles of it, and one shared-memory operand load per DFMA still leaves the load units
+// mostly idle.  What the tile size decides is the balance: a 64 x 64 tile of K = 392 holds its SM for
+// 0.4 ms, and the 165 such tiles of a pass at r = 14 took two of them (0.54 ms against 0.19 ms of DFMA
+// work).  So the tiles are small: 32 x 32 (2 x 2 outputs a thread) where every SM gets at least
+// GF_TILES_PER_SM of them, else 16 x 16 (one output a thread).
 #include "acse_internal.h"
 
 #define GEMM_F64_MAXP 40
-#define GF_BM 64
-#define GF_BN 64
-#define GF_BK 16
+#define GF_TPB 256
+// 32 x 32 tiles from this many per SM on: the last wave then idles at most a sixteenth of the launch, while
+// at r = 20 (6.5 a SM) 16 x 16 tiles finish earlier.
+#define GF_TILES_PER_SM 16
 
 struct GemmF64Batch {
     GemmF64 p[GEMM_F64_MAXP];
@@ -18,82 +22,86 @@ struct GemmF64Batch {
     int nprob;
 };
 
-__global__ void __launch_bounds__(256) k_gemm_f64(const __grid_constant__ GemmF64Batch b) {
+template <int BT>   // tile BT x BT, K blocks of 512 / BT: two elements of each operand a thread
+__global__ void __launch_bounds__(GF_TPB) k_gemm_f64(const __grid_constant__ GemmF64Batch b) {
+    constexpr int BK = 512 / BT, RT = BT / 16;   // RT x RT outputs a thread
     const int t = blockIdx.x;
     int pi = 0;
     while (pi + 1 < b.nprob && b.prefix[pi + 1] <= t) ++pi;
     const GemmF64& P = b.p[pi];
     const int local = t - b.prefix[pi];
-    const int m0 = (local / b.tiles_n[pi]) * GF_BM;
-    const int n0 = (local % b.tiles_n[pi]) * GF_BN;
+    const int m0 = (local / b.tiles_n[pi]) * BT;
+    const int n0 = (local % b.tiles_n[pi]) * BT;
 
-    __shared__ double As[GF_BK][GF_BM + 1];
-    __shared__ double Bs[GF_BK][GF_BN + 1];
+    __shared__ double As[BK][BT + 1];
+    __shared__ double Bs[BK][BT + 1];
 
-    const int tid = threadIdx.x;
-    const int tx = tid & 15;   // n direction
-    const int ty = tid >> 4;   // m direction
-    const int lrow = tid >> 2;          // 0..63 : row of the operand tile this thread loads
-    const int lk = (tid & 3) * 4;       // 0,4,8,12
-
-    double acc[4][4];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    double acc[RT][RT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RT; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < RT; ++j) acc[i][j] = 0.0;
 
     const int M = P.M, N = P.N, K = P.K;
-    const double* __restrict__ A = P.A;
-    const double* __restrict__ B = P.B;
-    const bool arow_ok = (m0 + lrow) < M;
-    const bool brow_ok = (n0 + lrow) < N;
-    // element (row, k) of each operand: row-major (K-major) or transposed storage
-    const size_t a_rs = P.transA ? 1 : (size_t)P.lda, a_ks = P.transA ? (size_t)P.lda : 1;
-    const size_t b_rs = P.transB ? 1 : (size_t)P.ldb, b_ks = P.transB ? (size_t)P.ldb : 1;
-    const double* Arow = A + (size_t)(m0 + lrow) * a_rs;
-    const double* Brow = B + (size_t)(n0 + lrow) * b_rs;
-
-    for (int k0 = 0; k0 < K; k0 += GF_BK) {
+    // this thread's two elements of an operand block: K-major storage runs along k, transposed along rows
+    int ar[2], ak[2], br[2], bk[2];
+    const double* asrc[2];
+    const double* bsrc[2];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = k0 + lk + q;
-            As[lk + q][lrow] = (arow_ok && k < K) ? Arow[(size_t)k * a_ks] : 0.0;
-            Bs[lk + q][lrow] = (brow_ok && k < K) ? Brow[(size_t)k * b_ks] : 0.0;
+    for (int u = 0; u < 2; ++u) {
+        const int e = tid + u * GF_TPB;
+        ar[u] = P.transA ? e % BT : e / BK;
+        ak[u] = P.transA ? e / BT : e % BK;
+        br[u] = P.transB ? e % BT : e / BK;
+        bk[u] = P.transB ? e / BT : e % BK;
+        const int m = m0 + ar[u], n = n0 + br[u];
+        asrc[u] = m < M ? P.A + (size_t)m * (P.transA ? 1 : P.lda) : nullptr;
+        bsrc[u] = n < N ? P.B + (size_t)n * (P.transB ? 1 : P.ldb) : nullptr;
+    }
+    const size_t a_ks = P.transA ? (size_t)P.lda : 1, b_ks = P.transB ? (size_t)P.ldb : 1;
+    double av[2], bv[2];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int ka = k0 + ak[u], kb = k0 + bk[u];
+            av[u] = asrc[u] && ka < K ? asrc[u][(size_t)ka * a_ks] : 0.0;
+            bv[u] = bsrc[u] && kb < K ? bsrc[u][(size_t)kb * b_ks] : 0.0;
+        }
+    };
+    load(0);
+    for (int k0 = 0; k0 < K; k0 += BK) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            As[ak[u]][ar[u]] = av[u];
+            Bs[bk[u]][br[u]] = bv[u];
         }
         __syncthreads();
+        if (k0 + BK < K) load(k0 + BK);   // in flight during the products
 #pragma unroll
-        for (int kk = 0; kk < GF_BK; ++kk) {
-            double a[4], bv[4];
+        for (int kk = 0; kk < BK; ++kk) {
+            double a[RT], c[RT];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < RT; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx + 16 * j];
+            for (int j = 0; j < RT; ++j) c[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RT; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
+                for (int j = 0; j < RT; ++j) acc[i][j] = fma(a[i], c[j], acc[i][j]);
         }
         __syncthreads();
     }
     const double alpha = P.alpha, beta = P.beta;
-    const int pr = P.perm_r, pR2 = pr * pr;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RT; ++i) {
         const int m = m0 + ty + 16 * i;
         if (m >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < RT; ++j) {
             const int n = n0 + tx + 16 * j;
             if (n >= N) continue;
-            size_t dst;
-            if (pr) {   // row (sK, k, j), column (sI, i, l) -> Cp[sK * nsb + sI][(i, j)][(k, l)]
-                const int nsb = N / pR2;
-                const int sK = m / pR2, kk = (m % pR2) / pr, jj = m % pr;
-                const int sI = n / pR2, ii = (n % pR2) / pr, ll = n % pr;
-                dst = ((size_t)(sK * nsb + sI) * pR2 + (size_t)ii * pr + jj) * pR2 + (size_t)kk * pr + ll;
-            } else {
-                dst = (size_t)m * P.ldc + n;
-            }
+            const size_t dst = (size_t)m * P.ldc + n;
             double v = alpha * acc[i][j];
             if (beta != 0.0) v += beta * P.C[dst];
             P.C[dst] = v;
@@ -107,6 +115,9 @@ int gemm_f64_grouped(acse_ctx* c, const GemmF64* probs, int nprob, cudaStream_t 
         GemmF64Batch b;
         int np = nprob - done;
         if (np > GEMM_F64_MAXP) np = GEMM_F64_MAXP;
+        long t32 = 0;
+        for (int i = 0; i < np; ++i) t32 += (long)((probs[done + i].M + 31) / 32) * ((probs[done + i].N + 31) / 32);
+        const int bt = t32 >= (long)GF_TILES_PER_SM * 152 ? 32 : 16;
         int tiles = 0;
         int used = 0;
         for (int i = 0; i < np; ++i) {
@@ -114,15 +125,16 @@ int gemm_f64_grouped(acse_ctx* c, const GemmF64* probs, int nprob, cudaStream_t 
             if (q.M <= 0 || q.N <= 0) continue;
             b.p[used] = q;
             b.prefix[used] = tiles;
-            b.tiles_n[used] = (q.N + GF_BN - 1) / GF_BN;
-            tiles += ((q.M + GF_BM - 1) / GF_BM) * b.tiles_n[used];
+            b.tiles_n[used] = (q.N + bt - 1) / bt;
+            tiles += ((q.M + bt - 1) / bt) * b.tiles_n[used];
             ++used;
         }
         b.prefix[used] = tiles;
         b.nprob = used;
         if (tiles > 0) {
             ACSE_TRY(prof_begin(c));
-            k_gemm_f64<<<tiles, 256, 0, s>>>(b);
+            if (bt == 32) k_gemm_f64<32><<<tiles, GF_TPB, 0, s>>>(b);
+            else k_gemm_f64<16><<<tiles, GF_TPB, 0, s>>>(b);
             ACSE_LAUNCHED(c);
             ACSE_TRY(prof_end(c));
         }

@@ -1183,7 +1183,7 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
     if (!root || slot < 0 || slot > 1 || n < 1 || n > OZ_MAXP) return ACSE_ERR_UNSUPPORTED;
     for (int i = 0; i < n; ++i) {
         int ex = 0;
-        if (frexp(g[i].alpha, &ex) != 0.5 || (g[i].beta != 0.0 && g[i].beta != 1.0) || g[i].perm_r) return ACSE_ERR_ARG;
+        if (frexp(g[i].alpha, &ex) != 0.5 || (g[i].beta != 0.0 && g[i].beta != 1.0)) return ACSE_ERR_ARG;
     }
     if (!root->lists[slot]) {
         const int s = oz_list_create(root, g, n, &root->lists[slot]);
