@@ -12,7 +12,9 @@
  *   * 2D^{pq}_{rs} = 1/2 <a+_p a+_q a_s a_r>;  Tr 2D = N(N-1)/2.
  *   * Spin blocks, spatial indices 0..r-1, full-square row-major [i][j][k][l]:
  *       X_aa = X^{ia ja}_{ka la},  X_ab = X^{ia jb}_{ka lb},  X_bb = X^{ib jb}_{kb lb}.
- *     Each block is r^4 doubles.  The aa and bb blocks are antisymmetric in (i,j) and in (k,l).
+ *     Each block is r^4 doubles.  The aa and bb blocks are antisymmetric in (i,j) and in (k,l), and every
+ *     block of a (real) 2-RDM is pair-Hermitian, X[ij][kl] = X[kl][ij]: the library relies on both and reads
+ *     entries that these symmetries relate once.
  *   * h: r x r one-electron integrals; V: r^4 two-electron integrals in chemist's notation
  *     (pq|rs) stored [p][q][r][s].
  *   * Reduced Hamiltonian (Eq. 2):  K = 1/2(<pq|rs> - <pq|sr>)
@@ -133,8 +135,8 @@ typedef struct {
  * context is ordered.  All device workspace of the forward calls is allocated here (about 40 r^4
  * doubles plus the split-precision operand copies, and the FP64-accurate context of a precision
  * schedule), so acse_energy, acse_residual and acse_step allocate nothing.  The one exception is
- * acse_residual_backward: its first call on a context allocates the adjoint workspace (about 65 r^4
- * doubles, 2.8 GB at r = 48) and, for a split precision, the ACSE_OZAKI companion context; both stay
+ * acse_residual_backward: its first call on a context allocates the adjoint workspace (about 75 r^4
+ * doubles, 3.2 GB at r = 48) and, for a split precision, the ACSE_OZAKI companion context; both stay
  * until acse_destroy.  On any failure *ctx is set to NULL (when ctx itself is not NULL) and nothing stays
  * allocated. */
 int acse_create(acse_ctx** ctx, const acse_opts* opts, const double* h, const double* V,
@@ -302,7 +304,7 @@ int acse_energy_noalloc(int r, int n_alpha, int n_beta, const double* h, const d
 
 /* Plan of the modular Ozaki GEMM (ACSE_OZAKI), on the host only (no device access; not part of the
  * method): for a context with oz_slices = S (4..10) whose longest O(r^6) contraction has length kmax
- * (2 r^2 for the pass; 1 <= kmax <= 8192), and one of its GEMMs of contraction length k (1 <= k <= kmax),
+ * (r (r + 1) for the pass; 1 <= kmax <= 8192), and one of its GEMMs of contraction length k (1 <= k <= kmax),
  * the number T of moduli (the least whose product P covers 4 kmax 2^(2 min(6S, 53))), the bits kept below
  * a row's leading bit (min(6S, 53), fewer only if P cannot cover the product at that k), the K chunks of
  * one residue product (64 * 64 elements at most each), and the moduli themselves (moduli: room for 19

@@ -98,8 +98,8 @@ static int alloc_d(void** p, size_t bytes, size_t* total) {
 
 static void free_work(acse_ctx* c) {
     Work& w = c->w;
-    void* ptrs[] = {w.Kh[0], w.Kh[1], w.Kh[2], w.gam, w.M[0], w.M[1], w.M[2], w.Md, w.Mf1, w.Mf2, w.Zd, w.Zf1,
-                    w.Zf2, w.w, w.Q, w.X[0], w.X[1], w.X[2], w.Y[0], w.Y[1], w.Y[2], w.X5d, w.X5f1, w.X5f2,
+    void* ptrs[] = {w.Kh[0], w.Kh[1], w.Kh[2], w.gam, w.M[0], w.M[1], w.M[2], w.Mp, w.Mm, w.Mf1, w.Wp, w.Wm, w.Wf1,
+                    w.V5d, w.V5f1, w.V5f2, w.Cp[0], w.Cp[1], w.pmap, w.w, w.Q, w.X[0], w.X[1], w.X[2], w.Y[0], w.Y[1], w.Y[2], w.X5d, w.X5f1, w.X5f2,
                     w.H[0], w.H[1], w.H[2], w.zdiag, w.A[0], w.A[1], w.A[2], w.U[0], w.U[1], w.U[2], w.Dt[0],
                     w.Dt[1], w.Dt[2], w.stage_in[0], w.stage_in[1], w.stage_in[2], w.stage_out[0],
                     w.stage_out[1], w.stage_out[2], w.h, w.V, w.scal, w.partial};
@@ -127,9 +127,19 @@ static int alloc_work(acse_ctx* c) {
         A_(w.zdiag, 4 * R2 * (size_t)c->r * sizeof(double));
         A_(w.w, 2 * R2 * sizeof(double));
         A_(w.Q, 2 * R2 * sizeof(double));
-        A_(w.Md, 4 * b4); A_(w.Mf1, b4); A_(w.Mf2, b4);
-        A_(w.Zd, 4 * b4); A_(w.Zf1, b4); A_(w.Zf2, b4);
+        const size_t S2 = (size_t)c->r * (c->r + 1), P2 = (size_t)c->r * (c->r - 1);   // pairs a <= b, a < b, two spins
+        A_(w.Mp, S2 * S2 * sizeof(double)); A_(w.Mm, P2 * P2 * sizeof(double)); A_(w.Mf1, b4);
+        A_(w.Wp, S2 * S2 * sizeof(double)); A_(w.Wm, S2 * P2 * sizeof(double)); A_(w.Wf1, b4);
+        A_(w.V5d, 4 * b4); A_(w.V5f1, b4); A_(w.V5f2, b4);
         A_(w.X5d, 4 * b4); A_(w.X5f1, b4); A_(w.X5f2, b4);
+        w.V1 = w.X5d;              // S2^2 + S2 P2 = 2 r^4 + 2 r^3 <= 4 r^4
+        w.V2 = w.X5d + S2 * S2;
+        for (int s = 0; s < 2; ++s) A_(w.Cp[s], P2 * P2 / 2 * sizeof(double));
+        A_(w.pmap, P2 / 2 * sizeof(int));
+        int hm[ACSE_MAX_R * (ACSE_MAX_R - 1) / 2];
+        for (int a = 0; a < c->r; ++a)
+            for (int b = a + 1; b < c->r; ++b) hm[pk_pair(c->r, a, b)] = a * c->r + b;
+        ACSE_CUDA_TRY(cudaMemcpy(w.pmap, hm, P2 / 2 * sizeof(int), cudaMemcpyHostToDevice));
     }
     A_(w.h, R2 * sizeof(double));
     A_(w.V, b4);
@@ -179,6 +189,7 @@ extern "C" int acse_create(acse_ctx** out, const acse_opts* o, const double* h, 
         return ACSE_ERR_CUDA;
     }
     int s = tiled_set_attrs();
+    if (s == ACSE_OK) s = ph_set_attrs();
     if (s == ACSE_OK) s = ny_set_attrs();
     if (s == ACSE_OK) s = alloc_work(c);
     if (s == ACSE_OK && c->opt.prec != ACSE_FP64) s = tc_plan_create(c);
@@ -254,7 +265,7 @@ extern "C" int acse_destroy(acse_ctx* c) {
 // ------------------------------------------------------------------------ contraction pass
 // G(W) for the current D: builds the operands, runs every O(r^6) GEMM of the pass in one
 // grouped launch, assembles B and G.  prep_D = 1 recomputes 1D, M and the ph layout of M.
-int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const W[3], int prep_D) {
+int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const W[3], int sW, int prep_D) {
     for (int s = 0; s < 3; ++s) {
         c->cur_D[s] = D[s];
         c->cur_W[s] = W[s];
@@ -262,45 +273,58 @@ int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const
     if (c->opt.prec == ACSE_FP64) {
         if (prep_D) {
             ACSE_TRY(launch_gamma_M(c, D));
-            ACSE_TRY(launch_pack_Mph(c));
+            ACSE_TRY(launch_ph_pack_M(c));
         }
-        ACSE_TRY(launch_W_intermediates(c, W));
-        return c->oz ? oz_slice_operands(c, prep_D) : ACSE_OK;
+        ACSE_TRY(launch_ph_pack_W(c, W, sW));
+        ACSE_TRY(launch_ph_w_diag(c, W));
+        ACSE_TRY(launch_w_sum(c));
+        return c->oz ? oz_slice_operands(c, prep_D, sW) : ACSE_OK;
     }
     if (prep_D) ACSE_TRY(launch_gamma(c, D));
     return tc_contract_pre(c, D, W, prep_D);
 }
 
-// The nine FP64 GEMMs of the pass whose operands acse_contract_pre prepared.
-int acse_gemm_list_f64(acse_ctx* c, GemmF64* g, int* n) {
+// The FP64 GEMMs of the pass whose operands acse_contract_pre prepared, longest contraction first: the
+// particle-hole products on symmetrised pairs (acse_ph.cu; with S, P the pairs a <= b, a < b, V1 has rows over
+// S and V2 over P for s = +1, the other way round for s = -1), the flip, X and Y of the mixed-spin pairs (their
+// (rs) sums count both orders, a factor 2) and of the same-spin pairs i < j (alpha 2 for the halved sum).
+int acse_gemm_list_f64(acse_ctx* c, int sW, GemmF64* g, int* n) {
     Work& w = c->w;
-    const int r = c->r, R2 = r * r, R22 = 2 * R2;
+    const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
+    const int n1 = sW > 0 ? S2 : P2, n2 = sW > 0 ? P2 : S2;
     int k = 0;
-    for (int s = 0; s < 3; ++s) {
-        const double f = (s == 1) ? 2.0 : 1.0;   // mixed-spin (rs) sums count both orders
-        g[k++] = GemmF64{w.M[s], c->cur_W[s], w.X[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0};
-        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], w.Y[s], R2, R2, R2, R2, R2, R2, f, 0.0, 0, 0};
+    g[k++] = GemmF64{w.Wp, w.Mp, w.V1, n1, S2, S2, S2, S2, S2, 1.0, 0.0, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wf1, w.Mf1, w.V5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr};
+    g[k++] = GemmF64{w.M[1], c->cur_W[1], w.X[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr};
+    g[k++] = GemmF64{c->cur_D[1], c->cur_W[1], w.Y[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wm, w.Mm, w.V2, n2, P2, P2, P2, P2, P2, 1.0, 0.0, nullptr, nullptr};
+    for (int s = 0; s < 3; s += 2) {
+        double* C = w.Cp[s / 2];
+        g[k++] = GemmF64{w.M[s], c->cur_W[s], C, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap};
+        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], C + (size_t)P * P, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap};
     }
-    g[k++] = GemmF64{w.Zd, w.Md, w.X5d, R22, R22, R22, R22, R22, R22, 1.0, 0.0, 0, 0};
-    g[k++] = GemmF64{w.Zf1, w.Mf1, w.X5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0};
-    g[k++] = GemmF64{w.Zf2, w.Mf2, w.X5f2, R2, R2, R2, R2, R2, R2, 1.0, 0.0, 0, 0};
     *n = k;
     return ACSE_OK;
 }
 
-int acse_contract_gemm(acse_ctx* c) {
-    if (c->oz) return oz_gemm_launch(c);
+int acse_contract_gemm(acse_ctx* c, int sW) {
+    if (c->oz) return oz_gemm_launch(c, sW);
     if (c->opt.prec == ACSE_FP64) {
-        GemmF64 g[9];
+        GemmF64 g[ACSE_F64_GEMMS];
         int n = 0;
-        ACSE_TRY(acse_gemm_list_f64(c, g, &n));
+        ACSE_TRY(acse_gemm_list_f64(c, sW, g, &n));
         return gemm_f64_grouped(c, g, n, c->stream);
     }
     return tc_gemm_launch(c);
 }
 
 int acse_contract_post(acse_ctx* c, int sW, double scale, int mask, double* const out[3], double* norm2_dst) {
-    if (c->opt.prec != ACSE_FP64) ACSE_TRY(tc_unpack_pairs(c));   // rows i < j of the same-spin [X; Y]
+    if (c->opt.prec != ACSE_FP64) {
+        ACSE_TRY(tc_unpack_pairs(c));   // rows i < j of the same-spin [X; Y]
+    } else {
+        ACSE_TRY(launch_pair_unpack(c));
+        ACSE_TRY(launch_ph_finish(c, sW));
+    }
     if (c->ny) ACSE_TRY(ny_pass(c));   // NY: the 3-cumulant term, added to B by the B kernel
     ACSE_TRY(launch_Q(c));
     ACSE_TRY(launch_build_B(c));
@@ -343,9 +367,9 @@ int acse_contract(acse_ctx* c, const double* const D[3], const double* const W[3
         ACSE_TRY(tc_mixed_prep_D(c, D));
         ACSE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_join[0], 0));
     } else {
-        ACSE_TRY(acse_contract_pre(c, D, W, prep_D));
+        ACSE_TRY(acse_contract_pre(c, D, W, sW, prep_D));
     }
-    ACSE_TRY(acse_contract_gemm(c));
+    ACSE_TRY(acse_contract_gemm(c, sW));
     return acse_contract_post(c, sW, scale, mask, out, norm2_dst);
 }
 

@@ -136,15 +136,15 @@ static int cgrid(size_t n) {
 }
 
 // --------------------------------------------------------------------------- one step
-static int gemm_pass(acse_batch* B) {
+static int gemm_pass(acse_batch* B, int sW) {
     if (B->prec == ACSE_FP64) {
-        // FP64: every instance's nine GEMMs in one grouped DFMA launch (split in chunks of 40 inside)
+        // FP64: every instance's GEMMs in one grouped DFMA launch (split in chunks of 40 inside)
         std::vector<GemmF64> all;
         for (int i = 0; i < B->n; ++i) {
             acse_ctx* c = B->ctx[i];
-            GemmF64 g[9];
+            GemmF64 g[ACSE_F64_GEMMS];
             int ng = 0;
-            ACSE_TRY(acse_gemm_list_f64(c, g, &ng));
+            ACSE_TRY(acse_gemm_list_f64(c, sW, g, &ng));
             all.insert(all.end(), g, g + ng);
         }
         return gemm_f64_grouped(B->ctx[0], all.data(), (int)all.size(), B->stream);
@@ -177,10 +177,10 @@ static int batch_step(acse_batch* B) {
         acse_ctx* c = B->ctx[i];
         const double* D[3] = {B->D[3 * i], B->D[3 * i + 1], B->D[3 * i + 2]};
         const double* Kh[3] = {c->w.Kh[0], c->w.Kh[1], c->w.Kh[2]};
-        ACSE_TRY(acse_contract_pre(c, D, Kh, 1));
+        ACSE_TRY(acse_contract_pre(c, D, Kh, +1, 1));
     }
     ACSE_TRY(join_all(B));
-    ACSE_TRY(gemm_pass(B));
+    ACSE_TRY(gemm_pass(B, +1));
     ACSE_TRY(fork_all(B));
     for (int i = 0; i < n; ++i) {
         acse_ctx* c = B->ctx[i];
@@ -196,10 +196,10 @@ static int batch_step(acse_batch* B) {
         ACSE_LAUNCHED(c);
         const double* D[3] = {B->D[3 * i], B->D[3 * i + 1], B->D[3 * i + 2]};
         const double* Ac[3] = {w.A[0], w.A[1], w.A[2]};
-        ACSE_TRY(acse_contract_pre(c, D, Ac, 0));
+        ACSE_TRY(acse_contract_pre(c, D, Ac, -1, 0));
     }
     ACSE_TRY(join_all(B));
-    ACSE_TRY(gemm_pass(B));
+    ACSE_TRY(gemm_pass(B, -1));
     ACSE_TRY(fork_all(B));
     for (int i = 0; i < n; ++i) {
         acse_ctx* c = B->ctx[i];
@@ -265,7 +265,7 @@ static int autotune(acse_batch* B) {
         acse_ctx* c = B->ctx[i];
         const double* D[3] = {B->D[3 * i], B->D[3 * i + 1], B->D[3 * i + 2]};
         const double* Kh[3] = {c->w.Kh[0], c->w.Kh[1], c->w.Kh[2]};
-        ACSE_TRY(acse_contract_pre(c, D, Kh, 1));
+        ACSE_TRY(acse_contract_pre(c, D, Kh, +1, 1));
         ACSE_CUDA_TRY(cudaStreamSynchronize(c->stream));
     }
     struct Cand { int choice, split; };
@@ -277,9 +277,9 @@ static int autotune(acse_batch* B) {
     ACSE_CUDA_TRY(cudaEventCreate(&e1));
     for (const Cand& cd : cands) {
         ACSE_TRY(build_tables(B, cd.choice, cd.split));
-        ACSE_TRY(gemm_pass(B));   // warm-up
+        ACSE_TRY(gemm_pass(B, +1));   // warm-up
         ACSE_CUDA_TRY(cudaEventRecord(e0, B->stream));
-        for (int rep = 0; rep < 3; ++rep) ACSE_TRY(gemm_pass(B));
+        for (int rep = 0; rep < 3; ++rep) ACSE_TRY(gemm_pass(B, +1));
         ACSE_CUDA_TRY(cudaEventRecord(e1, B->stream));
         ACSE_CUDA_TRY(cudaEventSynchronize(e1));
         float ms = 0.f;

@@ -12,7 +12,8 @@
 //     w^k_s  = sum_pr W^{kp}_{rs} 1D^p_r                              X2^{ij}_{kl} = sum_s w^k_s M^{ij}_{ls}
 //     Q^k_i  = sum_prs W^{kp}_{rs} M^{ip}_{rs}                        X4 = Q^k_i 1D^j_l,  X7 = Q^k_j 1D^i_l
 //     Z^{kp}_{js} = sum_r W^{kp}_{rs} 1D^j_r                          X5^{ij}_{kl} = sum_ps Z^{kp}_{js} M^{ip}_{ls}
-//     X8 = X5 with i <-> j                                             (particle-hole GEMM)
+//     X8 = X5 with i <-> j                                             (particle-hole GEMM; the FP64 and
+//                                                                      Ozaki paths: acse_ph.cu)
 // (the E^{ij}_{kl} intermediate of Appendix C is 2 X5 - X4), and the residual of
 // Eq. (residual) with the commutator sign convention becomes
 //     G(W) = 4 (Y - s Y^T) - 12 (B - B_{k<->l}) + 12 s (B^T - B^T_{i<->j}),   Y = D W^T,
@@ -134,50 +135,8 @@ int launch_gamma_M(acse_ctx* c, const double* const D[3]) {
     return ACSE_OK;
 }
 
-// ------------------------------------------------------------------ particle-hole layout of M
-// Diagonal ph sector: rows (sI,i,l), cols (sP,p,s) of M^{i sI, p sP}_{l sI, s sP}:
-//   (a,a) Maa[i][p][l][s]  (a,b) Mab[i][p][l][s]  (b,a) Mab[p][i][s][l]  (b,b) Mbb[i][p][l][s]
-// Spin-flip sectors (both Z and M carry a sign -1 there, which cancels in the product):
-//   F1: (I,L) = (ia, lb), (P,S) = (pb, sa):  Mf1[(i,l)][(p,s)] = Mab[i][p][s][l]
-//   F2: (I,L) = (ib, la), (P,S) = (pa, sb):  Mf2[(i,l)][(p,s)] = Mab[p][i][l][s]
-__global__ void k_pack_Mph(int r, const double* __restrict__ Maa, const double* __restrict__ Mab,
-                           const double* __restrict__ Mbb, double* __restrict__ Md, double* __restrict__ Mf1,
-                           double* __restrict__ Mf2) {
-    const size_t R2 = (size_t)r * r, n4 = R2 * R2;
-    const size_t nd = 4 * n4;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nd + 2 * n4; e += (size_t)gridDim.x * blockDim.x) {
-        if (e < nd) {
-            const size_t row = e / (2 * R2), col = e % (2 * R2);
-            const int sI = (int)(row / R2), sP = (int)(col / R2);
-            const int i = (int)((row % R2) / r), l = (int)(row % r);
-            const int p = (int)((col % R2) / r), s = (int)(col % r);
-            double v;
-            if (sI == 0 && sP == 0) v = Maa[((i * r + p) * (size_t)r + l) * r + s];
-            else if (sI == 0) v = Mab[((i * r + p) * (size_t)r + l) * r + s];
-            else if (sP == 0) v = Mab[((p * r + i) * (size_t)r + s) * r + l];
-            else v = Mbb[((i * r + p) * (size_t)r + l) * r + s];
-            Md[e] = v;
-        } else {
-            const size_t f = e - nd;
-            const int which = (int)(f / n4);
-            const size_t g = f % n4;
-            const int i = (int)(g / (R2 * r)), l = (int)((g / R2) % r), p = (int)((g / r) % r), s = (int)(g % r);
-            if (which == 0) Mf1[g] = Mab[((i * r + p) * (size_t)r + s) * r + l];
-            else Mf2[g] = Mab[((p * r + i) * (size_t)r + l) * r + s];
-        }
-    }
-}
-
-int launch_pack_Mph(acse_ctx* c) {
-    const int r = c->r;
-    const size_t n = (size_t)6 * r * r * r * r;
-    k_pack_Mph<<<grid_for(n), TPB, 0, c->stream>>>(r, c->w.M[0], c->w.M[1], c->w.M[2], c->w.Md, c->w.Mf1, c->w.Mf2);
-    ACSE_LAUNCHED(c);
-    return ACSE_OK;
-}
-
 // ------------------------------------------------------------------- W-dependent intermediates
-// Z, w (acse_tiled.cu) and Q (a partial trace of the pair GEMM output X).
+// w (acse_ph.cu, acse_tiled.cu) and Q (a partial trace of the pair GEMM output X).
 
 // Q^k_i = sum_prs W^{kp}_{rs} M^{ip}_{rs} is a partial trace of the pair GEMM output
 // X^{ij}_{kp} = sum_rs M^{ij}_{rs} W^{kp}_{rs}:  Q^k_i = sum_P X^{iP}_{kP}, i.e.
@@ -213,8 +172,6 @@ __global__ void __launch_bounds__(256) k_Q_from_X(int r, const T* __restrict__ X
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if (lane == 0) Qv[t] = acc;
 }
-
-int launch_W_intermediates(acse_ctx* c, const double* const W[3]) { return launch_Z_tiled(c, W, nullptr); }
 
 int launch_Q(acse_ctx* c) {
     const int r = c->r;

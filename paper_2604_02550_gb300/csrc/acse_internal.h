@@ -14,10 +14,21 @@
 // the row and column order of the packed same-spin GEMM operands and outputs of the split path.
 __host__ __device__ __forceinline__ int pk_pair(int r, int a, int b) { return a * r - a * (a + 1) / 2 + (b - a - 1); }
 
+// pair number among a <= b (row by row), and its inverse
+__host__ __device__ __forceinline__ int ps_pair(int r, int a, int b) { return a * r - a * (a - 1) / 2 + (b - a); }
+__device__ __forceinline__ void ps_unpair(int r, int u, int& a, int& b) {
+    const float h = 2.0f * (float)r + 1.0f;   // the float estimate is corrected by exact integer steps
+    int t = (int)(0.5f * (h - sqrtf(fmaxf(h * h - 8.0f * (float)u, 0.0f))));
+    t = max(0, min(r - 1, t));
+    while (t > 0 && ps_pair(r, t, t) > u) --t;
+    while (t + 1 < r && ps_pair(r, t + 1, t + 1) <= u) ++t;
+    a = t;
+    b = t + (u - ps_pair(r, t, t));
+}
+
 // ------------------------------------------------------------------------------------------
 // Dense GEMM problem: C[m*ldc + n] = alpha * sum_k A(m,k) B(n,k) (+ beta*C), with
-//   A(m,k) = A[m*lda + k] (transA = 0, K-major) or A[k*lda + m] (transA = 1),
-//   B(n,k) = B[n*ldb + k] (transB = 0, K-major) or B[k*ldb + n] (transB = 1).
+//   A(m,k) = A[mapA(m)*lda + mapA(k)],  B(n,k) = B[mapB(n)*ldb + mapB(k)]  (K-major).
 // ------------------------------------------------------------------------------------------
 struct GemmF64 {
     const double* A;
@@ -26,7 +37,8 @@ struct GemmF64 {
     int M, N, K;
     int lda, ldb, ldc;
     double alpha, beta;
-    int transA, transB;
+    const int* mapA;   // null, or the source row of every row of A and source column of every K index (the
+    const int* mapB;   // pair numbering of a packed same-spin operand); the same for B
 };
 
 // Split-precision operand problem for the tensor-core path.  A and B are 16-bit (BF16) or
@@ -85,14 +97,19 @@ struct Work {
     // 1-RDM per spin (r^2 each) and the M blocks (r^4 each)
     double* gam;          // [2][r][r]
     double* M[3];
-    // particle-hole layouts of M: diag (2r^2 x 2r^2), flips (r^2 x r^2)
-    double* Md;
+    // particle-hole operands on symmetrised pairs (acse_ph.cu): M+ (2S x 2S), M- (2P x 2P), flip (r^2 x r^2);
+    // W+ and W- (up to 2S x 2S and 2S x 2P), flip
+    double* Mp;
+    double* Mm;
     double* Mf1;
-    double* Mf2;
-    // per-W intermediates
-    double* Zd;
-    double* Zf1;
-    double* Zf2;
+    double* Wp;
+    double* Wm;
+    double* Wf1;
+    double* V1;           // their products (in X5d, which the transformation by 1D overwrites last)
+    double* V2;
+    double* V5d;          // V5 in full: 2r^2 x 2r^2, and the two flips
+    double* V5f1;
+    double* V5f2;
     double* w;            // [2][r][r]
     double* Q;            // [2][r][r]
     double* X[3];         // pair GEMM outputs M W^T (r^4 each)
@@ -101,7 +118,9 @@ struct Work {
     double* X5f1;
     double* X5f2;
     double* H[3];         // H_b = 4 Y_b - 12 (P - P'_{k<->l}) per block (r^4 each); G_b = H_b - s H_b^T
-    double* zdiag;        // [4][r][r][r]: diagonal rows j = p of Z (for w)
+    double* zdiag;        // [4][r][r][r]: the terms of w before the sum over p
+    double* Cp[2];        // packed [X; Y] of the aa and bb sectors (2P x P)
+    int* pmap;            // pair number -> i r + j (i < j), P entries
     // residual, update, trial D for the line search
     double* A[3];
     double* U[3];
@@ -242,13 +261,23 @@ int prof_end(acse_ctx* c);
 int launch_build_K(acse_ctx* c);
 int launch_gamma(acse_ctx* c, const double* const D[3]);
 int launch_gamma_M(acse_ctx* c, const double* const D[3]);
-int launch_pack_Mph(acse_ctx* c);
-int launch_W_intermediates(acse_ctx* c, const double* const W[3]);
+int launch_w_sum(acse_ctx* c);
+// particle-hole products on symmetrised pairs (acse_ph.cu)
+int launch_ph_pack_M(acse_ctx* c);
+int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW);
+int launch_ph_w_diag(acse_ctx* c, const double* const W[3]);
+int launch_ph_xform(acse_ctx* c, const double* const in[3], double* const out[3], int trans);
+int launch_ph_finish(acse_ctx* c, int sW);
+int launch_pair_unpack(acse_ctx* c);
+int ph_set_attrs();
 int launch_build_B(acse_ctx* c);
-int launch_Z_tiled(acse_ctx* c, const double* const W[3], const float* const W32[3]);
+int launch_Z_tiled(acse_ctx* c, const float* const W32[3]);
 int launch_B_tiled(acse_ctx* c);
 int launch_Z_tc(acse_ctx* c, const float* const W32[3], int ntypes, const int* tmap);   // acse_ztc.cu
-int launch_Z_oz(struct acse_ctx* c, const double* const W[3], int ntypes, const int* tmap);   // acse_zoz.cu
+int launch_xform_oz(struct acse_ctx* c, const double* const in[3], double* const out[3], int trans);   // acse_zoz.cu
+// out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] for eight classes (bit c of tt, gt: T, G read transposed)
+int launch_rows_oz(struct acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
+                   double* const out[8]);   // acse_zoz.cu
 int launch_Bx_oz(struct acse_ctx* c);                                                           // acse_zoz.cu
 int launch_Bx_tc(acse_ctx* c);                                                           // acse_btc.cu
 int tiled_set_attrs();
@@ -272,17 +301,18 @@ int tc_encode_map_bf16(void* map, const void* base, int rows, int inner_elems, i
 // Ozaki-scheme FP64 GEMMs of the contraction pass (gemm_oz.cu)
 int oz_plan_create(acse_ctx* c);
 void oz_plan_destroy(acse_ctx* c);
-int oz_slice_operands(acse_ctx* c, int prep_D);   // the pass's FP64 operands -> scaled bf16 slices
-int oz_gemm_launch(acse_ctx* c);                   // every GEMM of the pass, one persistent launch
+int oz_slice_operands(acse_ctx* c, int prep_D, int sW);   // the pass's FP64 operands -> scaled bf16 slices
+int oz_gemm_launch(acse_ctx* c, int sW);                  // every GEMM of the pass, one persistent launch
 int oz_set_wait_ns(acse_ctx* c, unsigned long long ns, int inject_stall);
-// Any list of up to 12 FP64 GEMMs (alpha a power of two, beta 0 or 1, operands possibly transposed) by
-// the Ozaki scheme; `slot` (0 or 1) names the list's plan, built on its first use (the adjoint's lists)
+// Any list of up to 12 FP64 GEMMs (alpha a power of two, beta 0, mapA null) by the Ozaki scheme; `slot` (0 or
+// 1) names the list's plan, built on its first use (the adjoint's lists)
 int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot);
 
 // contraction pass in three phases (acse_api.cu): operands, the O(r^6) GEMMs, assembly
-int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const W[3], int prep_D);
-int acse_contract_gemm(acse_ctx* c);
+int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const W[3], int sW, int prep_D);
+int acse_contract_gemm(acse_ctx* c, int sW);
 int acse_contract_post(acse_ctx* c, int sW, double scale, int mask, double* const out[3], double* norm2_dst);
-int acse_gemm_list_f64(acse_ctx* c, GemmF64* g, int* n);
+#define ACSE_F64_GEMMS 9   // entries acse_gemm_list_f64 fills
+int acse_gemm_list_f64(acse_ctx* c, int sW, GemmF64* g, int* n);
 int acse_contract(acse_ctx* c, const double* const D[3], const double* const W[3], int sW, double scale, int mask,
                   double* const out[3], double* norm2_dst, int prep_D);

@@ -451,7 +451,7 @@ int tc_mixed_prep_W(acse_ctx* c, const double* const W[3]) {
     else
         launch_pack_W<ACSE_TF32>(c, grid, W32, p);
     ACSE_LAUNCHED(c);
-    return launch_Z_tiled(c, W, W32);   // Z packs and w (the diagonal of Z)
+    return launch_Z_tiled(c, W32);   // Z packs and w (the diagonal of Z)
 }
 
 // ------------------------------------------------------------------------ workspace

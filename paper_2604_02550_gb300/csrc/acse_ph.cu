@@ -1,0 +1,353 @@
+// The particle-hole products of a contraction pass on symmetrised index pairs (FP64 and Ozaki paths).
+//
+// With V5[(k,q)][(i,l)] = sum_{p,t} W^{kp}_{qt} M^{ip}_{lt} (spin-conserving sector: (k,q) of one spin, (p,t) of
+// either, (i,l) of one spin), the operand of B is X5[(k,j)][(i,l)] = sum_q 1D^j_q V5[(k,q)][(i,l)] -- the
+// transformation by 1D commutes with the sum over (p,t), so it may follow the O(r^6) product instead of
+// preceding it, and then the product has a symmetry that halves both its output and its sum:
+//     M^{ip}_{lt} = M^{lt}_{ip} (Hermitian) and = M^{pi}_{tl}  =>  M[(i,l)][(p,t)] = M[(l,i)][(t,p)],
+//     W[(k,q)][(p,t)] = s W[(q,k)][(t,p)]  for a pair-Hermitian (s = +1) or anti-Hermitian (s = -1) W.
+// Split over the exchange of (p,t): W+- = (W[.][(p,t)] +- W[.][(t,p)]) / 2, M+- likewise.  M+ is symmetric in
+// (i,l) and M- antisymmetric; W+ is symmetric in (k,q) and W- antisymmetric for s = +1, the other way round
+// for s = -1.  The cross terms vanish, so
+//     V5 = V1 + V2,   V1 = 2 sum_{p<t} W+ M+ + sum_{p=t} W M,   V2 = 2 sum_{p<t} W- M-,
+// two products on pairs a <= b (S = r(r+1)/2 per spin) and a < b (P = r(r-1)/2): 4 r^6 flop in place of the
+// 16 r^6 of the full (2r^2)^3 product.  The spin-flip sectors are each other's image,
+// V5f2[(k,q)][(i,l)] = s V5f1[(q,k)][(l,i)], so one of them is multiplied: 2 r^6 in place of 4 r^6.
+// D (hence M) is taken as pair-Hermitian, which a 2-RDM is; entries are read at i <= l.
+//
+// Kernels here: the packing of both operands, the expansion of V1, V2, V5f1 into the full V5 (HBM-bound), the
+// diagonal sums behind w, and the transformation by 1D on the CUDA cores (an Ozaki context with r a
+// multiple of 16 runs it on the tensor cores, acse_zoz.cu).
+#include <type_traits>
+
+#include "acse_internal.h"
+#include "dfloat.cuh"
+
+// ------------------------------------------------------------------------------- packing
+// plus[(K,{kq})][(P',{p<=t})] = f (x + x') (x at p = t), minus[(K,{kq})][(P',{p<t})] = f (x - x'), with
+// x = T^{kp}_{qt}, x' = T^{kt}_{qp}, spins K of (k,q) and P' of (p,t); the rows of `plus` run over k <= q and
+// those of `minus` over k < q (plusS = 1), or the other way round (plusS = 0).  flip[(k,q)][(p,t)] =
+// T_ab[k][p][t][q].  W takes f = 1/2; M takes f = 1, the 2 of the halved sum over (p,t) included.
+//
+// Block (K, P', {k<=q}): the r x r slab of (p,t) goes through shared memory, both rows leave coalesced (the
+// b,a slab is read at stride r: its sectors are shared by the blocks of neighbouring q).  Block (k,p) of the
+// flips: an r x r transposition in shared memory.
+struct PhPack {
+    const double* src[3];
+    double* plus;
+    double* minus;
+    double* flip;
+    int r, plusS;
+    double f;
+};
+
+__global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack a) {
+    extern __shared__ double ph_sm[];   // [r][r + 1]
+    const int r = a.r, ld = r + 1, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
+    const size_t R2 = (size_t)r * r, r3 = R2 * r;
+    if ((int)blockIdx.x < 4 * S) {
+        const int kp = (int)blockIdx.x / S, u = (int)blockIdx.x - kp * S, K = kp >> 1, Q = kp & 1;
+        int k, q;
+        ps_unpair(r, u, k, q);
+        const double* src = a.src[K == Q ? 2 * K : 1];
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
+            const int p = e / r, t = e - p * r;
+            ph_sm[p * ld + t] = (K == 1 && Q == 0) ? src[p * r3 + k * R2 + (size_t)t * r + q]
+                                                   : src[k * r3 + p * R2 + (size_t)q * r + t];
+        }
+        __syncthreads();
+        const int rowS = K * S + u, rowA = k < q ? K * P + pk_pair(r, k, q) : -1;
+        const int rp = a.plusS ? rowS : rowA, rm = a.plusS ? rowA : rowS;
+        double* op = a.plus + (size_t)max(rp, 0) * 2 * S + (size_t)Q * S;
+        double* om = a.minus + (size_t)max(rm, 0) * 2 * P + (size_t)Q * P;
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
+            const int p = e / r, t = e - p * r;
+            if (t < p) continue;
+            const double x = ph_sm[p * ld + t], y = ph_sm[t * ld + p];
+            if (rp >= 0) op[ps_pair(r, p, t)] = p < t ? a.f * (x + y) : x;
+            if (rm >= 0 && p < t) om[pk_pair(r, p, t)] = a.f * (x - y);
+        }
+    } else {
+        const int kp = (int)blockIdx.x - 4 * S, k = kp / r, p = kp - k * r;
+        const double* src = a.src[1] + k * r3 + p * R2;
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) ph_sm[(e / r) * ld + e % r] = src[e];   // [t][q]
+        __syncthreads();
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
+            const int q = e / r, t = e - q * r;
+            a.flip[((size_t)k * r + q) * R2 + (size_t)p * r + t] = ph_sm[t * ld + q];
+        }
+    }
+}
+
+static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, double* minus, double* flip, int plusS,
+                          double f) {
+    const int r = c->r;
+    PhPack a;
+    for (int s = 0; s < 3; ++s) a.src[s] = T[s];
+    a.plus = plus;
+    a.minus = minus;
+    a.flip = flip;
+    a.r = r;
+    a.plusS = plusS;
+    a.f = f;
+    const int blocks = 4 * (r * (r + 1) / 2) + r * r;
+    k_ph_pack<<<blocks, 256, (size_t)r * (r + 1) * sizeof(double), c->stream>>>(a);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+int launch_ph_pack_M(acse_ctx* c) {
+    Work& w = c->w;
+    return launch_ph_pack(c, w.M, w.Mp, w.Mm, w.Mf1, 1, 1.0);
+}
+
+int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW) {
+    Work& w = c->w;
+    return launch_ph_pack(c, W, w.Wp, w.Wm, w.Wf1, sW > 0, 0.5);
+}
+
+// ------------------------------------------------------------------------------ expansion
+// V5 (rows (K,k,q), columns (I,i,l)) = V1 + V2 from the products on pairs, by the symmetries above: row (k,q),
+// k < q, is V1 + sg(i,l) V2 (sg = 1 for i < l, -1 for i > l, 0 for i = l), and row (q,k) s times V1 - sg V2
+// ... (s = +1: V1 is even and V2 odd in the exchange of k and q, s = -1: the other way round).  The diagonal
+// rows k = q have the even part alone.  V5f2[(k,q)][(i,l)] = s V5f1[(q,k)][(l,i)].
+struct PhUnpack {
+    const double* V1;
+    const double* V2;
+    const double* f1;
+    double* V;
+    double* f2;
+    int r, s;
+};
+
+__global__ void __launch_bounds__(256) k_ph_unpack(const __grid_constant__ PhUnpack a) {
+    extern __shared__ double ph_sm[];   // 2S + 2P = 2 r^2 doubles
+    const int r = a.r, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
+    const size_t R2 = (size_t)r * r;
+    if ((int)blockIdx.x < 2 * S) {
+        const int K = (int)blockIdx.x / S, u = (int)blockIdx.x - K * S;
+        int k, q;
+        ps_unpair(r, u, k, q);
+        const int rowS = K * S + u, rowA = k < q ? K * P + pk_pair(r, k, q) : -1;
+        const int r1 = a.s > 0 ? rowS : rowA, r2 = a.s > 0 ? rowA : rowS;
+        double* v1 = ph_sm;
+        double* v2 = ph_sm + 2 * S;
+        for (int e = threadIdx.x; e < 2 * S; e += blockDim.x) v1[e] = r1 >= 0 ? a.V1[(size_t)r1 * 2 * S + e] : 0.0;
+        for (int e = threadIdx.x; e < 2 * P; e += blockDim.x) v2[e] = r2 >= 0 ? a.V2[(size_t)r2 * 2 * P + e] : 0.0;
+        __syncthreads();
+        double* o1 = a.V + ((size_t)K * R2 + (size_t)k * r + q) * 2 * R2;
+        double* o2 = a.V + ((size_t)K * R2 + (size_t)q * r + k) * 2 * R2;
+        for (int e = threadIdx.x; e < 2 * (int)R2; e += blockDim.x) {
+            const int I = e >= (int)R2, c = e - I * (int)R2, i = c / r, l = c - i * r;
+            const double x = v1[I * S + (i <= l ? ps_pair(r, i, l) : ps_pair(r, l, i))];
+            double y = 0.0;
+            if (i < l) y = v2[I * P + pk_pair(r, i, l)];
+            else if (i > l) y = -v2[I * P + pk_pair(r, l, i)];
+            o1[e] = x + y;
+            if (k < q) o2[e] = a.s > 0 ? x - y : y - x;
+        }
+    } else {
+        const int kq = (int)blockIdx.x - 2 * S, k = kq / r, q = kq - k * r;
+        const double* src = a.f1 + ((size_t)q * r + k) * R2;
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) ph_sm[e] = src[e];
+        __syncthreads();
+        const double s = (double)a.s;
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
+            const int i = e / r, l = e - i * r;
+            a.f2[(size_t)kq * R2 + e] = s * ph_sm[l * r + i];
+        }
+    }
+}
+
+static int launch_ph_unpack(acse_ctx* c, int sW) {
+    const int r = c->r;
+    Work& w = c->w;
+    PhUnpack a;
+    a.V1 = w.V1;
+    a.V2 = w.V2;
+    a.f1 = w.V5f1;
+    a.V = w.V5d;
+    a.f2 = w.V5f2;
+    a.r = r;
+    a.s = sW;
+    k_ph_unpack<<<r * (r + 1) + r * r, 256, 2 * (size_t)r * r * sizeof(double), c->stream>>>(a);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// ------------------------------------------------------------------------ same-spin pairs
+// Same-spin pair GEMMs on packed pairs (as on the split path): in the aa and bb sectors the rows (ij),
+// the columns (kp) and the contraction (rs) of [M; D] W^T are antisymmetric pairs, so those GEMMs run
+// on pairs i < j only (P = r(r-1)/2; alpha 2 for the halved (rs) sum) and k_pair_unpack rebuilds the
+// full X and Y rows by antisymmetry (pairs numbered by pk_pair).
+//
+// X_s, Y_s (s = aa, bb; r^2 x r^2 FP64) from the packed [X; Y] (2P x P): one block per output row, the
+// packed source row staged in shared memory, the full row written two columns at a time.
+__global__ void __launch_bounds__(256) k_pair_unpack(int r, const double* __restrict__ Cp0, const double* __restrict__ Cp2,
+                                                   double* X0, double* Y0, double* X2, double* Y2) {
+    __shared__ double srow[ACSE_MAX_R * (ACSE_MAX_R - 1) / 2];
+    const int R2 = r * r, P = r * (r - 1) / 2;
+    const int sec = blockIdx.x / (2 * R2);
+    const int row = blockIdx.x - sec * 2 * R2;
+    const int part = row / R2, ij = row - part * R2, i = ij / r, j = ij - i * r;
+    double* dst = (sec == 0 ? (part ? Y0 : X0) : (part ? Y2 : X2)) + (size_t)ij * R2;
+    if (i == j) {   // block-uniform
+        for (int c = threadIdx.x; c < R2; c += blockDim.x) dst[c] = 0.0;
+        return;
+    }
+    const double si = i < j ? 1.0 : -1.0;
+    const double* src = (sec == 0 ? Cp0 : Cp2) + (size_t)(part * P + (i < j ? pk_pair(r, i, j) : pk_pair(r, j, i))) * P;
+    for (int e = threadIdx.x; e < P; e += blockDim.x) srow[e] = si * src[e];
+    __syncthreads();
+    auto val = [&](int k, int q) { return k == q ? 0.0 : (k < q ? srow[pk_pair(r, k, q)] : -srow[pk_pair(r, q, k)]); };
+    if ((R2 & 1) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+        for (int g = threadIdx.x; g < R2 / 2; g += blockDim.x) {
+            int k = (2 * g) / r, q = 2 * g - k * r;
+            const double v0 = val(k, q);
+            if (++q == r) { q = 0; ++k; }
+            reinterpret_cast<double2*>(dst)[g] = make_double2(v0, val(k, q));
+        }
+    } else {
+        for (int c = threadIdx.x; c < R2; c += blockDim.x) dst[c] = val(c / r, c - (c / r) * r);
+    }
+}
+
+int launch_pair_unpack(acse_ctx* c) {
+    Work& w = c->w;
+    k_pair_unpack<<<2 * 2 * c->r * c->r, 256, 0, c->stream>>>(c->r, w.Cp[0], w.Cp[1], w.X[0], w.Y[0], w.X[2], w.Y[2]);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// ------------------------------------------------------------------------------------- w
+// diag[slot][k][p][s], whose sum over p gives w (k_w_from_diag):
+//   slot 0: sum_q Waa[k][p][q][s] ga[p][q]    slot 1: sum_q Wbb[k][p][q][s] gb[p][q]
+//   slot 2: sum_q Wab[k][p][s][q] gb[p][q]    slot 3: sum_q Wab[p][k][q][s] ga[p][q]
+__global__ void __launch_bounds__(64) k_ph_w_diag(int r, const double* __restrict__ Waa, const double* __restrict__ Wab,
+                                                  const double* __restrict__ Wbb, const double* __restrict__ gam,
+                                                  double* __restrict__ diag) {
+    const int slot = (int)blockIdx.x / (r * r), kp = (int)blockIdx.x - slot * r * r, k = kp / r, p = kp - k * r;
+    const int s = threadIdx.x;
+    if (s >= r) return;
+    const size_t R2 = (size_t)r * r, r3 = R2 * r;
+    const double* g = gam + ((slot == 1 || slot == 2) ? R2 : 0) + (size_t)p * r;
+    const double* w = slot == 0 ? Waa + k * r3 + p * R2 : slot == 1 ? Wbb + k * r3 + p * R2
+                      : slot == 2 ? Wab + k * r3 + p * R2 + (size_t)s * r : Wab + p * r3 + k * R2;
+    double acc = 0.0;
+    if (slot == 2)
+        for (int q = 0; q < r; ++q) acc = fma(g[q], w[q], acc);
+    else
+        for (int q = 0; q < r; ++q) acc = fma(g[q], w[(size_t)q * r + s], acc);
+    diag[(size_t)blockIdx.x * r + s] = acc;
+}
+
+int launch_ph_w_diag(acse_ctx* c, const double* const W[3]) {
+    const int r = c->r;
+    k_ph_w_diag<<<4 * r * r, 64, 0, c->stream>>>(r, W[0], W[1], W[2], c->w.gam, c->w.zdiag);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// ------------------------------------------------------- transformation by 1D (CUDA cores)
+// out[(K,k,j)][(I,i,l)] = sum_q g_K[j][q] in[(K,k,q)][(I,i,l)] (trans: g_K[q][j]) for the six sectors t:
+// 0-3 the spin blocks (K, I) of the 2r^2 x 2r^2 array, 4 and 5 the two flips (1D of beta, of alpha).
+// Block (t, k, 64 columns): the columns' r rows and 1D sit in shared memory, each thread owns a 4 x 4 tile.
+// C: double on the FP64 path (bound by the DFMA pipe, 6 r^5), the double-float pair on the Ozaki path.
+#define PHT_COLS 64
+
+struct PhXform {
+    const double* in[3];   // spin blocks, flip 1, flip 2
+    double* out[3];
+    const double* gam;
+    int r, trans;
+};
+
+template <typename C>
+__global__ void __launch_bounds__(256) k_ph_xform(const __grid_constant__ PhXform a) {
+    extern __shared__ __align__(16) unsigned char ph_raw[];
+    const int r = a.r, rp = (r + 3) & ~3, R2 = r * r, nch = (R2 + PHT_COLS - 1) / PHT_COLS;
+    C* g = (C*)ph_raw;                      // [q][j], pitch rp
+    C* v = g + (size_t)r * rp;              // [q][64]
+    const int t = (int)blockIdx.x / (r * nch), rem = (int)blockIdx.x - t * r * nch, k = rem / nch;
+    const int c0 = (rem - k * nch) * PHT_COLS;
+    const int f = t < 4 ? 0 : t - 3, K = t < 4 ? t >> 1 : t == 4 ? 1 : 0;
+    const size_t ld = t < 4 ? 2 * (size_t)R2 : (size_t)R2;
+    const size_t base = (t < 4 ? (size_t)K * R2 * ld + (size_t)(t & 1) * R2 : 0) + (size_t)k * r * ld + c0;
+    const double* in = a.in[f] + base;
+    const double* gam = a.gam + (size_t)K * R2;
+    for (int e = threadIdx.x; e < r * rp; e += blockDim.x) {
+        const int q = e / rp, j = e - q * rp;
+        g[e] = tconv<C>(j < r ? (a.trans ? gam[q * r + j] : gam[j * r + q]) : 0.0);
+    }
+    for (int e = threadIdx.x; e < r * PHT_COLS; e += blockDim.x) {
+        const int q = e / PHT_COLS, c = e - q * PHT_COLS;
+        v[e] = tconv<C>(c0 + c < R2 ? in[(size_t)q * ld + c] : 0.0);
+    }
+    __syncthreads();
+    const int j0 = (threadIdx.x / (PHT_COLS / 4)) * 4, cc = (threadIdx.x % (PHT_COLS / 4)) * 4;
+    if (j0 >= r) return;
+    C acc[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) acc[u][x] = tconv<C>(0.0);
+#pragma unroll 2
+    for (int q = 0; q < r; ++q) {
+        C ga[4], vb[4];
+        ld4(g + (size_t)q * rp + j0, ga);
+        ld4(v + (size_t)q * PHT_COLS + cc, vb);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) tmac(acc[u][x], ga[u], vb[x]);
+    }
+    double* out = a.out[f] + base;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (j0 + u < r)
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (c0 + cc + x < R2) out[(size_t)(j0 + u) * ld + cc + x] = (double)acc[u][x];
+}
+
+static size_t ph_xform_smem(int r) { return (size_t)r * (((r + 3) & ~3) + PHT_COLS) * sizeof(double); }
+
+int launch_ph_xform(acse_ctx* c, const double* const in[3], double* const out[3], int trans) {
+    if (c->oz) {
+        const int s = launch_xform_oz(c, in, out, trans);
+        if (s != ACSE_ERR_UNSUPPORTED) return s;
+    }
+    const int r = c->r, nch = (r * r + PHT_COLS - 1) / PHT_COLS;
+    PhXform a;
+    for (int f = 0; f < 3; ++f) {
+        a.in[f] = in[f];
+        a.out[f] = out[f];
+    }
+    a.gam = c->w.gam;
+    a.r = r;
+    a.trans = trans;
+    const int threads = (((r + 3) / 4) * (PHT_COLS / 4) + 31) / 32 * 32;
+    if (c->oz) k_ph_xform<dfl><<<6 * r * nch, threads, ph_xform_smem(r), c->stream>>>(a);
+    else k_ph_xform<double><<<6 * r * nch, threads, ph_xform_smem(r), c->stream>>>(a);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// X5 of the pass from its products V1, V2 and V5f1.
+int launch_ph_finish(acse_ctx* c, int sW) {
+    Work& w = c->w;
+    ACSE_TRY(launch_ph_unpack(c, sW));
+    const double* in[3] = {w.V5d, w.V5f1, w.V5f2};
+    double* out[3] = {w.X5d, w.X5f1, w.X5f2};
+    return launch_ph_xform(c, in, out, 0);
+}
+
+int ph_set_attrs() {
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_ph_unpack, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double)));
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_ph_xform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)ph_xform_smem(ACSE_MAX_R)));
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_ph_xform<dfl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)ph_xform_smem(ACSE_MAX_R)));
+    return ACSE_OK;
+}

@@ -1,5 +1,5 @@
-// Shared-memory, register-tiled O(r^5) kernels of a contraction pass, for both arithmetic paths
-// (T = double for the FP64 path, T = float for the split-precision path).
+// Shared-memory, register-tiled O(r^5) kernels of a contraction pass: Z of the split path, and the B kernels
+// of both arithmetic paths (T = double for the FP64 path, T = float for the split-precision path).
 //
 //   Z^{kp}_{js} = sum_q W^{kp}_{qs} 1D^j_q  ->  for each (k, p): Z_kp = 1D . W_kp   (r x r x r)
 //   w^k_s = sum_pq W^{kp}_{qs} 1D^p_q = sum_p Z^{kp}_{ps}: the diagonal j = p of Z, so the Z kernel
@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "acse_internal.h"
+#include "dfloat.cuh"
 
 #define TL_TPB 256
 #define ZP_MAX_THREADS 288
@@ -26,68 +27,6 @@ __device__ __forceinline__ float tl_tf32(float x) {
 }
 
 __host__ __device__ __forceinline__ int pad4(int r) { return (r + 3) & ~3; }
-
-// 4 consecutive elements of a shared array (16-byte aligned: offsets are multiples of 4 elements).
-__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-}
-__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
-    const double2 x = *reinterpret_cast<const double2*>(p);
-    const double2 y = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-}
-
-// Double-float: an FP64 value carried as the unevaluated sum h + l of two floats (about 48 significant
-// bits).  The Ozaki path runs its O(r^5) products in it: FP32 arithmetic is many times faster than
-// FP64 on this GPU.  The all-zero bit pattern is 0.
-struct __align__(8) dfl {
-    float h, l;
-    __device__ __forceinline__ operator double() const { return (double)h + (double)l; }
-};
-// h = x rounded to the nearest float (ties to even), l = x - h rounded to the nearest float.  With integer
-// operations from the bit pattern where x is a normal double whose h and l are normal floats (the FP64
-// conversions run on the slow FP64 pipe); the same values through FP64 otherwise.
-__device__ __forceinline__ dfl to_dfl(double x) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
-    const int e = (int)((hi >> 20) & 0x7FFu);
-    if (e >= 949 && e <= 1149) {   // 2^(e - 1075) and h are normal floats
-        const unsigned sign = hi & 0x80000000u;
-        const unsigned m23 = ((hi & 0xFFFFFu) << 3) | (lo >> 29);    // the 23 fraction bits kept
-        const unsigned rem = lo & 0x1FFFFFFFu;                        // the 29 dropped ones
-        const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (m23 & 1u))) ? 1u : 0u;
-        const float h = __uint_as_float(sign | (((unsigned)(e - 1023 + 127) << 23) + m23 + up));
-        const int rr = up ? (int)rem - 0x20000000 : (int)rem;        // x - h in units of 2^(e - 1075)
-        const float scale = __uint_as_float((unsigned)(e - 1075 + 127) << 23);
-        const float l = __fmul_rn(__int2float_rn(sign ? -rr : rr), scale);
-        return dfl{h, l};
-    }
-    const float h = (float)x;
-    return dfl{h, (float)(x - (double)h)};   // x - h is exact in FP64
-}
-// acc += a b: the rounding error of the product by FMA (the l.l term is dropped), that of the sum by
-// Knuth's TwoSum; both go to acc.l.
-__device__ __forceinline__ void df_mac(dfl& acc, const dfl& a, const dfl& b) {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = fmaf(a.h, b.h, -p);
-    e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-    const float s = acc.h + p;
-    const float bb = s - acc.h;
-    const float t = (acc.h - (s - bb)) + (p - bb);
-    acc.h = s;
-    acc.l += t + e;
-}
-__device__ __forceinline__ void ld4(const dfl* p, dfl (&v)[4]) {
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    const float4 y = *reinterpret_cast<const float4*>(p + 2);
-    v[0] = dfl{x.x, x.y}; v[1] = dfl{x.z, x.w}; v[2] = dfl{y.x, y.y}; v[3] = dfl{y.z, y.w};
-}
-// conversions and multiply-add for the element types of the tiled kernels
-template <typename T> __device__ __forceinline__ T tconv(double x) { return (T)x; }
-template <> __device__ __forceinline__ dfl tconv<dfl>(double x) { return to_dfl(x); }
-template <typename T> __device__ __forceinline__ void tmac(T& acc, const T& a, const T& b) { acc += a * b; }
-template <> __device__ __forceinline__ void tmac<dfl>(dfl& acc, const dfl& a, const dfl& b) { df_mac(acc, a, b); }
 
 // acc[a][b] += sum_q A[q][i0 + a] * B[q][j0 + b]  (A, B: [rp][rp] shared arrays, rp % 4 == 0)
 template <typename T>
@@ -108,24 +47,21 @@ __device__ __forceinline__ void mma4x4(T (&acc)[4][4], const T* A, const T* B, i
 struct ZOut {
     void* Zd;      // (2 r^2) rows
     void* Zf[2];   // r^2 rows
-    int mode;      // 0 = FP64, 1 = BF16x3 (A pattern [hi|hi|lo]), 2 = TF32, 3 = TF32x3 ([hi|hi|lo])
+    int mode;      // 1 = BF16x3 (A pattern [hi|hi|lo]), 2 = TF32, 3 = TF32x3 ([hi|hi|lo])
     int ldd, ldf;  // row length in elements
-    int Kp1, Kp2;  // K segment length (split modes)
+    int Kp1, Kp2;  // K segment length
     void* diag;    // [4][r][r][r]: rows j = p of Zd(a,a), Zd(b,b), Zf1, Zf2
     int ntypes;    // spin types computed (6, or 3 with the spin-flip specialisation) ...
     int tmap[6];   // ... and which: block type index -> t
 };
 
-template <typename T>
-__device__ __forceinline__ void z_store(const ZOut& o, int which, size_t row, int col, T v) {
+__device__ __forceinline__ void z_store(const ZOut& o, int which, size_t row, int col, float v) {
     void* base = which < 0 ? o.Zd : o.Zf[which];
     const size_t ld = which < 0 ? (size_t)o.ldd : (size_t)o.ldf;
     const int Kp = which < 0 ? o.Kp2 : o.Kp1;
-    if (o.mode == 0) {
-        ((double*)base)[row * ld + col] = (double)v;
-    } else if (o.mode == 1) {
+    if (o.mode == 1) {
         __nv_bfloat16* p = (__nv_bfloat16*)base + row * ld;
-        const float x = (float)v;
+        const float x = v;
         const __nv_bfloat16 hi = __float2bfloat16_rn(x);
         const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
         p[col] = hi;
@@ -133,33 +69,29 @@ __device__ __forceinline__ void z_store(const ZOut& o, int which, size_t row, in
         p[2 * Kp + col] = lo;
     } else if (o.mode == 3) {
         float* p = (float*)base + row * ld;
-        const float hi = tl_tf32((float)v);
-        const float lo = tl_tf32((float)v - hi);
+        const float hi = tl_tf32(v);
+        const float lo = tl_tf32(v - hi);
         p[col] = hi;
         p[Kp + col] = hi;
         p[2 * Kp + col] = lo;
     } else {
-        ((float*)base + row * ld)[col] = tl_tf32((float)v);
+        ((float*)base + row * ld)[col] = tl_tf32(v);
     }
 }
 
 // Four consecutive columns col..col+3 of one output row (requires row * ld + col % 4 == 0); MODE is
 // the ZOut mode.
-template <int MODE, typename T>
-__device__ __forceinline__ void z_store4(const ZOut& o, int which, size_t row, int col, const T (&v)[4]) {
+template <int MODE>
+__device__ __forceinline__ void z_store4(const ZOut& o, int which, size_t row, int col, const float (&v)[4]) {
     void* base = which < 0 ? o.Zd : o.Zf[which];
     const size_t ld = which < 0 ? (size_t)o.ldd : (size_t)o.ldf;
     const int Kp = which < 0 ? o.Kp2 : o.Kp1;
-    if (MODE == 0 || MODE == 4) {
-        double* q = (double*)base + row * ld + col;
-        *reinterpret_cast<double2*>(q) = make_double2((double)v[0], (double)v[1]);
-        *reinterpret_cast<double2*>(q + 2) = make_double2((double)v[2], (double)v[3]);
-    } else if (MODE == 1) {
+    if (MODE == 1) {
         __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            hi[u] = __float2bfloat16_rn((float)v[u]);
-            lo[u] = __float2bfloat16_rn((float)v[u] - __bfloat162float(hi[u]));
+            hi[u] = __float2bfloat16_rn(v[u]);
+            lo[u] = __float2bfloat16_rn(v[u] - __bfloat162float(hi[u]));
         }
         uint2 H, L;
         memcpy(&H, hi, 8);
@@ -172,8 +104,8 @@ __device__ __forceinline__ void z_store4(const ZOut& o, int which, size_t row, i
         float hi[4], lo[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            hi[u] = tl_tf32((float)v[u]);
-            lo[u] = tl_tf32((float)v[u] - hi[u]);
+            hi[u] = tl_tf32(v[u]);
+            lo[u] = tl_tf32(v[u] - hi[u]);
         }
         float* q = (float*)base + row * ld + col;
         *reinterpret_cast<float4*>(q) = make_float4(hi[0], hi[1], hi[2], hi[3]);
@@ -182,7 +114,7 @@ __device__ __forceinline__ void z_store4(const ZOut& o, int which, size_t row, i
     } else {
         float* q = (float*)base + row * ld + col;
         *reinterpret_cast<float4*>(q) =
-            make_float4(tl_tf32((float)v[0]), tl_tf32((float)v[1]), tl_tf32((float)v[2]), tl_tf32((float)v[3]));
+            make_float4(tl_tf32(v[0]), tl_tf32(v[1]), tl_tf32(v[2]), tl_tf32(v[3]));
     }
 }
 
@@ -195,17 +127,12 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // The r x r slice W_kp[q][s] of spin type t (t = 0..5, see k_Z_pipe) and whether it is stored [s][q].
-template <typename WT>
-__device__ __forceinline__ const WT* z_slice(int t, int k, int p, int r, const WT* Waa, const WT* Wab, const WT* Wbb,
-                                             bool& transposed) {
+__device__ __forceinline__ const float* z_slice(int t, int k, int p, int r, const float* Waa, const float* Wab,
+                                                const float* Wbb, bool& transposed) {
     const size_t r3 = (size_t)r * r * r, R2 = (size_t)r * r;
     switch (t) {
         case 0: transposed = false; return Waa + k * r3 + p * R2;
@@ -223,27 +150,21 @@ __device__ __forceinline__ const WT* z_slice(int t, int k, int p, int r, const W
 //   t=4 Zf1:     W_kp[q][s] = Wab[k][p][s][q], gb      t=5 Zf2:     Wab[p][k][q][s], ga
 // (the spin-flip sectors drop a sign -1 that their M operand drops too).  The W slices of the next ipb
 // values of p are copied into shared memory (cp.async) while the current ipb slices are multiplied;
-// each thread owns one 4 x 4 output tile of one slice (ipb * (rp/4)^2 threads).  W is FP64 on the FP64
-// paths (MODE 0, and MODE 4, the Ozaki path: FP64 output as MODE 0, products in double-float) and the
-// FP32 copy of W on the split path (MODE 1-3), so that no FP64 conversion runs here.
-template <int MODE>
-using ZWT = typename std::conditional<MODE == 0 || MODE == 4, double, float>::type;
-
+// each thread owns one 4 x 4 output tile of one slice (ipb * (rp/4)^2 threads).  W is its FP32 copy, so that
+// no FP64 conversion runs here (split path; the FP64-accurate paths transform after the product, acse_ph.cu).
 template <int MODE, int RP = 0>   // RP > 0: compile-time padded size (product loop fully unrolled)
-__global__ void __launch_bounds__(ZP_MAX_THREADS, (MODE == 0 || MODE == 4) ? 2 : 3) k_Z_pipe(int r, int ipb, int pchunk, const ZWT<MODE>* __restrict__ Waa,
-                                                         const ZWT<MODE>* __restrict__ Wab,
-                                                         const ZWT<MODE>* __restrict__ Wbb,
-                                                         const double* __restrict__ gam, const __grid_constant__ ZOut o) {
-    using T = typename std::conditional<MODE == 0, double,
-                                        typename std::conditional<MODE == 4, dfl, float>::type>::type;
-    using WT = ZWT<MODE>;
-    constexpr int WV = 16 / sizeof(WT);                  // elements of a 16-byte copy
+__global__ void __launch_bounds__(ZP_MAX_THREADS, 3) k_Z_pipe(int r, int ipb, int pchunk, const float* __restrict__ Waa,
+                                                              const float* __restrict__ Wab,
+                                                              const float* __restrict__ Wbb,
+                                                              const double* __restrict__ gam,
+                                                              const __grid_constant__ ZOut o) {
+    constexpr int WV = 4;                                // elements of a 16-byte copy
     extern __shared__ __align__(16) unsigned char tl_smem[];
     const int rp = RP ? RP : pad4(r), ldw = rp + 4, R2 = r * r, R2e = (R2 + WV - 1) / WV * WV;
     const int nt = rp / 4, nt2 = nt * nt;
-    WT* stage = (WT*)tl_smem;                            // [ipb][R2e] raw W slices
-    T* gT = (T*)(stage + (size_t)ipb * R2e);             // [q][j] = 1D[j][q], row pitch ldw
-    T* Ws = gT + (size_t)rp * ldw;                       // [ipb][q][s], row pitch ldw
+    float* stage = (float*)tl_smem;                            // [ipb][R2e] raw W slices
+    float* gT = (float*)(stage + (size_t)ipb * R2e);             // [q][j] = 1D[j][q], row pitch ldw
+    float* Ws = gT + (size_t)rp * ldw;                       // [ipb][q][s], row pitch ldw
     const int nchunk = (r + pchunk - 1) / pchunk;
     const int tb = blockIdx.x / (r * nchunk);
     const int t = o.tmap[tb];
@@ -256,22 +177,20 @@ __global__ void __launch_bounds__(ZP_MAX_THREADS, (MODE == 0 || MODE == 4) ? 2 :
     const float invr = 1.f / (float)r;
     const bool vec_ld = R2 % WV == 0 && ((reinterpret_cast<uintptr_t>(Waa) | reinterpret_cast<uintptr_t>(Wab) |
                                           reinterpret_cast<uintptr_t>(Wbb)) & 15) == 0;
-    for (int e = threadIdx.x; e < (1 + ipb) * rp * ldw; e += blockDim.x) gT[e] = tconv<T>(0.0);
+    for (int e = threadIdx.x; e < (1 + ipb) * rp * ldw; e += blockDim.x) gT[e] = 0.f;
     __syncthreads();
     for (int e = threadIdx.x; e < R2; e += blockDim.x) {
         const int u = e / r, v = e - u * r;
-        gT[v * ldw + u] = tconv<T>(g[e]);                // g[j][q] -> gT[q][j]
+        gT[v * ldw + u] = (float)g[e];                // g[j][q] -> gT[q][j]
     }
     auto issue = [&](int p0) {
         const int n = min(ipb, pe - p0);
         for (int it = 0; it < n; ++it) {
             bool tr;
-            const WT* src = z_slice<WT>(t, k, p0 + it, r, Waa, Wab, Wbb, tr);
-            WT* dst = stage + (size_t)it * R2e;
+            const float* src = z_slice(t, k, p0 + it, r, Waa, Wab, Wbb, tr);
+            float* dst = stage + (size_t)it * R2e;
             if (vec_ld)
                 for (int e = threadIdx.x; e < R2 / WV; e += blockDim.x) cp_async16(dst + WV * e, src + WV * e);
-            else if (sizeof(WT) == 8)
-                for (int e = threadIdx.x; e < R2; e += blockDim.x) cp_async8(dst + e, src + e);
             else
                 for (int e = threadIdx.x; e < R2; e += blockDim.x) cp_async4(dst + e, src + e);
         }
@@ -291,14 +210,12 @@ __global__ void __launch_bounds__(ZP_MAX_THREADS, (MODE == 0 || MODE == 4) ? 2 :
         __syncthreads();                                 // slices landed; previous products done with Ws
         for (int it = 0; it < n; ++it) {
             bool tr;
-            z_slice<WT>(t, k, p0 + it, r, Waa, Wab, Wbb, tr);
-            const WT* st = stage + (size_t)it * R2e;
-            T* W = Ws + (size_t)it * rp * ldw;
+            z_slice(t, k, p0 + it, r, Waa, Wab, Wbb, tr);
+            const float* st = stage + (size_t)it * R2e;
+            float* W = Ws + (size_t)it * rp * ldw;
             for (int e = threadIdx.x; e < R2; e += blockDim.x) {
                 const int u = (int)(((float)e + 0.5f) * invr), v = e - u * r;   // e / r, see invr
-                T x;
-                if constexpr (std::is_same<T, WT>::value) x = st[e];   // FP32 W on the split path
-                else x = tconv<T>((double)st[e]);
+                const float x = st[e];
                 if (tr) W[v * ldw + u] = x;                // src[s][q] -> W[q][s]
                 else W[u * ldw + v] = x;
             }
@@ -307,46 +224,29 @@ __global__ void __launch_bounds__(ZP_MAX_THREADS, (MODE == 0 || MODE == 4) ? 2 :
         if (p0 + ipb < pe) issue(p0 + ipb);              // the next slices load during the products
         if (it_me >= n) continue;
         const int p = p0 + it_me;
-        T acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = tconv<T>(0.0);
-        const T* W = Ws + (size_t)it_me * rp * ldw;
+        float acc[4][4];
+        const float* W = Ws + (size_t)it_me * rp * ldw;
         // with RP the loop runs over the zero-padded rows too (q < RP), at a constant trip count
-        if constexpr (std::is_same<T, float>::value) {
-            // packed FP32x2 FMA, pairs along s (the same FMA sequence per element as scalar code)
-            float2 c2[4][2];
+        // packed FP32x2 FMA, pairs along s (the same FMA sequence per element as scalar code)
+        float2 c2[4][2];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) c2[u][0] = c2[u][1] = make_float2(0.f, 0.f);
+        for (int u = 0; u < 4; ++u) c2[u][0] = c2[u][1] = make_float2(0.f, 0.f);
 #pragma unroll 4
-            for (int q = 0; q < (RP ? RP : r); ++q) {
-                float a[4], b[4];
-                ld4(gT + q * ldw + j0, a);
-                ld4(W + q * ldw + s0, b);
-                const float2 b0 = make_float2(b[0], b[1]), b1 = make_float2(b[2], b[3]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float2 x = make_float2(a[u], a[u]);
-                    c2[u][0] = __ffma2_rn(x, b0, c2[u][0]);
-                    c2[u][1] = __ffma2_rn(x, b1, c2[u][1]);
-                }
-            }
+        for (int q = 0; q < (RP ? RP : r); ++q) {
+            float a[4], b[4];
+            ld4(gT + q * ldw + j0, a);
+            ld4(W + q * ldw + s0, b);
+            const float2 b0 = make_float2(b[0], b[1]), b1 = make_float2(b[2], b[3]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                acc[u][0] = c2[u][0].x; acc[u][1] = c2[u][0].y; acc[u][2] = c2[u][1].x; acc[u][3] = c2[u][1].y;
+                const float2 x = make_float2(a[u], a[u]);
+                c2[u][0] = __ffma2_rn(x, b0, c2[u][0]);
+                c2[u][1] = __ffma2_rn(x, b1, c2[u][1]);
             }
-        } else {
-#pragma unroll 4
-            for (int q = 0; q < (RP ? RP : r); ++q) {
-                T a[4], b[4];
-                ld4(gT + q * ldw + j0, a);
-                ld4(W + q * ldw + s0, b);
+        }
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) tmac(acc[u][v], a[u], b[v]);
-            }
+        for (int u = 0; u < 4; ++u) {
+            acc[u][0] = c2[u][0].x; acc[u][1] = c2[u][0].y; acc[u][2] = c2[u][1].x; acc[u][3] = c2[u][1].y;
         }
         const int col0 = sP * R2 + p * r + s0;
         const bool vec_st = s0 + 3 < r && ((size_t)col0 & 3) == 0 && (ld & 3) == 0;
@@ -355,18 +255,17 @@ __global__ void __launch_bounds__(ZP_MAX_THREADS, (MODE == 0 || MODE == 4) ? 2 :
             const int j = j0 + u;
             if (j >= r) continue;
             const size_t row = (size_t)sK * R2 + (size_t)k * r + j;
-            if (vec_st) z_store4<MODE, T>(o, which, row, col0, acc[u]);
+            if (vec_st) z_store4<MODE>(o, which, row, col0, acc[u]);
             else
 #pragma unroll
                 for (int v = 0; v < 4; ++v)
-                    if (s0 + v < r) z_store<T>(o, which, row, col0 + v, acc[u][v]);
+                    if (s0 + v < r) z_store(o, which, row, col0 + v, acc[u][v]);
             if (dslot >= 0 && j == p)
 #pragma unroll
                 for (int v = 0; v < 4; ++v)
                     if (s0 + v < r) {
                         const size_t di = ((size_t)dslot * R2 + (size_t)k * r + p) * r + s0 + v;
-                        if (MODE == 4) ((double*)o.diag)[di] = (double)acc[u][v];
-                        else ((T*)o.diag)[di] = acc[u][v];
+                        ((float*)o.diag)[di] = acc[u][v];
                     }
         }
     }
@@ -992,16 +891,15 @@ struct ZPlan {
     int ipb, threads, pchunk, blocks;
     size_t smem;
 };
-static ZPlan z_plan_compute(int r, size_t es, size_t ws, const void* kern) {   // es: tile, ws: W element bytes
+static ZPlan z_plan_compute(int r, const void* kern) {
     ZPlan z;
     const int rp = pad4(r), nt = rp / 4, nt2 = nt * nt;
     z.ipb = ZP_MAX_THREADS / nt2;
     if (z.ipb > 4) z.ipb = 4;
     if (z.ipb < 1) z.ipb = 1;
     z.threads = (z.ipb * nt2 + 31) / 32 * 32;
-    const int wv = (int)(16 / ws);
-    const int R2e = (r * r + wv - 1) / wv * wv;
-    z.smem = (size_t)z.ipb * R2e * ws + (size_t)(1 + z.ipb) * rp * (rp + 4) * es;
+    const int R2e = (r * r + 3) / 4 * 4;
+    z.smem = ((size_t)z.ipb * R2e + (size_t)(1 + z.ipb) * rp * (rp + 4)) * sizeof(float);
     int per_sm = 1, nsm = 152, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, z.threads, z.smem) != cudaSuccess || per_sm < 1) {
@@ -1021,18 +919,18 @@ static ZPlan z_plan_compute(int r, size_t es, size_t ws, const void* kern) {   /
 }
 
 // cached per host thread, output mode and r (the occupancy query is not free)
-static ZPlan z_plan(int r, int mode, size_t es, const void* kern) {
-    static thread_local int cached_r[5] = {-1, -1, -1, -1, -1};
-    static thread_local ZPlan cached[5];
+static ZPlan z_plan(int r, int mode, const void* kern) {
+    static thread_local int cached_r[4] = {-1, -1, -1, -1};
+    static thread_local ZPlan cached[4];
     if (cached_r[mode] != r) {
-        cached[mode] = z_plan_compute(r, es, (mode == 0 || mode == 4) ? sizeof(double) : sizeof(float), kern);
+        cached[mode] = z_plan_compute(r, kern);
         cached_r[mode] = r;
     }
     return cached[mode];
 }
 
-// W: the FP64 operand (FP64 and Ozaki paths); W32: its FP32 copy (split path).
-int launch_Z_tiled(acse_ctx* c, const double* const W[3], const float* const W32[3]) {
+// Z of the split path from the FP32 copy of W.
+int launch_Z_tiled(acse_ctx* c, const float* const W32[3]) {
     const int r = c->r;
     ZOut o;
     Work& w = c->w;
@@ -1043,53 +941,39 @@ int launch_Z_tiled(acse_ctx* c, const double* const W[3], const float* const W32
     o.ntypes = sf ? 3 : 6;
     const int tm_sf[6] = {0, 1, 4, 0, 0, 0};
     for (int k = 0; k < 6; ++k) o.tmap[k] = sf ? tm_sf[k] : k;
-    if (c->opt.prec == ACSE_FP64) {
-        o.Zd = w.Zd; o.Zf[0] = w.Zf1; o.Zf[1] = w.Zf2;
-        o.mode = 0; o.ldd = 2 * R2; o.ldf = R2; o.Kp1 = o.Kp2 = 0; o.diag = w.zdiag;
-        if (c->oz) {   // Ozaki path: the products on the tensor cores (acse_zoz.cu), else in double-float
-            const int zs = launch_Z_oz(c, W, o.ntypes, o.tmap);
-            if (zs == ACSE_OK) {
-                k_w_from_diag<double><<<2 * r, 256, 0, c->stream>>>(r, w.zdiag, w.w, 0);
-                ACSE_LAUNCHED(c);
-                return ACSE_OK;
-            }
-            if (zs != ACSE_ERR_UNSUPPORTED) return zs;
-            const ZPlan zp = z_plan(r, 4, sizeof(double), (const void*)k_Z_pipe<4>);
-            k_Z_pipe<4><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W[0], W[1], W[2], w.gam, o);
-        } else {
-            const ZPlan zp = z_plan(r, 0, sizeof(double), (const void*)k_Z_pipe<0>);
-            k_Z_pipe<0><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W[0], W[1], W[2], w.gam, o);
-        }
-        ACSE_LAUNCHED(c);
-        k_w_from_diag<double><<<2 * r, 256, 0, c->stream>>>(r, w.zdiag, w.w, 0);
-    } else {
-        o.Zd = w.tc_Zd; o.Zf[0] = w.tc_Zf[0]; o.Zf[1] = w.tc_Zf[1];
-        o.mode = c->opt.prec == ACSE_BF16X3 ? 1 : (c->opt.prec == ACSE_TF32X3 ? 3 : 2);
-        o.ldd = c->nsplit * w.Kp2; o.ldf = c->nsplit * w.Kp1; o.Kp1 = w.Kp1; o.Kp2 = w.Kp2; o.diag = w.zdiag32;
-        // BF16x3 with r a multiple of 16: the products on the tensor cores (acse_ztc.cu)
-        const int zs = launch_Z_tc(c, W32, o.ntypes, o.tmap);
-        if (zs == ACSE_OK) {
-            k_w_from_diag<float><<<2 * r, 256, 0, c->stream>>>(r, w.zdiag32, w.w32, sf ? 1 : 0);
-            ACSE_LAUNCHED(c);
-            return ACSE_OK;
-        }
-        if (zs != ACSE_ERR_UNSUPPORTED) return zs;
-        const bool r48 = o.mode == 1 && pad4(r) == 48;
-        const void* kern = r48 ? (const void*)k_Z_pipe<1, 48>
-                               : o.mode == 1 ? (const void*)k_Z_pipe<1> : o.mode == 3 ? (const void*)k_Z_pipe<3>
-                                                                                      : (const void*)k_Z_pipe<2>;
-        const ZPlan zp = z_plan(r, o.mode, sizeof(float), kern);
-        if (r48)
-            k_Z_pipe<1, 48><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
-        else if (o.mode == 1)
-            k_Z_pipe<1><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
-        else if (o.mode == 3)
-            k_Z_pipe<3><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
-        else
-            k_Z_pipe<2><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
-        ACSE_LAUNCHED(c);
+    o.Zd = w.tc_Zd; o.Zf[0] = w.tc_Zf[0]; o.Zf[1] = w.tc_Zf[1];
+    o.mode = c->opt.prec == ACSE_BF16X3 ? 1 : (c->opt.prec == ACSE_TF32X3 ? 3 : 2);
+    o.ldd = c->nsplit * w.Kp2; o.ldf = c->nsplit * w.Kp1; o.Kp1 = w.Kp1; o.Kp2 = w.Kp2; o.diag = w.zdiag32;
+    // BF16x3 with r a multiple of 16: the products on the tensor cores (acse_ztc.cu)
+    const int zs = launch_Z_tc(c, W32, o.ntypes, o.tmap);
+    if (zs == ACSE_OK) {
         k_w_from_diag<float><<<2 * r, 256, 0, c->stream>>>(r, w.zdiag32, w.w32, sf ? 1 : 0);
+        ACSE_LAUNCHED(c);
+        return ACSE_OK;
     }
+    if (zs != ACSE_ERR_UNSUPPORTED) return zs;
+    const bool r48 = o.mode == 1 && pad4(r) == 48;
+    const void* kern = r48 ? (const void*)k_Z_pipe<1, 48>
+                           : o.mode == 1 ? (const void*)k_Z_pipe<1> : o.mode == 3 ? (const void*)k_Z_pipe<3>
+                                                                                  : (const void*)k_Z_pipe<2>;
+    const ZPlan zp = z_plan(r, o.mode, kern);
+    if (r48)
+        k_Z_pipe<1, 48><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
+    else if (o.mode == 1)
+        k_Z_pipe<1><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
+    else if (o.mode == 3)
+        k_Z_pipe<3><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
+    else
+        k_Z_pipe<2><<<zp.blocks / 6 * o.ntypes, zp.threads, zp.smem, c->stream>>>(r, zp.ipb, zp.pchunk, W32[0], W32[1], W32[2], w.gam, o);
+    ACSE_LAUNCHED(c);
+    k_w_from_diag<float><<<2 * r, 256, 0, c->stream>>>(r, w.zdiag32, w.w32, sf ? 1 : 0);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// w of the FP64 and Ozaki paths from the terms of k_ph_w_diag.
+int launch_w_sum(acse_ctx* c) {
+    k_w_from_diag<double><<<2 * c->r, 256, 0, c->stream>>>(c->r, c->w.zdiag, c->w.w, 0);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -1212,14 +1096,12 @@ int tiled_set_attrs() {
                                        (int)b_smem(ACSE_MAX_R, sizeof(double), false)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_tiled<double, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)b_smem(ACSE_MAX_R, sizeof(double), false)));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_pipe<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k_smem_cap));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pipe<320, 2, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bp_smem(48)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pipe<320, 2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bp_smem(48)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pipe<BP_MAX_THREADS, 1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bp_smem(ACSE_MAX_R)));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_pipe<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k_smem_cap));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_pipe<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k_smem_cap));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_pipe<1, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k_smem_cap));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_pipe<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k_smem_cap));

@@ -1,10 +1,10 @@
-// Z = 1D . W_kp on the tensor cores in an FP64-accurate (Ozaki) context: the O(r^5) particle-hole operand
-// of a contraction pass, Z^{kp}_{js} = sum_q W^{kp}_{qs} 1D^j_q, by the error-free splitting of the Ozaki
-// scheme (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012) that gemm_oz.cu applies to the O(r^6)
-// GEMMs, instead of double-float FMAs on the CUDA cores.
+// The transformation of the particle-hole product by 1D on the tensor cores in an FP64-accurate (Ozaki)
+// context, X5[(k,j)][m] = sum_q 1D^j_q V5[(k,q)][m] (acse_ph.cu), by the error-free splitting of the Ozaki
+// scheme (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012) instead of double-float FMAs on the CUDA
+// cores; and the B products below.
 //
-// Tile: 128 consecutive (p, s) of one (spin type, k), rows m = p r + s, as in acse_ztc.cu:
-//     Z[m][j] = sum_q A[m][q] B[j][q],   A[m][q] = W_kp[q][s] (FP64),  B[j][q] = 1D[j][q] (FP64).
+// Tile: 128 consecutive columns m of one (sector, k):
+//     out[(k,j)][m] = sum_q A[m][q] B[j][q],   A[m][q] = V5[(k,q)][m] (FP64),  B[j][q] = 1D[j][q] (FP64).
 // Every row of A and of B gets a power-of-two scale 2^e (|x| 2^-e < 1/2 over the row) and each element the
 // fixed-point value X = round(x 2^(6S - e)), cut into S balanced base-64 digits (most significant first,
 // each exact in bf16).  The digit tiles A_s, B_t sit in shared memory in the 128-byte-swizzled K-major
@@ -19,9 +19,9 @@
 // range of tiles; the B tiles are rebuilt only when the spin of the tile's 1D changes.  Producer: four
 // threads per A row (partners in one warp share the row maximum); one thread issues the MMAs; epilogue:
 // each warp reads its TMEM lane quarter (one row m per thread) for a quarter of the columns j and writes the
-// FP64 rows of Zd / Zf (row (sK, k, j), column (sP, p, s)) and the diagonal rows j = p of w.  The wait for
+// output rows (consecutive m, coalesced).  The wait for
 // the MMAs is bounded; on expiry the kernel raises the device flag and stops.  Used for r a multiple of
-// 16 (r <= 64) and S <= 8; other cases take the double-float kernel of acse_tiled.cu.
+// 16 (r <= 64) and S <= 8; other cases take the double-float kernels of acse_ph.cu and acse_tiled.cu.
 #include <cuda_bf16.h>
 
 #include "acse_internal.h"
@@ -35,13 +35,10 @@
 #define ZOZ_WAIT_NS 4000000000ull
 
 struct ZozArgs {
-    const double* W[3];     // FP64 W blocks aa, ab, bb (r^4 each)
+    const double* in[3];    // spin blocks (2r^2 x 2r^2), flip 1, flip 2 (r^2 x r^2)
+    double* out[3];
     const double* gam;      // 1D per spin [2][r][r]
-    double* Zd;             // (2 r^2) rows of ldd doubles
-    double* Zf[2];          // r^2 rows of ldf doubles
-    double* diag;           // [4][r][r][r]: rows j = p of Zd(a,a), Zd(b,b), Zf1, Zf2
-    int ldd, ldf;
-    int tmap[6];            // block type index -> spin type t
+    int trans;              // transform by the transpose of 1D
     int S;                  // slices (<= ZOZ_SMAX)
     int* err;
 };
@@ -97,7 +94,7 @@ static __device__ __forceinline__ void zoz_tmem_ld4(uint32_t taddr, uint32_t (&v
 }
 
 template <int R>
-__global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__ ZozArgs a, int ntiles) {
+__global__ void __launch_bounds__(ZOZ_THREADS, 1) k_xform_oz(const __grid_constant__ ZozArgs a, int ntiles) {
     static_assert(R % 16 == 0 && R <= 64, "N = r a multiple of 16, K = r within one 64-element block");
     constexpr int R2 = R * R, NT = R2 / TC_BM, NCH = R / 8;   // 16-byte chunks of a digit row
     static_assert(R2 % TC_BM == 0, "whole tiles");
@@ -114,7 +111,6 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const size_t r3 = (size_t)R * R2;
     if (threadIdx.x < 65) tab[threadIdx.x] = __bfloat16_as_ushort(__float2bfloat16_rn((float)((int)threadIdx.x - 32)));
     // the K padding q >= R of every digit tile stays zero
     for (int e = threadIdx.x; e < (ZOZ_SMAX * ZOZ_A_SLICE + ZOZ_SMAX * B_SLICE) / 16; e += ZOZ_THREADS)
@@ -134,17 +130,19 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
     const int per = (ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
     const int t_end = min(ntiles, ((int)blockIdx.x + 1) * per);
     for (int tile = (int)blockIdx.x * per; tile < t_end && ok; ++tile, phase ^= 1) {
-        const int tb = tile / (R * NT);
-        const int t = a.tmap[tb];
-        const int rem = tile - tb * R * NT;
+        const int t = tile / (R * NT);   // sector: spin blocks (K, I) 0-3, the flips 4 and 5
+        const int rem = tile - t * R * NT;
         const int k = rem / NT;
         const int m0 = (rem - k * NT) * TC_BM;
-        const int sp = (t == 2 || t == 3 || t == 4) ? 1 : 0;
+        const int f = t < 4 ? 0 : t - 3, sp = t < 4 ? t >> 1 : t == 4 ? 1 : 0;
+        const size_t ld = t < 4 ? 2 * (size_t)R2 : (size_t)R2;
+        const size_t base = (t < 4 ? (size_t)sp * R2 * ld + (size_t)(t & 1) * R2 : 0) + (size_t)k * R * ld;
         if (sp != cur_sp) {   // B: the digits of 1D of this tile's spin, rows j, K = q (the last MMAs are done)
             const unsigned long long* g = reinterpret_cast<const unsigned long long*>(a.gam + (size_t)sp * R2);
+            const int gj = a.trans ? 1 : R, gq = a.trans ? R : 1;   // B[j][q] = 1D[j][q], or 1D[q][j]
             for (int j = threadIdx.x; j < R; j += ZOZ_THREADS) {
                 unsigned long long mx = 0;
-                for (int q = 0; q < R; ++q) mx = max(mx, g[j * R + q] & 0x7FFFFFFFFFFFFFFFull);
+                for (int q = 0; q < R; ++q) mx = max(mx, g[j * gj + q * gq] & 0x7FFFFFFFFFFFFFFFull);
                 eB[j] = zoz_row_exp(mx);
             }
             __syncthreads();
@@ -152,26 +150,15 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
                 const int j = e / NCH, c = e - j * NCH;
                 unsigned long long x[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = g[j * R + 8 * c + u];
+                for (int u = 0; u < 8; ++u) x[u] = g[j * gj + (8 * c + u) * gq];
                 zoz_digits8(x, eB[j], S, sB, B_SLICE, zoz_sw128(j, c), tab);
             }
             cur_sp = sp;
         }
-        // A: row m = p r + s of W_k^T, K = q: W_kp[q][s] of type t (see k_Z_pipe); ZOZ_TPR threads per row
+        // A: row m (a column of the sector), K = q: in[(k, q)][m]; ZOZ_TPR threads per row
         {
-            const int ml = threadIdx.x / ZOZ_TPR, half = threadIdx.x % ZOZ_TPR, m = m0 + ml;
-            const int p = m / R, s = m - p * R;
-            const double* base;
-            bool tr;
-            switch (t) {
-                case 0: tr = false; base = a.W[0] + k * r3 + (size_t)p * R2; break;
-                case 1: tr = false; base = a.W[1] + k * r3 + (size_t)p * R2; break;
-                case 2: tr = true; base = a.W[1] + (size_t)p * r3 + (size_t)k * R2; break;
-                case 3: tr = false; base = a.W[2] + k * r3 + (size_t)p * R2; break;
-                case 4: tr = true; base = a.W[1] + k * r3 + (size_t)p * R2; break;
-                default: tr = false; base = a.W[1] + (size_t)p * r3 + (size_t)k * R2; break;
-            }
-            const unsigned long long* b64 = reinterpret_cast<const unsigned long long*>(base);
+            const int ml = threadIdx.x / ZOZ_TPR, half = threadIdx.x % ZOZ_TPR;
+            const unsigned long long* b64 = reinterpret_cast<const unsigned long long*>(a.in[f] + base + m0 + ml);
             constexpr int MYCH = (NCH + ZOZ_TPR - 1) / ZOZ_TPR;   // chunks c = half, half + TPR, ... of this thread
             unsigned long long x[MYCH][8];
             unsigned long long mx = 0;
@@ -181,7 +168,7 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int q = 8 * c + u;
-                    x[i][u] = c < NCH ? (tr ? b64[(size_t)s * R + q] : b64[(size_t)q * R + s]) : 0ull;
+                    x[i][u] = c < NCH ? b64[(size_t)q * ld] : 0ull;
                     mx = max(mx, x[i][u] & 0x7FFFFFFFFFFFFFFFull);
                 }
             }
@@ -224,16 +211,9 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
             constexpr int NJG = ZOZ_THREADS / 128, JW = R / NJG;   // warps per lane quarter, columns each
             static_assert(JW % 4 == 0, "whole groups of four columns");
             const int q4 = warp & 3, jh = warp >> 2;
-            const int ml = q4 * 32 + lane, m = m0 + ml;
-            const int p = m / R, s = m - p * R;
+            const int ml = q4 * 32 + lane;
             const int em = eA[ml];
-            int which, sK, sP;
-            if (t < 4) { which = -1; sK = t >> 1; sP = t & 1; }
-            else { which = t - 4; sK = 0; sP = 0; }
-            const int dslot = t == 0 ? 0 : t == 3 ? 1 : t == 4 ? 2 : t == 5 ? 3 : -1;
-            double* zb = which < 0 ? a.Zd : a.Zf[which];
-            const size_t ld = which < 0 ? (size_t)a.ldd : (size_t)a.ldf;
-            const size_t col = (size_t)sP * R2 + m;
+            double* ob = a.out[f] + base + m0 + ml;
             for (int j0 = jh * JW; j0 < (jh + 1) * JW; j0 += 4) {
                 long long acc[4] = {0, 0, 0, 0};
                 for (int L = 2; L <= S + 1; ++L) {
@@ -250,10 +230,8 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
                 for (int jj = 0; jj < 4; ++jj) {
                     const int j = j0 + jj;
                     const int ej = eB[j];
-                    const double z = (em == ZOZ_BAD || ej == ZOZ_BAD) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                      : oz_ll_scaled(acc[jj], em + ej - 6 * (S + 1));
-                    zb[((size_t)sK * R2 + (size_t)k * R + j) * ld + col] = z;
-                    if (dslot >= 0 && j == p) a.diag[(((size_t)dslot * R2 + (size_t)k * R + p) * R) + s] = z;
+                    ob[(size_t)j * ld] = (em == ZOZ_BAD || ej == ZOZ_BAD) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                          : oz_ll_scaled(acc[jj], em + ej - 6 * (S + 1));
                 }
             }
         }
@@ -270,48 +248,43 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Z_oz(const __grid_constant__
 }
 
 template <int R>
-static int zoz_launch(const ZozArgs& a, int ntypes, cudaStream_t st) {
+static int zoz_launch(const ZozArgs& a, cudaStream_t st) {
     constexpr int R2 = R * R, NT = R2 / TC_BM;
     const size_t smem = 1024 + (size_t)ZOZ_SMAX * ZOZ_A_SLICE + (size_t)ZOZ_SMAX * R * 128 + 4 * (TC_BM + 64) + 2 * 72 + 64;
     static int nsm = 0;
     if (!nsm) {
-        ACSE_CUDA_TRY(cudaFuncSetAttribute(k_Z_oz<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        ACSE_CUDA_TRY(cudaFuncSetAttribute(k_xform_oz<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int dev = 0;
         ACSE_CUDA_TRY(cudaGetDevice(&dev));
         ACSE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     }
-    const int ntiles = ntypes * R * NT;
+    const int ntiles = 6 * R * NT;
     const int grid = ntiles < nsm ? ntiles : nsm;
-    k_Z_oz<R><<<grid, ZOZ_THREADS, smem, st>>>(a, ntiles);
+    k_xform_oz<R><<<grid, ZOZ_THREADS, smem, st>>>(a, ntiles);
     ACSE_CUDA_TRY(cudaGetLastError());
     return ACSE_OK;
 }
 
-// Z (FP64 rows of Zd, Zf) and the diagonal rows of w on the tensor cores for an Ozaki context with r a
-// multiple of 16 (r <= 64) and at most 8 slices; ACSE_ERR_UNSUPPORTED otherwise (the caller then runs
-// the double-float kernel).
-int launch_Z_oz(acse_ctx* c, const double* const W[3], int ntypes, const int* tmap) {
+// The transformation by 1D on the tensor cores for an Ozaki context with r a multiple of 16 (r <= 64) and at
+// most 8 slices; ACSE_ERR_UNSUPPORTED otherwise (the caller then runs the double-float kernel).
+int launch_xform_oz(acse_ctx* c, const double* const in[3], double* const out[3], int trans) {
     const int r = c->r;
     if (!c->oz || r % 16 != 0 || r > 64 || c->opt.oz_slices > ZOZ_SMAX) return ACSE_ERR_UNSUPPORTED;
-    Work& w = c->w;
     ZozArgs a;
-    for (int s = 0; s < 3; ++s) a.W[s] = W[s];
-    a.gam = w.gam;
-    a.Zd = w.Zd;
-    a.Zf[0] = w.Zf1;
-    a.Zf[1] = w.Zf2;
-    a.diag = w.zdiag;
-    a.ldd = 2 * r * r;
-    a.ldf = r * r;
-    for (int i = 0; i < 6; ++i) a.tmap[i] = tmap[i];
+    for (int f = 0; f < 3; ++f) {
+        a.in[f] = in[f];
+        a.out[f] = out[f];
+    }
+    a.gam = c->w.gam;
+    a.trans = trans;
     a.S = c->opt.oz_slices;
     a.err = c->w.tc_err;
     int s;
     switch (r) {
-        case 16: s = zoz_launch<16>(a, ntypes, c->stream); break;
-        case 32: s = zoz_launch<32>(a, ntypes, c->stream); break;
-        case 48: s = zoz_launch<48>(a, ntypes, c->stream); break;
-        default: s = zoz_launch<64>(a, ntypes, c->stream); break;
+        case 16: s = zoz_launch<16>(a, c->stream); break;
+        case 32: s = zoz_launch<32>(a, c->stream); break;
+        case 48: s = zoz_launch<48>(a, c->stream); break;
+        default: s = zoz_launch<64>(a, c->stream); break;
     }
     if (s == ACSE_OK) c->launches++;
     return s;
@@ -322,15 +295,15 @@ int launch_Z_oz(acse_ctx* c, const double* const W[3], int ntypes, const int* tm
 // of the FP64 paths, k_B_tiled, walks all r^2 pairs):
 //     x1[k][l] = sum_q X_ij[k][q] 1D[q][l]      (types 0, 1, 2; type 3 reads X_ij transposed)
 //     x2[k][l] = sum_p w[k][p] M_ij[l][p]       (types 0, 1, 3; type 2 reads M_ij transposed)
-// as tall GEMMs over the rows (ij, k) of x1 against 1D^T and (ij, l) of x2^T against w (the class
-// structure of acse_btc.cu), each by the Ozaki splitting of k_Z_oz: digit tiles in shared memory, one
-// exact FP32 accumulator per level, the levels added in int64 and rounded once to FP64.  Outputs: class
-// c = 2 t + (0: x1, 1: x2^T), rows (ij, .) of r doubles, read by k_B_tiled in its precomputed mode.
+// as tall GEMMs over the rows (ij, k) of x1 against 1D^T and (ij, l) of x2^T against w, and likewise the products
+// of the adjoint (acse_adjoint.cu): eight classes, each by the Ozaki splitting of k_xform_oz (digit tiles in
+// shared memory, one exact FP32 accumulator per level, the levels added in int64 and rounded once to FP64).
+// Outputs: rows (ij, .) of r doubles per class.
 struct BxozArgs {
-    const double* X[3];     // pair GEMM outputs (rows ij of r^2: X^{ij}_{kq} at [k][q])
-    const double* M[3];     // M blocks (rows ij: M^{ij}_{lp} at [l][p])
-    const double* gam;      // 1D per spin [2][r][r]
-    const double* w;        // w per spin [2][r][r], w[k][p]
+    const double* T[8];     // class c: rows ij of r^2, the operand of row `row`, element q at [row][q] ...
+    const double* G[8];     // r x r operand, G[n][q] ...
+    unsigned tt, gt;        // ... or transposed (bit c): [q][row], G[q][n]
+    int sel[8];             // classes with the same G (and transposition) share a number
     double* out[8];
     int S;
     int* err;
@@ -371,16 +344,14 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Bx_oz(const __grid_constant_
     const int t_end = min(ntiles, ((int)blockIdx.x + 1) * per);
     for (int tile = (int)blockIdx.x * per; tile < t_end && ok; ++tile, phase ^= 1) {
         const int c = tile / TPC;
-        const int t = c >> 1, x2 = c & 1;
         const int m0 = (tile - c * TPC) * TC_BM;
-        // x1: 1D^T of spin a for types 0, 3, b for 1, 2;  x2: w of spin a for types 0, 2, b for 1, 3
-        const int sel = x2 ? ((t == 0 || t == 2) ? 2 : 3) : ((t == 0 || t == 3) ? 0 : 1);
-        if (sel != cur_sel) {   // B rows n, K = q: 1D^T[n][q] = 1D[q][n], or w[n][q]
-            const unsigned long long* g =
-                reinterpret_cast<const unsigned long long*>((sel < 2 ? a.gam : a.w) + (size_t)(sel & 1) * R2);
+        const int sel = a.sel[c];
+        if (sel != cur_sel) {   // B rows n, K = q
+            const unsigned long long* g = reinterpret_cast<const unsigned long long*>(a.G[c]);
+            const int gn = (a.gt >> c) & 1 ? 1 : R, gq = (a.gt >> c) & 1 ? R : 1;
             for (int n = threadIdx.x; n < R; n += ZOZ_THREADS) {
                 unsigned long long mx = 0;
-                for (int q = 0; q < R; ++q) mx = max(mx, (sel < 2 ? g[q * R + n] : g[n * R + q]) & 0x7FFFFFFFFFFFFFFFull);
+                for (int q = 0; q < R; ++q) mx = max(mx, g[n * gn + q * gq] & 0x7FFFFFFFFFFFFFFFull);
                 eB[n] = zoz_row_exp(mx);
             }
             __syncthreads();
@@ -390,20 +361,18 @@ __global__ void __launch_bounds__(ZOZ_THREADS, 1) k_Bx_oz(const __grid_constant_
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int q = 8 * cc + u;
-                    x[u] = sel < 2 ? g[q * R + n] : g[n * R + q];
+                    x[u] = g[n * gn + q * gq];
                 }
                 zoz_digits8(x, eB[n], S, sB, B_SLICE, zoz_sw128(n, cc), tab);
             }
             cur_sel = sel;
         }
-        // A: row m = (ij, row) of X_ij (x1) or M_ij (x2), K = q; types 3 (x1) and 2 (x2) transposed
+        // A: row m = (ij, row) of T, K = q
         {
             const int ml = threadIdx.x / ZOZ_TPR, part = threadIdx.x % ZOZ_TPR, m = m0 + ml;
             const int ij = m / R, row = m - ij * R;
-            const int sec = t == 0 ? 0 : t == 1 ? 2 : 1;
-            const unsigned long long* base =
-                reinterpret_cast<const unsigned long long*>((x2 ? a.M[sec] : a.X[sec]) + (size_t)ij * R2);
-            const bool tr = x2 ? (t == 2) : (t == 3);
+            const unsigned long long* base = reinterpret_cast<const unsigned long long*>(a.T[c] + (size_t)ij * R2);
+            const bool tr = (a.tt >> c) & 1;
             constexpr int MYCH = (NCH + ZOZ_TPR - 1) / ZOZ_TPR;
             unsigned long long x[MYCH][8];
             unsigned long long mx = 0;
@@ -510,23 +479,28 @@ static int bxoz_launch(const BxozArgs& a, cudaStream_t st) {
     return ACSE_OK;
 }
 
-// x1 and x2^T of every B spin type and every pair into w.bx64 (Ozaki contexts with the scratch allocated:
-// r a multiple of 16, r <= 64, at most 8 slices); ACSE_ERR_UNSUPPORTED otherwise (the B kernel then forms
-// the products itself in double-float).
-int launch_Bx_oz(acse_ctx* c) {
+// The eight classes of tall products out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] in an Ozaki context with r a
+// multiple of 16 (r <= 64) and at most 8 slices; ACSE_ERR_UNSUPPORTED otherwise.
+int launch_rows_oz(acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
+                   double* const out[8]) {
     const int r = c->r;
-    Work& w = c->w;
-    if (!c->oz || !w.bx64[0] || r % 16 != 0 || r > 64 || c->opt.oz_slices > ZOZ_SMAX) return ACSE_ERR_UNSUPPORTED;
+    if (!c->oz || r % 16 != 0 || r > 64 || c->opt.oz_slices > ZOZ_SMAX) return ACSE_ERR_UNSUPPORTED;
     BxozArgs a;
-    for (int s = 0; s < 3; ++s) {
-        a.X[s] = w.X[s];
-        a.M[s] = w.M[s];
+    for (int k = 0; k < 8; ++k) {
+        a.T[k] = T[k];
+        a.G[k] = G[k];
+        a.out[k] = out[k];
+        a.sel[k] = k;
+        for (int m = 0; m < k; ++m)
+            if (G[m] == G[k] && ((gt >> m) & 1) == ((gt >> k) & 1)) {
+                a.sel[k] = m;
+                break;
+            }
     }
-    a.gam = w.gam;
-    a.w = w.w;
-    for (int k = 0; k < 8; ++k) a.out[k] = w.bx64[k];
+    a.tt = tt;
+    a.gt = gt;
     a.S = c->opt.oz_slices;
-    a.err = w.tc_err;
+    a.err = c->w.tc_err;
     int s;
     switch (r) {
         case 16: s = bxoz_launch<16>(a, c->stream); break;
@@ -536,4 +510,17 @@ int launch_Bx_oz(acse_ctx* c) {
     }
     if (s == ACSE_OK) c->launches++;
     return s;
+}
+
+// x1 and x2^T of every B spin type and every pair into w.bx64 (contexts with that scratch); ACSE_ERR_UNSUPPORTED
+// otherwise (the B kernel then forms the products itself in double-float).  Class 2 t: x1[k][l] of X against
+// 1D^T (type 3: X transposed); class 2 t + 1: x2^T[l][k] of M against w (type 2: M transposed).
+int launch_Bx_oz(acse_ctx* c) {
+    Work& w = c->w;
+    if (!w.bx64[0]) return ACSE_ERR_UNSUPPORTED;
+    const int R2 = c->r * c->r;
+    const double *ga = w.gam, *gb = w.gam + R2, *wa = w.w, *wb = w.w + R2;
+    const double* T[8] = {w.X[0], w.M[0], w.X[2], w.M[2], w.X[1], w.M[1], w.X[1], w.M[1]};
+    const double* G[8] = {ga, wa, gb, wb, gb, wa, ga, wb};
+    return launch_rows_oz(c, T, 1u << 6 | 1u << 5, G, 0x55u, w.bx64);
 }

@@ -44,37 +44,35 @@ __global__ void __launch_bounds__(GF_TPB) k_gemm_f64(const __grid_constant__ Gem
         for (int j = 0; j < RT; ++j) acc[i][j] = 0.0;
 
     const int M = P.M, N = P.N, K = P.K;
-    // this thread's two elements of an operand block: K-major storage runs along k, transposed along rows
-    int ar[2], ak[2], br[2], bk[2];
+    const int* __restrict__ mapA = P.mapA;
+    const int* __restrict__ mapB = P.mapB;
+    // this thread's two elements of an operand block: rows row and row + BT / 2, K offset kq
+    const int row = tid / BK, kq = tid % BK;
     const double* asrc[2];
     const double* bsrc[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-        const int e = tid + u * GF_TPB;
-        ar[u] = P.transA ? e % BT : e / BK;
-        ak[u] = P.transA ? e / BT : e % BK;
-        br[u] = P.transB ? e % BT : e / BK;
-        bk[u] = P.transB ? e / BT : e % BK;
-        const int m = m0 + ar[u], n = n0 + br[u];
-        asrc[u] = m < M ? P.A + (size_t)m * (P.transA ? 1 : P.lda) : nullptr;
-        bsrc[u] = n < N ? P.B + (size_t)n * (P.transB ? 1 : P.ldb) : nullptr;
+        const int m = m0 + row + u * (BT / 2), n = n0 + row + u * (BT / 2);
+        asrc[u] = m < M ? P.A + (size_t)(mapA ? mapA[m] : m) * P.lda : nullptr;
+        bsrc[u] = n < N ? P.B + (size_t)(mapB ? mapB[n] : n) * P.ldb : nullptr;
     }
-    const size_t a_ks = P.transA ? (size_t)P.lda : 1, b_ks = P.transB ? (size_t)P.ldb : 1;
     double av[2], bv[2];
     auto load = [&](int k0) {
+        const int k = k0 + kq;
+        const bool kok = k < K;
+        const int ka = mapA && kok ? mapA[k] : k, kb = mapB && kok ? mapB[k] : k;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int ka = k0 + ak[u], kb = k0 + bk[u];
-            av[u] = asrc[u] && ka < K ? asrc[u][(size_t)ka * a_ks] : 0.0;
-            bv[u] = bsrc[u] && kb < K ? bsrc[u][(size_t)kb * b_ks] : 0.0;
+            av[u] = asrc[u] && kok ? asrc[u][ka] : 0.0;
+            bv[u] = bsrc[u] && kok ? bsrc[u][kb] : 0.0;
         }
     };
     load(0);
     for (int k0 = 0; k0 < K; k0 += BK) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            As[ak[u]][ar[u]] = av[u];
-            Bs[bk[u]][br[u]] = bv[u];
+            As[kq][row + u * (BT / 2)] = av[u];
+            Bs[kq][row + u * (BT / 2)] = bv[u];
         }
         __syncthreads();
         if (k0 + BK < K) load(k0 + BK);   // in flight during the products

@@ -85,7 +85,6 @@ struct OzProb {
     int nb;             // operand rows rounded to X = round(a 2^(nb - e))
     int ngroups;        // T nch, modulus-major
     int tiles_n, tile_start;
-    int accum;          // 1: C += result (one FP64 addition), 0: C = result
 };
 
 struct __align__(128) OzBatch {
@@ -573,7 +572,7 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
             const double v = (ea == 0x7FF || eb == 0x7FF)
                                  ? __longlong_as_double(0x7ff8000000000000ll)
                                  : oz_crt_value<LB, NL>(acc[k], Pl, cp.pinvs, ea + eb - 2046 + P.ealpha - 2 * P.nb);
-            crow[j0 + k] = P.accum ? crow[j0 + k] + v : v;
+            crow[j0 + k] = v;
         }
     }
 }
@@ -603,48 +602,13 @@ static int oz_launch_crt(const OzBatch* host, const OzBatch* dev, int nsm, cudaS
     return ACSE_OK;
 }
 
-// Same-spin pair GEMMs on packed pairs (as on the split path): in the aa and bb sectors the rows (ij),
-// the columns (kp) and the contraction (rs) of [M; D] W^T are antisymmetric pairs, so those GEMMs run
-// on pairs i < j only (P = r(r-1)/2; alpha 2 for the halved (rs) sum) and k_oz_unpack rebuilds the
-// full X and Y rows by antisymmetry.  pk(a, b), a < b, numbers the pairs row by row.
-__host__ __device__ __forceinline__ int oz_pk(int r, int a, int b) { return a * r - a * (a + 1) / 2 + (b - a - 1); }
-
-// X_s, Y_s (s = aa, bb; r^2 x r^2 FP64) from the packed [X; Y] (2P x P): one block per output row, the
-// packed source row staged in shared memory, the full row written two columns at a time.
-__global__ void __launch_bounds__(256) k_oz_unpack(int r, const double* __restrict__ Cp0, const double* __restrict__ Cp2,
-                                                   double* X0, double* Y0, double* X2, double* Y2) {
-    __shared__ double srow[ACSE_MAX_R * (ACSE_MAX_R - 1) / 2];
-    const int R2 = r * r, P = r * (r - 1) / 2;
-    const int sec = blockIdx.x / (2 * R2);
-    const int row = blockIdx.x - sec * 2 * R2;
-    const int part = row / R2, ij = row - part * R2, i = ij / r, j = ij - i * r;
-    double* dst = (sec == 0 ? (part ? Y0 : X0) : (part ? Y2 : X2)) + (size_t)ij * R2;
-    if (i == j) {   // block-uniform
-        for (int c = threadIdx.x; c < R2; c += blockDim.x) dst[c] = 0.0;
-        return;
-    }
-    const double si = i < j ? 1.0 : -1.0;
-    const double* src = (sec == 0 ? Cp0 : Cp2) + (size_t)(part * P + (i < j ? oz_pk(r, i, j) : oz_pk(r, j, i))) * P;
-    for (int e = threadIdx.x; e < P; e += blockDim.x) srow[e] = si * src[e];
-    __syncthreads();
-    auto val = [&](int k, int q) { return k == q ? 0.0 : (k < q ? srow[oz_pk(r, k, q)] : -srow[oz_pk(r, q, k)]); };
-    if ((R2 & 1) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-        for (int g = threadIdx.x; g < R2 / 2; g += blockDim.x) {
-            int k = (2 * g) / r, q = 2 * g - k * r;
-            const double v0 = val(k, q);
-            if (++q == r) { q = 0; ++k; }
-            reinterpret_cast<double2*>(dst)[g] = make_double2(v0, val(k, q));
-        }
-    } else {
-        for (int c = threadIdx.x; c < R2; c += blockDim.x) dst[c] = val(c / r, c - (c / r) * r);
-    }
-}
-
 // --------------------------------------------------------------------------- host plan
-// Operands of the GEMMs of a pass (the products of acse_gemm_list_f64, the same-spin ones packed):
-//   A: [M_aa; D_aa] packed (2P x P), M_ab, D_ab (r^2 x r^2), [M_bb; D_bb] packed, Zd (2r^2 x 2r^2),
-//      Zf1, Zf2 (r^2 x r^2);
-//   B: W_aa packed (P x P), W_ab (r^2 x r^2), W_bb packed, Md (2r^2 x 2r^2), Mf1, Mf2 (r^2 x r^2).
+// Operands of the GEMMs of a pass (the products of acse_gemm_list_f64; S2 = r(r+1), P2 = r(r-1), P = P2 / 2):
+//   A: W+ and W- (rows S2 and P2 for s = +1, P2 and S2 for s = -1), Wf1, M_ab, D_ab (r^2 x r^2),
+//      [M_aa; D_aa], [M_bb; D_bb] packed (2P x P);
+//   B: M+ (S2 x S2), M- (P2 x P2), Mf1, W_ab (r^2 x r^2), W_aa, W_bb packed (P x P).
+// The problem table of s = +1 is the plan itself; that of s = -1 (`alt`) has the same operands with the
+// other row counts and borrows every buffer.
 struct OzOp {
     __nv_bfloat16* sl;
     double* scale;
@@ -665,15 +629,12 @@ struct OzPlan {
     int nsm;
     int tiles;
     OzOp A[OZ_MAXP], B[OZ_MAXP];
-    int* pmap;          // pair index -> i r + j (i < j), P entries
-    double* Cp[2];      // packed [X; Y] of the aa and bb sectors (2P x P)
     int* sched;         // tile lists of the persistent kernel (OzBatch::order, cta_start)
     int* err;
-    // GEMM lists of the adjoint (oz_gemm_list): a plan per list slot, and the column maps of the
-    // transposed operands (K index k -> source offset k ld)
-    struct OzPlan* lists[2];
-    int cm_K[4], cm_ld[4];
-    int* cm[4];
+    struct OzPlan* alt;       // the pass's table for s = -1
+    int borrowed;             // operands and staging belong to another plan
+    struct OzPlan* lists[2];  // GEMM lists of the adjoint (oz_gemm_list): a plan per list slot
+    int shareB[OZ_MAXP];      // lists: problem i reads the B operand of problem shareB[i] - 1 (0: its own)
 };
 
 static size_t oz_smem(int bn) { return (size_t)OZ_STAGES * (TC_BM + bn) * 128 + 1024 + 256; }
@@ -765,7 +726,10 @@ static int oz_op_alloc(OzPlan* pl, OzOp& o, int rows, int K) {
     return ACSE_OK;
 }
 
-static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, double alpha) {
+// One problem C = alpha A B^T; its residue staging is `stage` (borrowed) or allocated here for stage_rows >= M
+// rows.
+static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, double alpha, int stage_rows,
+                  unsigned char* stage) {
     OzBatch& B = *pl->host;
     if (B.nprob >= OZ_MAXP || a.K != b.K || a.Kp != b.Kp || a.nb != b.nb) return ACSE_ERR_SHAPE;
     const int n = B.nprob;
@@ -790,7 +754,8 @@ static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, 
     if (p.nch > OZ_MAXCH) return ACSE_ERR_SHAPE;
     p.cb = (p.kbs + p.nch - 1) / p.nch;
     p.ngroups = B.mods.T * p.nch;
-    if (cudaMalloc((void**)&p.stage, (size_t)p.ngroups * p.M * p.N) != cudaSuccess) {
+    p.stage = stage;
+    if (!stage && cudaMalloc((void**)&p.stage, (size_t)p.ngroups * stage_rows * p.N) != cudaSuccess) {
         cudaGetLastError();
         p.stage = nullptr;
         return ACSE_ERR_NOMEM;
@@ -874,12 +839,31 @@ extern "C" int acse_ozaki_plan_info(int oz_slices, int kmax, int k, int* moduli_
     return st;
 }
 
+// The seven products of a pass in the order of acse_gemm_list_f64 (the same-spin X and Y as one problem).
+static int oz_pass_table(acse_ctx* c, OzPlan* pl, const OzPlan* root) {
+    Work& w = c->w;
+    const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
+    const bool own = pl == root;
+    auto add = [&](int i, const OzOp& A, const OzOp& B, double* C, int ldc, double alpha, int stage_rows) {
+        return oz_add(pl, A, B, C, ldc, alpha, stage_rows, own ? nullptr : root->host->p[i].stage);
+    };
+    ACSE_TRY(add(0, pl->A[0], pl->B[0], w.V1, S2, 1.0, S2));
+    ACSE_TRY(add(1, pl->A[2], pl->B[2], w.V5f1, R2, 1.0, R2));
+    ACSE_TRY(add(2, pl->A[3], pl->B[3], w.X[1], R2, 2.0, R2));
+    ACSE_TRY(add(3, pl->A[4], pl->B[3], w.Y[1], R2, 2.0, R2));
+    ACSE_TRY(add(4, pl->A[1], pl->B[1], w.V2, P2, 1.0, S2));
+    ACSE_TRY(add(5, pl->A[5], pl->B[4], w.Cp[0], P, 2.0, 2 * P));
+    ACSE_TRY(add(6, pl->A[6], pl->B[5], w.Cp[1], P, 2.0, 2 * P));
+    return oz_plan_finish(pl);
+}
+
 int oz_plan_create(acse_ctx* c) {
     OzPlan* pl = (OzPlan*)calloc(1, sizeof(OzPlan));
     if (!pl) return ACSE_ERR_NOMEM;
     c->oz_plan = pl;
-    const int r = c->r, R2 = r * r, R22 = 2 * R2, P = r * (r - 1) / 2;
-    ACSE_TRY(oz_plan_init(pl, c->opt.oz_slices, R2 >= 256 ? OZ_BN : 128, c->opt.gemm_tile != 1, R22));
+    const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
+    const int bn = R2 >= 256 ? OZ_BN : 128, pair = c->opt.gemm_tile != 1;
+    ACSE_TRY(oz_plan_init(pl, c->opt.oz_slices, bn, pair, S2));
     // the B products on the tensor cores (acse_zoz.cu): x1 and x2^T of the four types for every pair
     if (r % 16 == 0 && r <= 64 && c->opt.oz_slices <= 8)
         for (int k = 0; k < 8; ++k)
@@ -888,37 +872,14 @@ int oz_plan_create(acse_ctx* c) {
                 c->w.bx64[k] = nullptr;
                 return ACSE_ERR_NOMEM;
             }
-    ACSE_TRY(oz_op_alloc(pl, pl->A[0], 2 * P, P));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[1], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[2], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[3], 2 * P, P));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[4], R22, R22));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[5], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->A[6], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[0], P, P));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[1], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[2], P, P));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[3], R22, R22));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[4], R2, R2));
-    ACSE_TRY(oz_op_alloc(pl, pl->B[5], R2, R2));
-    {
-        int* hm = (int*)malloc((size_t)P * sizeof(int));
-        if (!hm) return ACSE_ERR_NOMEM;
-        for (int a = 0; a < r; ++a)
-            for (int b = a + 1; b < r; ++b) hm[oz_pk(r, a, b)] = a * r + b;
-        const bool ok = cudaMalloc((void**)&pl->pmap, (size_t)P * sizeof(int)) == cudaSuccess &&
-                        cudaMemcpy(pl->pmap, hm, (size_t)P * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
-        free(hm);
-        if (!ok) {
-            cudaGetLastError();
-            return ACSE_ERR_NOMEM;
-        }
-    }
-    for (int s = 0; s < 2; ++s)
-        if (cudaMalloc((void**)&pl->Cp[s], (size_t)2 * P * P * sizeof(double)) != cudaSuccess) {
-            cudaGetLastError();
-            return ACSE_ERR_NOMEM;
-        }
+    ACSE_TRY(oz_op_alloc(pl, pl->A[0], S2, S2));
+    ACSE_TRY(oz_op_alloc(pl, pl->A[1], S2, P2));
+    for (int i = 2; i < 5; ++i) ACSE_TRY(oz_op_alloc(pl, pl->A[i], R2, R2));
+    for (int i = 5; i < 7; ++i) ACSE_TRY(oz_op_alloc(pl, pl->A[i], 2 * P, P));
+    ACSE_TRY(oz_op_alloc(pl, pl->B[0], S2, S2));
+    ACSE_TRY(oz_op_alloc(pl, pl->B[1], P2, P2));
+    for (int i = 2; i < 4; ++i) ACSE_TRY(oz_op_alloc(pl, pl->B[i], R2, R2));
+    for (int i = 4; i < 6; ++i) ACSE_TRY(oz_op_alloc(pl, pl->B[i], P, P));
     if (cudaMalloc((void**)&pl->err, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return ACSE_ERR_NOMEM;
@@ -926,17 +887,19 @@ int oz_plan_create(acse_ctx* c) {
     ACSE_CUDA_TRY(cudaMemset(pl->err, 0, sizeof(int)));
     if (!c->w.tc_err) c->w.tc_err = pl->err;   // read by acse_sync_status
     pl->host->err = pl->err;
-    Work& w = c->w;
-    // the largest-K GEMM first, then the mixed-spin pair GEMMs (X_ab = 2 M_ab W_ab^T, Y_ab = 2 D_ab W_ab^T),
-    // the spin-flip ones and the packed same-spin ones (alpha 2 for the halved (rs) sum)
-    ACSE_TRY(oz_add(pl, pl->A[4], pl->B[3], w.X5d, R22, 1.0));
-    ACSE_TRY(oz_add(pl, pl->A[1], pl->B[1], w.X[1], R2, 2.0));
-    ACSE_TRY(oz_add(pl, pl->A[2], pl->B[1], w.Y[1], R2, 2.0));
-    ACSE_TRY(oz_add(pl, pl->A[5], pl->B[4], w.X5f1, R2, 1.0));
-    ACSE_TRY(oz_add(pl, pl->A[6], pl->B[5], w.X5f2, R2, 1.0));
-    ACSE_TRY(oz_add(pl, pl->A[0], pl->B[0], pl->Cp[0], P, 2.0));
-    ACSE_TRY(oz_add(pl, pl->A[3], pl->B[2], pl->Cp[1], P, 2.0));
-    return oz_plan_finish(pl);
+    pl->A[1].rows = P2;   // s = +1: W+ over S2 rows, W- over P2
+    ACSE_TRY(oz_pass_table(c, pl, pl));
+    OzPlan* alt = (OzPlan*)calloc(1, sizeof(OzPlan));
+    if (!alt) return ACSE_ERR_NOMEM;
+    pl->alt = alt;
+    alt->borrowed = 1;
+    ACSE_TRY(oz_plan_init(alt, c->opt.oz_slices, bn, pair, S2));
+    alt->host->err = pl->err;
+    memcpy(alt->A, pl->A, sizeof(pl->A));
+    memcpy(alt->B, pl->B, sizeof(pl->B));
+    alt->A[0].rows = P2;   // s = -1: the other way round
+    alt->A[1].rows = S2;
+    return oz_pass_table(c, alt, pl);
 }
 
 // Longest-processing-time tile lists of the persistent kernel (tile cost: its K blocks over all groups)
@@ -981,22 +944,18 @@ static int oz_plan_finish(OzPlan* pl) {
 
 static void oz_plan_free(OzPlan* pl) {
     if (!pl) return;
-    for (int i = 0; i < OZ_MAXP; ++i) {
+    oz_plan_free(pl->alt);
+    for (int s = 0; s < 2; ++s) oz_plan_free(pl->lists[s]);
+    for (int i = 0; i < OZ_MAXP && !pl->borrowed; ++i) {
         if (pl->A[i].sl) cudaFree(pl->A[i].sl);
         if (pl->A[i].scale) cudaFree(pl->A[i].scale);
+        if (pl->shareB[i]) continue;   // an earlier problem's operand
         if (pl->B[i].sl) cudaFree(pl->B[i].sl);
         if (pl->B[i].scale) cudaFree(pl->B[i].scale);
     }
-    if (pl->pmap) cudaFree(pl->pmap);
     if (pl->sched) cudaFree(pl->sched);
-    for (int s = 0; s < 2; ++s) {
-        if (pl->Cp[s]) cudaFree(pl->Cp[s]);
-        oz_plan_free(pl->lists[s]);
-    }
-    for (int i = 0; i < 4; ++i)
-        if (pl->cm[i]) cudaFree(pl->cm[i]);
     if (pl->err) cudaFree(pl->err);
-    if (pl->host)
+    if (pl->host && !pl->borrowed)
         for (int i = 0; i < pl->host->nprob; ++i)
             if (pl->host->p[i].stage) cudaFree(pl->host->p[i].stage);
     if (pl->dev) cudaFree(pl->dev);
@@ -1066,100 +1025,68 @@ static int oz_slice_launch(acse_ctx* c, const OzSliceBatch& all, int rows) {
     return ACSE_OK;
 }
 
-int oz_slice_operands(acse_ctx* c, int prep_D) {
-    OzPlan* pl = (OzPlan*)c->oz_plan;
-    if (!pl) return ACSE_ERR_UNSUPPORTED;
-    const int r = c->r, P = r * (r - 1) / 2;
-    const size_t R2 = (size_t)r * r;
-    const int iR2 = (int)R2;
+int oz_slice_operands(acse_ctx* c, int prep_D, int sW) {
+    OzPlan* root = (OzPlan*)c->oz_plan;
+    if (!root) return ACSE_ERR_UNSUPPORTED;
+    const OzPlan* pl = sW > 0 ? root : root->alt;
+    const int r = c->r, P = r * (r - 1) / 2, R2 = r * r, S2 = r * (r + 1), P2 = 2 * P;
     Work& w = c->w;
     OzSliceBatch b;
     oz_slice_batch_init(b, pl->host->mods);
     int rows = 0;
-    const int* pm = pl->pmap;
+    const int* pm = w.pmap;
     // A residues as they are, B residues times y_t
     if (prep_D) {
-        oz_job(b, rows, pl->A[0], 0, P, w.M[0], R2, pm, pm, 0);
-        oz_job(b, rows, pl->A[0], P, P, c->cur_D[0], R2, pm, pm, 0);
-        oz_job(b, rows, pl->A[1], 0, iR2, w.M[1], R2, nullptr, nullptr, 0);
-        oz_job(b, rows, pl->A[2], 0, iR2, c->cur_D[1], R2, nullptr, nullptr, 0);
-        oz_job(b, rows, pl->A[3], 0, P, w.M[2], R2, pm, pm, 0);
-        oz_job(b, rows, pl->A[3], P, P, c->cur_D[2], R2, pm, pm, 0);
-        oz_job(b, rows, pl->B[3], 0, 2 * iR2, w.Md, 2 * R2, nullptr, nullptr, 1);
-        oz_job(b, rows, pl->B[4], 0, iR2, w.Mf1, R2, nullptr, nullptr, 1);
-        oz_job(b, rows, pl->B[5], 0, iR2, w.Mf2, R2, nullptr, nullptr, 1);
+        oz_job(b, rows, pl->A[5], 0, P, w.M[0], R2, pm, pm, 0);
+        oz_job(b, rows, pl->A[5], P, P, c->cur_D[0], R2, pm, pm, 0);
+        oz_job(b, rows, pl->A[3], 0, R2, w.M[1], R2, nullptr, nullptr, 0);
+        oz_job(b, rows, pl->A[4], 0, R2, c->cur_D[1], R2, nullptr, nullptr, 0);
+        oz_job(b, rows, pl->A[6], 0, P, w.M[2], R2, pm, pm, 0);
+        oz_job(b, rows, pl->A[6], P, P, c->cur_D[2], R2, pm, pm, 0);
+        oz_job(b, rows, pl->B[0], 0, S2, w.Mp, S2, nullptr, nullptr, 1);
+        oz_job(b, rows, pl->B[1], 0, P2, w.Mm, P2, nullptr, nullptr, 1);
+        oz_job(b, rows, pl->B[2], 0, R2, w.Mf1, R2, nullptr, nullptr, 1);
     }
-    oz_job(b, rows, pl->B[0], 0, P, c->cur_W[0], R2, pm, pm, 1);
-    oz_job(b, rows, pl->B[1], 0, iR2, c->cur_W[1], R2, nullptr, nullptr, 1);
-    oz_job(b, rows, pl->B[2], 0, P, c->cur_W[2], R2, pm, pm, 1);
-    oz_job(b, rows, pl->A[4], 0, 2 * iR2, w.Zd, 2 * R2, nullptr, nullptr, 0);
-    oz_job(b, rows, pl->A[5], 0, iR2, w.Zf1, R2, nullptr, nullptr, 0);
-    oz_job(b, rows, pl->A[6], 0, iR2, w.Zf2, R2, nullptr, nullptr, 0);
+    oz_job(b, rows, pl->B[3], 0, R2, c->cur_W[1], R2, nullptr, nullptr, 1);
+    oz_job(b, rows, pl->B[4], 0, P, c->cur_W[0], R2, pm, pm, 1);
+    oz_job(b, rows, pl->B[5], 0, P, c->cur_W[2], R2, pm, pm, 1);
+    oz_job(b, rows, pl->A[0], 0, pl->A[0].rows, w.Wp, S2, nullptr, nullptr, 0);
+    oz_job(b, rows, pl->A[1], 0, pl->A[1].rows, w.Wm, P2, nullptr, nullptr, 0);
+    oz_job(b, rows, pl->A[2], 0, R2, w.Wf1, R2, nullptr, nullptr, 0);
     return oz_slice_launch(c, b, rows);
 }
 
-int oz_gemm_launch(acse_ctx* c) {
-    OzPlan* pl = (OzPlan*)c->oz_plan;
-    if (!pl) return ACSE_ERR_UNSUPPORTED;
+int oz_gemm_launch(acse_ctx* c, int sW) {
+    OzPlan* root = (OzPlan*)c->oz_plan;
+    if (!root) return ACSE_ERR_UNSUPPORTED;
+    const OzPlan* pl = sW > 0 ? root : root->alt;
     if (pl->tiles == 0) return ACSE_OK;
     ACSE_TRY(prof_begin(c));
     ACSE_TRY(oz_launch_gemm(pl, c->stream));
     ACSE_LAUNCHED(c);
     ACSE_TRY(oz_launch_crt(pl->host, pl->dev, pl->nsm, c->stream));
     ACSE_LAUNCHED(c);
-    ACSE_TRY(prof_end(c));
-    Work& w = c->w;
-    k_oz_unpack<<<2 * 2 * c->r * c->r, 256, 0, c->stream>>>(c->r, pl->Cp[0], pl->Cp[1], w.X[0], w.Y[0], w.X[2], w.Y[2]);
-    ACSE_LAUNCHED(c);
-    return ACSE_OK;
+    return prof_end(c);
 }
 
 int oz_set_wait_ns(acse_ctx* c, unsigned long long ns, int inject_stall) {
     OzPlan* pl = (OzPlan*)c->oz_plan;
     if (!pl) return ACSE_ERR_UNSUPPORTED;
     ACSE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    pl->host->wait_ns = ns ? ns : OZ_WAIT_NS;
-    pl->host->inject_stall = inject_stall;
-    ACSE_CUDA_TRY(cudaMemcpy(pl->dev, pl->host, sizeof(OzBatch), cudaMemcpyHostToDevice));
+    for (OzPlan* q : {pl, pl->alt}) {
+        q->host->wait_ns = ns ? ns : OZ_WAIT_NS;
+        q->host->inject_stall = inject_stall;
+        ACSE_CUDA_TRY(cudaMemcpy(q->dev, q->host, sizeof(OzBatch), cudaMemcpyHostToDevice));
+    }
     return ACSE_OK;
 }
 
 // ------------------------------------------------------------------ GEMM lists of the adjoint
-// The reverse sweep's FP64 GEMMs (acse_adjoint.cu) of an Ozaki context run through the same kernels:
-// any list of up to OZ_MAXP GEMMs C (+)= alpha A B^T, alpha a power of two, beta 0 or 1, either operand
-// stored transposed (GemmF64::transA / transB).  A transposed operand is sliced through a column map
-// (K index k at source offset k ld, row n at offset n): its reads are strided, one 8-byte element per
-// 32-byte sector, cheap next to the GEMM.  One plan per list slot, built on the first call (its slices
-// and residue staging stay until the context is destroyed); a later call whose shapes differ from
-// the slot's plan is refused (ACSE_ERR_SHAPE).
-
-// Column map k -> k ld for K indices, cached per (K, ld).
-static int oz_colmap(OzPlan* root, int K, int ld, const int** out) {
-    for (int i = 0; i < 4; ++i)
-        if (root->cm[i] && root->cm_K[i] == K && root->cm_ld[i] == ld) {
-            *out = root->cm[i];
-            return ACSE_OK;
-        }
-    for (int i = 0; i < 4; ++i) {
-        if (root->cm[i]) continue;
-        int* h = (int*)malloc((size_t)K * sizeof(int));
-        if (!h) return ACSE_ERR_NOMEM;
-        for (int k = 0; k < K; ++k) h[k] = k * ld;
-        const bool ok = cudaMalloc((void**)&root->cm[i], (size_t)K * sizeof(int)) == cudaSuccess &&
-                        cudaMemcpy(root->cm[i], h, (size_t)K * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
-        free(h);
-        if (!ok) {
-            cudaGetLastError();
-            return ACSE_ERR_NOMEM;
-        }
-        root->cm_K[i] = K;
-        root->cm_ld[i] = ld;
-        *out = root->cm[i];
-        return ACSE_OK;
-    }
-    return ACSE_ERR_UNSUPPORTED;
-}
-
+// The reverse sweep's FP64 GEMMs (acse_adjoint.cu) of an Ozaki context run through the same kernels: any
+// list of up to OZ_MAXP GEMMs C = alpha A B^T, alpha a power of two, both operands K-major, B possibly through
+// a pair map; problems with the same B share its residues.  One plan per list slot, built on the first call
+// (its slices and residue staging stay until the context is destroyed); a later call whose shapes differ
+// from the slot's plan is refused (ACSE_ERR_SHAPE).
 static int oz_list_create(OzPlan* root, const GemmF64* g, int n, OzPlan** out) {
     OzPlan* pl = (OzPlan*)calloc(1, sizeof(OzPlan));
     if (!pl) return ACSE_ERR_NOMEM;
@@ -1171,9 +1098,13 @@ static int oz_list_create(OzPlan* root, const GemmF64* g, int n, OzPlan** out) {
     ACSE_TRY(oz_plan_init(pl, root->S, maxN >= 256 ? OZ_BN : 128, root->pair, maxK));
     pl->host->err = root->err;
     for (int i = 0; i < n; ++i) {
+        for (int k = 0; k < i && !pl->shareB[i]; ++k)
+            if (!pl->shareB[k] && g[k].B == g[i].B && g[k].N == g[i].N && g[k].K == g[i].K && g[k].mapB == g[i].mapB)
+                pl->shareB[i] = k + 1;
         ACSE_TRY(oz_op_alloc(pl, pl->A[i], g[i].M, g[i].K));
-        ACSE_TRY(oz_op_alloc(pl, pl->B[i], g[i].N, g[i].K));
-        ACSE_TRY(oz_add(pl, pl->A[i], pl->B[i], g[i].C, g[i].ldc, g[i].alpha));
+        if (!pl->shareB[i]) ACSE_TRY(oz_op_alloc(pl, pl->B[i], g[i].N, g[i].K));
+        else pl->B[i] = pl->B[pl->shareB[i] - 1];
+        ACSE_TRY(oz_add(pl, pl->A[i], pl->B[i], g[i].C, g[i].ldc, g[i].alpha, g[i].M, nullptr));
     }
     return oz_plan_finish(pl);
 }
@@ -1183,7 +1114,7 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
     if (!root || slot < 0 || slot > 1 || n < 1 || n > OZ_MAXP) return ACSE_ERR_UNSUPPORTED;
     for (int i = 0; i < n; ++i) {
         int ex = 0;
-        if (frexp(g[i].alpha, &ex) != 0.5 || (g[i].beta != 0.0 && g[i].beta != 1.0)) return ACSE_ERR_ARG;
+        if (frexp(g[i].alpha, &ex) != 0.5 || g[i].beta != 0.0 || g[i].mapA) return ACSE_ERR_ARG;
     }
     if (!root->lists[slot]) {
         const int s = oz_list_create(root, g, n, &root->lists[slot]);
@@ -1196,21 +1127,21 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
     OzPlan* pl = root->lists[slot];
     OzBatch& B = *pl->host;
     if (B.nprob != n) return ACSE_ERR_SHAPE;
-    for (int i = 0; i < n; ++i)
+    for (int i = 0; i < n; ++i) {
         if (B.p[i].M != g[i].M || B.p[i].N != g[i].N || pl->A[i].K != g[i].K) return ACSE_ERR_SHAPE;
+        const int k = pl->shareB[i] - 1;
+        if (k >= 0 && (g[k].B != g[i].B || g[k].ldb != g[i].ldb || g[k].mapB != g[i].mapB)) return ACSE_ERR_SHAPE;
+    }
     // residues of every operand (B times y_t), at most OZ_MAXJ jobs a launch
     OzSliceBatch sb;
     oz_slice_batch_init(sb, B.mods);
     int rows = 0;
     for (int i = 0; i < n; ++i) {
         for (int side = 0; side < 2; ++side) {
-            const double* src = side ? g[i].B : g[i].A;
-            const int tr = side ? g[i].transB : g[i].transA;
-            const int ld = side ? g[i].ldb : g[i].lda;
+            if (side && pl->shareB[i]) continue;
             const OzOp& o = side ? pl->B[i] : pl->A[i];
-            const int* cm = nullptr;
-            if (tr) ACSE_TRY(oz_colmap(root, o.K, ld, &cm));
-            oz_job(sb, rows, o, 0, o.rows, src, tr ? 1 : (size_t)ld, nullptr, cm, side);
+            const int* map = side ? g[i].mapB : nullptr;
+            oz_job(sb, rows, o, 0, o.rows, side ? g[i].B : g[i].A, (size_t)(side ? g[i].ldb : g[i].lda), map, map, side);
             if (sb.njobs == OZ_MAXJ) {
                 ACSE_TRY(oz_slice_launch(c, sb, rows));
                 oz_slice_batch_init(sb, B.mods);
@@ -1219,7 +1150,7 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
         }
     }
     ACSE_TRY(oz_slice_launch(c, sb, rows));
-    // this call's outputs, scales and accumulation
+    // this call's outputs and scales
     for (int i = 0; i < n; ++i) {
         OzProb& p = B.p[i];
         int ex = 0;
@@ -1228,7 +1159,6 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
         p.ldc = g[i].ldc;
         p.alpha = g[i].alpha;
         p.ealpha = ex - 1;
-        p.accum = g[i].beta != 0.0;
     }
     B.wait_ns = root->host->wait_ns;
     B.inject_stall = root->host->inject_stall;
