@@ -74,7 +74,10 @@ struct OzMods {
 
 struct OzProb {
     double* C;
-    unsigned char* stage;   // [ngroups][M][N]: the residue w + 128 of each (modulus, chunk) group
+    unsigned char* stage;   // [ngroups][M][ns]: the residue w + 128 of each (modulus, chunk) group
+    int ns;                 // row pitch of stage: N rounded up to 32, so that a thread's 32 residues always leave
+                            // as two aligned 16-byte stores (byte stores for odd N held the GEMM of r = 30 at
+                            // 1.32 ms, 8 times its work)
     const double* sa;   // 2^ea per row of A
     const double* sb;   // 2^eb per row of B
     double alpha;
@@ -388,8 +391,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
             const int m0 = (local / P.tiles_n) * BM + (int)rank * TC_BM, n0 = (local % P.tiles_n) * BN;
             const int row = m0 + q * 32 + lane;
             const bool rok = row < P.M;
-            // 16- or 8-byte stores of a row's 32 residues when the row starts on such a boundary
-            const int vec = (reinterpret_cast<uintptr_t>(P.stage) & 15) ? 0 : (P.N & 15) == 0 ? 16 : (P.N & 7) == 0 ? 8 : 0;
             for (int gi = 0; gi < P.ngroups; ++gi, ++lt) {
                 const int ab = lt & 1, use = lt >> 1;
                 int go = 0;
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
                 const float pm = b.mods.p[tm], pinv = b.mods.pinv[tm];
                 // the chunk sum is an integer of magnitude at most 2^24 (exact in FP32); its residue w modulo
                 // p_t (|w| <= 65) goes out as the byte w + 128 (the low byte of the float w + 128 + 1.5 * 2^23)
-                unsigned char* srow = P.stage + (size_t)gi * P.M * P.N + (size_t)(rok ? row : 0) * P.N;
+                unsigned char* srow = P.stage + ((size_t)gi * P.M + (rok ? row : 0)) * P.ns;
 #pragma unroll 1
                 for (int c = 0; c < BN / 32; ++c) {
                     uint32_t v[32];
@@ -425,18 +426,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
                             x[i] = __float_as_uint(oz_bal_mod(__uint_as_float(v[j + i]), pm, pinv) + 12583040.0f);
                         wd[j / 4] = __byte_perm(__byte_perm(x[0], x[1], 0x0040), __byte_perm(x[2], x[3], 0x0040), 0x5410);
                     }
-                    if (col0 + 32 <= P.N && vec == 16) {
-                        *reinterpret_cast<uint4*>(srow + col0) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                        *reinterpret_cast<uint4*>(srow + col0 + 16) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-                    } else if (col0 + 32 <= P.N && vec == 8) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) *reinterpret_cast<uint2*>(srow + col0 + 8 * j) = make_uint2(wd[2 * j], wd[2 * j + 1]);
-                    } else {
-                        const int nc = min(32, P.N - col0);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (j < nc) srow[col0 + j] = (unsigned char)((wd[j / 4] >> (8 * (j & 3))) & 0xFF);
-                    }
+                    *reinterpret_cast<uint4*>(srow + col0) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+                    *reinterpret_cast<uint4*>(srow + col0 + 16) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -520,21 +511,22 @@ struct OzCrtParams {
     int T;
 };
 
-// Two consecutive elements of one row per thread (16-bit loads of their residue bytes when N is even):
-// every residue word of the element pair (all moduli and chunks) is loaded before any is used, so that
+// Two consecutive elements of one row per thread (16-bit loads of their residue bytes; the second one of an odd
+// row's last pair is padding): every residue word of the element pair (all moduli and chunks) is loaded before any is used, so that
 // about 2 KB per warp is in flight.  A byte b = w + 128 becomes the float 2^23 + b by a byte permute
 // (exact), so w = that - (2^23 + 128).
-template <int NCH, int VW>
+template <int NCH>
 __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& cp) {
     constexpr int LB = NCH == 1 ? OZ_LB1 : OZ_LB2, NL = NCH == 1 ? OZ_NL1 : OZ_NL2;
     const float(*qt)[NL] = NCH == 1 ? (const float(*)[NL])cp.q11 : (const float(*)[NL])cp.q10;
     const float* Pl = NCH == 1 ? cp.P11 : cp.P10;
-    const int T = cp.T, N = P.N;
-    const size_t MN = (size_t)P.M * N;
-    const size_t nunit = MN / VW;
+    constexpr int VW = 2;
+    const int T = cp.T, N = P.N, nh = (N + 1) / 2;
+    const size_t MN = (size_t)P.M * P.ns;   // bytes of a (modulus, chunk) group
+    const size_t nunit = (size_t)P.M * nh;
     for (size_t u = (size_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunit; u += (size_t)gridDim.x * blockDim.x) {
-        const size_t e = u * VW;
-        const unsigned char* __restrict__ sp = P.stage + e;
+        const int i = (int)(u / nh), j0 = 2 * (int)(u - (size_t)i * nh);
+        const unsigned char* __restrict__ sp = P.stage + (size_t)i * P.ns + j0;
         unsigned int xw[OZ_NMOD][NCH];
 #pragma unroll
         for (int t = 0; t < OZ_NMOD; ++t)
@@ -542,7 +534,7 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
             for (int c = 0; c < NCH; ++c) {
                 xw[t][c] = 0x8080u;   // w = 0 past the last modulus
                 if (t < T) {
-                    xw[t][c] = VW == 2 ? (unsigned int)__ldg(reinterpret_cast<const unsigned short*>(sp)) : (unsigned int)__ldg(sp);
+                    xw[t][c] = (unsigned int)__ldg(reinterpret_cast<const unsigned short*>(sp));
                     sp += MN;
                 }
             }
@@ -563,11 +555,11 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
                 for (int l = 0; l < NL; ++l) acc[k][l] = fmaf(w, qt[t][l], acc[k][l]);
             }
         }
-        const int i = (int)(e / N), j0 = (int)(e - (size_t)i * N);
         const int ea = (int)((__double_as_longlong(P.sa[i]) >> 52) & 0x7FF);   // row scales are powers of two
         double* crow = P.C + (size_t)i * P.ldc;
 #pragma unroll
         for (int k = 0; k < VW; ++k) {
+            if (j0 + k >= N) break;
             const int eb = (int)((__double_as_longlong(P.sb[j0 + k]) >> 52) & 0x7FF);
             const double v = (ea == 0x7FF || eb == 0x7FF)
                                  ? __longlong_as_double(0x7ff8000000000000ll)
@@ -581,9 +573,8 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
 // an element are read once, coalesced, and C is written once.
 __global__ void __launch_bounds__(256, OZ_CRT_MINB) k_oz_crt(const OzBatch* __restrict__ bp, const __grid_constant__ OzCrtParams cp) {
     const OzProb& P = bp->p[blockIdx.y];
-    const bool v2 = (P.N & 1) == 0;
-    if (P.nch == 1) v2 ? oz_crt_rows<1, 2>(P, cp) : oz_crt_rows<1, 1>(P, cp);
-    else v2 ? oz_crt_rows<2, 2>(P, cp) : oz_crt_rows<2, 1>(P, cp);
+    if (P.nch == 1) oz_crt_rows<1>(P, cp);
+    else oz_crt_rows<2>(P, cp);
 }
 
 // The reconstruction launch of a plan.
@@ -747,6 +738,7 @@ static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, 
     p.M = a.rows;
     p.N = b.rows;
     p.ldc = ldc;
+    p.ns = (p.N + 31) / 32 * 32;
     p.kbs = a.Kp / 64;
     p.nb = a.nb;
     // chunks of at most OZ_CHUNK_KB blocks: every partial sum of residue products stays below 2^24
@@ -755,7 +747,7 @@ static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, 
     p.cb = (p.kbs + p.nch - 1) / p.nch;
     p.ngroups = B.mods.T * p.nch;
     p.stage = stage;
-    if (!stage && cudaMalloc((void**)&p.stage, (size_t)p.ngroups * stage_rows * p.N) != cudaSuccess) {
+    if (!stage && cudaMalloc((void**)&p.stage, (size_t)p.ngroups * stage_rows * p.ns) != cudaSuccess) {
         cudaGetLastError();
         p.stage = nullptr;
         return ACSE_ERR_NOMEM;
