@@ -73,10 +73,10 @@ typedef enum {
  *                sums exact in FP32, T the least count that covers the product: 17 at r = 48 with 8
  *                slices) and rebuilt exactly by the Chinese remainder theorem, with one rounding to FP64.
  *                With the default 8 (48 bits) the GEMM error is of the order of 2^-48 |A||B| K, below
- *                that of FP64 FMA.  The O(r^5) products of the pass (Z and the B products, r a multiple
- *                of 16) run by the six-bit slice form of the scheme (error-free splitting, Ozaki, Ogita,
- *                Oishi and Rump, Numer. Algorithms 59, 2012) with `oz_slices` slices.  The adjoint's
- *                O(r^6) GEMMs run by the modular form. */
+ *                that of FP64 FMA.  The O(r^5) products (the transformation by 1D and the products of the pairs)
+ *                run with 8 slices or fewer by the digit form of the scheme (error-free splitting, Ozaki, Ogita,
+ *                Oishi and Rump, Numer. Algorithms 59, 2012) in ceil(6 oz_slices / 8) eight-bit digits, with
+ *                more in double-float FP32.  The adjoint's O(r^6) GEMMs run by the modular form. */
 typedef enum { ACSE_FP64 = 0, ACSE_BF16X3 = 1, ACSE_TF32 = 2, ACSE_TF32X3 = 3, ACSE_OZAKI = 4 } acse_prec;
 /* 3-RDM reconstruction (Eq. 3rdm_recon / Eq. NY):
  *   ACSE_RECON_V   Valdemoro: the 3-cumulant is neglected;
@@ -107,8 +107,8 @@ typedef struct {
                         * n_beta.  The library does not symmetrise D: on an asymmetric D the
                         * beta-beta results are those of the alpha-alpha block.             */
     int oz_slices;     /* ACSE_OZAKI: accuracy in 6-bit units, 4..10; 0 -> 8: the O(r^6) GEMM
-                        * operands keep min(6 oz_slices, 53) bits, the O(r^5) products use
-                        * oz_slices six-bit slices                                          */
+                        * operands keep min(6 oz_slices, 53) bits, the O(r^5) products at least
+                        * min(6 oz_slices, 48)                                              */
     int refine;        /* precision schedule of acse_step: 0 off; 1 the steps run in `prec` (any precision,
                         * ACSE_OZAKI with oz_slices included) until the switch rule fires, every later step
                         * in ACSE_OZAKI with refine_slices slices (FP64-accurate), from the same D and

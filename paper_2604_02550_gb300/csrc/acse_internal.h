@@ -278,6 +278,7 @@ int launch_xform_oz(struct acse_ctx* c, const double* const in[3], double* const
 // out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] for eight classes (bit c of tt, gt: T, G read transposed)
 int launch_rows_oz(struct acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
                    double* const out[8]);   // acse_zoz.cu
+bool rows_oz_applies(const struct acse_ctx* c);   // the digit kernels of acse_zoz.cu serve this context
 int launch_Bx_oz(struct acse_ctx* c);                                                           // acse_zoz.cu
 int launch_Bx_tc(acse_ctx* c);                                                           // acse_btc.cu
 int tiled_set_attrs();

@@ -857,7 +857,7 @@ int oz_plan_create(acse_ctx* c) {
     const int bn = R2 >= 256 ? OZ_BN : 128, pair = c->opt.gemm_tile != 1;
     ACSE_TRY(oz_plan_init(pl, c->opt.oz_slices, bn, pair, S2));
     // the B products on the tensor cores (acse_zoz.cu): x1 and x2^T of the four types for every pair
-    if (r % 16 == 0 && r <= 64 && c->opt.oz_slices <= 8)
+    if (rows_oz_applies(c))
         for (int k = 0; k < 8; ++k)
             if (cudaMalloc((void**)&c->w.bx64[k], (size_t)R2 * R2 * sizeof(double)) != cudaSuccess) {
                 cudaGetLastError();
