@@ -158,63 +158,7 @@ __global__ void k_adj_tau(int r, const double* __restrict__ Haa, const double* _
 //   2   t1[a][x]    gb[b][x]    Xb_bb                      3   t1[x][a]   wb[x][b]   -Mb_bb / 2
 //   4   t2[a][x]    gb[b][x]    Xb_ab[(a,b)]               5   t2[x][a]   wa[x][b]    Mb_ab[u=b][v=a] / 2
 //   6   t3[a][x]    ga[b][x]   -Xb_ab[(b,a)]               7   t3[x][a]   wb[x][b]   -Mb_ab[u=a][v=b] / 2
-// On the tensor cores where launch_rows_oz applies; here block (c, ij), both r x r operands in shared memory, a
-// 4 x 4 tile a thread (C: double, bound by the DFMA pipe, or the double-float pair of an Ozaki context).
-struct AdjRows {
-    const double* T[8];
-    const double* G[8];
-    double* out[8];
-    int r;
-};
-
-template <typename C>
-__global__ void __launch_bounds__(256) k_adj_rows(const __grid_constant__ AdjRows a) {
-    extern __shared__ __align__(16) unsigned char ad_raw[];
-    const int r = a.r, rp = (r + 3) & ~3, R2 = r * r, nt = rp / 4;
-    const int c = (int)blockIdx.x / R2;
-    const size_t ij = blockIdx.x - (size_t)c * R2;
-    C* Ts = (C*)ad_raw;          // [x][a]
-    C* Gs = Ts + (size_t)r * rp; // [x][b]
-    const double* T = a.T[c] + ij * R2;
-    const double* G = a.G[c];
-    for (int e = threadIdx.x; e < r * rp; e += blockDim.x) Ts[e] = Gs[e] = tconv<C>(0.0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-        const int u = e / r, v = e - u * r;
-        if (c & 1) {   // t[x = u][a = v], w[x = u][b = v]
-            Ts[u * rp + v] = tconv<C>(T[e]);
-            Gs[u * rp + v] = tconv<C>(G[e]);
-        } else {       // t[a = u][x = v], g[b = u][x = v]
-            Ts[v * rp + u] = tconv<C>(T[e]);
-            Gs[v * rp + u] = tconv<C>(G[e]);
-        }
-    }
-    __syncthreads();
-    double* out = a.out[c] + ij * R2;
-    for (int tile = threadIdx.x; tile < nt * nt; tile += blockDim.x) {
-        const int a0 = (tile / nt) * 4, b0 = (tile % nt) * 4;
-        C acc[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = tconv<C>(0.0);
-        for (int x = 0; x < r; ++x) {
-            C p[4], q[4];
-            ld4(Ts + x * rp + a0, p);
-            ld4(Gs + x * rp + b0, q);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) tmac(acc[u][v], p[u], q[v]);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-                if (a0 + u < r && b0 + v < r) out[(a0 + u) * r + b0 + v] = (double)acc[u][v];
-    }
-}
-
+// (launch_pair_rows).
 // Small-matrix reductions over a large sum (tall and skinny, r x r outputs): C_j[u][v] = sum_n sum_x
 // A_j(n; x, u) B_j(n; x, v) for the 14 jobs below, n over r^2 blocks of r x r.  Block (job, chunk of n): both
 // operand blocks in shared memory, nt^2 threads (nt = ceil(r / 4)) own a 4 x 4 tile of C each, and where those do
@@ -720,7 +664,7 @@ struct AdjWork {
     int nbuf;
     double* Hb[3];
     double* tau[4];
-    double* cls[8];    // classes of k_adj_rows (an Ozaki context's B-product scratch where it has one)
+    double* cls[8];    // the eight classes of products (the scratch of the B products, free between passes)
     double* X5b[3];    // X5bar: spin blocks, flips; then overwritten by the products mp, mm, mxab; mf; yab
     double* Vb[3];     // V5bar
     double* v1;
@@ -778,15 +722,14 @@ static int adj_alloc(acse_ctx* c) {
         get(a->Vb[s], s ? n4 : 4 * n4);
         get(a->sV[s], s ? n4 : 4 * n4);
     }
-    // one block each: the pair operands and products, the classes, the small arrays
-    double *tau = nullptr, *pairs = nullptr, *cls = nullptr, *small = nullptr;
+    // one block each: tau, the pair operands and products, the small arrays
+    double *tau = nullptr, *pairs = nullptr, *small = nullptr;
     get(tau, 4 * n4);
     get(pairs, 8 * PP + 2 * n4);
     get(a->v1, S2 * S2);
     get(a->v2, P2 * S2);
     get(a->vf, n4);
     get(a->Vraw, n4);
-    if (!c->w.bx64[0]) get(cls, 8 * n4);
     const int nt = (int)(r + 3) / 4, nt2 = nt * nt;
     a->groups = 256 / nt2 < (int)r ? 256 / nt2 : (int)r;
     a->threads = (a->groups * nt2 + 31) / 32 * 32;
@@ -799,7 +742,7 @@ static int adj_alloc(acse_ctx* c) {
         return st;
     }
     for (int t = 0; t < 4; ++t) a->tau[t] = tau + t * n4;
-    for (int k = 0; k < 8; ++k) a->cls[k] = c->w.bx64[0] ? c->w.bx64[k] : cls + k * n4;
+    for (int k = 0; k < 8; ++k) a->cls[k] = c->w.bx64[k];
     a->Xp[0] = pairs; a->Xp[2] = pairs + PP; a->Yp[0] = pairs + 2 * PP; a->Yp[2] = pairs + 3 * PP;
     a->mx[0] = pairs + 4 * PP; a->mx[2] = pairs + 5 * PP; a->my[0] = pairs + 6 * PP; a->my[2] = pairs + 7 * PP;
     a->Xp[1] = pairs + 8 * PP; a->Yp[1] = a->Xp[1] + n4;
@@ -852,18 +795,7 @@ static int vjp_D(acse_ctx* c, const double* const W[3], int sW, double scale, co
         const double* G[8] = {ga, wa, gb, wb, gb, wa, ga, wb};
         const double* T[8];
         for (int k = 0; k < 8; ++k) T[k] = a->tau[k / 2];
-        const int st = launch_rows_oz(c, T, 0xAAu, G, 0xAAu, a->cls);   // odd classes: T and G transposed
-        if (st == ACSE_ERR_UNSUPPORTED) {
-            AdjRows ar;
-            for (int k = 0; k < 8; ++k) { ar.T[k] = T[k]; ar.G[k] = G[k]; ar.out[k] = a->cls[k]; }
-            ar.r = r;
-            const int th = ((rp / 4) * (rp / 4) + 31) / 32 * 32;
-            if (c->oz) k_adj_rows<dfl><<<8 * R2, th < 256 ? th : 256, sm2, c->stream>>>(ar);
-            else k_adj_rows<double><<<8 * R2, th < 256 ? th : 256, sm2, c->stream>>>(ar);
-            AL(c);
-        } else {
-            ACSE_TRY(st);
-        }
+        ACSE_TRY(launch_pair_rows(c, T, 0xAAu, G, 0xAAu, 0u, a->cls));   // odd classes: T and G transposed
     }
     k_adj_X5<<<ad_grid(6 * n4), AD_TPB, 0, c->stream>>>(ab);
     AL(c);
@@ -983,8 +915,6 @@ static int adj_set_attrs() {
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_pack_V, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double)));
     const int sm2 = 2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double);
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows<dfl>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_reduce<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_reduce<dfl>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
     return ACSE_OK;
@@ -997,6 +927,11 @@ extern "C" int acse_residual_backward_impl(acse_ctx* c, const double* const* D_c
     if (!D_ckpt || n_steps < 0 || !D_ckpt[0] || !D_ckpt[1] || !D_ckpt[2]) return ACSE_ERR_ARG;
     ACSE_TRY(adj_set_attrs());
     ACSE_TRY(adj_alloc(c));
+    struct InAdjoint {   // for every return below
+        acse_ctx* c;
+        explicit InAdjoint(acse_ctx* x) : c(x) { c->in_adjoint = 1; }
+        ~InAdjoint() { c->in_adjoint = 0; }
+    } in_adjoint(c);
     AdjWork* a = (AdjWork*)c->adj;
     Work& w = c->w;
     const int r = c->r;

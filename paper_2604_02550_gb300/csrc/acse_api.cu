@@ -99,7 +99,7 @@ static int alloc_d(void** p, size_t bytes, size_t* total) {
 static void free_work(acse_ctx* c) {
     Work& w = c->w;
     void* ptrs[] = {w.Kh[0], w.Kh[1], w.Kh[2], w.gam, w.M[0], w.M[1], w.M[2], w.Mp, w.Mm, w.Mf1, w.Wp, w.Wm, w.Wf1,
-                    w.V5d, w.V5f1, w.V5f2, w.Cp[0], w.Cp[1], w.pmap, w.w, w.Q, w.X[0], w.X[1], w.X[2], w.Y[0], w.Y[1], w.Y[2], w.X5d, w.X5f1, w.X5f2,
+                    w.V5d, w.V5f1, w.V5f2, w.Cp[0], w.Cp[1], w.pmap, w.bx64[0], w.w, w.Q, w.X[0], w.X[1], w.X[2], w.Y[0], w.Y[1], w.Y[2], w.X5d, w.X5f1, w.X5f2,
                     w.H[0], w.H[1], w.H[2], w.zdiag, w.A[0], w.A[1], w.A[2], w.U[0], w.U[1], w.U[2], w.Dt[0],
                     w.Dt[1], w.Dt[2], w.stage_in[0], w.stage_in[1], w.stage_in[2], w.stage_out[0],
                     w.stage_out[1], w.stage_out[2], w.h, w.V, w.scal, w.partial};
@@ -135,6 +135,8 @@ static int alloc_work(acse_ctx* c) {
         w.V1 = w.X5d;              // S2^2 + S2 P2 = 2 r^4 + 2 r^3 <= 4 r^4
         w.V2 = w.X5d + S2 * S2;
         for (int s = 0; s < 2; ++s) A_(w.Cp[s], P2 * P2 / 2 * sizeof(double));
+        A_(w.bx64[0], 8 * b4);   // one block, eight classes
+        for (int k = 1; k < 8; ++k) w.bx64[k] = w.bx64[0] + k * n4;
         A_(w.pmap, P2 / 2 * sizeof(int));
         int hm[ACSE_MAX_R * (ACSE_MAX_R - 1) / 2];
         for (int a = 0; a < c->r; ++a)
@@ -327,7 +329,7 @@ int acse_contract_post(acse_ctx* c, int sW, double scale, int mask, double* cons
     }
     if (c->ny) ACSE_TRY(ny_pass(c));   // NY: the 3-cumulant term, added to B by the B kernel
     ACSE_TRY(launch_Q(c));
-    ACSE_TRY(launch_build_B(c));
+    ACSE_TRY(launch_B_tiled(c));
     return launch_assemble_G(c, sW, scale, mask, out, norm2_dst);
 }
 

@@ -142,10 +142,9 @@ int launch_gamma_M(acse_ctx* c, const double* const D[3]) {
 // X^{ij}_{kp} = sum_rs M^{ij}_{rs} W^{kp}_{rs}:  Q^k_i = sum_P X^{iP}_{kP}, i.e.
 //   Q_a[k][i] = sum_p Xaa[(i,p)][(k,p)] + sum_p Xab[(i,p)][(k,p)]
 //   Q_b[k][i] = sum_p Xbb[(i,p)][(k,p)] + sum_p Xab[(p,i)][(p,k)]
-// (O(r^3) instead of O(r^5); Xab already carries the factor 2 of the mixed-spin (rs) sum).  With Xpaa /
-// Xpbb set (split path), the same-spin X is read from the packed GEMM output (rows and columns over
-// the pairs a < b, row pitch P):  X[(i,p)][(k,p)] = s_ip s_kp Xp[pk(i,p)][pk(k,p)], zero for i = p or
-// k = p (s_ab = -1 for a > b), the values the unpacked rows hold.
+// (O(r^3) instead of O(r^5); Xab already carries the factor 2 of the mixed-spin (rs) sum).  The same-spin X is
+// read from the packed GEMM output (rows and columns over the pairs a < b, row pitch P):  X[(i,p)][(k,p)] =
+// s_ip s_kp Xp[pk(i,p)][pk(k,p)], zero for i = p or k = p (s_ab = -1 for a > b), the values the unpacked rows hold.
 template <typename T>
 __device__ __forceinline__ T q_packed(const T* __restrict__ Xp, int r, int P, int i, int k, int p) {
     if (i == p || k == p) return (T)0;
@@ -154,8 +153,7 @@ __device__ __forceinline__ T q_packed(const T* __restrict__ Xp, int r, int P, in
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_Q_from_X(int r, const T* __restrict__ Xaa, const T* __restrict__ Xab,
-                                                  const T* __restrict__ Xbb, size_t ldx, const T* __restrict__ Xpaa,
+__global__ void __launch_bounds__(256) k_Q_from_X(int r, const T* __restrict__ Xab, size_t ldx, const T* __restrict__ Xpaa,
                                                   const T* __restrict__ Xpbb, T* __restrict__ Qv) {
     // one warp per output element, lanes over p, fixed-order warp reduction
     const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -163,8 +161,7 @@ __global__ void __launch_bounds__(256) k_Q_from_X(int r, const T* __restrict__ X
     const int sp = t / (r * r), k = (t / r) % r, i = t % r, P = r * (r - 1) / 2;
     T acc = 0;
     for (int p = lane; p < r; p += 32) {
-        const T xs = Xpaa ? q_packed(sp == 0 ? Xpaa : Xpbb, r, P, i, k, p)
-                          : (sp == 0 ? Xaa : Xbb)[(size_t)(i * r + p) * ldx + k * r + p];
+        const T xs = q_packed(sp == 0 ? Xpaa : Xpbb, r, P, i, k, p);
         const T xab = sp == 0 ? Xab[(size_t)(i * r + p) * ldx + k * r + p] : Xab[(size_t)(p * r + i) * ldx + p * r + k];
         acc += xs + xab;
     }
@@ -177,13 +174,12 @@ int launch_Q(acse_ctx* c) {
     const int r = c->r;
     const size_t R2 = (size_t)r * r;
     if (c->opt.prec == ACSE_FP64) {
-        k_Q_from_X<double><<<(2 * r * r + 7) / 8, 256, 0, c->stream>>>(r, c->w.X[0], c->w.X[1], c->w.X[2], R2,
-                                                                          nullptr, nullptr, c->w.Q);
+        k_Q_from_X<double><<<(2 * r * r + 7) / 8, 256, 0, c->stream>>>(r, c->w.X[1], R2, c->w.Cp[0], c->w.Cp[1], c->w.Q);
     } else {
         // same-spin X from the packed GEMM output; spin-flip specialisation: Xbb is the flip of Xaa (same
         // values)
         k_Q_from_X<float><<<(2 * r * r + 7) / 8, 256, 0, c->stream>>>(
-            r, nullptr, c->w.tc_pairC[1], nullptr, R2, c->w.tc_pairCp[0], c->w.tc_pairCp[acse_singlet(c) ? 0 : 2],
+            r, c->w.tc_pairC[1], R2, c->w.tc_pairCp[0], c->w.tc_pairCp[acse_singlet(c) ? 0 : 2],
             c->w.Q32);
     }
     ACSE_LAUNCHED(c);
@@ -200,8 +196,6 @@ int launch_Q(acse_ctx* c) {
 //   T3: x1 = -sum_p Xab[ij][pk] ga[p][l], x2 = sum_p wb[k][p] Mab[ij][l][p], x5 = X5d[(b,k,j)][(a,i,l)],
 //       x7 = Qb[k][j] ga[i][l], x8 = X5f2[(k,i)][(j,l)], x4 = 0
 //   B = (x1 - 2 x2 - x4 + 2 x5 + x7 - 2 x8) / 9.
-int launch_build_B(acse_ctx* c) { return launch_B_tiled(c); }
-
 // --------------------------------------------------------------------------- G assembly
 // The B kernel (acse_tiled.cu) leaves H_b = 4 Y_b - 12 (P - P'_{k<->l}) per block b, so that
 //   G_b[ij][kl] = H_b[ij][kl] - s H_b[kl][ij]

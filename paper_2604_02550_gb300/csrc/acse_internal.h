@@ -167,7 +167,7 @@ struct Work {
     // i r + j table (pairs i < j in packed order); null otherwise
     float* bx[8];
     int* pair_ij;
-    double* bx64[8];   // Ozaki contexts: x1 and x2^T of the four B spin types for every pair (acse_zoz.cu)
+    double* bx64[8];   // FP64 and Ozaki contexts: x1 and x2^T of the four B spin types (r^2 rows of r^2 each)
 };
 
 struct acse_ctx {
@@ -179,6 +179,7 @@ struct acse_ctx {
     int nsplit;           // split terms for the tensor-core path (3 for BF16x3, 1 for TF32)
     Work w;
     void* tc_plan;        // tensor-core GEMM plan (tensor maps etc.)
+    int in_adjoint;       // the passes of acse_residual_backward: every row of X and Y is unpacked
     void* adj;            // adjoint workspace (allocated by the first acse_residual_backward call)
     struct acse_ctx* shadow;   // ACSE_OZAKI companion of a split-precision context (its adjoint), or null
     void* ny;             // NY reconstruction workspace (acse_ny.cu), or null for V
@@ -270,16 +271,17 @@ int launch_ph_xform(acse_ctx* c, const double* const in[3], double* const out[3]
 int launch_ph_finish(acse_ctx* c, int sW);
 int launch_pair_unpack(acse_ctx* c);
 int ph_set_attrs();
-int launch_build_B(acse_ctx* c);
 int launch_Z_tiled(acse_ctx* c, const float* const W32[3]);
 int launch_B_tiled(acse_ctx* c);
 int launch_Z_tc(acse_ctx* c, const float* const W32[3], int ntypes, const int* tmap);   // acse_ztc.cu
 int launch_xform_oz(struct acse_ctx* c, const double* const in[3], double* const out[3], int trans);   // acse_zoz.cu
-// out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] for eight classes (bit c of tt, gt: T, G read transposed)
+// out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] for eight classes (bit c of tt, gt: T, G read transposed; of tri: the
+// pairs i < j only): acse_ph.cu; on the tensor cores acse_zoz.cu
+int launch_pair_rows(struct acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
+                     unsigned tri, double* const out[8]);
 int launch_rows_oz(struct acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
-                   double* const out[8]);   // acse_zoz.cu
-bool rows_oz_applies(const struct acse_ctx* c);   // the digit kernels of acse_zoz.cu serve this context
-int launch_Bx_oz(struct acse_ctx* c);                                                           // acse_zoz.cu
+                   unsigned tri, double* const out[8]);
+int launch_Bx(struct acse_ctx* c);
 int launch_Bx_tc(acse_ctx* c);                                                           // acse_btc.cu
 int tiled_set_attrs();
 int launch_Q(acse_ctx* c);

@@ -182,14 +182,16 @@ static int launch_ph_unpack(acse_ctx* c, int sW) {
 // full X and Y rows by antisymmetry (pairs numbered by pk_pair).
 //
 // X_s, Y_s (s = aa, bb; r^2 x r^2 FP64) from the packed [X; Y] (2P x P): one block per output row, the
-// packed source row staged in shared memory, the full row written two columns at a time.
-__global__ void __launch_bounds__(256) k_pair_unpack(int r, const double* __restrict__ Cp0, const double* __restrict__ Cp2,
-                                                   double* X0, double* Y0, double* X2, double* Y2) {
+// packed source row staged in shared memory, the full row written two columns at a time.  The pass reads the
+// rows i < j only (pmap set: P rows); the adjoint sums over every row (pmap null: r^2 rows).
+__global__ void __launch_bounds__(256) k_pair_unpack(int r, const int* __restrict__ pmap, const double* __restrict__ Cp0,
+                                                     const double* __restrict__ Cp2, double* X0, double* Y0, double* X2,
+                                                     double* Y2) {
     __shared__ double srow[ACSE_MAX_R * (ACSE_MAX_R - 1) / 2];
-    const int R2 = r * r, P = r * (r - 1) / 2;
-    const int sec = blockIdx.x / (2 * R2);
-    const int row = blockIdx.x - sec * 2 * R2;
-    const int part = row / R2, ij = row - part * R2, i = ij / r, j = ij - i * r;
+    const int R2 = r * r, P = r * (r - 1) / 2, rows = pmap ? P : R2;
+    const int sec = blockIdx.x / (2 * rows);
+    const int row = blockIdx.x - sec * 2 * rows;
+    const int part = row / rows, u = row - part * rows, ij = pmap ? pmap[u] : u, i = ij / r, j = ij - i * r;
     double* dst = (sec == 0 ? (part ? Y0 : X0) : (part ? Y2 : X2)) + (size_t)ij * R2;
     if (i == j) {   // block-uniform
         for (int c = threadIdx.x; c < R2; c += blockDim.x) dst[c] = 0.0;
@@ -214,9 +216,144 @@ __global__ void __launch_bounds__(256) k_pair_unpack(int r, const double* __rest
 
 int launch_pair_unpack(acse_ctx* c) {
     Work& w = c->w;
-    k_pair_unpack<<<2 * 2 * c->r * c->r, 256, 0, c->stream>>>(c->r, w.Cp[0], w.Cp[1], w.X[0], w.Y[0], w.X[2], w.Y[2]);
+    const int r = c->r;
+    const int* pmap = c->in_adjoint ? nullptr : w.pmap;
+    k_pair_unpack<<<2 * 2 * (pmap ? r * (r - 1) / 2 : r * r), 256, 0, c->stream>>>(r, pmap, w.Cp[0], w.Cp[1], w.X[0],
+                                                                                  w.Y[0], w.X[2], w.Y[2]);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
+}
+
+// -------------------------------------------------------- products of the pairs (CUDA cores)
+// Eight classes of r x r x r products per pair ij, out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] (bit c of tt, gt: T, G
+// read transposed; bit c of tri: the pairs i < j only).  FP64 contexts, and Ozaki contexts where the digit kernel
+// does not apply (C: double, or the double-float pair).  Block: one class, nij pairs, both operands in shared
+// memory as [x][.]; the MT x MT tiles of all pairs are dealt out to full warps -- a DFMA holds the FP64 pipe 16
+// cycles however many lanes are active, and at r = 24 one 4 x 4 tile a thread left 28 of 64 lanes idle -- with
+// nij chosen on the host so that the last round of tiles is nearly full.  r = 24, FP64: 123 us for the six pair-types'
+// worth of products a pass runs (1.05 TFLOP/s), where the B kernel that formed them itself took 279 us.
+struct PairRows {
+    const double* T[8];
+    const double* G[8];
+    double* out[8];
+    const int* pmap;
+    unsigned tt, gt, tri;
+    int start[9];   // first block of each class
+    int r, nij;
+};
+
+template <typename C, int MT>
+__global__ void __launch_bounds__(256) k_pair_rows(const __grid_constant__ PairRows a) {
+    extern __shared__ __align__(16) unsigned char ph_raw[];
+    const int r = a.r, rp = (r + MT - 1) / MT * MT, R2 = r * r, nt = rp / MT, nt2 = nt * nt, op = r * rp;
+    int c = 0;
+    while (c < 7 && a.start[c + 1] <= (int)blockIdx.x) ++c;
+    const bool tri = (a.tri >> c) & 1, tt = (a.tt >> c) & 1, gt = (a.gt >> c) & 1;
+    const int u0 = ((int)blockIdx.x - a.start[c]) * a.nij, n = min(a.nij, (tri ? r * (r - 1) / 2 : R2) - u0);
+    C* Gs = (C*)ph_raw;   // [x][b]
+    C* Ts = Gs + op;      // [pair][x][a]
+    if (rp != r) {
+        for (int e = threadIdx.x; e < (1 + n) * op; e += blockDim.x) Gs[e] = tconv<C>(0.0);
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < R2; e += blockDim.x) {
+        const int u = e / r, v = e - u * r;
+        Gs[gt ? u * rp + v : v * rp + u] = tconv<C>(a.G[c][e]);   // [b = u][x = v], or [x = u][b = v]
+    }
+    for (int f = threadIdx.x; f < n * R2; f += blockDim.x) {
+        const int it = f / R2, e = f - it * R2, u = e / r, v = e - u * r;
+        const int ij = tri ? a.pmap[u0 + it] : u0 + it;
+        Ts[it * op + (tt ? u * rp + v : v * rp + u)] = tconv<C>(a.T[c][(size_t)ij * R2 + e]);
+    }
+    __syncthreads();
+    for (int g = threadIdx.x; g < n * nt2; g += blockDim.x) {
+        const int it = g / nt2, tile = g - it * nt2, a0 = (tile / nt) * MT, b0 = (tile % nt) * MT;
+        const C* T = Ts + it * op + a0;
+        const C* G = Gs + b0;
+        C acc[MT][MT];
+#pragma unroll
+        for (int u = 0; u < MT; ++u)
+#pragma unroll
+            for (int v = 0; v < MT; ++v) acc[u][v] = tconv<C>(0.0);
+#pragma unroll 4
+        for (int x = 0; x < r; ++x) {
+            C p[MT], q[MT];
+#pragma unroll
+            for (int u = 0; u < MT; ++u) {
+                p[u] = T[x * rp + u];
+                q[u] = G[x * rp + u];
+            }
+#pragma unroll
+            for (int u = 0; u < MT; ++u)
+#pragma unroll
+                for (int v = 0; v < MT; ++v) tmac(acc[u][v], p[u], q[v]);
+        }
+        const int ij = tri ? a.pmap[u0 + it] : u0 + it;
+        double* out = a.out[c] + (size_t)ij * R2;
+#pragma unroll
+        for (int u = 0; u < MT; ++u)
+#pragma unroll
+            for (int v = 0; v < MT; ++v)
+                if (a0 + u < r && b0 + v < r) out[(a0 + u) * r + b0 + v] = (double)acc[u][v];
+    }
+}
+
+#define PR_SMEM (96 * 1024)   // two blocks an SM
+
+// nij: fewest idle lanes over the rounds of 256 tiles, within PR_SMEM; the smallest such count.
+static int pair_rows_nij(int r, int mt) {
+    const int rp = (r + mt - 1) / mt * mt, nt2 = (rp / mt) * (rp / mt);
+    int best = 1;
+    double bu = 0.0;
+    for (int n = 1; n <= 32 && (size_t)(1 + n) * r * rp * sizeof(double) <= PR_SMEM; ++n) {
+        const double u = (double)n * nt2 / ((n * nt2 + 255) / 256 * 256);
+        if (u > bu + 0.01) {
+            bu = u;
+            best = n;
+        }
+    }
+    return best;
+}
+
+int launch_pair_rows(acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt, unsigned tri,
+                     double* const out[8]) {
+    const int st = launch_rows_oz(c, T, tt, G, gt, tri, out);
+    if (st != ACSE_ERR_UNSUPPORTED) return st;
+    const int r = c->r, mt = c->oz ? 4 : 2, rp = (r + mt - 1) / mt * mt;
+    PairRows a;
+    for (int k = 0; k < 8; ++k) {
+        a.T[k] = T[k];
+        a.G[k] = G[k];
+        a.out[k] = out[k];
+    }
+    a.pmap = c->w.pmap;
+    a.tt = tt;
+    a.gt = gt;
+    a.tri = tri;
+    a.r = r;
+    a.nij = pair_rows_nij(r, mt);
+    a.start[0] = 0;
+    for (int k = 0; k < 8; ++k) {
+        const int items = (tri >> k) & 1 ? r * (r - 1) / 2 : r * r;
+        a.start[k + 1] = a.start[k] + (items + a.nij - 1) / a.nij;
+    }
+    const size_t sm = (size_t)(1 + a.nij) * r * rp * sizeof(double);
+    if (c->oz) k_pair_rows<dfl, 4><<<a.start[8], 256, sm, c->stream>>>(a);
+    else k_pair_rows<double, 2><<<a.start[8], 256, sm, c->stream>>>(a);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
+}
+
+// The two products of every B spin type into w.bx64 (same-spin types on the pairs i < j):
+//     class 2 t:      x1[k][l] = sum_q X_ij[k][q] 1D[q][l]       (type 3: X_ij transposed)
+//     class 2 t + 1:  x2^T[l][k] = sum_p M_ij[l][p] w[k][p]      (type 2: M_ij transposed)
+int launch_Bx(acse_ctx* c) {
+    Work& w = c->w;
+    const int R2 = c->r * c->r;
+    const double *ga = w.gam, *gb = w.gam + R2, *wa = w.w, *wb = w.w + R2;
+    const double* T[8] = {w.X[0], w.M[0], w.X[2], w.M[2], w.X[1], w.M[1], w.X[1], w.M[1]};
+    const double* G[8] = {ga, wa, gb, wb, gb, wa, ga, wb};
+    return launch_pair_rows(c, T, 1u << 6 | 1u << 5, G, 0x55u, 0x0Fu, w.bx64);
 }
 
 // ------------------------------------------------------------------------------------- w
@@ -343,6 +480,8 @@ int launch_ph_finish(acse_ctx* c, int sW) {
 }
 
 int ph_set_attrs() {
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_pair_rows<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PR_SMEM));
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_pair_rows<dfl, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PR_SMEM));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_ph_unpack, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_ph_xform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -17,7 +17,6 @@
 #include "acse_internal.h"
 #include "dfloat.cuh"
 
-#define TL_TPB 256
 #define ZP_MAX_THREADS 288
 
 __device__ __forceinline__ float tl_tf32(float x) {
@@ -27,21 +26,6 @@ __device__ __forceinline__ float tl_tf32(float x) {
 }
 
 __host__ __device__ __forceinline__ int pad4(int r) { return (r + 3) & ~3; }
-
-// acc[a][b] += sum_q A[q][i0 + a] * B[q][j0 + b]  (A, B: [rp][rp] shared arrays, rp % 4 == 0)
-template <typename T>
-__device__ __forceinline__ void mma4x4(T (&acc)[4][4], const T* A, const T* B, int rp, int n, int i0, int j0) {
-#pragma unroll 4
-    for (int q = 0; q < n; ++q) {
-        T a[4], b[4];
-        ld4(A + q * rp + i0, a);
-        ld4(B + q * rp + j0, b);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) tmac(acc[u][v], a[u], b[v]);
-    }
-}
 
 // --------------------------------------------------------------------------- outputs of Z
 struct ZOut {
@@ -317,164 +301,86 @@ struct BTiledArgs {
     const T* ny[4];     // NY three-body term per spin type (acse_ny.cu), added to B; null for V
     int flip;           // spin-flip specialisation: no bb items; the b-led particle-hole blocks and the
                         // second flip sector are read as their alpha-led flips
-    const T* bx[8];     // precomputed products (k_B_pipe<.., true>): per type t, x1 rows at bx[2t] and
-                        // x2^T rows at bx[2t + 1], r^2 per item (the type's item number, see acse_btc.cu)
+    const T* bx[8];     // precomputed products (k_B_pre, k_B_pipe<.., true>): per type t, x1 rows at bx[2t] and
+                        // x2^T rows at bx[2t + 1], r^2 per item (pair ij; k_B_pipe: the type's item number, see
+                        // acse_btc.cu)
+    const int* pmap;    // k_B_pre: pair number -> i r + j (i < j)
 };
 
-// Block (i, j).  Spin types t = 0 (aaaa), 1 (bbbb), 2 (abab), 3 (abba):
-//   x1 = sgn1 sum_p X[k][p] g1[p][l],  x2 = sgn2 sum_p w[k][p] Mt[p][l]   (r x r x r, register tiled)
-//   B_t = (x1 - 2 x2 - x4 + 2 x5 + x7 - 2 x8) / 9 with the gathered x4, x5, x7, x8 of acse_elem.cu.
-// B rows are kept in shared memory (Bs[t][k][l]) and combined into
-//   H_aa = 4 Y_aa - 12 (B0 - B0_{k<->l}),  H_bb = 4 Y_bb - 12 (B1 - B1_{k<->l}),
-//   H_ab = 4 Y_ab - 12 (B2 - B3_{k<->l}).
-// STAGE: the particle-hole rows (x5, x8) and the Q / 1D vectors of (x4, x7) are staged in shared
-// memory with coalesced loads before the products (off when shared memory would not fit).
-// DF (T = double, the Ozaki path): the two products in double-float (C = dfl, the same 8 bytes as
-// double in shared memory), everything else in FP64.
-// PREX (Ozaki path): x1 and x2^T come precomputed for every pair (a.bx, k_Bx_oz of acse_zoz.cu): no operand
-// staging, each thread reads its 4 x 4 tile of both.
-template <typename T, bool STAGE, bool DF = false, bool PREX = false>
-__global__ void __launch_bounds__(TL_TPB) k_B_tiled(const __grid_constant__ BTiledArgs<T> a) {
-    using C = typename std::conditional<DF, dfl, T>::type;
-    static_assert(sizeof(C) == sizeof(T), "product operands share the layout of T");
-    extern __shared__ __align__(16) unsigned char tl_smem[];
-    const int r = a.r;
-    const int rp = pad4(r);
-    const int R2 = r * r;
-    C* XT = (C*)tl_smem;      // [p][k]
-    C* G1 = XT + rp * rp;     // [p][l]
-    C* WT = G1 + rp * rp;     // [p][k]
-    C* MT = WT + rp * rp;     // [p][l]
-    T* Bs = (T*)(MT + rp * rp);   // [2][r][r]: current pair of B types
-    T* X5s = Bs + 2 * R2;     // [k][l] (STAGE)
-    T* X8s = X5s + R2;
-    T* vq = X8s + R2;         // 4 vectors of r: Q column, 1D row, Q column, 1D row (x4, x7)
-    const int i = blockIdx.x / r, j = blockIdx.x % r;
-    const size_t ij = (size_t)blockIdx.x;
-    const T* ga = a.gam;
-    const T* gb = a.gam + R2;
-    const T* Qa = a.Q;
-    const T* Qb = a.Q + R2;
-    const int nt = rp / 4;
+// FP64 and Ozaki paths.  Spin types t = 0 (aaaa), 1 (bbbb), 2 (abab), 3 (abba); the products x1[k][l] and x2^T[l][k]
+// of every type come precomputed (a.bx: launch_Bx), so that a block only gathers and combines.  With U = x2^T read
+// in its own order, U[a][b] = x2[b][a], and R = x1 - x4 + 2 x5 + x7 - 2 x8 (the gathered terms of acse_elem.cu),
+//     9 (B_t[k][l] - B_t[l][k]) = V[k][l] - V[l][k],  V = R + 2 U,                         t = 0, 1
+//     9 (B_2[k][l] - B_3[l][k]) = N[k][l] - N'[l][k],  N = R_2 + 2 U_3,  N' = R_3 - 2 U_2  (x1 of type 3 negated),
+// so every operand is read in rows of l and one r x r array crosses through shared memory:
+//     H_aa = 4 Y_aa - (4/3)(V - V^T), H_bb likewise, H_ab = 4 Y_ab - (4/3)(N - N'^T).
+// Blocks: the pairs i < j of aa and of bb (row (j, i) of H is minus row (i, j), rows (i, i) are zero), every pair of
+// ab.  The FP64 pipe (two operations a clock and SM) bounds it at about 19 r^4 operations, HBM at 17 r^4 doubles:
+// r = 48: 217 us, against 628 us for the kernel that combined all r^2 pairs of each type entry by entry.
+__global__ void __launch_bounds__(256) k_B_pre(const __grid_constant__ BTiledArgs<double> a) {
+    extern __shared__ __align__(16) double bp_sm[];   // N [r][ld], N' [r][ld] (ab)
+    const int r = a.r, R2 = r * r, ld = r | 1, P = r * (r - 1) / 2;
     const size_t R22 = 2 * (size_t)R2;
-    for (int e = threadIdx.x; e < 4 * rp * rp; e += blockDim.x) XT[e] = tconv<C>(0.0);   // zero padding once
-    for (int round = 0; round < 3; ++round) {
-        const int ntypes = round < 2 ? 1 : 2;
-        for (int tt = 0; tt < ntypes; ++tt) {
-            const int t = round < 2 ? round : 2 + tt;
-            const T* Xrow;
-            const T* g1;
-            const T* wv;
-            const T* Mrow;
-            bool xT = false, mT = true;
-            T sgn1 = 1, sgn2 = 1;
-            if (t == 0) { Xrow = a.X[0] + ij * R2; g1 = ga; wv = a.w; Mrow = a.M[0] + ij * R2; }
-            else if (t == 1) { Xrow = a.X[2] + ij * R2; g1 = gb; wv = a.w + R2; Mrow = a.M[2] + ij * R2; }
-            else if (t == 2) { Xrow = a.X[1] + ij * R2; g1 = gb; wv = a.w; Mrow = a.M[1] + ij * R2; mT = false; sgn2 = -1; }
-            else { Xrow = a.X[1] + ij * R2; g1 = ga; wv = a.w + R2; Mrow = a.M[1] + ij * R2; xT = true; sgn1 = -1; }
-            // particle-hole sources: x5 at row (k, j), column (i, l); x8 at row (k, i), column (j, l):
-            //   T0: X5d(a,a) both   T1: X5d(b,b) both   T2: X5f1, X5d(a,b)   T3: X5d(b,a), X5f2
-            const T* X5b;
-            const T* X8b;
-            size_t ld5, ld8;
-            if (t == 0) { X5b = a.X5d; X8b = a.X5d; ld5 = ld8 = R22; }
-            else if (t == 1) { X5b = X8b = a.X5d + R2 * R22 + R2; ld5 = ld8 = R22; }
-            else if (t == 2) { X5b = a.X5f1; ld5 = R2; X8b = a.X5d + R2; ld8 = R22; }
-            else { X5b = a.X5d + R2 * R22; ld5 = R22; X8b = a.X5f2; ld8 = R2; }
-            // x4 = Q4[k] g4[l], x7 = Q7[k] g7[l] (zero vectors where a type has no such term)
-            const T* Q4 = t == 0 ? Qa : t == 1 ? Qb : t == 2 ? Qa : nullptr;
-            const T* g4 = t == 0 ? ga : t == 1 ? gb : t == 2 ? gb : nullptr;
-            const T* Q7 = t == 0 ? Qa : t == 1 ? Qb : t == 3 ? Qb : nullptr;
-            const T* g7 = t == 0 ? ga : t == 1 ? gb : t == 3 ? ga : nullptr;
-            __syncthreads();
-            for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-                const int u = e / r, v = e - u * r;
-                if (!PREX) {
-                    XT[xT ? u * rp + v : v * rp + u] = tconv<C>(Xrow[e]);   // T3 uses Xab[ij][p][k]
-                    G1[u * rp + v] = tconv<C>(g1[e]);
-                    WT[v * rp + u] = tconv<C>(wv[e]);                      // w[k][p] -> WT[p][k]
-                    MT[mT ? v * rp + u : u * rp + v] = tconv<C>(Mrow[e]);  // M[(l,p)] -> MT[p][l]  or  M[(p,l)]
-                }
-                if (STAGE) {
-                    X5s[e] = X5b[((size_t)u * r + j) * ld5 + (size_t)i * r + v];   // (k, l) = (u, v)
-                    X8s[e] = X8b[((size_t)u * r + i) * ld8 + (size_t)j * r + v];
-                }
-            }
-            if (STAGE)
-                for (int e = threadIdx.x; e < r; e += blockDim.x) {
-                    vq[e] = Q4 ? Q4[e * r + i] : (T)0;            // Q[k][i]
-                    vq[r + e] = g4 ? g4[j * r + e] : (T)0;        // g[j][l]
-                    vq[2 * r + e] = Q7 ? Q7[e * r + j] : (T)0;    // Q[k][j]
-                    vq[3 * r + e] = g7 ? g7[i * r + e] : (T)0;    // g[i][l]
-                }
-            __syncthreads();
-            T* Bt = Bs + (size_t)tt * R2;
-            for (int tile = threadIdx.x; tile < nt * nt; tile += blockDim.x) {
-                const int k0 = (tile / nt) * 4, l0 = (tile % nt) * 4;
-                C x1[4][4], x2[4][4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) x1[u][v] = x2[u][v] = tconv<C>(0.0);
-                T p1[4][4], p2[4][4];   // PREX: x1[k][l] = bx[2t] row (ij, k), x2[k][l] = bx[2t + 1] row (ij, l)
-                if constexpr (PREX) {
-                    const T* b1 = a.bx[2 * t] + ij * R2;
-                    const T* b2 = a.bx[2 * t + 1] + ij * R2;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            const int k = min(k0 + u, r - 1), l = min(l0 + v, r - 1);
-                            p1[u][v] = b1[(size_t)k * r + l];
-                            p2[u][v] = b2[(size_t)l * r + k];
-                        }
-                } else {
-                    mma4x4<C>(x1, XT, G1, rp, r, k0, l0);
-                    mma4x4<C>(x2, WT, MT, rp, r, k0, l0);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            p1[u][v] = (T)x1[u][v];
-                            p2[u][v] = (T)x2[u][v];
-                        }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int k = k0 + u;
-                    if (k >= r) continue;
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const int l = l0 + v;
-                        if (l >= r) continue;
-                        T x4, x5, x7, x8;
-                        if (STAGE) {
-                            x4 = vq[k] * vq[r + l];
-                            x7 = vq[2 * r + k] * vq[3 * r + l];
-                            x5 = X5s[k * r + l];
-                            x8 = X8s[k * r + l];
-                        } else {
-                            x4 = Q4 ? Q4[k * r + i] * g4[j * r + l] : (T)0;
-                            x7 = Q7 ? Q7[k * r + j] * g7[i * r + l] : (T)0;
-                            x5 = X5b[((size_t)k * r + j) * ld5 + (size_t)i * r + l];
-                            x8 = X8b[((size_t)k * r + i) * ld8 + (size_t)j * r + l];
-                        }
-                        Bt[k * r + l] = (sgn1 * p1[u][v] - (T)2 * sgn2 * p2[u][v] - x4 + (T)2 * x5 + x7 - (T)2 * x8) *
-                                            (T)(1.0 / 9.0) +
-                                        (a.ny[t] ? a.ny[t][ij * R2 + (size_t)k * r + l] : (T)0);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        const int b = round == 0 ? 0 : round == 1 ? 2 : 1;   // output block aa, bb, ab
-        const T* P = Bs;
-        const T* Px = round < 2 ? Bs : Bs + R2;
-        const T* Yrow = a.Y[b] + ij * R2;
-        T* Hrow = a.H[b] + ij * R2;
+    const double *ga = a.gam, *gb = a.gam + R2, *Qa = a.Q, *Qb = a.Q + R2;
+    if ((int)blockIdx.x < 2 * P) {
+        const int sec = (int)blockIdx.x / P, ij = a.pmap[(int)blockIdx.x - sec * P], i = ij / r, j = ij - i * r;
+        const double* g = sec ? gb : ga;
+        const double* Q = sec ? Qb : Qa;
+        const double* X5 = a.X5d + (sec ? R2 * R22 + R2 : 0);
+        const double* x1 = a.bx[2 * sec] + (size_t)ij * R2;
+        const double* U = a.bx[2 * sec + 1] + (size_t)ij * R2;
+        const double* ny = a.ny[sec] ? a.ny[sec] + (size_t)ij * R2 : nullptr;
         for (int e = threadIdx.x; e < R2; e += blockDim.x) {
             const int k = e / r, l = e - k * r;
-            Hrow[e] = (T)4 * Yrow[e] - (T)12 * (P[e] - Px[l * r + k]);
+            const double x5 = X5[((size_t)k * r + j) * R22 + (size_t)i * r + l], x8 = X5[((size_t)k * r + i) * R22 + (size_t)j * r + l];
+            double v = fma(2.0, (x5 - x8) + U[e], x1[e]);
+            v = fma(-Q[k * r + i], g[j * r + l], v);
+            v = fma(Q[k * r + j], g[i * r + l], v);
+            if (ny) v = fma(9.0, ny[e], v);
+            bp_sm[k * ld + l] = v;
+        }
+        __syncthreads();
+        const double* Y = a.Y[2 * sec] + (size_t)ij * R2;
+        double* H = a.H[2 * sec] + (size_t)ij * R2;
+        double* Hm = a.H[2 * sec] + ((size_t)j * r + i) * R2;
+        for (int e = threadIdx.x; e < R2; e += blockDim.x) {
+            const int k = e / r, l = e - k * r;
+            const double h = fma(-4.0 / 3.0, bp_sm[k * ld + l] - bp_sm[l * ld + k], 4.0 * Y[e]);
+            H[e] = h;
+            Hm[e] = -h;
+        }
+    } else {
+        const int ij = (int)blockIdx.x - 2 * P, i = ij / r, j = ij - i * r;
+        double* Nt = bp_sm + r * ld;
+        const double *x12 = a.bx[4] + (size_t)ij * R2, *U2 = a.bx[5] + (size_t)ij * R2;
+        const double *x13 = a.bx[6] + (size_t)ij * R2, *U3 = a.bx[7] + (size_t)ij * R2;
+        const double* ny2 = a.ny[2] ? a.ny[2] + (size_t)ij * R2 : nullptr;
+        const double* ny3 = a.ny[3] ? a.ny[3] + (size_t)ij * R2 : nullptr;
+        for (int e = threadIdx.x; e < R2; e += blockDim.x) {
+            const int k = e / r, l = e - k * r;
+            // type 2: x5 = X5f1, x8 = X5d(a,b), x4 = Qa 1Db;  type 3: x5 = X5d(b,a), x8 = X5f2, x7 = Qb 1Da
+            const double x52 = a.X5f1[((size_t)k * r + j) * R2 + (size_t)i * r + l];
+            const double x82 = a.X5d[((size_t)k * r + i) * R22 + R2 + (size_t)j * r + l];
+            const double x53 = a.X5d[(R2 + (size_t)k * r + j) * R22 + (size_t)i * r + l];
+            const double x83 = a.X5f2[((size_t)k * r + i) * R2 + (size_t)j * r + l];
+            double n = fma(2.0, (x52 - x82) + U3[e], x12[e]);
+            n = fma(-Qa[k * r + i], gb[j * r + l], n);
+            double m = fma(2.0, (x53 - x83) - U2[e], -x13[e]);
+            m = fma(Qb[k * r + j], ga[i * r + l], m);
+            if (ny2) {
+                n = fma(9.0, ny2[e], n);
+                m = fma(9.0, ny3[e], m);
+            }
+            bp_sm[k * ld + l] = n;
+            Nt[k * ld + l] = m;
+        }
+        __syncthreads();
+        const double* Y = a.Y[1] + (size_t)ij * R2;
+        double* H = a.H[1] + (size_t)ij * R2;
+        for (int e = threadIdx.x; e < R2; e += blockDim.x) {
+            const int k = e / r, l = e - k * r;
+            H[e] = fma(-4.0 / 3.0, bp_sm[k * ld + l] - Nt[l * ld + k], 4.0 * Y[e]);
+            if (i == j) a.H[0][(size_t)ij * R2 + e] = a.H[2][(size_t)ij * R2 + e] = 0.0;
         }
     }
 }
@@ -978,9 +884,7 @@ int launch_w_sum(acse_ctx* c) {
     return ACSE_OK;
 }
 
-static size_t b_smem(int r, size_t es, bool stage) {
-    return (4 * (size_t)pad4(r) * pad4(r) + (stage ? 4 : 2) * (size_t)r * r + (stage ? 4 * (size_t)r : 0)) * es;
-}
+static size_t b_smem(int r) { return 2 * (size_t)r * (r | 1) * sizeof(double); }
 static const size_t k_smem_cap = 227 * 1024;
 
 int launch_B_tiled(acse_ctx* c) {
@@ -995,24 +899,10 @@ int launch_B_tiled(acse_ctx* c) {
         a.flip = 0;
         for (int t = 0; t < 4; ++t) a.ny[t] = (const double*)ny_terms(c, t);
         a.gam = w.gam; a.w = w.w; a.Q = w.Q;
-        const bool st = b_smem(r, sizeof(double), true) <= k_smem_cap;
-        const size_t sm = b_smem(r, sizeof(double), st);
-        if (c->oz) {
-            // Ozaki path: the products on the tensor cores (acse_zoz.cu) where it applies, else in
-            // double-float; without staging two blocks fit an SM
-            const int bs = launch_Bx_oz(c);
-            if (bs == ACSE_OK) {
-                for (int k = 0; k < 8; ++k) a.bx[k] = w.bx64[k];
-                k_B_tiled<double, false, true, true><<<R2, TL_TPB, b_smem(r, sizeof(double), false), c->stream>>>(a);
-            } else if (bs == ACSE_ERR_UNSUPPORTED) {
-                k_B_tiled<double, false, true><<<R2, TL_TPB, b_smem(r, sizeof(double), false), c->stream>>>(a);
-            } else {
-                return bs;
-            }
-        } else {
-            if (st) k_B_tiled<double, true><<<R2, TL_TPB, sm, c->stream>>>(a);
-            else k_B_tiled<double, false><<<R2, TL_TPB, sm, c->stream>>>(a);
-        }
+        a.pmap = w.pmap;
+        ACSE_TRY(launch_Bx(c));
+        for (int k = 0; k < 8; ++k) a.bx[k] = w.bx64[k];
+        k_B_pre<<<r * (r - 1) + R2, 256, b_smem(r), c->stream>>>(a);
     } else {
         BTiledArgs<float> a;
         a.r = r;
@@ -1088,14 +978,7 @@ int launch_B_tiled(acse_ctx* c) {
 }
 
 int tiled_set_attrs() {
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_tiled<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)k_smem_cap));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_tiled<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)b_smem(ACSE_MAX_R, sizeof(double), false)));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_tiled<double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)b_smem(ACSE_MAX_R, sizeof(double), false)));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_tiled<double, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)b_smem(ACSE_MAX_R, sizeof(double), false)));
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_smem(ACSE_MAX_R)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pipe<320, 2, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bp_smem(48)));
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_B_pipe<320, 2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,

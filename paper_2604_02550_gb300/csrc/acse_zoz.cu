@@ -31,7 +31,7 @@
 // digits and the int64 normalisation, about half busy) and the chain TMEM read - MMA - TMEM read; HBM at 2 TB/s.
 // Every wait is bounded, and on expiry the kernel raises the device flag and stops.
 //
-// Used for S <= 8; more slices take the double-float kernels of acse_ph.cu, acse_tiled.cu and acse_adjoint.cu.
+// Used for S <= 8; more slices take the double-float kernels of acse_ph.cu.
 #include <cuda_bf16.h>
 
 #include "acse_internal.h"
@@ -53,8 +53,11 @@ struct RowsArgs {
     double* out[8];
     unsigned tt, gt;        // ... or transposed (bit c): A at [q][a], G[q][n]
     int sel[8];             // MODE 0: classes with the same G (and transposition) share a number
+    unsigned tri;           // MODE 0, bit c: the pairs i < j only (numbered through pmap)
+    const int* pmap;
     int r, D;
-    int tpg;                // tiles per group (MODE 0: class; MODE 1: (sector, k))
+    int start[9];           // MODE 0: first tile of each class
+    int tpg;                // MODE 1: tiles per group (sector, k)
     int ntiles;
     int* err;
 };
@@ -159,22 +162,27 @@ struct RzTile {
     const double* A;
     double* out;
     const double* G;
-    int m0, nrow, sel, gt, tr;
+    int m0, nrow, sel, gt, tr, tri;
     size_t ld;
     __device__ __forceinline__ RzTile(const RowsArgs& a, int tile) {
         const int r = a.r, R2 = r * r;
-        const int g = tile / a.tpg;
-        m0 = (tile - g * a.tpg) * TC_BM;
         if (MODE == 0) {
+            int g = 0;
+            while (g < 7 && a.start[g + 1] <= tile) ++g;
+            m0 = (tile - a.start[g]) * TC_BM;
+            tri = (a.tri >> g) & 1;
             A = a.A[g];
             out = a.out[g];
             G = a.G[g];
             sel = a.sel[g];
             gt = (a.gt >> g) & 1;
             tr = (a.tt >> g) & 1;
-            nrow = r * R2;
+            nrow = r * (tri ? r * (r - 1) / 2 : R2);
             ld = r;
         } else {   // g = (sector t, k): spin blocks (K, I) 0-3, the flips 4 (1D of beta) and 5 (of alpha)
+            const int g = tile / a.tpg;
+            m0 = (tile - g * a.tpg) * TC_BM;
+            tri = 0;
             const int t = g / r, k = g - t * r, f = t < 4 ? 0 : t - 3;
             sel = t < 4 ? t >> 1 : t == 4 ? 1 : 0;
             ld = t < 4 ? 2 * (size_t)R2 : (size_t)R2;
@@ -188,6 +196,12 @@ struct RzTile {
         }
     }
 };
+
+// Row m = (pair number, a) of a class on the pairs i < j as the row (ij, a) of the full array.
+static __device__ __forceinline__ int rz_pair_row(const RowsArgs& a, int m) {
+    const int u = m / a.r;
+    return a.pmap[u] * a.r + (m - u * a.r);
+}
 
 template <int RP, int MODE>
 __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant__ RowsArgs a) {
@@ -328,12 +342,13 @@ __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant
             size_t sq = 1;
             bool vec = false;
             if (MODE == 0) {
+                const int row = T.tri && ok ? rz_pair_row(a, m) : m;
                 if (T.tr) {
-                    const int ij = m / r;
-                    src += (size_t)ij * r * r + (m - ij * r);
+                    const int ij = row / r;
+                    src += (size_t)ij * r * r + (row - ij * r);
                     sq = r;
                 } else {
-                    src += (size_t)m * r;
+                    src += (size_t)row * r;
                     vec = (r & 1) == 0 && (reinterpret_cast<uintptr_t>(T.A) & 15) == 0;
                 }
             } else {
@@ -409,7 +424,7 @@ __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant
             const int m = T.m0 + ml;
             if (m >= T.nrow) continue;
             const int* eb = eB + slot * 64 + half * CW;
-            double* o = T.out + (MODE == 0 ? (size_t)m * r + half * CW : (size_t)(half * CW) * T.ld + m);
+            double* o = T.out + (MODE == 0 ? (size_t)(T.tri ? rz_pair_row(a, m) : m) * r + half * CW : (size_t)(half * CW) * T.ld + m);
             const bool v2 = MODE == 0 && (r & 1) == 0 && (reinterpret_cast<uintptr_t>(T.out) & 15) == 0;
 #pragma unroll
             for (int n = 0; n < CW; n += 2) {
@@ -470,7 +485,7 @@ static int rows_dispatch(acse_ctx* c, RowsArgs& a) {
     return s;
 }
 
-bool rows_oz_applies(const acse_ctx* c) { return c->oz && c->opt.oz_slices <= RZ_SMAX; }
+static bool rows_oz_applies(const acse_ctx* c) { return c->oz && c->opt.oz_slices <= RZ_SMAX; }
 
 // The transformation by 1D (trans: by its transpose) of the three arrays; ACSE_ERR_UNSUPPORTED where the kernel
 // does not apply.
@@ -490,9 +505,8 @@ int launch_xform_oz(acse_ctx* c, const double* const in[3], double* const out[3]
     return rows_dispatch<1>(c, a);
 }
 
-// The eight classes of tall products out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x]; ACSE_ERR_UNSUPPORTED where the
-// kernel does not apply.
-int launch_rows_oz(acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt,
+// The eight classes of tall products of launch_pair_rows; ACSE_ERR_UNSUPPORTED where the kernel does not apply.
+int launch_rows_oz(acse_ctx* c, const double* const T[8], unsigned tt, const double* const G[8], unsigned gt, unsigned tri,
                    double* const out[8]) {
     if (!rows_oz_applies(c)) return ACSE_ERR_UNSUPPORTED;
     const int r = c->r;
@@ -507,25 +521,13 @@ int launch_rows_oz(acse_ctx* c, const double* const T[8], unsigned tt, const dou
                 a.sel[k] = m;
                 break;
             }
+        const int items = (tri >> k) & 1 ? r * (r - 1) / 2 : r * r;
+        a.start[k + 1] = a.start[k] + (items * r + TC_BM - 1) / TC_BM;
     }
     a.tt = tt;
     a.gt = gt;
-    a.tpg = (r * r * r + TC_BM - 1) / TC_BM;
-    a.ntiles = 8 * a.tpg;
+    a.tri = tri;
+    a.pmap = c->w.pmap;
+    a.ntiles = a.start[8];
     return rows_dispatch<0>(c, a);
-}
-
-// The two r x r x r products of every B spin type and every pair (i, j) (the B kernel of the FP64 paths walks all
-// r^2 pairs) into w.bx64:
-//     class 2 t:      x1[k][l] = sum_q X_ij[k][q] 1D[q][l]       (type 3: X_ij transposed)
-//     class 2 t + 1:  x2^T[l][k] = sum_p M_ij[l][p] w[k][p]      (type 2: M_ij transposed)
-// ACSE_ERR_UNSUPPORTED without that scratch (the B kernel then forms the products itself in double-float).
-int launch_Bx_oz(acse_ctx* c) {
-    Work& w = c->w;
-    if (!w.bx64[0]) return ACSE_ERR_UNSUPPORTED;
-    const int R2 = c->r * c->r;
-    const double *ga = w.gam, *gb = w.gam + R2, *wa = w.w, *wb = w.w + R2;
-    const double* T[8] = {w.X[0], w.M[0], w.X[2], w.M[2], w.X[1], w.M[1], w.X[1], w.M[1]};
-    const double* G[8] = {ga, wa, gb, wb, gb, wa, ga, wb};
-    return launch_rows_oz(c, T, 1u << 6 | 1u << 5, G, 0x55u, w.bx64);
 }

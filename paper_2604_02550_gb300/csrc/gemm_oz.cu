@@ -856,14 +856,6 @@ int oz_plan_create(acse_ctx* c) {
     const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
     const int bn = R2 >= 256 ? OZ_BN : 128, pair = c->opt.gemm_tile != 1;
     ACSE_TRY(oz_plan_init(pl, c->opt.oz_slices, bn, pair, S2));
-    // the B products on the tensor cores (acse_zoz.cu): x1 and x2^T of the four types for every pair
-    if (rows_oz_applies(c))
-        for (int k = 0; k < 8; ++k)
-            if (cudaMalloc((void**)&c->w.bx64[k], (size_t)R2 * R2 * sizeof(double)) != cudaSuccess) {
-                cudaGetLastError();
-                c->w.bx64[k] = nullptr;
-                return ACSE_ERR_NOMEM;
-            }
     ACSE_TRY(oz_op_alloc(pl, pl->A[0], S2, S2));
     ACSE_TRY(oz_op_alloc(pl, pl->A[1], S2, P2));
     for (int i = 2; i < 5; ++i) ACSE_TRY(oz_op_alloc(pl, pl->A[i], R2, R2));
@@ -956,11 +948,6 @@ static void oz_plan_free(OzPlan* pl) {
 }
 
 void oz_plan_destroy(acse_ctx* c) {
-    for (int k = 0; k < 8; ++k)
-        if (c->w.bx64[k]) {
-            cudaFree(c->w.bx64[k]);
-            c->w.bx64[k] = nullptr;
-        }
     OzPlan* pl = (OzPlan*)c->oz_plan;
     if (!pl) return;
     if (pl->err && c->w.tc_err == pl->err) c->w.tc_err = nullptr;
