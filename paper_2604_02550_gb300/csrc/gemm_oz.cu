@@ -13,12 +13,12 @@
 //   * the tensor cores multiply the residue matrices of each modulus in FP32; a chunk of at most 64 * 64
 //     K elements keeps every partial sum an integer of magnitude at most 64 * 64 * 64^2 = 2^24, so the
 //     accumulation is exact, and the epilogue stores a residue w (|w| <= 65) of the chunk sum (one byte);
-//   * the reconstruction kernel forms s = sum_t w_t (P / p_t) exactly in FP32 sums of 10- or 11-bit
-//     limbs, which is congruent to X_A X_B^T modulo every p_t and hence modulo P (Chinese remainder theorem), takes
-//     q = round(s / P) (the product lies within P / 4 of zero, so a float estimate of s / P decides q),
-//     and x = s - q P is the exact integer product, rounded once to FP64 and scaled by alpha 2^(ea + eb - 2 nb).
+//   * the reconstruction kernel takes x / P = sum_t w_t / p_t modulo 1 (Chinese remainder theorem: w_t is the residue
+//     of x (P / p_t)^-1) in fixed point, the wrap-around modulo 2^96 being the reduction modulo 1; |x| <= P / 4, so the
+//     signed fraction is x / P itself, and x = P (x / P) is rounded once to FP64 and scaled by alpha 2^(ea + eb - 2 nb).
 // The result is the FP64 product up to the rounding of the operands to nb - 1 bits below each row's
-// leading bit and one final rounding: no product level is dropped.  Against the six-bit slice form of
+// leading bit, the 2^-69 P of the fraction's constants (2^-10 of the operand rounding or less) and one final
+// rounding: no product level is dropped.  Against the six-bit slice form of
 // the scheme (36 slice products at S = 8) this takes 17 residue products at S = 8 and r = 48.
 //
 // Kernels: the persistent tcgen05 GEMM of gemm_tc.cu with the accumulation unit changed from a tile
@@ -45,15 +45,8 @@
 #define OZ2_STAGES 6         // ring depth of the CTA-pair form (32 KB a stage per CTA)
 #define OZ_DRAIN_NS 2000000000ull
 #define OZ_WAIT_NS 4000000000ull
-// limbs of the reconstruction: 14 of 10 bits for two K chunks, 12 of 11 bits for one (their limb sums stay
-// below 2^22 in magnitude either way)
-#define OZ_LB2 10
-#define OZ_NL2 14
-#define OZ_LB1 11
-#define OZ_NL1 12
-#ifndef OZ_CRT_MINB
-#define OZ_CRT_MINB 3        // resident blocks of 256 threads per SM the reconstruction is compiled for
-#endif
+#define OZ_FL 11                       // bytes of the reconstruction's constants 2^88 / p_t
+#define OZ_NQ (OZ_NMOD * OZ_MAXCH + 3) / 4   // (modulus, chunk) groups in fours
 
 // Pairwise coprime moduli, largest first: 127, 5^3, 3 * 41, 11^2, 7 * 17 and the primes 113 .. 59.
 static const int oz_moduli[OZ_NMOD] = {127, 125, 123, 121, 119, 113, 109, 107, 103, 101, 97, 89, 83, 79, 73, 71, 67, 61, 59};
@@ -65,11 +58,8 @@ struct OzMods {
     float pinv[OZ_NMOD];      // 1 / p_t, rounded
     float cA[OZ_NMOD][4];     // 2^(14 l) mod p_t, l = 0..3 (limb weights of an A row)
     float cB[OZ_NMOD][4];     // 2^(14 l) y_t mod p_t, y_t = (P / p_t)^-1 mod p_t (limb weights of a B row)
-    float q10[OZ_NMOD][OZ_NL2];   // P / p_t in base-2^10 limbs, least significant first (exact floats)
-    float P10[OZ_NL2];            // P in base-2^10 limbs
-    float q11[OZ_NMOD][OZ_NL1];   // the same in base-2^11 limbs
-    float P11[OZ_NL1];
-    float pinvs;              // 2^120 / P, rounded (between 2^-5 and 2^114)
+    unsigned long long Pm;    // P = Pm 2^Pe, Pm with bit 63 set (truncated where P has more than 64 bits)
+    int Pe;
 };
 
 struct OzProb {
@@ -450,130 +440,135 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
 }
 
 // --------------------------------------------------------------------------- reconstruction
-// s = sum_t w_t (P / p_t) is accumulated in NL float limb sums of weight 2^(LB l): each is a sum of w_t
-// times a limb of P / p_t below 2^LB, so with T <= 19 it stays an integer below 2^22 in magnitude
-// (|w_t| <= 130 with two chunks and 10-bit limbs: 2^21.3; |w_t| <= 65 with one chunk and 11-bit limbs:
-// 2^21.3) -- exact, and within the range of the float-to-int step below.
-
-// x = s - round(s / P) P from the limb sums, rounded once to FP64 and scaled by 2^ex.  The product lies
-// within P / 4 of zero, so q needs s / P to within 1/4: the estimate is summed from the limb sums as they
-// are (each a sum of w_t times non-negative limbs of P / p_t, so the float rounding errors stay near
-// 2^-20 sum_t |w_t| / p_t of s / P).  x's limbs (integers below 2^22) become int32 through the float
-// 1.5 * 2^23 + x, carries normalise them to [0, 2^LB) under a signed top limb, the value is assembled
-// modulo 2^128 (|x| < 2^123), and a negative x is negated as a 128-bit two's complement.
-template <int LB, int NL>
-__device__ __forceinline__ double oz_crt_value(const float* a, const float* Pl, float pinvs, int ex) {
-    float sf = 0.0f;
-#pragma unroll
-    for (int l = 0; l < NL; ++l) sf = fmaf(a[l], __int_as_float((127 + LB * l - 120) << 23), sf);   // s 2^-120
-    const float q = fmaf(sf, pinvs, 12582912.0f) - 12582912.0f;
-    int x[NL];
-#pragma unroll
-    for (int l = 0; l < NL; ++l) x[l] = __float_as_int(fmaf(-q, Pl[l], a[l]) + 12582912.0f) - 0x4B400000;
-    int c = x[0];
-#pragma unroll
-    for (int l = 0; l < NL - 1; ++l) {
-        const int cl = c;
-        x[l] = cl & ((1 << LB) - 1);
-        c = (cl >> LB) + x[l + 1];   // arithmetic shift: floor
-    }
-    typedef unsigned long long u64;
-    u64 lo = 0, hi = 0;
-#pragma unroll
-    for (int l = 0; l < NL - 1; ++l) {   // limbs in [0, 2^LB) at bit LB l
-        const int pos = LB * l;
-        const u64 v = (u64)(unsigned int)x[l];
-        if (pos < 64) {
-            lo |= v << pos;
-            if (pos + LB > 64) hi |= v >> (64 - pos);
-        } else if (pos < 128) {
-            hi |= v << (pos - 64);
-        }
-    }
-    constexpr int TOP = LB * (NL - 1);   // the signed top limb c: sign-extended, modulo 2^128
-    if constexpr (TOP < 128) hi |= (u64)(long long)c << (TOP - 64);
-    if (c < 0) {   // |x| = -(the assembled value) modulo 2^128, since |x| < 2^128
-        const u64 nlo = 0ull - lo;
-        hi = ~hi + (lo == 0 ? 1ull : 0ull);
-        return oz_u128_scaled(hi, nlo, true, ex);
-    }
-    return oz_u128_scaled(hi, lo, false, ex);
-}
-
-// The constants of the reconstruction, passed as a kernel parameter: with the modulus and limb loops
-// unrolled, every limb of P / p_t is an immediate constant-bank operand of its FMA (no load).
+// x / P = sum over the (modulus, chunk) groups of w / p_t modulo 1, in units of 2^-88: F = sum_g w_g C_t modulo 2^88
+// with C_t = round(2^88 / p_t), eleven bytes.  The four residue bytes b = w + 128 of four groups meet each byte of
+// their constants in one dp4a (the 128 sum C_t comes off at the start): 5 x 11 of them for 17 moduli, where the sums
+// of s = sum w_t P / p_t in float limbs took 17 x 12 FMAs, an estimate of s / P and a subtraction of its multiple
+// (r = 48: 31.6 M elements a pass, 733 -> 244 us, 3.2 TB/s; issue-bound, dp4a at half rate).  The
+// constants are off by at most 1/2, so F by sum |w| / 2 <= 38 x 65 / 2 < 2^11 units: 2^-77 of P, against an operand
+// rounding of at least 2^-67 of P (the longest list, 53 bits).  An F of that size is a zero (exact cancellations stay
+// zero).  Wrap-around modulo 2^96 (F shifted by a byte) is the reduction modulo 1, and |x| <= P / 4 leaves the sign in
+// the top bit.
 struct OzCrtParams {
-    float q10[OZ_NMOD][OZ_NL2];
-    float P10[OZ_NL2];
-    float q11[OZ_NMOD][OZ_NL1];
-    float P11[OZ_NL1];
-    float pinvs;
-    int T;
+    unsigned c1[5][OZ_FL], c2[OZ_NQ][OZ_FL];   // one or two K chunks: byte l of the constants of groups 4u .. 4u + 3
+    int i1[OZ_FL], i2[OZ_FL];                  // -128 sum_g (byte l of C)
+    unsigned long long Pm;
+    int Pe, T;
 };
 
-// Two consecutive elements of one row per thread (16-bit loads of their residue bytes; the second one of an odd
-// row's last pair is padding): every residue word of the element pair (all moduli and chunks) is loaded before any is used, so that
-// about 2 KB per warp is in flight.  A byte b = w + 128 becomes the float 2^23 + b by a byte permute
-// (exact), so w = that - (2^23 + 128).
+// The FP64 value of x 2^ex from the eleven byte sums a_l (weight 2^(8 l) of F): carries into three 32-bit words of
+// 2^8 F, magnitude, its leading 64 bits times P, rounded to 53 bits.
+__device__ __forceinline__ double oz_frac_value(const int (&a)[OZ_FL], unsigned long long Pm, int ex) {
+    // bytes in pairs, pairs in 64-bit words of weight 2^32 (every sum below 2^21 in magnitude)
+    const long long t0 = (long long)(a[0] * 256) + (long long)(a[1] + a[2] * 256) * 65536;
+    const long long t1 = (long long)(a[3] + a[4] * 256) + (long long)(a[5] + a[6] * 256) * 65536;
+    const long long t2 = (long long)(a[7] + a[8] * 256) + (long long)(a[9] + a[10] * 256) * 65536;
+    const long long u1 = t1 + (t0 >> 32), u2 = t2 + (u1 >> 32);
+    const unsigned int sg = (unsigned int)((int)u2 >> 31);   // 0, or all ones for a negative x
+    unsigned int w0 = (unsigned int)t0 ^ sg, w1 = (unsigned int)u1 ^ sg, w2 = (unsigned int)u2 ^ sg;
+    if (w2 == 0) {   // |x| < 2^-32 P
+        if (w1 == 0 && w0 < (1u << 19)) return 0.0;
+        w2 = w1;
+        w1 = w0;
+        w0 = 0;
+        ex -= 32;
+        if (w2 == 0) {
+            w2 = w1;
+            w1 = 0;
+            ex -= 32;
+        }
+    }
+    const int n = __clz(w2);
+    const unsigned long long top = ((unsigned long long)__funnelshift_l(w1, w2, n) << 32) | __funnelshift_l(w0, w1, n);
+    unsigned long long m = __umul64hi(top, Pm);   // in [2^62, 2^64)
+    int e = ex - n;                                // x = m 2^e
+    const int s = (int)(m >> 63) ^ 1;
+    m <<= s;
+    e -= s;
+    const int E = e + 63 + 1022;   // exponent field less one: the significand's leading bit adds it
+    if (E < 1 || E > 2044) return oz_ll_scaled(sg ? -(long long)(m >> 1) : (long long)(m >> 1), e + 1);
+    return __longlong_as_double((long long)(((m >> 11) + ((m >> 10) & 1ull) + ((unsigned long long)(unsigned)E << 52)) |
+                                            ((unsigned long long)(sg & 0x80000000u) << 32)));
+}
+
+// Four consecutive elements of one row per thread: a 32-bit load of residue bytes per group, all issued first; the
+// words of four groups are transposed into one word per element by eight byte permutes.
 template <int NCH>
 __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& cp) {
-    constexpr int LB = NCH == 1 ? OZ_LB1 : OZ_LB2, NL = NCH == 1 ? OZ_NL1 : OZ_NL2;
-    const float(*qt)[NL] = NCH == 1 ? (const float(*)[NL])cp.q11 : (const float(*)[NL])cp.q10;
-    const float* Pl = NCH == 1 ? cp.P11 : cp.P10;
-    constexpr int VW = 2;
-    const int T = cp.T, N = P.N, nh = (N + 1) / 2;
-    const size_t MN = (size_t)P.M * P.ns;   // bytes of a (modulus, chunk) group
-    const size_t nunit = (size_t)P.M * nh;
-    for (size_t u = (size_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunit; u += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(u / nh), j0 = 2 * (int)(u - (size_t)i * nh);
+    constexpr int NQ = NCH == 1 ? 5 : OZ_NQ;
+    const unsigned(*ct)[OZ_FL] = NCH == 1 ? cp.c1 : cp.c2;
+    const int* ci = NCH == 1 ? cp.i1 : cp.i2;
+    const int G = cp.T * NCH, N = P.N;
+    const unsigned nq = (unsigned)(N + 3) / 4, nunit = (unsigned)P.M * nq;
+    const size_t MN = (size_t)P.M * P.ns;   // bytes of a group
+    const bool v2 = (P.ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(P.C) & 15) == 0;
+    for (unsigned u = blockIdx.x * blockDim.x + threadIdx.x; u < nunit; u += gridDim.x * blockDim.x) {
+        const int i = (int)(u / nq), j0 = 4 * (int)(u - (unsigned)i * nq);
         const unsigned char* __restrict__ sp = P.stage + (size_t)i * P.ns + j0;
-        unsigned int xw[OZ_NMOD][NCH];
+        unsigned int x[NQ][4];
 #pragma unroll
-        for (int t = 0; t < OZ_NMOD; ++t)
+        for (int g = 0; g < 4 * NQ; ++g) {
+            x[g / 4][g & 3] = 0u;   // past the last group: the constants are zero
+            if (g < G) x[g / 4][g & 3] = __ldg(reinterpret_cast<const unsigned int*>(sp + g * MN));
+        }
 #pragma unroll
-            for (int c = 0; c < NCH; ++c) {
-                xw[t][c] = 0x8080u;   // w = 0 past the last modulus
-                if (t < T) {
-                    xw[t][c] = (unsigned int)__ldg(reinterpret_cast<const unsigned short*>(sp));
-                    sp += MN;
-                }
-            }
-        float acc[VW][NL];
-#pragma unroll
-        for (int k = 0; k < VW; ++k)
-#pragma unroll
-            for (int l = 0; l < NL; ++l) acc[k][l] = 0.0f;
-#pragma unroll
-        for (int t = 0; t < OZ_NMOD; ++t) {
-            if (t >= T) break;
-#pragma unroll
-            for (int k = 0; k < VW; ++k) {
-                float w = 0.0f;
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) w += __uint_as_float(__byte_perm(xw[t][c], 0x4B000000u, 0x7540u | k)) - 8388736.0f;
-#pragma unroll
-                for (int l = 0; l < NL; ++l) acc[k][l] = fmaf(w, qt[t][l], acc[k][l]);
-            }
+        for (int q = 0; q < NQ; ++q) {
+            const unsigned a = __byte_perm(x[q][0], x[q][1], 0x5140), b = __byte_perm(x[q][2], x[q][3], 0x5140);
+            const unsigned c = __byte_perm(x[q][0], x[q][1], 0x7362), d = __byte_perm(x[q][2], x[q][3], 0x7362);
+            x[q][0] = __byte_perm(a, b, 0x5410);
+            x[q][1] = __byte_perm(a, b, 0x7632);
+            x[q][2] = __byte_perm(c, d, 0x5410);
+            x[q][3] = __byte_perm(c, d, 0x7632);
         }
         const int ea = (int)((__double_as_longlong(P.sa[i]) >> 52) & 0x7FF);   // row scales are powers of two
-        double* crow = P.C + (size_t)i * P.ldc;
+        double* crow = P.C + (size_t)i * P.ldc + j0;
+#pragma unroll 1
+        for (int h = 0; h < 4 && j0 + h < N; h += 2) {   // two elements a round (fully unrolled the kernel spills)
+            unsigned acc[2][OZ_FL];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) {
-            if (j0 + k >= N) break;
-            const int eb = (int)((__double_as_longlong(P.sb[j0 + k]) >> 52) & 0x7FF);
-            const double v = (ea == 0x7FF || eb == 0x7FF)
-                                 ? __longlong_as_double(0x7ff8000000000000ll)
-                                 : oz_crt_value<LB, NL>(acc[k], Pl, cp.pinvs, ea + eb - 2046 + P.ealpha - 2 * P.nb);
-            crow[j0 + k] = v;
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int l = 0; l < OZ_FL; ++l) acc[k][l] = (unsigned)ci[l];
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                if (NCH > 1 && 4 * q >= G) break;
+#pragma unroll
+                for (int l = 0; l < OZ_FL; ++l) {
+                    acc[0][l] = __dp4a(x[q][0], ct[q][l], acc[0][l]);
+                    acc[1][l] = __dp4a(x[q][1], ct[q][l], acc[1][l]);
+                }
+                x[q][0] = x[q][2];   // the next round's
+                x[q][1] = x[q][3];
+            }
+            double v[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                int a[OZ_FL];
+#pragma unroll
+                for (int l = 0; l < OZ_FL; ++l) a[l] = (int)acc[k][l];
+                const int eb = (int)((__double_as_longlong(P.sb[min(j0 + h + k, N - 1)]) >> 52) & 0x7FF);
+                v[k] = (ea == 0x7FF || eb == 0x7FF) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                    : oz_frac_value(a, cp.Pm, ea + eb - 2046 + P.ealpha - 2 * P.nb + cp.Pe);
+            }
+            if (v2 && j0 + h + 1 < N) {
+                *reinterpret_cast<double2*>(crow + h) = make_double2(v[0], v[1]);
+            } else {
+                crow[h] = v[0];
+                if (j0 + h + 1 < N) crow[h + 1] = v[1];
+            }
         }
     }
 }
 
 // C = alpha 2^(e_i + e_j - 2 nb) x for every element, x rebuilt from the staged residues.  The residues of
 // an element are read once, coalesced, and C is written once.
-__global__ void __launch_bounds__(256, OZ_CRT_MINB) k_oz_crt(const OzBatch* __restrict__ bp, const __grid_constant__ OzCrtParams cp) {
+// TWO: some problem has two K chunks (r = 64), whose twice as many residue words take the registers of two resident
+// blocks; without, three.
+template <bool TWO>
+__global__ void __launch_bounds__(256, TWO ? 2 : 3) k_oz_crt(const OzBatch* __restrict__ bp,
+                                                             const __grid_constant__ OzCrtParams cp) {
     const OzProb& P = bp->p[blockIdx.y];
-    if (P.nch == 1) oz_crt_rows<1>(P, cp);
+    if (!TWO || P.nch == 1) oz_crt_rows<1>(P, cp);
     else oz_crt_rows<2>(P, cp);
 }
 
@@ -583,12 +578,27 @@ static int oz_launch_crt(const OzBatch* host, const OzBatch* dev, int nsm, cudaS
     memset(&cp, 0, sizeof(cp));
     const OzMods& m = host->mods;
     cp.T = m.T;
-    memcpy(cp.q10, m.q10, sizeof(cp.q10));
-    memcpy(cp.P10, m.P10, sizeof(cp.P10));
-    memcpy(cp.q11, m.q11, sizeof(cp.q11));
-    memcpy(cp.P11, m.P11, sizeof(cp.P11));
-    cp.pinvs = m.pinvs;
-    k_oz_crt<<<dim3(2 * nsm, host->nprob), 256, 0, st>>>(dev, cp);
+    cp.Pm = m.Pm;
+    cp.Pe = m.Pe;
+    for (int t = 0; t < m.T; ++t) {
+        const unsigned __int128 one = (unsigned __int128)1 << 88;
+        const int p = oz_moduli[t];
+        unsigned __int128 C = (one + p / 2) / p;
+        for (int l = 0; l < OZ_FL; ++l, C >>= 8) {
+            const unsigned byte = (unsigned)(C & 255);
+            cp.c1[t / 4][l] |= byte << (8 * (t & 3));
+            cp.i1[l] -= 128 * (int)byte;
+            for (int c = 0; c < 2; ++c) {
+                const int g = 2 * t + c;
+                cp.c2[g / 4][l] |= byte << (8 * (g & 3));
+                cp.i2[l] -= 128 * (int)byte;
+            }
+        }
+    }
+    bool two = false;
+    for (int p = 0; p < host->nprob; ++p) two = two || host->p[p].nch > 1;
+    if (two) k_oz_crt<true><<<dim3(2 * nsm, host->nprob), 256, 0, st>>>(dev, cp);
+    else k_oz_crt<false><<<dim3(3 * nsm, host->nprob), 256, 0, st>>>(dev, cp);
     ACSE_CUDA_TRY(cudaGetLastError());
     return ACSE_OK;
 }
@@ -672,7 +682,6 @@ static int oz_mods_init(OzPlan* pl, int S, long long Kmax) {
     OzMods& m = pl->host->mods;
     memset(&m, 0, sizeof(m));
     m.T = T;
-    const unsigned __int128 m10 = ((unsigned __int128)1 << OZ_LB2) - 1, m11 = ((unsigned __int128)1 << OZ_LB1) - 1;
     for (int t = 0; t < T; ++t) {
         const int pt = oz_moduli[t];
         const unsigned __int128 Q = P / (unsigned __int128)pt;
@@ -686,12 +695,11 @@ static int oz_mods_init(OzPlan* pl, int S, long long Kmax) {
             m.cA[t][l] = (float)cl;
             m.cB[t][l] = (float)((cl * y) % pt);
         }
-        for (int l = 0; l < OZ_NL2; ++l) m.q10[t][l] = (float)(int)((Q >> (OZ_LB2 * l)) & m10);
-        for (int l = 0; l < OZ_NL1; ++l) m.q11[t][l] = (float)(int)((Q >> (OZ_LB1 * l)) & m11);
     }
-    for (int l = 0; l < OZ_NL2; ++l) m.P10[l] = (float)(int)((P >> (OZ_LB2 * l)) & m10);
-    for (int l = 0; l < OZ_NL1; ++l) m.P11[l] = (float)(int)((P >> (OZ_LB1 * l)) & m11);
-    m.pinvs = (float)(ldexp(1.0, 120) / (double)P);
+    int bits = 0;
+    while (bits < 127 && (P >> bits) > 1) ++bits;   // leading bit of P
+    m.Pe = bits - 63;
+    m.Pm = (unsigned long long)(m.Pe >= 0 ? P >> m.Pe : P << -m.Pe);
     return ACSE_OK;
 }
 
