@@ -272,6 +272,7 @@ int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const
         c->cur_D[s] = D[s];
         c->cur_W[s] = W[s];
     }
+    c->cur_prep = prep_D;
     if (c->opt.prec == ACSE_FP64) {
         if (prep_D) {
             ACSE_TRY(launch_gamma_M(c, D));

@@ -193,6 +193,8 @@ struct acse_ctx {
     void* oz_plan;
     const double* cur_D[3];   // operands of the contraction pass in flight (FP64 GEMM list)
     const double* cur_W[3];
+    int cur_prep;              // the pass in flight prepares its D (1D, M and, for NY, 2Delta)
+    const float* cur_W32[3];   // split path: the FP32 copies of cur_W
     // profiling: kernel launch count and CUDA-event timing of the O(r^6) GEMM launches
     long long launches;
     int prof_on;

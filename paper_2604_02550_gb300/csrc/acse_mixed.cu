@@ -443,6 +443,7 @@ int tc_mixed_prep_W(acse_ctx* c, const double* const W[3]) {
         ACSE_TRY(to_f32(c, W, w.W32s));
         for (int s = 0; s < 3; ++s) W32[s] = w.W32s[s];
     }
+    for (int s = 0; s < 3; ++s) c->cur_W32[s] = W32[s];
     const dim3 grid((r * r / 4 + 128) / 128, (acse_singlet(c) ? 2 : 3) * r * r);   // no bb pair GEMM under the spin flip
     if (c->opt.prec == ACSE_BF16X3)
         launch_pack_W<ACSE_BF16X3>(c, grid, W32, p);

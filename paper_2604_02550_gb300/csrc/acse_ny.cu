@@ -23,15 +23,17 @@
 // one r^2 x r^2 problem of one grouped launch (FP64 DFMA or tcgen05).  A final kernel forms T for
 // the four spin types of the B kernel, which adds it to B.
 #include <math.h>
+#include <type_traits>
 
 #include "acse_internal.h"
 #include "acse_split.cuh"
+#include "dfloat.cuh"
 
 struct NyWork {
     int n;                 // spin orbitals
     size_t n2, n4;
     int Kb;                // padded r^2: K elements of one spin block per split term
-    double* delta[3];      // 2Delta blocks aa, ab, bb (FP64)
+    void* delta[3];        // 2Delta blocks aa, ab, bb (double; float on the split path)
     double* sig;           // [n] sigma_a
     void* opA[3];          // operand rows of the three GEMMs of a stage
     void* opB[3];
@@ -47,13 +49,13 @@ struct NyWork {
 
 // Element T^{x1 x2}_{x3 x4} (spin-orbital indices, alpha first) of a pair-antisymmetric tensor stored
 // as its aa, ab, bb blocks (the other nonzero blocks follow by antisymmetry within each pair).
-__device__ __forceinline__ double so_get(const double* aa, const double* ab, const double* bb, int r, int x1, int x2,
-                                         int x3, int x4) {
+template <typename T>
+__device__ __forceinline__ T so_get(const T* aa, const T* ab, const T* bb, int r, int x1, int x2, int x3, int x4) {
     const int s1 = x1 >= r, s2 = x2 >= r, s3 = x3 >= r, s4 = x4 >= r;
     const int a = x1 - s1 * r, b = x2 - s2 * r, c = x3 - s3 * r, d = x4 - s4 * r;
     const size_t R = r;
-    auto at = [&](const double* t, int i, int j, int k, int l) { return t[((i * R + j) * R + k) * R + l]; };
-    if (s1 + s2 != s3 + s4) return 0.0;
+    auto at = [&](const T* t, int i, int j, int k, int l) { return t[((i * R + j) * R + k) * R + l]; };
+    if (s1 + s2 != s3 + s4) return (T)0;
     if (s1 == s2) return s1 ? at(bb, a, b, c, d) : at(aa, a, b, c, d);
     if (s1 == 0 && s3 == 0) return at(ab, a, b, c, d);     // (a b | a b)
     if (s1 == 1 && s3 == 1) return at(ab, b, a, d, c);     // (b a | b a)
@@ -62,17 +64,17 @@ __device__ __forceinline__ double so_get(const double* aa, const double* ab, con
 }
 
 // 2Delta = 2D - 1D^1D per block: aa/bb: D - 1/2 (g_ik g_jl - g_jk g_il), ab: D - 1/2 ga_ik gb_jl.
+template <typename T>   // formed in FP64, rounded once to T
 __global__ void k_ny_delta(int r, const double* __restrict__ gam, const double* __restrict__ Daa,
-                           const double* __restrict__ Dab, const double* __restrict__ Dbb, double* daa, double* dab,
-                           double* dbb) {
+                           const double* __restrict__ Dab, const double* __restrict__ Dbb, T* daa, T* dab, T* dbb) {
     const size_t R2 = (size_t)r * r, n4 = R2 * R2;
     const double* ga = gam;
     const double* gb = gam + R2;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
         const int l = (int)(e % r), k = (int)((e / r) % r), j = (int)((e / R2) % r), i = (int)(e / (R2 * r));
-        daa[e] = Daa[e] - 0.5 * (ga[i * r + k] * ga[j * r + l] - ga[j * r + k] * ga[i * r + l]);
-        dbb[e] = Dbb[e] - 0.5 * (gb[i * r + k] * gb[j * r + l] - gb[j * r + k] * gb[i * r + l]);
-        dab[e] = Dab[e] - 0.5 * ga[i * r + k] * gb[j * r + l];
+        daa[e] = (T)(Daa[e] - 0.5 * (ga[i * r + k] * ga[j * r + l] - ga[j * r + k] * ga[i * r + l]));
+        dbb[e] = (T)(Dbb[e] - 0.5 * (gb[i * r + k] * gb[j * r + l] - gb[j * r + k] * gb[i * r + l]));
+        dab[e] = (T)(Dab[e] - 0.5 * ga[i * r + k] * gb[j * r + l]);
     }
 }
 
@@ -95,65 +97,103 @@ __device__ __forceinline__ T ny_dense(const T* t, int r, int x1, int x2, int x3,
     return t[ny_pidx(r, x1, x2) * (size_t)(4 * r * r) + ny_pidx(r, x3, x4)];
 }
 
-// Operand row `row` (spin-major pair (u0, u1)); K position (q, t): spin block q holds the pair
-// korder[q], t = u2' r + u3'.  Value [sigma[u2]] * src(u[P0], u[P1], u[P2], u[P3]), src a
-// pair-antisymmetric tensor given by blocks (blk != null) or a dense intermediate.  FP64: rows of
-// 4 r^2 doubles (block q at q r^2); split: rows of 4 Kbw elements (block q at q Kbw, its hi/lo
-// segments Kb apart).
-struct NyPack {
-    const double* blk[3];
-    const void* dense;     // double (FP64 path) or float (split path)
-    int P[4];
-    int use_sigma;
-    const double* sig;
+// Packing of the six operands of a stage, one launch.  A piece is one spin block of one operand: rows (u0, u1) of row
+// block rb, K positions t = u2 r + u3 of K block position q, value sign sigma[u2] src[base + sum_m u_m st_m].  The
+// source is contiguous in u3, u2 or u1 (mode 0, 1, 2); a block takes nslab r x r slabs of u3 against u2 (modes 0, 1; fixed
+// u0, u1: r^2 consecutive K positions of one row) or u1 (mode 2; fixed u0, u2) through shared memory, so that reads and
+// writes are both coalesced and about 16 loads a thread are in flight.  (A thread per output element read the permuted
+// source at stride r or r^2 in FP64 with four integer divisions an element: 34 us a launch at r = 32, 24 launches a
+// step; one slab a block 146 us a stage, 97 now for 36 pieces: 230 MB written and 150 read.)
+// Values are those of the FP64 source rounded once (2Delta and W are read as their FP32 copies on the split path).
+struct NyPiece {
+    const void* src;
+    size_t base;
+    int st[4];
     void* dst;
-    size_t ld;             // row length of dst in elements
-    int Kb, Kbw;
-    int korder[4];
-    int need[4];           // per row block: bit kb set when some problem reads K spin block kb
+    int rb, q, mode, sp2;   // sp2: spin of u2
+    int pat, use_sigma;
+    float sign;
+};
+#define NY_MAXPC 96   // six operands of at most 16 spin blocks
+struct NyPackList {
+    NyPiece p[NY_MAXPC];
+    const double* sig;
+    size_t ld;              // row length of dst in elements
+    int Kb, Kbw;            // K elements of a spin block per split term, and in all
 };
 
-template <int PREC, int PAT>
-__global__ void __launch_bounds__(256) k_ny_pack(int r, const __grid_constant__ NyPack a) {
-    const int R2 = r * r;
-    const int row = blockIdx.x;
-    const int rb = row / R2, rr = row - rb * R2;
-    const int u0 = (rb >> 1) * r + rr / r, u1 = (rb & 1) * r + rr % r;
-    const bool vec = (R2 & 3) == 0;
-    const int ngroups = vec ? R2 / 4 : R2;
-    const int per = vec ? 4 : 1;
-    for (int e = threadIdx.x; e < 4 * ngroups; e += blockDim.x) {
-        const int q = e / ngroups, t0 = (e - q * ngroups) * per;
-        const int code = a.korder[q];
-        if (!(a.need[rb] >> code & 1)) continue;   // no problem reads this block
-        float xf[4];
-        double xd[4];
-        for (int c = 0; c < per; ++c) {
-            const int t = t0 + c;
-            const int u2 = (code >> 1) * r + t / r, u3 = (code & 1) * r + t % r;
-            const int u[4] = {u0, u1, u2, u3};
-            const int s0 = u[a.P[0]], s1 = u[a.P[1]], s2 = u[a.P[2]], s3 = u[a.P[3]];
-            double v;
-            if (a.blk[0]) v = so_get(a.blk[0], a.blk[1], a.blk[2], r, s0, s1, s2, s3);
-            else if (PREC == ACSE_FP64) v = ny_dense((const double*)a.dense, r, s0, s1, s2, s3);
-            else v = (double)ny_dense((const float*)a.dense, r, s0, s1, s2, s3);
-            if (a.use_sigma) v *= a.sig[u2];
-            xd[c] = v;
-            xf[c] = (float)v;
+template <int PREC>
+__global__ void __launch_bounds__(256) k_ny_pack(int r, int nslab, const __grid_constant__ NyPackList a) {
+    using T = typename std::conditional<PREC == ACSE_FP64, double, float>::type;
+    extern __shared__ __align__(16) unsigned char ny_smem[];
+    T* tile = (T*)ny_smem;   // [nslab][r][r + 1]
+    const int R2 = r * r, ld = r + 1, nblk = (R2 + nslab - 1) / nslab;
+    const float invr = 1.f / (float)r, invR2 = 1.f / (float)R2;   // e / r as (int)((e + 1/2) / r), exact for e < 2^16
+    const int ip = blockIdx.x / nblk;
+    const NyPiece& pc = a.p[ip];
+    const int fb = (blockIdx.x - ip * nblk) * nslab, nf = min(nslab, R2 - fb);   // slabs (u0, u1), or (u0, u2) in mode 2
+    const int mode = pc.mode;
+    const bool m2 = mode == 2;
+    const int sf0 = pc.st[0], sf1 = pc.st[m2 ? 2 : 1], slow = mode == 0 ? pc.st[2] : pc.st[3];
+    const T* src = (const T*)pc.src + pc.base;
+    // sigma in T once a block: a conversion from FP64 runs at 1/64 of the FP32 rate
+    __shared__ T sig[ACSE_MAX_R];
+    if (threadIdx.x < r) sig[threadIdx.x] = (T)a.sig[pc.sp2 * r + threadIdx.x];
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nf * R2; e += 256) {
+        const int w = (int)(((float)e + 0.5f) * invR2), g = e - w * R2;
+        const int s = (int)(((float)g + 0.5f) * invr), c = g - s * r;
+        const int f = fb + w, f0 = (int)(((float)f + 0.5f) * invr), f1 = f - f0 * r;
+        const T v = src[(size_t)f0 * sf0 + (size_t)f1 * sf1 + (size_t)s * slow + c];
+        tile[w * r * ld + (mode == 0 ? s * ld + c : c * ld + s)] = v;   // [u2 or u1][u3]
+    }
+    __syncthreads();
+    const T sign = (T)pc.sign;
+    const int use_sigma = pc.use_sigma, pat = pc.pat;
+    const size_t rows0 = (size_t)pc.rb * R2;
+    if constexpr (PREC == ACSE_FP64) {
+        for (int e = threadIdx.x; e < nf * R2; e += 256) {
+            const int w = e / R2, g = e - w * R2, d = g / r, u3 = g - d * r;
+            const int f0 = (fb + w) / r, f1 = fb + w - f0 * r;
+            T v = sign * tile[w * r * ld + d * ld + u3];
+            if (use_sigma) v = sig[m2 ? f1 : d] * v;
+            const size_t row = rows0 + (size_t)f0 * r + (m2 ? d : f1);
+            ((double*)pc.dst)[row * a.ld + (size_t)pc.q * R2 + (m2 ? f1 * r + u3 : g)] = v;
         }
-        if (PREC == ACSE_FP64) {
-            double* d = (double*)a.dst + (size_t)row * a.ld + (size_t)q * R2 + t0;
-            if (vec) {
-                *reinterpret_cast<double2*>(d) = make_double2(xd[0], xd[1]);
-                *reinterpret_cast<double2*>(d + 2) = make_double2(xd[2], xd[3]);
-            } else {
-                d[0] = xd[0];
+    } else {
+        // groups of four K positions where they start on a multiple of four (a K block does)
+        const size_t off = (size_t)pc.q * a.Kbw;
+        void* base = PREC == ACSE_BF16X3 ? (void*)((__nv_bfloat16*)pc.dst + off) : (void*)((float*)pc.dst + off);
+        const int n4 = !m2 || (r & 3) == 0 ? R2 / 4 : 0;
+        const float invn4 = n4 ? 1.f / (float)n4 : 0.f;
+        for (int h = threadIdx.x; h < nf * n4; h += 256) {
+            const int w = (int)(((float)h + 0.5f) * invn4), g = h - w * n4;
+            const int f = fb + w, f0 = (int)(((float)f + 0.5f) * invr), f1 = f - f0 * r;
+            const int d = (int)(((float)(4 * g) + 0.5f) * invr);
+            const T* tw = tile + w * r * ld;
+            int u2 = d, u3 = 4 * g - d * r;
+            const int k = m2 ? f1 * r + u3 : 4 * g;
+            float x[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                x[c] = sign * tw[u2 * ld + u3];
+                if (use_sigma) x[c] = sig[m2 ? f1 : u2] * x[c];
+                if (++u3 == r) { u3 = 0; ++u2; }   // mode 2: r % 4 == 0, the group stays in its row
             }
-        } else {
-            const size_t off = (size_t)q * a.Kbw;    // elements; the block's segments start here
-            void* base = PREC == ACSE_BF16X3 ? (void*)((__nv_bfloat16*)a.dst + off) : (void*)((float*)a.dst + off);
-            if (vec) put4<PREC, PAT>(base, (size_t)row, a.ld, a.Kb, t0, xf);
-            else put<PREC, PAT>(base, (size_t)row, a.ld, a.Kb, t0, xf[0]);
+            const size_t row = rows0 + (size_t)f0 * r + (m2 ? d : f1);
+            if (pat) put4<PREC, 1>(base, row, a.ld, a.Kb, k, x);
+            else put4<PREC, 0>(base, row, a.ld, a.Kb, k, x);
+        }
+        const int nrest = R2 - 4 * n4;
+        for (int h = threadIdx.x; h < nf * nrest; h += 256) {
+            const int w = h / nrest, g = 4 * n4 + h - w * nrest, d = g / r, u3 = g - d * r;
+            const int f0 = (fb + w) / r, f1 = fb + w - f0 * r;
+            float v = sign * tile[w * r * ld + d * ld + u3];
+            if (use_sigma) v = sig[m2 ? f1 : d] * v;
+            const size_t row = rows0 + (size_t)f0 * r + (m2 ? d : f1);
+            const int k = m2 ? f1 * r + u3 : g;
+            if (pat) put<PREC, 1>(base, row, a.ld, a.Kb, k, v);
+            else put<PREC, 0>(base, row, a.ld, a.Kb, k, v);
         }
     }
 }
@@ -173,38 +213,77 @@ __global__ void __launch_bounds__(256) k_ny_Q(int r, const T* __restrict__ X, T*
 }
 
 // T for the spin type tt of block (i', j') (types of the B kernel: 0 aaaa, 1 bbbb, 2 (ia jb | ka lb),
-// 3 (ia jb | kb la)); threads over (k', l').  S3 from factors staged in shared memory:
-// qs[a][k'] = sigma_a Q[a][k], dv[a][l'] = 2Delta^{ji}_{al}.
+// 3 (ia jb | kb la)).  S3 from factors staged in shared memory, qs[a][k'] = sigma_a Q[a][k], dv[a][l'] =
+// 2Delta^{ji}_{al} (rows padded to rp = r rounded up to 4): a thread owns 2 x 4 outputs (k', l'), two vector loads for eight
+// FMAs of the a loop (one output a thread took two loads a FMA: 109 us a launch at r = 32, 73 now).
 template <typename T>
 __global__ void __launch_bounds__(256) k_ny_assemble(int r, const T* __restrict__ S1, const T* __restrict__ S4,
                                                      const T* __restrict__ S6, const T* __restrict__ Q,
-                                                     const double* __restrict__ daa, const double* __restrict__ dab,
-                                                     const double* __restrict__ dbb, const double* __restrict__ sig,
+                                                     const T* __restrict__ daa, const T* __restrict__ dab,
+                                                     const T* __restrict__ dbb, const double* __restrict__ sig,
                                                      T* t0, T* t1, T* t2, T* t3) {
     extern __shared__ __align__(16) unsigned char ny_smem[];
-    const int n = 2 * r, R2 = r * r;
-    T* qs = (T*)ny_smem;           // [n][r]
-    T* dv = qs + (size_t)n * r;    // [n][r]
+    const int n = 2 * r, R2 = r * r, rp = (r + 3) & ~3;
+    T* qs = (T*)ny_smem;            // [n][rp]
+    T* dv = qs + (size_t)n * rp;    // [n][rp]
     const int tt = blockIdx.x / R2, ij = blockIdx.x % R2;
     const int ip = ij / r, jp = ij % r;
     const int si = tt == 1, sj = tt == 0 ? 0 : 1, sk = tt == 1 || tt == 3, sl = tt == 1 || tt == 2;
     const int i = si * r + ip, j = sj * r + jp;
-    for (int e = threadIdx.x; e < n * r; e += blockDim.x) {
-        const int aa_ = e / r, c = e % r;
-        qs[e] = (T)(sig[aa_] * (double)Q[(size_t)aa_ * n + sk * r + c]);
-        dv[e] = (T)so_get(daa, dab, dbb, r, j, i, aa_, sl * r + c);
+    __shared__ T sg[2 * ACSE_MAX_R];   // +-1: exact in T
+    if (threadIdx.x < n) sg[threadIdx.x] = (T)sig[threadIdx.x];
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * rp; e += blockDim.x) {
+        const int aa_ = e / rp, c = e - aa_ * rp;
+        qs[e] = c < r ? sg[aa_] * Q[(size_t)aa_ * n + sk * r + c] : (T)0;
+        dv[e] = c < r ? so_get<T>(daa, dab, dbb, r, j, i, aa_, sl * r + c) : (T)0;
     }
     __syncthreads();
-    T* out = tt == 0 ? t0 : tt == 1 ? t1 : tt == 2 ? t2 : t3;
-    for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-        const int kp = e / r, lp = e % r;
-        const int k = sk * r + kp, l = sl * r + lp;
-        T s3 = 0;
-        for (int a_ = 0; a_ < n; ++a_) s3 += qs[a_ * r + kp] * dv[a_ * r + lp];
-        const T s1a = ny_dense(S1, r, k, i, j, l), s1b = ny_dense(S1, r, k, j, i, l);
-        const T s4a = ny_dense(S4, r, k, j, i, l), s4b = ny_dense(S4, r, k, i, j, l);
-        const T s6 = ny_dense(S6, r, j, i, k, l);
-        out[(size_t)ij * R2 + e] = (T)(4.0 / 6.0) * (s1a - s1b - s3 - (T)2 * s4a + (T)2 * s4b + (T)2 * s6);
+    T* out = (tt == 0 ? t0 : tt == 1 ? t1 : tt == 2 ? t2 : t3) + (size_t)ij * R2;
+    const int nl = rp / 4, nk = rp / 2;
+    for (int g = threadIdx.x; g < nk * nl; g += blockDim.x) {
+        const int k0 = 2 * (g / nl), l0 = 4 * (g % nl);
+        T s3[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) s3[u][v] = (T)0;
+#pragma unroll 4
+        for (int a_ = 0; a_ < n; ++a_) {
+            T q[2], d[4];
+            q[0] = qs[a_ * rp + k0];
+            q[1] = qs[a_ * rp + k0 + 1];
+            ld4(dv + a_ * rp + l0, d);
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) s3[u][v] += q[u] * d[v];
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int kp = k0 + u;
+            if (kp >= r) continue;
+            const int k = sk * r + kp, l = sl * r + l0;
+            const T *p1a = &S1[ny_pidx(r, k, i) * (size_t)(4 * R2) + ny_pidx(r, j, l)],
+                    *p1b = &S1[ny_pidx(r, k, j) * (size_t)(4 * R2) + ny_pidx(r, i, l)];
+            const T *p4a = &S4[ny_pidx(r, k, j) * (size_t)(4 * R2) + ny_pidx(r, i, l)],
+                    *p4b = &S4[ny_pidx(r, k, i) * (size_t)(4 * R2) + ny_pidx(r, j, l)];
+            const T* p6 = &S6[ny_pidx(r, j, i) * (size_t)(4 * R2) + ny_pidx(r, k, l)];
+            T s1a[4], s1b[4], s4a[4], s4b[4], s6[4];
+            if ((r & 3) == 0) {   // rows of l start on 16-byte boundaries
+                ld4(p1a, s1a); ld4(p1b, s1b); ld4(p4a, s4a); ld4(p4b, s4b); ld4(p6, s6);
+            } else {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int o = l0 + v < r ? v : 0;
+                    s1a[v] = p1a[o]; s1b[v] = p1b[o]; s4a[v] = p4a[o]; s4b[v] = p4b[o]; s6[v] = p6[o];
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (l0 + v < r)
+                    out[kp * r + l0 + v] = (T)(4.0 / 6.0) * (s1a[v] - s1b[v] - s3[u][v] - (T)2 * s4a[v] + (T)2 * s4b[v] + (T)2 * s6[v]);
+        }
     }
 }
 
@@ -230,27 +309,6 @@ void ny_free(acse_ctx* c) {
         if (y->st[s].host) tc_table_free(&y->st[s]);
     free(y);
     c->ny = nullptr;
-}
-
-static int ny_pack_launch(acse_ctx* c, const NyPack& pk, int pat) {
-    const int r = c->r, n2 = 4 * r * r;
-    switch (c->opt.prec) {
-        case ACSE_FP64: k_ny_pack<ACSE_FP64, 0><<<n2, 256, 0, c->stream>>>(r, pk); break;
-        case ACSE_BF16X3:
-            if (pat) k_ny_pack<ACSE_BF16X3, 1><<<n2, 256, 0, c->stream>>>(r, pk);
-            else k_ny_pack<ACSE_BF16X3, 0><<<n2, 256, 0, c->stream>>>(r, pk);
-            break;
-        case ACSE_TF32X3:
-            if (pat) k_ny_pack<ACSE_TF32X3, 1><<<n2, 256, 0, c->stream>>>(r, pk);
-            else k_ny_pack<ACSE_TF32X3, 0><<<n2, 256, 0, c->stream>>>(r, pk);
-            break;
-        default:
-            if (pat) k_ny_pack<ACSE_TF32, 1><<<n2, 256, 0, c->stream>>>(r, pk);
-            else k_ny_pack<ACSE_TF32, 0><<<n2, 256, 0, c->stream>>>(r, pk);
-            break;
-    }
-    ACSE_LAUNCHED(c);
-    return ACSE_OK;
 }
 
 // Operands of the six GEMMs (stage 1: X, Y4, Y6; stage 2: S1, S4, S6).  src: 0 = 2Delta blocks,
@@ -341,7 +399,7 @@ int ny_alloc(acse_ctx* c) {
     const bool f64 = c->opt.prec == ACSE_FP64;
     const size_t es = f64 ? 8 : 4;                                  // GEMM output / T element
     for (int g = 0; g < 6; ++g) ACSE_TRY(ny_plan_gemm(y, g));
-    for (int b = 0; b < 3; ++b) ACSE_TRY(ny_malloc((void**)&y->delta[b], r4 * sizeof(double)));
+    for (int b = 0; b < 3; ++b) ACSE_TRY(ny_malloc(&y->delta[b], r4 * es));
     ACSE_TRY(ny_malloc((void**)&y->sig, n * sizeof(double)));
     size_t op_bytes;
     if (f64) {
@@ -392,29 +450,87 @@ int ny_alloc(acse_ctx* c) {
     return ACSE_OK;
 }
 
-static NyPack ny_pk(NyWork* y, int g, int side, const double* const Dl[3], const double* const W[3], void* dst,
-                    size_t ld) {
+// The pieces of operand `side` of GEMM g (the spin blocks that some problem reads), appended to list k.  S[0], S[1]:
+// the 2Delta and W blocks (aa, ab, bb) in the element type of the path.
+static int ny_pieces(NyWork* y, int r, int g, int side, const void* const S[2][3], void* dst, NyPackList* k, int n) {
     const NyOp& op = k_ny_ops[g][side];
-    NyPack k;
-    const double* const* blk = op.src == 0 ? Dl : op.src == 1 ? W : nullptr;
-    for (int b = 0; b < 3; ++b) k.blk[b] = blk ? blk[b] : nullptr;
-    k.dense = op.src >= 2 ? y->out[op.src - 2] : nullptr;
-    for (int q = 0; q < 4; ++q) {
-        k.P[q] = op.P[q];
-        k.korder[q] = y->korder[g][q];
-    }
-    for (int b = 0; b < 4; ++b) k.need[b] = 0;
-    for (int p = 0; p < y->nprob[g]; ++p) {   // row block of this operand -> K blocks its problems read
-        const int rowb = y->prob[g][p][side];
-        for (int q = y->prob[g][p][2]; q < y->prob[g][p][2] + y->prob[g][p][3]; ++q) k.need[rowb] |= 1 << y->korder[g][q];
-    }
-    k.use_sigma = op.sigma;
+    const int R2 = r * r;
+    int need[4] = {0, 0, 0, 0};
+    for (int p = 0; p < y->nprob[g]; ++p)
+        for (int q = y->prob[g][p][2]; q < y->prob[g][p][2] + y->prob[g][p][3]; ++q)
+            need[y->prob[g][p][side]] |= 1 << y->korder[g][q];
+    for (int rb = 0; rb < 4; ++rb)
+        for (int q = 0; q < 4; ++q) {
+            const int kb = y->korder[g][q];
+            if (!(need[rb] >> kb & 1)) continue;
+            NyPiece& pc = k->p[n++];
+            const int su[4] = {rb >> 1, rb & 1, kb >> 1, kb & 1};
+            int sx[4], xst[4];   // spins and strides of the source's four indices
+            for (int m = 0; m < 4; ++m) sx[m] = su[op.P[m]];
+            pc.sign = 1.0f;
+            pc.base = 0;
+            if (op.src < 2) {   // pair-antisymmetric tensor by its aa, ab, bb blocks (as so_get)
+                int pos[4] = {0, 1, 2, 3};
+                int blk = sx[0] == sx[1] ? 2 * sx[0] : 1;
+                if (blk == 1) {
+                    if (sx[0] == 1) { pos[0] = 1; pos[1] = 0; }
+                    // lower indices: alpha first
+                    if (sx[2] == 1) { pos[2] = 3; pos[3] = 2; }
+                    if (sx[0] != sx[2]) pc.sign = -1.0f;
+                }
+                const int stride[4] = {R2 * r, R2, r, 1};
+                for (int m = 0; m < 4; ++m) xst[m] = stride[pos[m]];
+                pc.src = S[op.src][blk];
+            } else {
+                const int n2 = (int)y->n2;
+                const int stride[4] = {r * n2, n2, r, 1};
+                for (int m = 0; m < 4; ++m) xst[m] = stride[m];
+                pc.src = y->out[op.src - 2];
+                pc.base = (size_t)(2 * sx[0] + sx[1]) * R2 * n2 + (size_t)(2 * sx[2] + sx[3]) * R2;
+            }
+            for (int m = 0; m < 4; ++m) pc.st[op.P[m]] = xst[m];
+            if (pc.st[3] == 1) pc.mode = 0;
+            else if (pc.st[2] == 1) pc.mode = 1;
+            else if (pc.st[1] == 1) pc.mode = 2;
+            else return -1;   // contiguous in u0: no operand is
+            pc.dst = dst;
+            pc.rb = rb;
+            pc.q = q;
+            pc.sp2 = su[2];
+            pc.pat = side;
+            pc.use_sigma = op.sigma;
+        }
+    return n;
+}
+
+static int ny_pack_stage(acse_ctx* c, NyWork* y, int s, const void* const S[2][3]) {
+    const int r = c->r;
+    NyPackList k;
+    int n = 0;
+    for (int g = 3 * s; g < 3 * s + 3; ++g)
+        for (int side = 0; side < 2; ++side) {
+            n = ny_pieces(y, r, g, side, S, side ? y->opB[g % 3] : y->opA[g % 3], &k, n);
+            if (n < 0) return ACSE_ERR_UNSUPPORTED;
+        }
     k.sig = y->sig;
-    k.dst = dst;
-    k.ld = ld;
+    k.ld = (size_t)4 * y->Kbw;
     k.Kb = y->Kb;
     k.Kbw = y->Kbw;
-    return k;
+    const size_t es = c->opt.prec == ACSE_FP64 ? sizeof(double) : sizeof(float);
+    // about 4096 elements a block (16 a thread), within the 48 KB of shared memory that need no opt-in
+    int nslab = 4096 / (r * r);
+    nslab = nslab < 1 ? 1 : nslab > 16 ? 16 : nslab;
+    while (nslab > 1 && nslab * (size_t)r * (r + 1) * es > 40 * 1024) --nslab;
+    const size_t sm = nslab * (size_t)r * (r + 1) * es;
+    const int blocks = n * ((r * r + nslab - 1) / nslab);
+    switch (c->opt.prec) {
+        case ACSE_FP64: k_ny_pack<ACSE_FP64><<<blocks, 256, sm, c->stream>>>(r, nslab, k); break;
+        case ACSE_BF16X3: k_ny_pack<ACSE_BF16X3><<<blocks, 256, sm, c->stream>>>(r, nslab, k); break;
+        case ACSE_TF32X3: k_ny_pack<ACSE_TF32X3><<<blocks, 256, sm, c->stream>>>(r, nslab, k); break;
+        default: k_ny_pack<ACSE_TF32><<<blocks, 256, sm, c->stream>>>(r, nslab, k); break;
+    }
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
 }
 
 // The NY term T for the pass in flight (D = c->cur_D, W = c->cur_W, 1D in c->w.gam), left in the
@@ -424,17 +540,23 @@ int ny_pass(acse_ctx* c) {
     if (!y) return ACSE_ERR_UNSUPPORTED;
     const int r = c->r, R2 = r * r;
     const bool f64 = c->opt.prec == ACSE_FP64;
-    k_ny_delta<<<152 * 8, 256, 0, c->stream>>>(r, c->w.gam, c->cur_D[0], c->cur_D[1], c->cur_D[2], y->delta[0],
-                                               y->delta[1], y->delta[2]);
-    ACSE_LAUNCHED(c);
-    const double* Dl[3] = {y->delta[0], y->delta[1], y->delta[2]};
-    const double* W[3] = {c->cur_W[0], c->cur_W[1], c->cur_W[2]};
+    if (c->cur_prep) {   // 2Delta is that of D: the update pass finds the residual pass's
+        if (f64)
+            k_ny_delta<double><<<152 * 8, 256, 0, c->stream>>>(r, c->w.gam, c->cur_D[0], c->cur_D[1], c->cur_D[2],
+                                                               (double*)y->delta[0], (double*)y->delta[1], (double*)y->delta[2]);
+        else
+            k_ny_delta<float><<<152 * 8, 256, 0, c->stream>>>(r, c->w.gam, c->cur_D[0], c->cur_D[1], c->cur_D[2],
+                                                              (float*)y->delta[0], (float*)y->delta[1], (float*)y->delta[2]);
+        ACSE_LAUNCHED(c);
+    }
+    const void* S[2][3];
+    for (int b = 0; b < 3; ++b) {
+        S[0][b] = y->delta[b];
+        S[1][b] = f64 ? (const void*)c->cur_W[b] : (const void*)c->cur_W32[b];
+    }
     const size_t ld = (size_t)4 * y->Kbw;
     for (int s = 0; s < 2; ++s) {
-        for (int g = 3 * s; g < 3 * s + 3; ++g) {
-            ACSE_TRY(ny_pack_launch(c, ny_pk(y, g, 0, Dl, W, y->opA[g % 3], ld), 0));
-            ACSE_TRY(ny_pack_launch(c, ny_pk(y, g, 1, Dl, W, y->opB[g % 3], ld), 1));
-        }
+        ACSE_TRY(ny_pack_stage(c, y, s, S));
         if (f64) {
             GemmF64 gl[48];
             int ng = 0;
@@ -453,19 +575,19 @@ int ny_pass(acse_ctx* c) {
         }
     }
     const int n = y->n;
-    const size_t smem = 2 * (size_t)n * r * (f64 ? sizeof(double) : sizeof(float));
+    const size_t smem = 2 * (size_t)n * ((r + 3) & ~3) * (f64 ? sizeof(double) : sizeof(float));
     if (f64) {
         k_ny_Q<double><<<(n * n + 7) / 8, 256, 0, c->stream>>>(r, (const double*)y->out[0], (double*)y->Q);
         ACSE_LAUNCHED(c);
         k_ny_assemble<double><<<4 * R2, 256, smem, c->stream>>>(
-            r, (const double*)y->out[3], (const double*)y->out[4], (const double*)y->out[5], (const double*)y->Q, Dl[0],
-            Dl[1], Dl[2], y->sig, (double*)y->tny[0], (double*)y->tny[1], (double*)y->tny[2], (double*)y->tny[3]);
+            r, (const double*)y->out[3], (const double*)y->out[4], (const double*)y->out[5], (const double*)y->Q,
+            (const double*)y->delta[0], (const double*)y->delta[1], (const double*)y->delta[2], y->sig, (double*)y->tny[0], (double*)y->tny[1], (double*)y->tny[2], (double*)y->tny[3]);
     } else {
         k_ny_Q<float><<<(n * n + 7) / 8, 256, 0, c->stream>>>(r, (const float*)y->out[0], (float*)y->Q);
         ACSE_LAUNCHED(c);
         k_ny_assemble<float><<<4 * R2, 256, smem, c->stream>>>(
-            r, (const float*)y->out[3], (const float*)y->out[4], (const float*)y->out[5], (const float*)y->Q, Dl[0],
-            Dl[1], Dl[2], y->sig, (float*)y->tny[0], (float*)y->tny[1], (float*)y->tny[2], (float*)y->tny[3]);
+            r, (const float*)y->out[3], (const float*)y->out[4], (const float*)y->out[5], (const float*)y->Q,
+            (const float*)y->delta[0], (const float*)y->delta[1], (const float*)y->delta[2], y->sig, (float*)y->tny[0], (float*)y->tny[1], (float*)y->tny[2], (float*)y->tny[3]);
     }
     ACSE_LAUNCHED(c);
     return ACSE_OK;
