@@ -25,6 +25,11 @@ __device__ __forceinline__ void ps_unpair(int r, int u, int& a, int& b) {
     a = t;
     b = t + (u - ps_pair(r, t, t));
 }
+// The pair a < b of number u of pk_pair (the pairs a <= b - 1 of r - 1 indices).
+__device__ __forceinline__ void pk_unpair(int r, int u, int& a, int& b) {
+    ps_unpair(r - 1, u, a, b);
+    ++b;
+}
 
 // ------------------------------------------------------------------------------------------
 // Dense GEMM problem: C[m*ldc + n] = alpha * sum_k A(m,k) B(n,k) (+ beta*C), with

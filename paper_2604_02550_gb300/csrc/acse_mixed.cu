@@ -53,19 +53,23 @@ static MxPtrs mx_ptrs(acse_ctx* c) {
 // M = 3 2D - 2 (1D^1D) in FP32 (App. C), stored plain (M32) and as rows 0..r^2-1 of the pair
 // operand [M; D]; rows r^2..2r^2-1 hold D.  Also rounds the FP64 1-RDM to FP32.  One block per
 // (sector, pair ij): the D row ij is read and rounded to FP32 once and gives both the M row ij and the
-// D row r^2 + ij (the FP64 -> FP32 conversions run on the slow FP64 pipe); each thread handles groups
-// of four consecutive columns (16-byte loads and vector stores when r is even); the two 1-RDM rows the
-// M row needs are staged in shared memory.  RC: r as a compile-time constant (0: runtime r).
+// D row r^2 + ij (the FP64 -> FP32 conversions run on the slow FP64 pipe); the two 1-RDM rows the
+// M row needs are staged in shared memory.  The mixed sector of an even r goes straight from the 16-byte loads to the
+// vector stores; otherwise the M and D rows pass through shared memory, from which the operand rows (16-byte aligned
+// for every r) are written in groups of four K positions: consecutive columns, or consecutive packed pairs a < b of a
+// same-spin row.  (Single stores of packed pairs and of an odd r: 54 us at r = 48 and 53 at r = 31, now 49 and 26.)
+// RC: r as a compile-time constant (0: runtime r).
 template <int PREC, int RC>
 __global__ void __launch_bounds__(192) k_mx_prepD(int r_, const double* __restrict__ gam, const double* __restrict__ Daa,
                                                   const double* __restrict__ Dab, const double* __restrict__ Dbb,
                                                   const __grid_constant__ MxPtrs p) {
+    extern __shared__ __align__(16) float pd_smem[];   // x [R4], m [R4]; R4 = r^2 rounded up to 4
     __shared__ float g1[ACSE_MAX_R], g2[ACSE_MAX_R];
     const int r = RC ? RC : r_;
-    const int R2 = r * r;
-    const int c4 = (R2 + 3) >> 2;
+    const int R2 = r * r, R4 = (R2 + 3) & ~3;
     const int s = blockIdx.x / R2;
     const int row = blockIdx.x - s * R2;   // pair ij: M row ij and D row r^2 + ij
+    float *xs = pd_smem, *ms = pd_smem + R4;
     if (blockIdx.x == 0)
         for (int e = threadIdx.x; e < 2 * R2; e += blockDim.x) p.gam32[e] = (float)gam[e];
     const int i = row / r, j = row - (row / r) * r;
@@ -83,67 +87,87 @@ __global__ void __launch_bounds__(192) k_mx_prepD(int r_, const double* __restri
     const size_t ldP = (size_t)p.ns * p.KpP;
     // packed rows of a same-spin sector (pairs i < j only): M at pk(i, j), D at P + pk(i, j)
     const int P = r * (r - 1) / 2;
-    const int prow = i < j ? pk_pair(r, i, j) : -1;
+    const int prow = s != 1 && i < j ? pk_pair(r, i, j) : -1;
     const double* D = (s == 0 ? Daa : (s == 1 ? Dab : Dbb)) + (size_t)row * R2;
     float* Mrow = p.M32[s] + (size_t)row * R2;
-    const bool vec = (r & 1) == 0 && ((reinterpret_cast<uintptr_t>(s == 0 ? Daa : (s == 1 ? Dab : Dbb)) & 15) == 0);
-    for (int q4 = threadIdx.x; q4 < c4; q4 += blockDim.x) {
-        const int k0 = q4 * 4;
-        const int nk = R2 - k0 < 4 ? R2 - k0 : 4;
-        float x[4] = {0.f, 0.f, 0.f, 0.f}, m[4] = {0.f, 0.f, 0.f, 0.f};
-        if (vec && nk == 4) {
+    // (int)((e + 1/2) / r) = e / r for e < r^2: the fraction stays at least 1/(2r) from an integer
+    const float invr = 1.f / (float)r;
+    if ((r & 1) == 0 && ((reinterpret_cast<uintptr_t>(s == 0 ? Daa : (s == 1 ? Dab : Dbb)) & 15) == 0)) {
+        for (int q4 = threadIdx.x; q4 < R2 / 4; q4 += blockDim.x) {
+            const int k0 = q4 * 4;
+            float x[4], m[4];
             const double2 d01 = *reinterpret_cast<const double2*>(D + k0);
             const double2 d23 = *reinterpret_cast<const double2*>(D + k0 + 2);
             x[0] = (float)d01.x; x[1] = (float)d01.y; x[2] = (float)d23.x; x[3] = (float)d23.y;
-        } else {
-            for (int u = 0; u < nk; ++u) x[u] = (float)D[k0 + u];
-        }
-        {
-            int kk = k0 / r, l = k0 - kk * r;
+            int kk = RC ? k0 / r : (int)(((float)k0 + 0.5f) * invr), l = k0 - kk * r;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (u < nk) m[u] = s == 1 ? 3.0f * x[u] - g1[kk] * g2[l] : 3.0f * x[u] - (g1[kk] * g2[l] - g2[kk] * g1[l]);
+                m[u] = s == 1 ? 3.0f * x[u] - g1[kk] * g2[l] : 3.0f * x[u] - (g1[kk] * g2[l] - g2[kk] * g1[l]);
                 if (++l == r) { l = 0; ++kk; }
             }
-        }
-        if (vec && nk == 4) *reinterpret_cast<float4*>(Mrow + k0) = make_float4(m[0], m[1], m[2], m[3]);
-        else
-            for (int u = 0; u < nk; ++u) Mrow[k0 + u] = m[u];
-        if (s == 1) {
-            if (vec && nk == 4) {
+            *reinterpret_cast<float4*>(Mrow + k0) = make_float4(m[0], m[1], m[2], m[3]);
+            if (s == 1) {
                 put4<PREC, 0>(p.pairA[s], row, ld, p.Kp1, k0, m);
                 put4<PREC, 0>(p.pairA[s], (size_t)R2 + row, ld, p.Kp1, k0, x);
-            } else {
-                for (int u = 0; u < nk; ++u) {
-                    put<PREC, 0>(p.pairA[s], row, ld, p.Kp1, k0 + u, m[u]);
-                    put<PREC, 0>(p.pairA[s], (size_t)R2 + row, ld, p.Kp1, k0 + u, x[u]);
-                }
-            }
-        } else if (prow >= 0) {
-            // same-spin sector: rows and K restricted to pairs a < b (antisymmetry; the GEMM's alpha
-            // carries the factor 2 of the (r, s) sum)
-            int kk = k0 / r, l = k0 - kk * r;
-            for (int u = 0; u < nk; ++u) {
-                if (kk < l) {
-                    const int kq = pk_pair(r, kk, l);
-                    put<PREC, 0>(p.pairA[s], (size_t)prow, ldP, p.KpP, kq, m[u]);
-                    put<PREC, 0>(p.pairA[s], (size_t)(P + prow), ldP, p.KpP, kq, x[u]);
-                }
-                if (++l == r) { l = 0; ++kk; }
+            } else if (prow >= 0) {
+                *reinterpret_cast<float4*>(xs + k0) = make_float4(x[0], x[1], x[2], x[3]);
+                *reinterpret_cast<float4*>(ms + k0) = make_float4(m[0], m[1], m[2], m[3]);
             }
         }
+        if (prow < 0) return;
+    } else {
+#pragma unroll 4
+        for (int e = threadIdx.x; e < R4; e += blockDim.x) {
+            float x = 0.f, m = 0.f;
+            if (e < R2) {
+                const int kk = (int)(((float)e + 0.5f) * invr), l = e - kk * r;
+                x = (float)D[e];
+                m = s == 1 ? 3.0f * x - g1[kk] * g2[l] : 3.0f * x - (g1[kk] * g2[l] - g2[kk] * g1[l]);
+                Mrow[e] = m;
+            }
+            xs[e] = x;
+            ms[e] = m;
+        }
+        if (s != 1 && prow < 0) return;
+    }
+    __syncthreads();
+    if (s == 1) {   // columns from r^2 to R4: zeros, as in the rows' padding
+        for (int q4 = threadIdx.x; q4 < R4 / 4; q4 += blockDim.x) {
+            const int k0 = 4 * q4;
+            const float x[4] = {xs[k0], xs[k0 + 1], xs[k0 + 2], xs[k0 + 3]}, m[4] = {ms[k0], ms[k0 + 1], ms[k0 + 2], ms[k0 + 3]};
+            put4<PREC, 0>(p.pairA[s], row, ld, p.Kp1, k0, m);
+            put4<PREC, 0>(p.pairA[s], (size_t)R2 + row, ld, p.Kp1, k0, x);
+        }
+        return;
+    }
+    // same-spin sector: rows and K restricted to pairs a < b (antisymmetry; the GEMM's alpha carries the factor 2
+    // of the (r, s) sum); the positions from P to the next multiple of four are zeros, as the padding
+    for (int q4 = threadIdx.x; q4 < (P + 3) / 4; q4 += blockDim.x) {
+        int a, b;
+        pk_unpair(r, 4 * q4, a, b);
+        float x[4], m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool in = 4 * q4 + u < P;
+            x[u] = in ? xs[a * r + b] : 0.f;
+            m[u] = in ? ms[a * r + b] : 0.f;
+            if (++b >= r) { ++a; b = a + 1; }
+        }
+        put4<PREC, 0>(p.pairA[s], (size_t)prow, ldP, p.KpP, 4 * q4, m);
+        put4<PREC, 0>(p.pairA[s], (size_t)(P + prow), ldP, p.KpP, 4 * q4, x);
     }
 }
 
 template <int PREC>
 static void launch_prepD(acse_ctx* c, int nsec, const double* const D[3], const MxPtrs& p) {
     const int r = c->r, g = nsec * r * r;
+    const size_t sm = 2 * (size_t)((r * r + 3) & ~3) * sizeof(float);   // 32 KB at r = 64
     switch (r) {
-        case 16: k_mx_prepD<PREC, 16><<<g, 192, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
-        case 32: k_mx_prepD<PREC, 32><<<g, 192, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
-        case 48: k_mx_prepD<PREC, 48><<<g, 192, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
-        case 64: k_mx_prepD<PREC, 64><<<g, 192, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
-        default: k_mx_prepD<PREC, 0><<<g, 192, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
+        case 16: k_mx_prepD<PREC, 16><<<g, 192, sm, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
+        case 32: k_mx_prepD<PREC, 32><<<g, 192, sm, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
+        case 48: k_mx_prepD<PREC, 48><<<g, 192, sm, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
+        case 64: k_mx_prepD<PREC, 64><<<g, 192, sm, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
+        default: k_mx_prepD<PREC, 0><<<g, 192, sm, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], p); break;
     }
 }
 
@@ -151,41 +175,50 @@ static void launch_prepD(acse_ctx* c, int nsec, const double* const D[3], const 
 //   t=0 Md(a,a) rows (a,i,l) cols (a,p,s) <- Maa[i][p][l][s]      t=1 Md(a,b) <- Mab[i][p][l][s]
 //   t=2 Md(b,a) rows (b,i,l) cols (a,p,s) <- Mab[p][i][s][l]      t=3 Md(b,b) <- Mbb[i][p][l][s]
 //   t=4 Mf1[(i,l)][(p,s)] <- Mab[i][p][s][l]                        t=5 Mf2[(i,l)][(p,s)] <- Mab[p][i][l][s]
-// (transposed source blocks go through shared memory so that reads and writes stay coalesced).
+// (transposed source blocks go through shared memory so that reads and writes stay coalesced).  A block takes np
+// consecutive p, whose columns follow one another in the row: longer runs of stores, and an r that is not a multiple of
+// four still writes groups of four columns (the row's first and last few singly).  One p a block and, for such r, single
+// stores took 104 us at r = 48, 75 at r = 40 (TF32x3) and 23 at r = 31; now 60, 47 and 19.
 template <int PREC, int RC>
-__global__ void __launch_bounds__(256) k_mx_pack_Mph(int r_, const __grid_constant__ MxPtrs p) {
-    __shared__ float tile[ACSE_MAX_R][ACSE_MAX_R + 1];
+__global__ void __launch_bounds__(256) k_mx_pack_Mph(int r_, int np, const __grid_constant__ MxPtrs p) {
+    extern __shared__ __align__(16) float pm_smem[];   // [np][r][r + 1]
     const int r = RC ? RC : r_;   // compile-time r where it is one of the tensor-core sizes
-    const int R2 = r * r;
-    const int t = blockIdx.x / R2, ip = blockIdx.x % R2;
-    const int i = ip / r, pp = ip % r;
+    const int R2 = r * r, ldt = r + 1, npb = (r + np - 1) / np;
+    const int t = blockIdx.x / (r * npb), ip = blockIdx.x - t * r * npb;
+    const int i = ip / npb, pp = (ip - i * npb) * np, n = min(np, r - pp);
     const size_t r3 = (size_t)R2 * r;
+    const float invr = 1.f / (float)r, invR2 = 1.f / (float)R2;   // quotients below 2^16, as in k_mx_prepD
     const float* src;
     bool tr;
+    size_t sp;   // from one p to the next
     switch (t) {
-        case 0: src = p.M32[0] + i * r3 + (size_t)pp * R2; tr = false; break;
-        case 1: src = p.M32[1] + i * r3 + (size_t)pp * R2; tr = false; break;
-        case 2: src = p.M32[1] + pp * r3 + (size_t)i * R2; tr = true; break;
-        case 3: src = p.M32[2] + i * r3 + (size_t)pp * R2; tr = false; break;
-        case 4: src = p.M32[1] + i * r3 + (size_t)pp * R2; tr = true; break;
-        default: src = p.M32[1] + pp * r3 + (size_t)i * R2; tr = false; break;
+        case 0: src = p.M32[0] + i * r3 + (size_t)pp * R2; sp = R2; tr = false; break;
+        case 1: src = p.M32[1] + i * r3 + (size_t)pp * R2; sp = R2; tr = false; break;
+        case 2: src = p.M32[1] + pp * r3 + (size_t)i * R2; sp = r3; tr = true; break;
+        case 3: src = p.M32[2] + i * r3 + (size_t)pp * R2; sp = R2; tr = false; break;
+        case 4: src = p.M32[1] + i * r3 + (size_t)pp * R2; sp = R2; tr = true; break;
+        default: src = p.M32[1] + pp * r3 + (size_t)i * R2; sp = r3; tr = false; break;
     }
     if ((r & 1) == 0) {   // r^2 % 4 == 0 and every source block starts on a 16-byte boundary
-        for (int e4 = threadIdx.x; e4 < R2 / 4; e4 += blockDim.x) {
-            const float4 q = reinterpret_cast<const float4*>(src)[e4];
+        for (int e4 = threadIdx.x; e4 < n * (R2 / 4); e4 += blockDim.x) {
+            const int w = RC ? 4 * e4 / R2 : (int)(((float)(4 * e4) + 0.5f) * invR2);
+            const int g = 4 * e4 - w * R2;
+            const float4 q = *reinterpret_cast<const float4*>(src + w * sp + g);
             const float qv[4] = {q.x, q.y, q.z, q.w};
+            float* tile = pm_smem + (size_t)w * r * ldt;
+            int u = RC ? g / r : (int)(((float)g + 0.5f) * invr), v = g - u * r;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const int e = 4 * e4 + c, u = e / r, v = e - u * r;
-                if (tr) tile[v][u] = qv[c];
-                else tile[u][v] = qv[c];
+                tile[tr ? v * ldt + u : u * ldt + v] = qv[c];
+                if (++v == r) { v = 0; ++u; }
             }
         }
     } else {
-        for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-            const int u = e / r, v = e % r;
-            if (tr) tile[v][u] = src[e];
-            else tile[u][v] = src[e];
+#pragma unroll 4
+        for (int e = threadIdx.x; e < n * R2; e += blockDim.x) {
+            const int w = (int)(((float)e + 0.5f) * invR2), g = e - w * R2;
+            const int u = (int)(((float)g + 0.5f) * invr), v = g - u * r;
+            pm_smem[(size_t)w * r * ldt + (tr ? v * ldt + u : u * ldt + v)] = src[w * sp + g];
         }
     }
     __syncthreads();
@@ -199,29 +232,40 @@ __global__ void __launch_bounds__(256) k_mx_pack_Mph(int r_, const __grid_consta
         dst = p.Mf[t - 4]; ld = (size_t)p.ns * p.Kp1; Kp = p.Kp1;
         rowbase = i * r; colbase = pp * r;
     }
-    if ((r & 3) == 0) {   // four consecutive columns of one row per thread, vector stores
-        for (int g = threadIdx.x; g < R2 / 4; g += blockDim.x) {
-            const int l = (4 * g) / r, s0 = 4 * g - l * r;
-            const float x[4] = {tile[l][s0], tile[l][s0 + 1], tile[l][s0 + 2], tile[l][s0 + 3]};
-            put4<PREC, 1>(dst, (size_t)rowbase + l, ld, Kp, colbase + s0, x);
+    const int nc = n * r;   // columns colbase .. colbase + nc - 1 of rows rowbase .. rowbase + r - 1
+    const int head = min(nc, (4 - (colbase & 3)) & 3), n4 = (nc - head) / 4, single = nc - 4 * n4;
+    const float invn4 = n4 ? 1.f / (float)n4 : 0.f;
+    for (int g = threadIdx.x; g < r * n4; g += blockDim.x) {
+        const int l = (int)(((float)g + 0.5f) * invn4), x0 = head + 4 * (g - l * n4);
+        int w = (int)(((float)x0 + 0.5f) * invr), s0 = x0 - w * r;
+        float x[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            x[c] = pm_smem[(size_t)(w * r + l) * ldt + s0];
+            if (++s0 == r) { s0 = 0; ++w; }
         }
-    } else {
-        for (int e = threadIdx.x; e < R2; e += blockDim.x) {
-            const int l = e / r, s2 = e % r;
-            put<PREC, 1>(dst, (size_t)rowbase + l, ld, Kp, colbase + s2, tile[l][s2]);
-        }
+        put4<PREC, 1>(dst, (size_t)rowbase + l, ld, Kp, colbase + x0, x);
+    }
+    for (int e = threadIdx.x; e < r * single; e += blockDim.x) {
+        const int l = e / single, q = e - l * single, x0 = q < head ? q : 4 * n4 + q;
+        const int w = x0 / r, s0 = x0 - w * r;
+        put<PREC, 1>(dst, (size_t)rowbase + l, ld, Kp, colbase + x0, pm_smem[(size_t)(w * r + l) * ldt + s0]);
     }
 }
 
 template <int PREC>
 static void launch_pack_Mph(acse_ctx* c, int nph, const MxPtrs& q) {
-    const int r = c->r, g = nph * r * r;
+    const int r = c->r;
+    int np = 4;   // as far as 48 KB hold them
+    while (np > 1 && np * (size_t)r * (r + 1) * sizeof(float) > 48 * 1024) --np;
+    const int g = nph * r * ((r + np - 1) / np);
+    const size_t sm = np * (size_t)r * (r + 1) * sizeof(float);
     switch (r) {
-        case 16: k_mx_pack_Mph<PREC, 16><<<g, 256, 0, c->stream>>>(r, q); break;
-        case 32: k_mx_pack_Mph<PREC, 32><<<g, 256, 0, c->stream>>>(r, q); break;
-        case 48: k_mx_pack_Mph<PREC, 48><<<g, 256, 0, c->stream>>>(r, q); break;
-        case 64: k_mx_pack_Mph<PREC, 64><<<g, 256, 0, c->stream>>>(r, q); break;
-        default: k_mx_pack_Mph<PREC, 0><<<g, 256, 0, c->stream>>>(r, q); break;
+        case 16: k_mx_pack_Mph<PREC, 16><<<g, 256, sm, c->stream>>>(r, np, q); break;
+        case 32: k_mx_pack_Mph<PREC, 32><<<g, 256, sm, c->stream>>>(r, np, q); break;
+        case 48: k_mx_pack_Mph<PREC, 48><<<g, 256, sm, c->stream>>>(r, np, q); break;
+        case 64: k_mx_pack_Mph<PREC, 64><<<g, 256, sm, c->stream>>>(r, np, q); break;
+        default: k_mx_pack_Mph<PREC, 0><<<g, 256, sm, c->stream>>>(r, np, q); break;
     }
 }
 
@@ -266,30 +310,30 @@ __global__ void k_mx_pack_W(int r_, const float* __restrict__ Waa, const float* 
     const size_t ld = (size_t)p.ns * p.Kp1;
     const float* W = (s == 0 ? Waa : (s == 1 ? Wab : Wbb)) + (size_t)row * R2;   // FP32 copy of W
     const int k0 = q4 * 4;
-    const int nk = R2 - k0 < 4 ? R2 - k0 : 4;
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    if ((r & 1) == 0 && nk == 4) {   // r^2 % 4 == 0: every row starts on a 16-byte boundary
-        const float4 v = *reinterpret_cast<const float4*>(W + k0);
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-    } else {
-        for (int u = 0; u < nk; ++u) x[u] = W[k0 + u];
-    }
-    if (s == 1) {
-        if ((r & 1) == 0 && nk == 4) put4<PREC, 1>(p.pairB[s], row, ld, p.Kp1, k0, x);
-        else
-            for (int u = 0; u < nk; ++u) put<PREC, 1>(p.pairB[s], row, ld, p.Kp1, k0 + u, x[u]);
+    float x[4];
+    if (s == 1) {   // columns from r^2 to the next multiple of four: zeros, as the rows' padding
+        if ((r & 1) == 0) {   // r^2 % 4 == 0: every row starts on a 16-byte boundary
+            const float4 v = *reinterpret_cast<const float4*>(W + k0);
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = k0 + u < R2 ? W[k0 + u] : 0.f;
+        }
+        put4<PREC, 1>(p.pairB[s], row, ld, p.Kp1, k0, x);
         return;
     }
-    // same-spin sector: rows (k, p) and K (r, s) restricted to pairs a < b
-    const int kr = row / r, pr = row - (row / r) * r;
-    if (kr >= pr) return;
+    // same-spin sector: rows (k, p) and K (r, s) restricted to pairs a < b, four packed positions a thread
+    const int kr = row / r, pr = row - (row / r) * r, P = r * (r - 1) / 2;
+    if (kr >= pr || k0 >= P) return;
     const size_t ldP = (size_t)p.ns * p.KpP;
-    const int prow = pk_pair(r, kr, pr);
-    int a = k0 / r, b = k0 - a * r;
-    for (int u = 0; u < nk; ++u) {
-        if (a < b) put<PREC, 1>(p.pairB[s], (size_t)prow, ldP, p.KpP, pk_pair(r, a, b), x[u]);
-        if (++b == r) { b = 0; ++a; }
+    int a, b;
+    pk_unpair(r, k0, a, b);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        x[u] = k0 + u < P ? W[a * r + b] : 0.f;
+        if (++b >= r) { ++a; b = a + 1; }
     }
+    put4<PREC, 1>(p.pairB[s], (size_t)pk_pair(r, kr, pr), ldP, p.KpP, k0, x);
 }
 
 // Rows (i, j), i < j, of [X; Y] of a same-spin sector from the packed GEMM output:

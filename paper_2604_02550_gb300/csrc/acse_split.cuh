@@ -39,7 +39,7 @@ __device__ __forceinline__ void put(void* base, size_t row, size_t ld, int Kp, i
 }
 
 // Four consecutive K positions k..k+3 of one row at once (8-byte stores for BF16, 16-byte for TF32);
-// requires k % 4 == 0 and a row length that keeps 8/16-byte alignment (true when r is even).
+// requires k % 4 == 0 (every K segment is a multiple of 128 bytes long, whatever r).
 template <int PREC, int PAT>
 __device__ __forceinline__ void put4(void* base, size_t row, size_t ld, int Kp, int k, const float (&x)[4]) {
     if (PREC == ACSE_BF16X3) {

@@ -524,6 +524,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     } else {
         const int q = warp & 3;   // TMEM lane quadrant this warp may access
         const uint32_t acce0 = mapa_rank(smem_u32(acce), 0);
+        float* est = (float*)((uint8_t*)full + 256) + q * (32 * 33);
         int lt = 0;
         for (int qi = q0; qi < q1; ++qi, ++lt) {
             const int t = b.order[qi];
@@ -551,8 +552,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * BN + c * 32), v);   // warp-collective
                 const int col0 = n0 + c * 32;
-                if (store && row < P.M && col0 < P.N) {
-                    if (vec && col0 + 32 <= P.N) {
+                if (!store || col0 >= P.N) continue;
+                if (vec && col0 + 32 <= P.N) {
+                    if (row < P.M) {
 #pragma unroll
                         for (int j = 0; j < 32; j += 4) {
                             float4 o = make_float4(P.alpha * __uint_as_float(v[j]), P.alpha * __uint_as_float(v[j + 1]),
@@ -560,8 +562,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
                                                    P.alpha * __uint_as_float(v[j + 3]));
                             *reinterpret_cast<float4*>(Crow + col0 + j) = o;
                         }
-                    } else {
-                        for (int j = 0; j < 32 && col0 + j < P.N; ++j) Crow[col0 + j] = P.alpha * __uint_as_float(v[j]);
+                    }
+                } else {
+                    // rows that start on no 16-byte boundary (r odd) or end within the chunk: 32 x 32 values through
+                    // shared memory, a row a store (a thread per row took 32 sectors a store: r = 31 96 -> 66 us)
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) est[lane * 33 + j] = P.alpha * __uint_as_float(v[j]);
+                    __syncwarp();
+                    const int nrow = min(32, P.M - (row - lane));
+                    if (col0 + lane < P.N) {
+                        float* Cc = Crow - (size_t)lane * P.ldc + col0 + lane;
+#pragma unroll 8
+                        for (int j = 0; j < nrow; ++j) Cc[(size_t)j * P.ldc] = est[j * 33 + lane];
                     }
                 }
             }
@@ -594,7 +606,8 @@ static size_t smem_for(int bn, int stages) { return (size_t)stages * (TC_BM + bn
 #ifndef TC2_STAGES
 #define TC2_STAGES 6                         // ring depth of the CTA-pair kernel (32 KB a stage per CTA)
 #endif
-static size_t smem_pair() { return (size_t)TC2_STAGES * (TC_BM + 128) * 128 + 1024 + 256; }
+// ring, alignment, barriers, and the four epilogue warps' 32 x 33 staging
+static size_t smem_pair() { return (size_t)TC2_STAGES * (TC_BM + 128) * 128 + 1024 + 256 + 4 * 32 * 33 * sizeof(float); }
 
 // Clusters of the CTA-pair kernel that fit on the device at once (its persistent grid).
 template <int KIND>
