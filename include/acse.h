@@ -12,9 +12,11 @@
  *   * 2D^{pq}_{rs} = 1/2 <a+_p a+_q a_s a_r>;  Tr 2D = N(N-1)/2.
  *   * Spin blocks, spatial indices 0..r-1, full-square row-major [i][j][k][l]:
  *       X_aa = X^{ia ja}_{ka la},  X_ab = X^{ia jb}_{ka lb},  X_bb = X^{ib jb}_{kb lb}.
- *     Each block is r^4 doubles.  The aa and bb blocks are antisymmetric in (i,j) and in (k,l), and every
- *     block of a (real) 2-RDM is pair-Hermitian, X[ij][kl] = X[kl][ij]: the library relies on both and reads
- *     entries that these symmetries relate once.
+ *     Each block is r^4 doubles.  The aa and bb blocks are antisymmetric in (i,j) and in (k,l): the library
+ *     relies on it and reads entries that it relates once.  Every block of a (real) 2-RDM is also
+ *     pair-Hermitian, X[ij][kl] = X[kl][ij].  A D that is not, by more than 2^-47 of its largest entry, is
+ *     contracted as given, at about 1.5 times the cost in ACSE_FP64 and ACSE_OZAKI (the commutator form of
+ *     Appendix B has used the Hermiticity of K and D, so A is then that form's value, not a commutator's).
  *   * h: r x r one-electron integrals; V: r^4 two-electron integrals in chemist's notation
  *     (pq|rs) stored [p][q][r][s].
  *   * Reduced Hamiltonian (Eq. 2):  K = 1/2(<pq|rs> - <pq|sr>)
@@ -178,7 +180,8 @@ int acse_step(acse_ctx* ctx, double* Daa, double* Dab, double* Dbb, double eps,
  * D_ckpt: n_steps+1 checkpoints, D_ckpt[3k+0..2] = (Daa, Dab, Dbb) of D_k (any of them may be
  * NULL except D_0; missing ones are recomputed from the previous one).  dh and dV are
  * symmetrised (h: p<->q; V: the 8-fold permutational symmetry); dD is projected onto tensors
- * with the symmetries of a 2-RDM (antisymmetric within pairs, pair-Hermitian).  Each output
+ * with the symmetries of a 2-RDM (antisymmetric within pairs, pair-Hermitian), which the checkpoints
+ * must have: the reverse sweep rests on the commutator's antisymmetry, which holds for those.  Each output
  * may be NULL.  The reverse sweep is FP64-accurate: FP64 FMA GEMMs in an ACSE_FP64 context, GEMMs by
  * the Ozaki scheme on the tensor cores in an ACSE_OZAKI context; a context in a split precision runs it
  * in an ACSE_OZAKI companion context the library creates on first use (same integrals and options,

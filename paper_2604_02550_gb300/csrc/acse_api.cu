@@ -98,7 +98,7 @@ static int alloc_d(void** p, size_t bytes, size_t* total) {
 
 static void free_work(acse_ctx* c) {
     Work& w = c->w;
-    void* ptrs[] = {w.Kh[0], w.Kh[1], w.Kh[2], w.gam, w.M[0], w.M[1], w.M[2], w.Mp, w.Mm, w.Mf1, w.Wp, w.Wm, w.Wf1,
+    void* ptrs[] = {w.Kh[0], w.Kh[1], w.Kh[2], w.gam, w.M[0], w.M[1], w.M[2], w.Mp, w.Mm, w.Mf1, w.Mf2, w.dmax, w.asym, w.Wp, w.Wm, w.Wf1,
                     w.V5d, w.V5f1, w.V5f2, w.Cp[0], w.Cp[1], w.pmap, w.bx64[0], w.w, w.Q, w.X[0], w.X[1], w.X[2], w.Y[0], w.Y[1], w.Y[2], w.X5d, w.X5f1, w.X5f2,
                     w.H[0], w.H[1], w.H[2], w.zdiag, w.A[0], w.A[1], w.A[2], w.U[0], w.U[1], w.U[2], w.Dt[0],
                     w.Dt[1], w.Dt[2], w.stage_in[0], w.stage_in[1], w.stage_in[2], w.stage_out[0],
@@ -128,12 +128,14 @@ static int alloc_work(acse_ctx* c) {
         A_(w.w, 2 * R2 * sizeof(double));
         A_(w.Q, 2 * R2 * sizeof(double));
         const size_t S2 = (size_t)c->r * (c->r + 1), P2 = (size_t)c->r * (c->r - 1);   // pairs a <= b, a < b, two spins
-        A_(w.Mp, S2 * S2 * sizeof(double)); A_(w.Mm, P2 * P2 * sizeof(double)); A_(w.Mf1, b4);
+        A_(w.Mp, 2 * R2 * S2 * sizeof(double)); A_(w.Mm, 2 * R2 * P2 * sizeof(double)); A_(w.Mf1, b4); A_(w.Mf2, b4);
+        A_(w.dmax, 2 * sizeof(unsigned long long)); A_(w.asym, sizeof(int));
+        ACSE_CUDA_TRY(cudaMemsetAsync(w.dmax, 0, 2 * sizeof(unsigned long long), c->stream));
         A_(w.Wp, S2 * S2 * sizeof(double)); A_(w.Wm, S2 * P2 * sizeof(double)); A_(w.Wf1, b4);
         A_(w.V5d, 4 * b4); A_(w.V5f1, b4); A_(w.V5f2, b4);
         A_(w.X5d, 4 * b4); A_(w.X5f1, b4); A_(w.X5f2, b4);
-        w.V1 = w.X5d;              // S2^2 + S2 P2 = 2 r^4 + 2 r^3 <= 4 r^4
-        w.V2 = w.X5d + S2 * S2;
+        w.V1 = w.X5d;              // S2 and P2 rows of 2 r^2 (s = -1: P2 and S2): 4 r^4 together
+        w.Vf2 = w.X5f1;
         for (int s = 0; s < 2; ++s) A_(w.Cp[s], P2 * P2 / 2 * sizeof(double));
         A_(w.bx64[0], 8 * b4);   // one block, eight classes
         for (int k = 1; k < 8; ++k) w.bx64[k] = w.bx64[0] + k * n4;
@@ -290,22 +292,27 @@ int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const
 // The FP64 GEMMs of the pass whose operands acse_contract_pre prepared, longest contraction first: the
 // particle-hole products on symmetrised pairs (acse_ph.cu; with S, P the pairs a <= b, a < b, V1 has rows over
 // S and V2 over P for s = +1, the other way round for s = -1), the flip, X and Y of the mixed-spin pairs (their
-// (rs) sums count both orders, a factor 2) and of the same-spin pairs i < j (alpha 2 for the halved sum).
+// (rs) sums count both orders, a factor 2) and of the same-spin pairs i < j (alpha 2 for the halved sum); last the three
+// products of a D that is not pair-Hermitian.
 int acse_gemm_list_f64(acse_ctx* c, int sW, GemmF64* g, int* n) {
     Work& w = c->w;
     const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
     const int n1 = sW > 0 ? S2 : P2, n2 = sW > 0 ? P2 : S2;
     int k = 0;
-    g[k++] = GemmF64{w.Wp, w.Mp, w.V1, n1, S2, S2, S2, S2, S2, 1.0, 0.0, nullptr, nullptr};
-    g[k++] = GemmF64{w.Wf1, w.Mf1, w.V5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr};
-    g[k++] = GemmF64{w.M[1], c->cur_W[1], w.X[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr};
-    g[k++] = GemmF64{c->cur_D[1], c->cur_W[1], w.Y[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr};
-    g[k++] = GemmF64{w.Wm, w.Mm, w.V2, n2, P2, P2, P2, P2, P2, 1.0, 0.0, nullptr, nullptr};
+    double* const V2 = ph_V2(c, sW);
+    g[k++] = GemmF64{w.Wp, w.Mp, w.V1, n1, S2, S2, S2, S2, 2 * R2, 1.0, 0.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wf1, w.Mf1, w.V5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.M[1], c->cur_W[1], w.X[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{c->cur_D[1], c->cur_W[1], w.Y[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wm, w.Mm, V2, n2, P2, P2, P2, P2, 2 * R2, 1.0, 0.0, nullptr, nullptr, nullptr};
     for (int s = 0; s < 3; s += 2) {
         double* C = w.Cp[s / 2];
-        g[k++] = GemmF64{w.M[s], c->cur_W[s], C, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap};
-        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], C + (size_t)P * P, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap};
+        g[k++] = GemmF64{w.M[s], c->cur_W[s], C, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap, nullptr};
+        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], C + (size_t)P * P, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap, nullptr};
     }
+    g[k++] = GemmF64{w.Wp, w.Mp + (size_t)S2 * S2, w.V1 + S2, n1, P2, S2, S2, S2, 2 * R2, 1.0, 0.0, nullptr, nullptr, w.asym};
+    g[k++] = GemmF64{w.Wm, w.Mm + (size_t)P2 * P2, V2 + P2, n2, S2, P2, P2, P2, 2 * R2, 1.0, 0.0, nullptr, nullptr, w.asym};
+    g[k++] = GemmF64{w.Wf1, w.Mf2, w.Vf2, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr, w.asym};
     *n = k;
     return ACSE_OK;
 }

@@ -138,7 +138,7 @@ static int cgrid(size_t n) {
 // --------------------------------------------------------------------------- one step
 static int gemm_pass(acse_batch* B, int sW) {
     if (B->prec == ACSE_FP64) {
-        // FP64: every instance's GEMMs in one grouped DFMA launch (split in chunks of 40 inside)
+        // FP64: every instance's GEMMs in one grouped DFMA launch (split in chunks of 54 inside)
         std::vector<GemmF64> all;
         for (int i = 0; i < B->n; ++i) {
             acse_ctx* c = B->ctx[i];

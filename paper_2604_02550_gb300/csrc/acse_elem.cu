@@ -80,13 +80,64 @@ int launch_build_K(acse_ctx* c) {
     return ACSE_OK;
 }
 
+// Tile pair u of the upper triangle (ti <= tj, row by row) of an n x n tile grid: row ti starts at
+// ti n - ti (ti - 1) / 2.  The float estimate is corrected by exact integer steps.
+__device__ __forceinline__ void tri_decode(int u, int n, int& ti, int& tj) {
+    const float b = 2.0f * (float)n + 1.0f;
+    int t = (int)(0.5f * (b - sqrtf(fmaxf(b * b - 8.0f * (float)u, 0.0f))));
+    t = max(0, min(n - 1, t));
+    while (t > 0 && t * n - t * (t - 1) / 2 > u) --t;
+    while (t + 1 < n && (t + 1) * n - (t + 1) * t / 2 <= u) ++t;
+    ti = t;
+    tj = t + (u - (t * n - t * (t - 1) / 2));
+}
+
 // ------------------------------------------------------------------------------ 1D and M
+// Largest |D| and |D - D^T| (pair transpose) of a block D over tile pair w of its 32 x 32 tiles, as bit patterns (those
+// of non-negative doubles order like the values; a NaN is the largest) into dmax[0], dmax[1].
+__device__ void d_asymmetry(int r, int w, const double* __restrict__ D, unsigned long long* dmax) {
+    __shared__ double Q[32][33];
+    const int R2 = r * r, nT = (R2 + 31) / 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
+    int ti, tj;
+    tri_decode(w, nT, ti, tj);
+    for (int y = ty; y < 32; y += 8) {
+        const int qr = tj * 32 + y, qc = ti * 32 + tx;
+        Q[y][tx] = qr < R2 && qc < R2 ? D[(size_t)qr * R2 + qc] : 0.0;
+    }
+    __syncthreads();
+    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; };
+    unsigned long long mx = 0, ma = 0;
+    for (int y = ty; y < 32; y += 8) {
+        const int pr = ti * 32 + y, pc = tj * 32 + tx;
+        if (pr >= R2 || pc >= R2) continue;
+        const double p = D[(size_t)pr * R2 + pc], q = Q[tx][y];
+        mx = max(mx, max(bits(p), bits(q)));
+        ma = max(ma, bits(p - q));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+    }
+    if (tx == 0) {
+        if (mx) atomicMax(dmax, mx);
+        if (ma) atomicMax(dmax + 1, ma);
+    }
+}
+
 // 1D^p_r = 2/(N-1) sum_q 2D^{pq}_{rq} over spin orbitals (App. C):
 //   g_a[p][r] = c sum_q (Daa[p][q][r][q] + Dab[p][q][r][q]);  g_b[p][r] = c sum_q (Dbb[p][q][r][q] + Dab[q][p][q][r]).
-// One warp per output element (lanes over q, fixed-order warp reduction).
+// One warp per output element (lanes over q, fixed-order warp reduction).  With dmax (FP64 and Ozaki contexts) the blocks
+// past those of 1D take the asymmetry of the three blocks of D, which k_build_M turns into `asym`.
 __global__ void __launch_bounds__(256) k_gamma(int r, double cN, const double* __restrict__ Daa,
                                                const double* __restrict__ Dab, const double* __restrict__ Dbb,
-                                               double* __restrict__ gam) {
+                                               double* __restrict__ gam, unsigned long long* __restrict__ dmax) {
+    const int ng = (2 * r * r + 7) / 8;
+    if ((int)blockIdx.x >= ng) {
+        const int nT = (r * r + 31) / 32, ntri = nT * (nT + 1) / 2, w = (int)blockIdx.x - ng, b = w / ntri;
+        d_asymmetry(r, w - b * ntri, b == 0 ? Daa : b == 1 ? Dab : Dbb, dmax);
+        return;
+    }
     const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (t >= 2 * r * r) return;
     const int sp = t / (r * r), p = (t / r) % r, rr = t % r;
@@ -106,8 +157,14 @@ __global__ void __launch_bounds__(256) k_gamma(int r, double cN, const double* _
 // the exchange piece vanishes in the ab block (1D is spin diagonal).
 __global__ void k_build_M(int r, const double* __restrict__ gam, const double* __restrict__ Daa,
                           const double* __restrict__ Dab, const double* __restrict__ Dbb, double* __restrict__ Maa,
-                          double* __restrict__ Mab, double* __restrict__ Mbb) {
+                          double* __restrict__ Mab, double* __restrict__ Mbb, unsigned long long* __restrict__ dmax,
+                          int* __restrict__ asym) {
     const size_t n = (size_t)r * r * r * r;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // D is pair-Hermitian to 2^-47 of its largest entry, or not (acse_ph.cu)
+        const double mx = __longlong_as_double((long long)dmax[0]), ma = __longlong_as_double((long long)dmax[1]);
+        *asym = ma <= mx * 0x1p-47 ? 0 : 1;   // NaN: not
+        dmax[0] = dmax[1] = 0;
+    }
     const double* ga = gam;
     const double* gb = gam + r * r;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
@@ -121,7 +178,8 @@ __global__ void k_build_M(int r, const double* __restrict__ gam, const double* _
 
 int launch_gamma(acse_ctx* c, const double* const D[3]) {
     const int r = c->r;
-    k_gamma<<<(2 * r * r + 7) / 8, 256, 0, c->stream>>>(r, 2.0 / (c->N - 1), D[0], D[1], D[2], c->w.gam);
+    const int nT = (r * r + 31) / 32, nasym = c->w.dmax ? 3 * (nT * (nT + 1) / 2) : 0;
+    k_gamma<<<(2 * r * r + 7) / 8 + nasym, 256, 0, c->stream>>>(r, 2.0 / (c->N - 1), D[0], D[1], D[2], c->w.gam, c->w.dmax);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -130,7 +188,8 @@ int launch_gamma_M(acse_ctx* c, const double* const D[3]) {
     const int r = c->r;
     ACSE_TRY(launch_gamma(c, D));
     const size_t n = (size_t)r * r * r * r;
-    k_build_M<<<grid_for(n), TPB, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], c->w.M[0], c->w.M[1], c->w.M[2]);
+    k_build_M<<<grid_for(n), TPB, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], c->w.M[0], c->w.M[1], c->w.M[2],
+                                                 c->w.dmax, c->w.asym);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -216,18 +275,6 @@ struct GArgs {
 
 #define G_GRID (152 * 16)
 #define G_ASM_GRID (152 * 8)   // k_assemble_G: eight resident blocks of 256 threads per SM, one wave
-
-// Tile pair u of the upper triangle (ti <= tj, row by row) of an n x n tile grid: row ti starts at
-// ti n - ti (ti - 1) / 2.  The float estimate is corrected by exact integer steps.
-__device__ __forceinline__ void tri_decode(int u, int n, int& ti, int& tj) {
-    const float b = 2.0f * (float)n + 1.0f;
-    int t = (int)(0.5f * (b - sqrtf(fmaxf(b * b - 8.0f * (float)u, 0.0f))));
-    t = max(0, min(n - 1, t));
-    while (t > 0 && t * n - t * (t - 1) / 2 > u) --t;
-    while (t + 1 < n && (t + 1) * n - (t + 1) * t / 2 <= u) ++t;
-    ti = t;
-    tj = t + (u - (t * n - t * (t - 1) / 2));
-}
 
 // Per-thread accumulator of the norm: FP64 on the FP64 path; on the FP32 path a double-float pair
 // (hi, lo) fed with exact products (v*v and its FMA residual) through Knuth's TwoSum, so that the

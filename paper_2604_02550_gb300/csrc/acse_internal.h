@@ -44,6 +44,7 @@ struct GemmF64 {
     double alpha, beta;
     const int* mapA;   // null, or the source row of every row of A and source column of every K index (the
     const int* mapB;   // pair numbering of a packed same-spin operand); the same for B
+    const int* gate;   // null, or the product is formed only where *gate (device memory) is not zero
 };
 
 // Split-precision operand problem for the tensor-core path.  A and B are 16-bit (BF16) or
@@ -102,16 +103,20 @@ struct Work {
     // 1-RDM per spin (r^2 each) and the M blocks (r^4 each)
     double* gam;          // [2][r][r]
     double* M[3];
-    // particle-hole operands on symmetrised pairs (acse_ph.cu): M+ (2S x 2S), M- (2P x 2P), flip (r^2 x r^2);
-    // W+ and W- (up to 2S x 2S and 2S x 2P), flip
+    // particle-hole operands on symmetrised pairs (acse_ph.cu): M+ (2r^2 x 2S: 2S rows even in (i,l), 2P odd), M-
+    // (2r^2 x 2P: 2P rows odd, 2S even), flips (r^2 x r^2); W+ and W- (up to 2S x 2S and 2S x 2P), flip
     double* Mp;
     double* Mm;
     double* Mf1;
+    double* Mf2;
+    unsigned long long* dmax;   // largest |D| and |D - D^T| of the D being prepared (bit patterns; zero between passes)
+    int* asym;                  // not zero: that D is not pair-Hermitian (k_build_M)
     double* Wp;
     double* Wm;
     double* Wf1;
-    double* V1;           // their products (in X5d, which the transformation by 1D overwrites last)
-    double* V2;
+    double* V1;           // their products, rows of 2r^2: V1, then V2 (ph_V2), in X5d, which the transformation by 1D
+                          // overwrites last
+    double* Vf2;          // product behind the second flip for a D that is not pair-Hermitian (in X5f1)
     double* V5d;          // V5 in full: 2r^2 x 2r^2, and the two flips
     double* V5f1;
     double* V5f2;
@@ -276,6 +281,10 @@ int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW);
 int launch_ph_w_diag(acse_ctx* c, const double* const W[3]);
 int launch_ph_xform(acse_ctx* c, const double* const in[3], double* const out[3], int trans);
 int launch_ph_finish(acse_ctx* c, int sW);
+// V2 of a pass: behind the r(r+1) rows (s = +1) or r(r-1) rows (s = -1) of V1.
+static inline double* ph_V2(const acse_ctx* c, int sW) {
+    return c->w.V1 + (size_t)c->r * (c->r + (sW > 0 ? 1 : -1)) * 2 * c->r * c->r;
+}
 int launch_pair_unpack(acse_ctx* c);
 int ph_set_attrs();
 int launch_Z_tiled(acse_ctx* c, const float* const W32[3]);
@@ -322,7 +331,7 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot);
 int acse_contract_pre(acse_ctx* c, const double* const D[3], const double* const W[3], int sW, int prep_D);
 int acse_contract_gemm(acse_ctx* c, int sW);
 int acse_contract_post(acse_ctx* c, int sW, double scale, int mask, double* const out[3], double* norm2_dst);
-#define ACSE_F64_GEMMS 9   // entries acse_gemm_list_f64 fills
+#define ACSE_F64_GEMMS 12   // entries acse_gemm_list_f64 fills
 int acse_gemm_list_f64(acse_ctx* c, int sW, GemmF64* g, int* n);
 int acse_contract(acse_ctx* c, const double* const D[3], const double* const W[3], int sW, double scale, int mask,
                   double* const out[3], double* norm2_dst, int prep_D);

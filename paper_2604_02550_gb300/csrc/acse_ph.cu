@@ -13,11 +13,18 @@
 // two products on pairs a <= b (S = r(r+1)/2 per spin) and a < b (P = r(r-1)/2): 4 r^6 flop in place of the
 // 16 r^6 of the full (2r^2)^3 product.  The spin-flip sectors are each other's image,
 // V5f2[(k,q)][(i,l)] = s V5f1[(q,k)][(l,i)], so one of them is multiplied: 2 r^6 in place of 4 r^6.
-// D (hence M) is taken as pair-Hermitian, which a 2-RDM is; entries are read at i <= l.
+//
+// W always has that symmetry, a 2-RDM D does, but the caller's D (sampled, truncated, one-sided) need not. M+ then
+// also has a part that is antisymmetric in (i,l), M- one that is symmetric, and the second flip is a product of its
+// own: V1, V2 get those columns too (2P and 2S of them) by three more products, 6 r^6, which every context holds and
+// runs where k_build_M found max |D - D^T| > 2^-47 max |D| in the D being prepared (`asym`, on the device: no
+// read-back, and a captured step decides anew on every replay).  That bound is 32 units in the last place of the
+// largest entry: a D that is Hermitian but for the rounding of an orbital transformation (1.2 2^-50 measured at r = 48)
+// stays below it, and what is dropped of its asymmetry is below the rounding of its own entries.
 //
 // Kernels here: the packing of both operands, the expansion of V1, V2, V5f1 into the full V5 (HBM-bound), the
-// diagonal sums behind w, and the transformation by 1D on the CUDA cores (an Ozaki context with r a
-// multiple of 16 runs it on the tensor cores, acse_zoz.cu).
+// diagonal sums behind w, and the transformation by 1D on the CUDA cores (an Ozaki context runs it on the tensor
+// cores where acse_zoz.cu applies).
 #include <type_traits>
 
 #include "acse_internal.h"
@@ -28,6 +35,9 @@
 // x = T^{kp}_{qt}, x' = T^{kt}_{qp}, spins K of (k,q) and P' of (p,t); the rows of `plus` run over k <= q and
 // those of `minus` over k < q (plusS = 1), or the other way round (plusS = 0).  flip[(k,q)][(p,t)] =
 // T_ab[k][p][t][q].  W takes f = 1/2; M takes f = 1, the 2 of the halved sum over (p,t) included.
+// An M that is not pair-Hermitian (asym, not zero): x and x' are averaged over the exchange of k and q, half their
+// differences go to 2P more rows of `plus` (k < q) and 2S more of `minus` (k <= q), and flip2[(k,q)][(p,t)] =
+// T_ab[t][q][k][p] is the second flip with both its pairs exchanged (for a Hermitian T equal to flip).
 //
 // Block (K, P', {k<=q}): the r x r slab of (p,t) goes through shared memory, both rows leave coalesced (the
 // b,a slab is read at stride r: its sectors are shared by the blocks of neighbouring q).  Block (k,p) of the
@@ -37,6 +47,8 @@ struct PhPack {
     double* plus;
     double* minus;
     double* flip;
+    double* flip2;     // M: the second flip ...
+    const int* asym;   // ... where *asym is not zero; null for W
     int r, plusS;
     double f;
 };
@@ -45,6 +57,7 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
     extern __shared__ double ph_sm[];   // [r][r + 1]
     const int r = a.r, ld = r + 1, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
     const size_t R2 = (size_t)r * r, r3 = R2 * r;
+    const bool gen = a.asym && *a.asym;
     if ((int)blockIdx.x < 4 * S) {
         const int kp = (int)blockIdx.x / S, u = (int)blockIdx.x - kp * S, K = kp >> 1, Q = kp & 1;
         int k, q;
@@ -63,9 +76,23 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
         for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
             const int p = e / r, t = e - p * r;
             if (t < p) continue;
-            const double x = ph_sm[p * ld + t], y = ph_sm[t * ld + p];
+            double x = ph_sm[p * ld + t], y = ph_sm[t * ld + p];
+            if (gen) {   // the slab of (q,k), read as it is stored
+                const bool tr = K == 1 && Q == 0;
+                const double x2 = tr ? src[p * r3 + q * R2 + (size_t)t * r + k] : src[q * r3 + p * R2 + (size_t)k * r + t];
+                const double y2 = tr ? src[t * r3 + q * R2 + (size_t)p * r + k] : src[q * r3 + t * R2 + (size_t)k * r + p];
+                const double dx = 0.5 * (x - x2), dy = 0.5 * (y - y2);
+                x = 0.5 * (x + x2);
+                y = 0.5 * (y + y2);
+                if (rowA >= 0) a.plus[((size_t)2 * S + rowA) * 2 * S + Q * S + ps_pair(r, p, t)] = p < t ? a.f * (dx + dy) : dx;
+                if (p < t) {
+                    a.minus[((size_t)2 * P + rowS) * 2 * P + Q * P + pk_pair(r, p, t)] = a.f * (x - y);
+                    if (rowA >= 0) om[pk_pair(r, p, t)] = a.f * (dx - dy);
+                }
+            } else if (rm >= 0 && p < t) {
+                om[pk_pair(r, p, t)] = a.f * (x - y);
+            }
             if (rp >= 0) op[ps_pair(r, p, t)] = p < t ? a.f * (x + y) : x;
-            if (rm >= 0 && p < t) om[pk_pair(r, p, t)] = a.f * (x - y);
         }
     } else {
         const int kp = (int)blockIdx.x - 4 * S, k = kp / r, p = kp - k * r;
@@ -75,18 +102,21 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
         for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
             const int q = e / r, t = e - q * r;
             a.flip[((size_t)k * r + q) * R2 + (size_t)p * r + t] = ph_sm[t * ld + q];
+            if (gen) a.flip2[((size_t)k * r + q) * R2 + (size_t)p * r + t] = a.src[1][t * r3 + q * R2 + (size_t)k * r + p];
         }
     }
 }
 
-static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, double* minus, double* flip, int plusS,
-                          double f) {
+static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, double* minus, double* flip, double* flip2,
+                          int plusS, double f) {
     const int r = c->r;
     PhPack a;
     for (int s = 0; s < 3; ++s) a.src[s] = T[s];
     a.plus = plus;
     a.minus = minus;
     a.flip = flip;
+    a.flip2 = flip2;
+    a.asym = flip2 ? c->w.asym : nullptr;
     a.r = r;
     a.plusS = plusS;
     a.f = f;
@@ -98,12 +128,12 @@ static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, d
 
 int launch_ph_pack_M(acse_ctx* c) {
     Work& w = c->w;
-    return launch_ph_pack(c, w.M, w.Mp, w.Mm, w.Mf1, 1, 1.0);
+    return launch_ph_pack(c, w.M, w.Mp, w.Mm, w.Mf1, w.Mf2, 1, 1.0);
 }
 
 int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW) {
     Work& w = c->w;
-    return launch_ph_pack(c, W, w.Wp, w.Wm, w.Wf1, sW > 0, 0.5);
+    return launch_ph_pack(c, W, w.Wp, w.Wm, w.Wf1, nullptr, sW > 0, 0.5);
 }
 
 // ------------------------------------------------------------------------------ expansion
@@ -111,10 +141,14 @@ int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW) {
 // k < q, is V1 + sg(i,l) V2 (sg = 1 for i < l, -1 for i > l, 0 for i = l), and row (q,k) s times V1 - sg V2
 // ... (s = +1: V1 is even and V2 odd in the exchange of k and q, s = -1: the other way round).  The diagonal
 // rows k = q have the even part alone.  V5f2[(k,q)][(i,l)] = s V5f1[(q,k)][(l,i)].
+// Rows of V1: the 2S pairs i <= l, and with asym the 2P pairs i < l of its part antisymmetric in (i,l); of V2: the 2P
+// pairs i < l, and with asym the 2S pairs i <= l of its symmetric part.
 struct PhUnpack {
     const double* V1;
     const double* V2;
     const double* f1;
+    const double* g2;   // with asym: the product behind the second flip, in the place of f1
+    const int* asym;
     double* V;
     double* f2;
     int r, s;
@@ -124,6 +158,7 @@ __global__ void __launch_bounds__(256) k_ph_unpack(const __grid_constant__ PhUnp
     extern __shared__ double ph_sm[];   // 2S + 2P = 2 r^2 doubles
     const int r = a.r, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
     const size_t R2 = (size_t)r * r;
+    const bool gen = *a.asym;
     if ((int)blockIdx.x < 2 * S) {
         const int K = (int)blockIdx.x / S, u = (int)blockIdx.x - K * S;
         int k, q;
@@ -132,23 +167,29 @@ __global__ void __launch_bounds__(256) k_ph_unpack(const __grid_constant__ PhUnp
         const int r1 = a.s > 0 ? rowS : rowA, r2 = a.s > 0 ? rowA : rowS;
         double* v1 = ph_sm;
         double* v2 = ph_sm + 2 * S;
-        for (int e = threadIdx.x; e < 2 * S; e += blockDim.x) v1[e] = r1 >= 0 ? a.V1[(size_t)r1 * 2 * S + e] : 0.0;
-        for (int e = threadIdx.x; e < 2 * P; e += blockDim.x) v2[e] = r2 >= 0 ? a.V2[(size_t)r2 * 2 * P + e] : 0.0;
+        const double* p1 = a.V1 + (size_t)max(r1, 0) * 2 * R2;
+        const double* p2 = a.V2 + (size_t)max(r2, 0) * 2 * R2;
+        for (int e = threadIdx.x; e < 2 * S; e += blockDim.x) v1[e] = r1 >= 0 ? p1[e] : 0.0;
+        for (int e = threadIdx.x; e < 2 * P; e += blockDim.x) v2[e] = r2 >= 0 ? p2[e] : 0.0;
         __syncthreads();
         double* o1 = a.V + ((size_t)K * R2 + (size_t)k * r + q) * 2 * R2;
         double* o2 = a.V + ((size_t)K * R2 + (size_t)q * r + k) * 2 * R2;
         for (int e = threadIdx.x; e < 2 * (int)R2; e += blockDim.x) {
             const int I = e >= (int)R2, c = e - I * (int)R2, i = c / r, l = c - i * r;
-            const double x = v1[I * S + (i <= l ? ps_pair(r, i, l) : ps_pair(r, l, i))];
-            double y = 0.0;
+            const int us = I * S + (i <= l ? ps_pair(r, i, l) : ps_pair(r, l, i));
+            double x = v1[us], y = 0.0;
             if (i < l) y = v2[I * P + pk_pair(r, i, l)];
             else if (i > l) y = -v2[I * P + pk_pair(r, l, i)];
+            if (gen) {
+                if (r1 >= 0 && i != l) x += i < l ? p1[2 * S + I * P + pk_pair(r, i, l)] : -p1[2 * S + I * P + pk_pair(r, l, i)];
+                if (r2 >= 0) y += p2[2 * P + us];
+            }
             o1[e] = x + y;
             if (k < q) o2[e] = a.s > 0 ? x - y : y - x;
         }
     } else {
         const int kq = (int)blockIdx.x - 2 * S, k = kq / r, q = kq - k * r;
-        const double* src = a.f1 + ((size_t)q * r + k) * R2;
+        const double* src = (gen ? a.g2 : a.f1) + ((size_t)q * r + k) * R2;
         for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) ph_sm[e] = src[e];
         __syncthreads();
         const double s = (double)a.s;
@@ -164,8 +205,10 @@ static int launch_ph_unpack(acse_ctx* c, int sW) {
     Work& w = c->w;
     PhUnpack a;
     a.V1 = w.V1;
-    a.V2 = w.V2;
+    a.V2 = ph_V2(c, sW);
     a.f1 = w.V5f1;
+    a.g2 = w.Vf2;
+    a.asym = w.asym;
     a.V = w.V5d;
     a.f2 = w.V5f2;
     a.r = r;

@@ -9,7 +9,7 @@
 // GF_TILES_PER_SM of them, else 16 x 16 (one output a thread).
 #include "acse_internal.h"
 
-#define GEMM_F64_MAXP 40
+#define GEMM_F64_MAXP 54
 #define GF_TPB 256
 // 32 x 32 tiles from this many per SM on: the last wave then idles at most a sixteenth of the launch, while
 // at r = 20 (6.5 a SM) 16 x 16 tiles finish earlier.
@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(GF_TPB) k_gemm_f64(const __grid_constant__ Gem
     int pi = 0;
     while (pi + 1 < b.nprob && b.prefix[pi + 1] <= t) ++pi;
     const GemmF64& P = b.p[pi];
+    if (P.gate && !*P.gate) return;
     const int local = t - b.prefix[pi];
     const int m0 = (local / b.tiles_n[pi]) * BT;
     const int n0 = (local % b.tiles_n[pi]) * BT;
@@ -114,7 +115,8 @@ int gemm_f64_grouped(acse_ctx* c, const GemmF64* probs, int nprob, cudaStream_t 
         int np = nprob - done;
         if (np > GEMM_F64_MAXP) np = GEMM_F64_MAXP;
         long t32 = 0;
-        for (int i = 0; i < np; ++i) t32 += (long)((probs[done + i].M + 31) / 32) * ((probs[done + i].N + 31) / 32);
+        for (int i = 0; i < np; ++i)   // (gated products are rare)
+            if (!probs[done + i].gate) t32 += (long)((probs[done + i].M + 31) / 32) * ((probs[done + i].N + 31) / 32);
         const int bt = t32 >= (long)GF_TILES_PER_SM * 152 ? 32 : 16;
         int tiles = 0;
         int used = 0;

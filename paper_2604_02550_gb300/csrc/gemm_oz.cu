@@ -38,7 +38,7 @@
 #define OZ_CHUNK_KB 64       // 64-element K blocks of one exactly accumulated chunk: 64 * 64 * 64^2 = 2^24
 #define OZ_MAXCH 2           // chunks of one residue product (K <= 2 * 64 * 64 = 8192)
 #define OZ_MAXP 12           // GEMMs of one launch
-#define OZ_MAXJ 16           // operands of one slicing launch
+#define OZ_MAXJ 18           // operands of one slicing launch
 #define OZ_THREADS 192
 #define OZ_BN 256
 #define OZ_STAGES 4
@@ -88,6 +88,7 @@ struct __align__(128) OzBatch {
     int nprob;
     int total_tiles;
     int* err;
+    const int* gate;      // null, or the launch is skipped where *gate is zero
     unsigned long long wait_ns;
     int inject_stall;
     const int* order;     // tiles of CTA c: order[cta_start[c] .. cta_start[c+1]) (longest first)
@@ -123,6 +124,7 @@ struct OzSliceJob {
     __nv_bfloat16* dst;     // first output row of the job
     size_t ldd;             // T * Kp
     double* scale;          // 2^e per output row (NaN for a row with a non-finite entry)
+    const int* gate;        // null, or the job is skipped where *gate is zero
     int rows, K, Kp, nb, mul_y, row0;
 };
 
@@ -142,6 +144,7 @@ __global__ void __launch_bounds__(256) k_oz_rowscale(const __grid_constant__ OzS
     int ji = 0;
     while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
     const OzSliceJob& J = b.j[ji];
+    if (J.gate && !*J.gate) return;
     const int row = grow - J.row0;
     const int srow = J.rowmap ? J.rowmap[row] : row;
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(J.src + (size_t)srow * J.lds);
@@ -182,6 +185,7 @@ __global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSl
     int ji = 0;
     while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
     const OzSliceJob& J = b.j[ji];
+    if (J.gate && !*J.gate) return;
     const int K = J.K;
     const int qi = (int)blockIdx.x * 256 + (int)threadIdx.x;
     if (qi >= (K + 3) >> 2) return;
@@ -227,6 +231,7 @@ __global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSl
 template <int BN, int STAGES, bool PAIR>
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __restrict__ bp) {
     const OzBatch& b = *bp;
+    if (b.gate && !*b.gate) return;   // the whole grid, before any barrier or tensor memory
     constexpr int A_BYTES = TC_BM * 128;
     constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * 128;
     constexpr int BM = PAIR ? 2 * TC_BM : TC_BM;   // rows of an output tile
@@ -567,6 +572,7 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
 template <bool TWO>
 __global__ void __launch_bounds__(256, TWO ? 2 : 3) k_oz_crt(const OzBatch* __restrict__ bp,
                                                              const __grid_constant__ OzCrtParams cp) {
+    if (bp->gate && !*bp->gate) return;
     const OzProb& P = bp->p[blockIdx.y];
     if (!TWO || P.nch == 1) oz_crt_rows<1>(P, cp);
     else oz_crt_rows<2>(P, cp);
@@ -609,7 +615,9 @@ static int oz_launch_crt(const OzBatch* host, const OzBatch* dev, int nsm, cudaS
 //      [M_aa; D_aa], [M_bb; D_bb] packed (2P x P);
 //   B: M+ (S2 x S2), M- (P2 x P2), Mf1, W_ab (r^2 x r^2), W_aa, W_bb packed (P x P).
 // The problem table of s = +1 is the plan itself; that of s = -1 (`alt`) has the same operands with the
-// other row counts and borrows every buffer.
+// other row counts and borrows every buffer.  `gen`: the three products of a D that is not pair-Hermitian, with the same
+// A and B operands of their own (the 2P odd rows of M+, the 2S even ones of M-, the second flip of M), skipped on the
+// device (Work::asym) for the others.
 struct OzOp {
     __nv_bfloat16* sl;
     double* scale;
@@ -633,7 +641,9 @@ struct OzPlan {
     int* sched;         // tile lists of the persistent kernel (OzBatch::order, cta_start)
     int* err;
     struct OzPlan* alt;       // the pass's table for s = -1
+    struct OzPlan* gen;       // the products of a D that is not pair-Hermitian
     int borrowed;             // operands and staging belong to another plan
+    int borrowedA;            // the A operands do
     struct OzPlan* lists[2];  // GEMM lists of the adjoint (oz_gemm_list): a plan per list slot
     int shareB[OZ_MAXP];      // lists: problem i reads the B operand of problem shareB[i] - 1 (0: its own)
 };
@@ -840,21 +850,50 @@ extern "C" int acse_ozaki_plan_info(int oz_slices, int kmax, int k, int* moduli_
 }
 
 // The seven products of a pass in the order of acse_gemm_list_f64 (the same-spin X and Y as one problem).
-static int oz_pass_table(acse_ctx* c, OzPlan* pl, const OzPlan* root) {
+static int oz_pass_table(acse_ctx* c, OzPlan* pl, const OzPlan* root, int sW) {
     Work& w = c->w;
     const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
     const bool own = pl == root;
     auto add = [&](int i, const OzOp& A, const OzOp& B, double* C, int ldc, double alpha, int stage_rows) {
         return oz_add(pl, A, B, C, ldc, alpha, stage_rows, own ? nullptr : root->host->p[i].stage);
     };
-    ACSE_TRY(add(0, pl->A[0], pl->B[0], w.V1, S2, 1.0, S2));
+    ACSE_TRY(add(0, pl->A[0], pl->B[0], w.V1, 2 * R2, 1.0, S2));
     ACSE_TRY(add(1, pl->A[2], pl->B[2], w.V5f1, R2, 1.0, R2));
     ACSE_TRY(add(2, pl->A[3], pl->B[3], w.X[1], R2, 2.0, R2));
     ACSE_TRY(add(3, pl->A[4], pl->B[3], w.Y[1], R2, 2.0, R2));
-    ACSE_TRY(add(4, pl->A[1], pl->B[1], w.V2, P2, 1.0, S2));
+    ACSE_TRY(add(4, pl->A[1], pl->B[1], ph_V2(c, sW), 2 * R2, 1.0, S2));
     ACSE_TRY(add(5, pl->A[5], pl->B[4], w.Cp[0], P, 2.0, 2 * P));
     ACSE_TRY(add(6, pl->A[6], pl->B[5], w.Cp[1], P, 2.0, 2 * P));
     return oz_plan_finish(pl);
+}
+
+// The gated products of table pl (the plan of s = +1, root, or alt): operands of their own in root's.
+static int oz_gen_table(acse_ctx* c, OzPlan* pl, const OzPlan* root, int sW) {
+    Work& w = c->w;
+    const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1);
+    OzPlan* g = (OzPlan*)calloc(1, sizeof(OzPlan));
+    if (!g) return ACSE_ERR_NOMEM;
+    pl->gen = g;
+    g->borrowed = pl != root;
+    g->borrowedA = 1;
+    ACSE_TRY(oz_plan_init(g, pl->S, pl->bn, pl->pair, S2));
+    g->host->err = root->err;
+    g->host->gate = w.asym;
+    memcpy(g->A, pl->A, 3 * sizeof(OzOp));
+    if (g->borrowed) {
+        memcpy(g->B, root->gen->B, 3 * sizeof(OzOp));
+    } else {
+        ACSE_TRY(oz_op_alloc(g, g->B[0], P2, S2));
+        ACSE_TRY(oz_op_alloc(g, g->B[1], S2, P2));
+        ACSE_TRY(oz_op_alloc(g, g->B[2], R2, R2));
+    }
+    auto add = [&](int i, double* C, int ldc, int stage_rows) {
+        return oz_add(g, g->A[i], g->B[i], C, ldc, 1.0, stage_rows, g->borrowed ? root->gen->host->p[i].stage : nullptr);
+    };
+    ACSE_TRY(add(0, w.V1 + S2, 2 * R2, S2));
+    ACSE_TRY(add(1, ph_V2(c, sW) + P2, 2 * R2, S2));
+    ACSE_TRY(add(2, w.Vf2, R2, R2));
+    return oz_plan_finish(g);
 }
 
 int oz_plan_create(acse_ctx* c) {
@@ -880,7 +919,8 @@ int oz_plan_create(acse_ctx* c) {
     if (!c->w.tc_err) c->w.tc_err = pl->err;   // read by acse_sync_status
     pl->host->err = pl->err;
     pl->A[1].rows = P2;   // s = +1: W+ over S2 rows, W- over P2
-    ACSE_TRY(oz_pass_table(c, pl, pl));
+    ACSE_TRY(oz_pass_table(c, pl, pl, +1));
+    ACSE_TRY(oz_gen_table(c, pl, pl, +1));
     OzPlan* alt = (OzPlan*)calloc(1, sizeof(OzPlan));
     if (!alt) return ACSE_ERR_NOMEM;
     pl->alt = alt;
@@ -891,7 +931,8 @@ int oz_plan_create(acse_ctx* c) {
     memcpy(alt->B, pl->B, sizeof(pl->B));
     alt->A[0].rows = P2;   // s = -1: the other way round
     alt->A[1].rows = S2;
-    return oz_pass_table(c, alt, pl);
+    ACSE_TRY(oz_pass_table(c, alt, pl, -1));
+    return oz_gen_table(c, alt, pl, -1);
 }
 
 // Longest-processing-time tile lists of the persistent kernel (tile cost: its K blocks over all groups)
@@ -937,10 +978,11 @@ static int oz_plan_finish(OzPlan* pl) {
 static void oz_plan_free(OzPlan* pl) {
     if (!pl) return;
     oz_plan_free(pl->alt);
+    oz_plan_free(pl->gen);
     for (int s = 0; s < 2; ++s) oz_plan_free(pl->lists[s]);
     for (int i = 0; i < OZ_MAXP && !pl->borrowed; ++i) {
-        if (pl->A[i].sl) cudaFree(pl->A[i].sl);
-        if (pl->A[i].scale) cudaFree(pl->A[i].scale);
+        if (pl->A[i].sl && !pl->borrowedA) cudaFree(pl->A[i].sl);
+        if (pl->A[i].scale && !pl->borrowedA) cudaFree(pl->A[i].scale);
         if (pl->shareB[i]) continue;   // an earlier problem's operand
         if (pl->B[i].sl) cudaFree(pl->B[i].sl);
         if (pl->B[i].scale) cudaFree(pl->B[i].scale);
@@ -980,8 +1022,9 @@ static void oz_slice_batch_init(OzSliceBatch& b, const OzMods& m) {
 // One slicing job: `rows` rows of operand o starting at output row `orow`, read from src (row stride
 // lds) through the optional row / column maps; mul_y for a B operand (residues times y_t).
 static void oz_job(OzSliceBatch& b, int& rows, const OzOp& o, int orow, int nrows, const double* src, size_t lds,
-                   const int* rowmap, const int* colmap, int mul_y) {
+                   const int* rowmap, const int* colmap, int mul_y, const int* gate = nullptr) {
     OzSliceJob& j = b.j[b.njobs++];
+    j.gate = gate;
     j.src = src;
     j.lds = lds;
     j.rowmap = rowmap;
@@ -1033,6 +1076,10 @@ int oz_slice_operands(acse_ctx* c, int prep_D, int sW) {
         oz_job(b, rows, pl->B[0], 0, S2, w.Mp, S2, nullptr, nullptr, 1);
         oz_job(b, rows, pl->B[1], 0, P2, w.Mm, P2, nullptr, nullptr, 1);
         oz_job(b, rows, pl->B[2], 0, R2, w.Mf1, R2, nullptr, nullptr, 1);
+        const OzOp* gB = root->gen->B;
+        oz_job(b, rows, gB[0], 0, P2, w.Mp + (size_t)S2 * S2, S2, nullptr, nullptr, 1, w.asym);
+        oz_job(b, rows, gB[1], 0, S2, w.Mm + (size_t)P2 * P2, P2, nullptr, nullptr, 1, w.asym);
+        oz_job(b, rows, gB[2], 0, R2, w.Mf2, R2, nullptr, nullptr, 1, w.asym);
     }
     oz_job(b, rows, pl->B[3], 0, R2, c->cur_W[1], R2, nullptr, nullptr, 1);
     oz_job(b, rows, pl->B[4], 0, P, c->cur_W[0], R2, pm, pm, 1);
@@ -1053,14 +1100,19 @@ int oz_gemm_launch(acse_ctx* c, int sW) {
     ACSE_LAUNCHED(c);
     ACSE_TRY(oz_launch_crt(pl->host, pl->dev, pl->nsm, c->stream));
     ACSE_LAUNCHED(c);
-    return prof_end(c);
+    ACSE_TRY(prof_end(c));
+    ACSE_TRY(oz_launch_gemm(pl->gen, c->stream));
+    ACSE_LAUNCHED(c);
+    ACSE_TRY(oz_launch_crt(pl->gen->host, pl->gen->dev, pl->gen->nsm, c->stream));
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
 }
 
 int oz_set_wait_ns(acse_ctx* c, unsigned long long ns, int inject_stall) {
     OzPlan* pl = (OzPlan*)c->oz_plan;
     if (!pl) return ACSE_ERR_UNSUPPORTED;
     ACSE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    for (OzPlan* q : {pl, pl->alt}) {
+    for (OzPlan* q : {pl, pl->alt, pl->gen, pl->alt->gen}) {
         q->host->wait_ns = ns ? ns : OZ_WAIT_NS;
         q->host->inject_stall = inject_stall;
         ACSE_CUDA_TRY(cudaMemcpy(q->dev, q->host, sizeof(OzBatch), cudaMemcpyHostToDevice));
