@@ -164,7 +164,8 @@ __global__ void k_adj_tau(int r, const double* __restrict__ Haa, const double* _
 // operand blocks in shared memory, nt^2 threads (nt = ceil(r / 4)) own a 4 x 4 tile of C each, and where those do
 // not fill the block, groups of them take every G-th x; the groups meet in shared memory and the block
 // writes one partial C, summed in a fixed order by k_adj_small.  (One block per output element, as before, read
-// every operand r times from L2: 2.4 ms for the 14 jobs at r = 32, FP64.)
+// every operand r times from L2: 2.4 ms for the 14 jobs at r = 32.)  FP64 in every context: in double-float pairs (48
+// bits, the range of FP32) the gradients of an Ozaki context lost bits, and more of them the smaller the cotangent.
 //   job 0-3   gbar from x1:  Xaa[ij][x][u] t0[ij][x][v],  Xbb t1,  Xab[ij][x][u] t2[ij][x][v],  Xab[ij][u][x] t3[ij][x][v]
 //   job 4-7   wbar from x2:  t0[ij][u][x] Maa[ij][x][v],  t1 Mbb,  t2[ij][u][x] Mab[ij][v][x],  t3[ij][u][x] Mab[ij][x][v]
 //   job 8-13  gbar from X5 = 1D V5: X5b_t[(k,u)][(i,x)] V5_t[(k,v)][(i,x)], n = (k, i), sectors t = 0-3 and the flips
@@ -179,22 +180,21 @@ struct AdjRed {
     int r, nb, groups;
 };
 
-template <typename C>
 __global__ void __launch_bounds__(256) k_adj_reduce(const __grid_constant__ AdjRed a) {
     extern __shared__ __align__(16) unsigned char ad_raw[];
     const int r = a.r, rp = (r + 3) & ~3, R2 = r * r, nt = rp / 4, nt2 = nt * nt;
     const int job = (int)blockIdx.x / a.nb, chunk = (int)blockIdx.x - job * a.nb;
-    C* As = (C*)ad_raw;          // [x][u]
-    C* Bs = As + (size_t)r * rp; // [x][v]
+    double* As = (double*)ad_raw;     // [x][u]
+    double* Bs = As + (size_t)r * rp; // [x][v]
     const int g = threadIdx.x / nt2, tile = threadIdx.x - g * nt2;
     const bool active = g < a.groups;
     const int u0 = (tile / nt) * 4, v0 = (tile % nt) * 4;
-    C acc[4][4];
+    double acc[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = tconv<C>(0.0);
-    for (int e = threadIdx.x; e < r * rp; e += blockDim.x) As[e] = Bs[e] = tconv<C>(0.0);
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+    for (int e = threadIdx.x; e < r * rp; e += blockDim.x) As[e] = Bs[e] = 0.0;
     const int per = (R2 + a.nb - 1) / a.nb, n1 = min(R2, (chunk + 1) * per);
     for (int n = chunk * per; n < n1; ++n) {
         const size_t off = (size_t)(n / r) * a.sn_hi[job] + (size_t)(n % r) * a.sn_lo[job];
@@ -204,20 +204,20 @@ __global__ void __launch_bounds__(256) k_adj_reduce(const __grid_constant__ AdjR
         for (int e = threadIdx.x; e < R2; e += blockDim.x) {   // consecutive threads along the unit stride
             const int hi = e / r, lo = e - hi * r;
             const int ax = a.asx[job] == 1 ? lo : hi, au = a.asx[job] == 1 ? hi : lo;
-            As[ax * rp + au] = tconv<C>(A[(size_t)ax * a.asx[job] + (size_t)au * a.asu[job]]);
+            As[ax * rp + au] = A[(size_t)ax * a.asx[job] + (size_t)au * a.asu[job]];
             const int bx = a.bsx[job] == 1 ? lo : hi, bv = a.bsx[job] == 1 ? hi : lo;
-            Bs[bx * rp + bv] = tconv<C>(B[(size_t)bx * a.bsx[job] + (size_t)bv * a.bsv[job]]);
+            Bs[bx * rp + bv] = B[(size_t)bx * a.bsx[job] + (size_t)bv * a.bsv[job]];
         }
         __syncthreads();
         if (active)
             for (int x = g; x < r; x += a.groups) {
-                C p[4], q[4];
+                double p[4], q[4];
                 ld4(As + x * rp + u0, p);
                 ld4(Bs + x * rp + v0, q);
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) tmac(acc[u][v], p[u], q[v]);
+                    for (int v = 0; v < 4; ++v) acc[u][v] = fma(p[u], q[v], acc[u][v]);
             }
     }
     __syncthreads();
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) k_adj_reduce(const __grid_constant__ AdjR
                 for (int v = 0; v < 4; ++v)
                     if (u0 + u < r) {
                         double* d = sh + (size_t)(u0 + u) * rp + v0 + v;
-                        *d = (h ? *d : 0.0) + (double)acc[u][v];
+                        *d = (h ? *d : 0.0) + acc[u][v];
                     }
         __syncthreads();
     }
@@ -824,8 +824,7 @@ static int vjp_D(acse_ctx* c, const double* const W[3], int sW, double scale, co
             const double* B = t < 4 ? w.V5d + o : t == 4 ? w.V5f1 : w.V5f2;
             set(8 + t, A, true, B, true, ld, ld, (size_t)r * ld, r);
         }
-        if (c->oz) k_adj_reduce<dfl><<<AD_JOBS * a->nb, a->threads, sm2, c->stream>>>(d);
-        else k_adj_reduce<double><<<AD_JOBS * a->nb, a->threads, sm2, c->stream>>>(d);
+        k_adj_reduce<<<AD_JOBS * a->nb, a->threads, sm2, c->stream>>>(d);
         AL(c);
     }
     k_adj_small<<<6 * R2, 128, 0, c->stream>>>(ab);
@@ -915,8 +914,7 @@ static int adj_set_attrs() {
     ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_pack_V, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double)));
     const int sm2 = 2 * ACSE_MAX_R * ACSE_MAX_R * (int)sizeof(double);
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_reduce<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
-    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_reduce<dfl>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
+    ACSE_CUDA_TRY(cudaFuncSetAttribute(k_adj_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
     return ACSE_OK;
 }
 

@@ -270,7 +270,7 @@ int launch_pair_unpack(acse_ctx* c) {
 // -------------------------------------------------------- products of the pairs (CUDA cores)
 // Eight classes of r x r x r products per pair ij, out_c[ij][a][b] = sum_x T_c(a, x) G_c[b][x] (bit c of tt, gt: T, G
 // read transposed; bit c of tri: the pairs i < j only).  FP64 contexts, and Ozaki contexts where the digit kernel
-// does not apply (C: double, or the double-float pair).  Block: one class, nij pairs, both operands in shared
+// does not apply (C: double, or the double-float pair where acse_use_dfl).  Block: one class, nij pairs, both operands in shared
 // memory as [x][.]; the MT x MT tiles of all pairs are dealt out to full warps -- a DFMA holds the FP64 pipe 16
 // cycles however many lanes are active, and at r = 24 one 4 x 4 tile a thread left 28 of 64 lanes idle -- with
 // nij chosen on the host so that the last round of tiles is nearly full.  r = 24, FP64: 123 us for the six pair-types'
@@ -362,7 +362,8 @@ int launch_pair_rows(acse_ctx* c, const double* const T[8], unsigned tt, const d
                      double* const out[8]) {
     const int st = launch_rows_oz(c, T, tt, G, gt, tri, out);
     if (st != ACSE_ERR_UNSUPPORTED) return st;
-    const int r = c->r, mt = c->oz ? 4 : 2, rp = (r + mt - 1) / mt * mt;
+    const bool df = acse_use_dfl(c);
+    const int r = c->r, mt = df ? 4 : 2, rp = (r + mt - 1) / mt * mt;
     PairRows a;
     for (int k = 0; k < 8; ++k) {
         a.T[k] = T[k];
@@ -381,7 +382,7 @@ int launch_pair_rows(acse_ctx* c, const double* const T[8], unsigned tt, const d
         a.start[k + 1] = a.start[k] + (items + a.nij - 1) / a.nij;
     }
     const size_t sm = (size_t)(1 + a.nij) * r * rp * sizeof(double);
-    if (c->oz) k_pair_rows<dfl, 4><<<a.start[8], 256, sm, c->stream>>>(a);
+    if (df) k_pair_rows<dfl, 4><<<a.start[8], 256, sm, c->stream>>>(a);
     else k_pair_rows<double, 2><<<a.start[8], 256, sm, c->stream>>>(a);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
@@ -432,7 +433,7 @@ int launch_ph_w_diag(acse_ctx* c, const double* const W[3]) {
 // out[(K,k,j)][(I,i,l)] = sum_q g_K[j][q] in[(K,k,q)][(I,i,l)] (trans: g_K[q][j]) for the six sectors t:
 // 0-3 the spin blocks (K, I) of the 2r^2 x 2r^2 array, 4 and 5 the two flips (1D of beta, of alpha).
 // Block (t, k, 64 columns): the columns' r rows and 1D sit in shared memory, each thread owns a 4 x 4 tile.
-// C: double on the FP64 path (bound by the DFMA pipe, 6 r^5), the double-float pair on the Ozaki path.
+// C: double (bound by the DFMA pipe, 6 r^5), or the double-float pair where acse_use_dfl.
 #define PHT_COLS 64
 
 struct PhXform {
@@ -507,7 +508,7 @@ int launch_ph_xform(acse_ctx* c, const double* const in[3], double* const out[3]
     a.r = r;
     a.trans = trans;
     const int threads = (((r + 3) / 4) * (PHT_COLS / 4) + 31) / 32 * 32;
-    if (c->oz) k_ph_xform<dfl><<<6 * r * nch, threads, ph_xform_smem(r), c->stream>>>(a);
+    if (acse_use_dfl(c)) k_ph_xform<dfl><<<6 * r * nch, threads, ph_xform_smem(r), c->stream>>>(a);
     else k_ph_xform<double><<<6 * r * nch, threads, ph_xform_smem(r), c->stream>>>(a);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
