@@ -130,7 +130,6 @@ static int alloc_work(acse_ctx* c) {
         const size_t S2 = (size_t)c->r * (c->r + 1), P2 = (size_t)c->r * (c->r - 1);   // pairs a <= b, a < b, two spins
         A_(w.Mp, 2 * R2 * S2 * sizeof(double)); A_(w.Mm, 2 * R2 * P2 * sizeof(double)); A_(w.Mf1, b4); A_(w.Mf2, b4);
         A_(w.dmax, 2 * sizeof(unsigned long long)); A_(w.asym, sizeof(int));
-        ACSE_CUDA_TRY(cudaMemsetAsync(w.dmax, 0, 2 * sizeof(unsigned long long), c->stream));
         A_(w.Wp, S2 * S2 * sizeof(double)); A_(w.Wm, S2 * P2 * sizeof(double)); A_(w.Wf1, b4);
         A_(w.V5d, 4 * b4); A_(w.V5f1, b4); A_(w.V5f2, b4);
         A_(w.X5d, 4 * b4); A_(w.X5f1, b4); A_(w.X5f2, b4);

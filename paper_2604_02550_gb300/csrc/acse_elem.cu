@@ -93,51 +93,14 @@ __device__ __forceinline__ void tri_decode(int u, int n, int& ti, int& tj) {
 }
 
 // ------------------------------------------------------------------------------ 1D and M
-// Largest |D| and |D - D^T| (pair transpose) of a block D over tile pair w of its 32 x 32 tiles, as bit patterns (those
-// of non-negative doubles order like the values; a NaN is the largest) into dmax[0], dmax[1].
-__device__ void d_asymmetry(int r, int w, const double* __restrict__ D, unsigned long long* dmax) {
-    __shared__ double Q[32][33];
-    const int R2 = r * r, nT = (R2 + 31) / 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
-    int ti, tj;
-    tri_decode(w, nT, ti, tj);
-    for (int y = ty; y < 32; y += 8) {
-        const int qr = tj * 32 + y, qc = ti * 32 + tx;
-        Q[y][tx] = qr < R2 && qc < R2 ? D[(size_t)qr * R2 + qc] : 0.0;
-    }
-    __syncthreads();
-    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; };
-    unsigned long long mx = 0, ma = 0;
-    for (int y = ty; y < 32; y += 8) {
-        const int pr = ti * 32 + y, pc = tj * 32 + tx;
-        if (pr >= R2 || pc >= R2) continue;
-        const double p = D[(size_t)pr * R2 + pc], q = Q[tx][y];
-        mx = max(mx, max(bits(p), bits(q)));
-        ma = max(ma, bits(p - q));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-    }
-    if (tx == 0) {
-        if (mx) atomicMax(dmax, mx);
-        if (ma) atomicMax(dmax + 1, ma);
-    }
-}
-
 // 1D^p_r = 2/(N-1) sum_q 2D^{pq}_{rq} over spin orbitals (App. C):
 //   g_a[p][r] = c sum_q (Daa[p][q][r][q] + Dab[p][q][r][q]);  g_b[p][r] = c sum_q (Dbb[p][q][r][q] + Dab[q][p][q][r]).
-// One warp per output element (lanes over q, fixed-order warp reduction).  With dmax (FP64 and Ozaki contexts) the blocks
-// past those of 1D take the asymmetry of the three blocks of D, which k_build_M turns into `asym`.
+// One warp per output element (lanes over q, fixed-order warp reduction).  dmax (FP64 and Ozaki contexts) is cleared
+// for k_build_M.
 __global__ void __launch_bounds__(256) k_gamma(int r, double cN, const double* __restrict__ Daa,
                                                const double* __restrict__ Dab, const double* __restrict__ Dbb,
                                                double* __restrict__ gam, unsigned long long* __restrict__ dmax) {
-    const int ng = (2 * r * r + 7) / 8;
-    if ((int)blockIdx.x >= ng) {
-        const int nT = (r * r + 31) / 32, ntri = nT * (nT + 1) / 2, w = (int)blockIdx.x - ng, b = w / ntri;
-        d_asymmetry(r, w - b * ntri, b == 0 ? Daa : b == 1 ? Dab : Dbb, dmax);
-        return;
-    }
+    if (dmax && blockIdx.x == 0 && threadIdx.x < 2) dmax[threadIdx.x] = 0;
     const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (t >= 2 * r * r) return;
     const int sp = t / (r * r), p = (t / r) % r, rr = t % r;
@@ -153,21 +116,73 @@ __global__ void __launch_bounds__(256) k_gamma(int r, double cN, const double* _
     if (lane == 0) gam[t] = cN * s;
 }
 
-// M = 3 2Delta + 1D^1D = 3 2D - 2 (1D^1D), (1D^1D)^{ij}_{kl} = 1/2(g^i_k g^j_l - g^j_k g^i_l) (App. C);
-// the exchange piece vanishes in the ab block (1D is spin diagonal).
-__global__ void k_build_M(int r, const double* __restrict__ gam, const double* __restrict__ Daa,
-                          const double* __restrict__ Dab, const double* __restrict__ Dbb, double* __restrict__ Maa,
-                          double* __restrict__ Mab, double* __restrict__ Mbb, unsigned long long* __restrict__ dmax,
-                          int* __restrict__ asym) {
-    const size_t n = (size_t)r * r * r * r;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {   // D is pair-Hermitian to 2^-47 of its largest entry, or not (acse_ph.cu)
-        const double mx = __longlong_as_double((long long)dmax[0]), ma = __longlong_as_double((long long)dmax[1]);
-        *asym = ma <= mx * 0x1p-47 ? 0 : 1;   // NaN: not
-        dmax[0] = dmax[1] = 0;
+// Largest |D| and |D - D^T| (pair transpose) of the three blocks over the pairs of 32 x 32 tiles w, w + stride, .., as
+// bit patterns (those of non-negative doubles order like the values; a NaN is the largest) into dmax[0], dmax[1], which
+// k_gamma has cleared and k_ph_pack_asym reads.  One atomic a block at most: with one a warp of every tile pair it
+// took 90 us at r = 48 (127 MB).
+__device__ void d_asymmetry(int r, int w, int stride, const double* __restrict__ Daa, const double* __restrict__ Dab,
+                            const double* __restrict__ Dbb, unsigned long long* dmax) {
+    __shared__ double Q[32][33];
+    __shared__ unsigned long long sh[2][8];
+    const int R2 = r * r, nT = (R2 + 31) / 32, ntri = nT * (nT + 1) / 2;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
+    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull; };
+    unsigned long long mx = 0, ma = 0;
+    for (; w < 3 * ntri; w += stride) {
+        const int b = w / ntri;
+        const double* D = b == 0 ? Daa : b == 1 ? Dab : Dbb;
+        int ti, tj;
+        tri_decode(w - b * ntri, nT, ti, tj);
+        double p[4], q[4];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            const int pr = ti * 32 + ty + 8 * y, pc = tj * 32 + tx, qr = tj * 32 + ty + 8 * y, qc = ti * 32 + tx;
+            p[y] = pr < R2 && pc < R2 ? D[(size_t)pr * R2 + pc] : 0.0;
+            q[y] = qr < R2 && qc < R2 ? D[(size_t)qr * R2 + qc] : 0.0;
+        }
+#pragma unroll
+        for (int y = 0; y < 4; ++y) Q[ty + 8 * y][tx] = q[y];
+        __syncthreads();
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            mx = max(mx, max(bits(p[y]), bits(q[y])));
+            ma = max(ma, bits(p[y] - Q[tx][ty + 8 * y]));
+        }
+        __syncthreads();
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+    }
+    if (tx == 0) {
+        sh[0][ty] = mx;
+        sh[1][ty] = ma;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        unsigned long long v = 0;
+        for (int y = 0; y < 8; ++y) v = max(v, sh[threadIdx.x][y]);
+        if (v) atomicMax(dmax + threadIdx.x, v);
+    }
+}
+
+// M = 3 2Delta + 1D^1D = 3 2D - 2 (1D^1D), (1D^1D)^{ij}_{kl} = 1/2(g^i_k g^j_l - g^j_k g^i_l) (App. C);
+// the exchange piece vanishes in the ab block (1D is spin diagonal).  The first nasym blocks take the asymmetry of D
+// beside it: this part is bound by the FP64 pipe, that one by memory.
+__global__ void __launch_bounds__(TPB) k_build_M(int r, int nasym, const double* __restrict__ gam,
+                                                 const double* __restrict__ Daa, const double* __restrict__ Dab,
+                                                 const double* __restrict__ Dbb, double* __restrict__ Maa,
+                                                 double* __restrict__ Mab, double* __restrict__ Mbb,
+                                                 unsigned long long* __restrict__ dmax) {
+    if ((int)blockIdx.x < nasym) {
+        d_asymmetry(r, blockIdx.x, nasym, Daa, Dab, Dbb, dmax);
+        return;
+    }
+    const size_t n = (size_t)r * r * r * r, step = (size_t)(gridDim.x - nasym) * blockDim.x;
     const double* ga = gam;
     const double* gb = gam + r * r;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    for (size_t e = (blockIdx.x - nasym) * (size_t)blockDim.x + threadIdx.x; e < n; e += step) {
         const int l = (int)(e % r), k = (int)((e / r) % r), j = (int)((e / ((size_t)r * r)) % r),
                   i = (int)(e / ((size_t)r * r * r));
         Maa[e] = 3.0 * Daa[e] - (ga[i * r + k] * ga[j * r + l] - ga[j * r + k] * ga[i * r + l]);
@@ -178,8 +193,7 @@ __global__ void k_build_M(int r, const double* __restrict__ gam, const double* _
 
 int launch_gamma(acse_ctx* c, const double* const D[3]) {
     const int r = c->r;
-    const int nT = (r * r + 31) / 32, nasym = c->w.dmax ? 3 * (nT * (nT + 1) / 2) : 0;
-    k_gamma<<<(2 * r * r + 7) / 8 + nasym, 256, 0, c->stream>>>(r, 2.0 / (c->N - 1), D[0], D[1], D[2], c->w.gam, c->w.dmax);
+    k_gamma<<<(2 * r * r + 7) / 8, 256, 0, c->stream>>>(r, 2.0 / (c->N - 1), D[0], D[1], D[2], c->w.gam, c->w.dmax);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -188,8 +202,9 @@ int launch_gamma_M(acse_ctx* c, const double* const D[3]) {
     const int r = c->r;
     ACSE_TRY(launch_gamma(c, D));
     const size_t n = (size_t)r * r * r * r;
-    k_build_M<<<grid_for(n), TPB, 0, c->stream>>>(r, c->w.gam, D[0], D[1], D[2], c->w.M[0], c->w.M[1], c->w.M[2],
-                                                 c->w.dmax, c->w.asym);
+    const int nT = (r * r + 31) / 32, ntri = 3 * (nT * (nT + 1) / 2), nasym = ntri < 152 * 2 ? ntri : 152 * 2;
+    k_build_M<<<nasym + grid_for(n), TPB, 0, c->stream>>>(r, nasym, c->w.gam, D[0], D[1], D[2], c->w.M[0], c->w.M[1],
+                                                          c->w.M[2], c->w.dmax);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }

@@ -109,8 +109,8 @@ struct Work {
     double* Mm;
     double* Mf1;
     double* Mf2;
-    unsigned long long* dmax;   // largest |D| and |D - D^T| of the D being prepared (bit patterns; zero between passes)
-    int* asym;                  // not zero: that D is not pair-Hermitian (k_build_M)
+    unsigned long long* dmax;   // largest |D| and |D - D^T| of the D being prepared (bit patterns, k_build_M)
+    int* asym;                  // not zero: that D is not pair-Hermitian (k_ph_pack_asym)
     double* Wp;
     double* Wm;
     double* Wf1;

@@ -17,7 +17,7 @@
 // W always has that symmetry, a 2-RDM D does, but the caller's D (sampled, truncated, one-sided) need not. M+ then
 // also has a part that is antisymmetric in (i,l), M- one that is symmetric, and the second flip is a product of its
 // own: V1, V2 get those columns too (2P and 2S of them) by three more products, 6 r^6, which every context holds and
-// runs where k_build_M found max |D - D^T| > 2^-47 max |D| in the D being prepared (`asym`, on the device: no
+// runs where k_ph_pack_asym finds max |D - D^T| > 2^-47 max |D| in the D being prepared (`asym`, on the device: no
 // read-back, and a captured step decides anew on every replay).  That bound is 32 units in the last place of the
 // largest entry: a D that is Hermitian but for the rounding of an orbital transformation (1.2 2^-50 measured at r = 48)
 // stays below it, and what is dropped of its asymmetry is below the rounding of its own entries.
@@ -35,10 +35,6 @@
 // x = T^{kp}_{qt}, x' = T^{kt}_{qp}, spins K of (k,q) and P' of (p,t); the rows of `plus` run over k <= q and
 // those of `minus` over k < q (plusS = 1), or the other way round (plusS = 0).  flip[(k,q)][(p,t)] =
 // T_ab[k][p][t][q].  W takes f = 1/2; M takes f = 1, the 2 of the halved sum over (p,t) included.
-// An M that is not pair-Hermitian (asym, not zero): x and x' are averaged over the exchange of k and q, half their
-// differences go to 2P more rows of `plus` (k < q) and 2S more of `minus` (k <= q), and flip2[(k,q)][(p,t)] =
-// T_ab[t][q][k][p] is the second flip with both its pairs exchanged (for a Hermitian T equal to flip).
-//
 // Block (K, P', {k<=q}): the r x r slab of (p,t) goes through shared memory, both rows leave coalesced (the
 // b,a slab is read at stride r: its sectors are shared by the blocks of neighbouring q).  Block (k,p) of the
 // flips: an r x r transposition in shared memory.
@@ -47,8 +43,6 @@ struct PhPack {
     double* plus;
     double* minus;
     double* flip;
-    double* flip2;     // M: the second flip ...
-    const int* asym;   // ... where *asym is not zero; null for W
     int r, plusS;
     double f;
 };
@@ -57,7 +51,6 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
     extern __shared__ double ph_sm[];   // [r][r + 1]
     const int r = a.r, ld = r + 1, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
     const size_t R2 = (size_t)r * r, r3 = R2 * r;
-    const bool gen = a.asym && *a.asym;
     if ((int)blockIdx.x < 4 * S) {
         const int kp = (int)blockIdx.x / S, u = (int)blockIdx.x - kp * S, K = kp >> 1, Q = kp & 1;
         int k, q;
@@ -76,23 +69,9 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
         for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
             const int p = e / r, t = e - p * r;
             if (t < p) continue;
-            double x = ph_sm[p * ld + t], y = ph_sm[t * ld + p];
-            if (gen) {   // the slab of (q,k), read as it is stored
-                const bool tr = K == 1 && Q == 0;
-                const double x2 = tr ? src[p * r3 + q * R2 + (size_t)t * r + k] : src[q * r3 + p * R2 + (size_t)k * r + t];
-                const double y2 = tr ? src[t * r3 + q * R2 + (size_t)p * r + k] : src[q * r3 + t * R2 + (size_t)k * r + p];
-                const double dx = 0.5 * (x - x2), dy = 0.5 * (y - y2);
-                x = 0.5 * (x + x2);
-                y = 0.5 * (y + y2);
-                if (rowA >= 0) a.plus[((size_t)2 * S + rowA) * 2 * S + Q * S + ps_pair(r, p, t)] = p < t ? a.f * (dx + dy) : dx;
-                if (p < t) {
-                    a.minus[((size_t)2 * P + rowS) * 2 * P + Q * P + pk_pair(r, p, t)] = a.f * (x - y);
-                    if (rowA >= 0) om[pk_pair(r, p, t)] = a.f * (dx - dy);
-                }
-            } else if (rm >= 0 && p < t) {
-                om[pk_pair(r, p, t)] = a.f * (x - y);
-            }
+            const double x = ph_sm[p * ld + t], y = ph_sm[t * ld + p];
             if (rp >= 0) op[ps_pair(r, p, t)] = p < t ? a.f * (x + y) : x;
+            if (rm >= 0 && p < t) om[pk_pair(r, p, t)] = a.f * (x - y);
         }
     } else {
         const int kp = (int)blockIdx.x - 4 * S, k = kp / r, p = kp - k * r;
@@ -102,21 +81,18 @@ __global__ void __launch_bounds__(256) k_ph_pack(const __grid_constant__ PhPack 
         for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
             const int q = e / r, t = e - q * r;
             a.flip[((size_t)k * r + q) * R2 + (size_t)p * r + t] = ph_sm[t * ld + q];
-            if (gen) a.flip2[((size_t)k * r + q) * R2 + (size_t)p * r + t] = a.src[1][t * r3 + q * R2 + (size_t)k * r + p];
         }
     }
 }
 
-static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, double* minus, double* flip, double* flip2,
-                          int plusS, double f) {
+static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, double* minus, double* flip, int plusS,
+                          double f) {
     const int r = c->r;
     PhPack a;
     for (int s = 0; s < 3; ++s) a.src[s] = T[s];
     a.plus = plus;
     a.minus = minus;
     a.flip = flip;
-    a.flip2 = flip2;
-    a.asym = flip2 ? c->w.asym : nullptr;
     a.r = r;
     a.plusS = plusS;
     a.f = f;
@@ -126,14 +102,81 @@ static int launch_ph_pack(acse_ctx* c, const double* const T[3], double* plus, d
     return ACSE_OK;
 }
 
+// Is D pair-Hermitian (the maxima of k_build_M), for the kernels behind this one in `asym`; and where it is not (otherwise
+// the blocks leave at once, 1.6 us): M+ and M- with x and x' averaged over
+// the exchange of k and q, half their differences in 2P more rows of M+ (k < q) and 2S more of M- (k <= q), and
+// flip2[(k,q)][(p,t)] = M_ab[t][q][k][p], the second flip with both its pairs exchanged (for a Hermitian M the first).
+// Read straight from global memory: the rare case.
+struct PhPackAsym {
+    const double* src[3];
+    double* plus;
+    double* minus;
+    double* flip2;
+    const unsigned long long* dmax;
+    int* asym;
+    int r;
+};
+
+__global__ void __launch_bounds__(256) k_ph_pack_asym(const __grid_constant__ PhPackAsym a) {
+    const double mx = __longlong_as_double((long long)a.dmax[0]), ma = __longlong_as_double((long long)a.dmax[1]);
+    const bool sym = ma <= mx * 0x1p-47;   // NaN: not
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.asym = sym ? 0 : 1;
+    if (sym) return;
+    const int r = a.r, S = r * (r + 1) / 2, P = r * (r - 1) / 2;
+    const size_t R2 = (size_t)r * r, r3 = R2 * r;
+    for (int w = blockIdx.x; w < 4 * S + (int)R2; w += gridDim.x) {
+        const int kp = w < 4 * S ? w / S : 0, u = w - kp * S, K = kp >> 1, Q = kp & 1;
+        int k, q;
+        if (w < 4 * S) {
+            ps_unpair(r, u, k, q);
+        } else {
+            k = (w - 4 * S) / r;
+            q = w - 4 * S - k * r;
+        }
+        const double* src = a.src[w < 4 * S && K == Q ? 2 * K : 1];
+        // T^{kp}_{qt} of the spins K of (k,q) and Q of (p,t)
+        auto at = [&](int k, int q, int p, int t) {
+            return K == 1 && Q == 0 ? src[p * r3 + k * R2 + (size_t)t * r + q] : src[k * r3 + p * R2 + (size_t)q * r + t];
+        };
+        const int rowS = K * S + u, rowA = k < q ? K * P + pk_pair(r, k, q) : -1;
+        for (int e = threadIdx.x; e < (int)R2; e += blockDim.x) {
+            const int p = e / r, t = e - p * r;
+            if (w >= 4 * S) {
+                a.flip2[((size_t)k * r + q) * R2 + e] = src[t * r3 + q * R2 + (size_t)k * r + p];
+                continue;
+            }
+            if (t < p) continue;
+            const double x1 = at(k, q, p, t), x2 = at(q, k, p, t), y1 = at(k, q, t, p), y2 = at(q, k, t, p);
+            const double x = 0.5 * (x1 + x2), y = 0.5 * (y1 + y2), dx = 0.5 * (x1 - x2), dy = 0.5 * (y1 - y2);
+            const size_t cs = (size_t)Q * S + ps_pair(r, p, t), ca = (size_t)Q * P + (p < t ? pk_pair(r, p, t) : 0);
+            a.plus[(size_t)rowS * 2 * S + cs] = p < t ? x + y : x;
+            if (p < t) a.minus[((size_t)2 * P + rowS) * 2 * P + ca] = x - y;
+            if (rowA < 0) continue;
+            a.plus[((size_t)2 * S + rowA) * 2 * S + cs] = p < t ? dx + dy : dx;
+            if (p < t) a.minus[(size_t)rowA * 2 * P + ca] = dx - dy;
+        }
+    }
+}
+
 int launch_ph_pack_M(acse_ctx* c) {
     Work& w = c->w;
-    return launch_ph_pack(c, w.M, w.Mp, w.Mm, w.Mf1, w.Mf2, 1, 1.0);
+    ACSE_TRY(launch_ph_pack(c, w.M, w.Mp, w.Mm, w.Mf1, 1, 1.0));
+    PhPackAsym a;
+    for (int s = 0; s < 3; ++s) a.src[s] = w.M[s];
+    a.plus = w.Mp;
+    a.minus = w.Mm;
+    a.flip2 = w.Mf2;
+    a.dmax = w.dmax;
+    a.asym = w.asym;
+    a.r = c->r;
+    k_ph_pack_asym<<<152 * 2, 256, 0, c->stream>>>(a);
+    ACSE_LAUNCHED(c);
+    return ACSE_OK;
 }
 
 int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW) {
     Work& w = c->w;
-    return launch_ph_pack(c, W, w.Wp, w.Wm, w.Wf1, nullptr, sW > 0, 0.5);
+    return launch_ph_pack(c, W, w.Wp, w.Wm, w.Wf1, sW > 0, 0.5);
 }
 
 // ------------------------------------------------------------------------------ expansion

@@ -38,7 +38,7 @@
 #define OZ_CHUNK_KB 64       // 64-element K blocks of one exactly accumulated chunk: 64 * 64 * 64^2 = 2^24
 #define OZ_MAXCH 2           // chunks of one residue product (K <= 2 * 64 * 64 = 8192)
 #define OZ_MAXP 12           // GEMMs of one launch
-#define OZ_MAXJ 18           // operands of one slicing launch
+#define OZ_MAXJ 16           // operands of one slicing launch
 #define OZ_THREADS 192
 #define OZ_BN 256
 #define OZ_STAGES 4
@@ -124,12 +124,12 @@ struct OzSliceJob {
     __nv_bfloat16* dst;     // first output row of the job
     size_t ldd;             // T * Kp
     double* scale;          // 2^e per output row (NaN for a row with a non-finite entry)
-    const int* gate;        // null, or the job is skipped where *gate is zero
     int rows, K, Kp, nb, mul_y, row0;
 };
 
 struct OzSliceBatch {
     OzSliceJob j[OZ_MAXJ];
+    const int* gate;        // null, or the launch is skipped where *gate is zero
     int njobs;
     int T;
     float p[OZ_NMOD], pinv[OZ_NMOD];
@@ -140,11 +140,10 @@ struct OzSliceBatch {
 // fixes e (|a| 2^-e < 1/2); scale = 2^e, NaN for a row with a non-finite entry.
 __global__ void __launch_bounds__(256) k_oz_rowscale(const __grid_constant__ OzSliceBatch b, int rows) {
     const int grow = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (grow >= rows) return;
+    if (grow >= rows || (b.gate && !*b.gate)) return;
     int ji = 0;
     while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
     const OzSliceJob& J = b.j[ji];
-    if (J.gate && !*J.gate) return;
     const int row = grow - J.row0;
     const int srow = J.rowmap ? J.rowmap[row] : row;
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(J.src + (size_t)srow * J.lds);
@@ -180,12 +179,10 @@ __device__ __forceinline__ void oz_limbs(unsigned long long bits, int nb, int e,
     L[3] = sg * (__uint_as_float(0x4B000000u | l3) - 8388608.0f);
 }
 
-__global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSliceBatch b) {
-    const int grow = (int)blockIdx.y;
+__device__ __forceinline__ void oz_residue_row(const OzSliceBatch& b, int grow) {
     int ji = 0;
     while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
     const OzSliceJob& J = b.j[ji];
-    if (J.gate && !*J.gate) return;
     const int K = J.K;
     const int qi = (int)blockIdx.x * 256 + (int)threadIdx.x;
     if (qi >= (K + 3) >> 2) return;
@@ -221,6 +218,18 @@ __global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSl
                 if (i < nk) reinterpret_cast<unsigned short*>(dst)[i] = (unsigned short)(h[i] >> 16);
         }
     }
+}
+
+// A block row per operand row, or (gated) a few that take every gridDim.y-th: r = 48, 7000 gated rows left at once took
+// 20 us as block rows of their own.
+template <bool GATED>
+__global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSliceBatch b, int rows) {
+    if (!GATED) {
+        oz_residue_row(b, (int)blockIdx.y);
+        return;
+    }
+    if (!*b.gate) return;
+    for (int grow = (int)blockIdx.y; grow < rows; grow += (int)gridDim.y) oz_residue_row(b, grow);
 }
 
 // ------------------------------------------------------------------------------- GEMM
@@ -617,7 +626,7 @@ static int oz_launch_crt(const OzBatch* host, const OzBatch* dev, int nsm, cudaS
 // The problem table of s = +1 is the plan itself; that of s = -1 (`alt`) has the same operands with the
 // other row counts and borrows every buffer.  `gen`: the three products of a D that is not pair-Hermitian, with the same
 // A and B operands of their own (the 2P odd rows of M+, the 2S even ones of M-, the second flip of M), skipped on the
-// device (Work::asym) for the others.
+// device (Work::asym) for any other D: its launches leave at once, 2-3 us each.
 struct OzOp {
     __nv_bfloat16* sl;
     double* scale;
@@ -1022,9 +1031,8 @@ static void oz_slice_batch_init(OzSliceBatch& b, const OzMods& m) {
 // One slicing job: `rows` rows of operand o starting at output row `orow`, read from src (row stride
 // lds) through the optional row / column maps; mul_y for a B operand (residues times y_t).
 static void oz_job(OzSliceBatch& b, int& rows, const OzOp& o, int orow, int nrows, const double* src, size_t lds,
-                   const int* rowmap, const int* colmap, int mul_y, const int* gate = nullptr) {
+                   const int* rowmap, const int* colmap, int mul_y) {
     OzSliceJob& j = b.j[b.njobs++];
-    j.gate = gate;
     j.src = src;
     j.lds = lds;
     j.rowmap = rowmap;
@@ -1050,7 +1058,8 @@ static int oz_slice_launch(acse_ctx* c, const OzSliceBatch& all, int rows) {
     ACSE_LAUNCHED(c);
     int maxq = 1;
     for (int i = 0; i < all.njobs; ++i) maxq = (all.j[i].K + 3) / 4 > maxq ? (all.j[i].K + 3) / 4 : maxq;
-    k_oz_residue<<<dim3((maxq + 255) / 256, rows), 256, 0, c->stream>>>(all);
+    if (all.gate) k_oz_residue<true><<<dim3((maxq + 255) / 256, rows < 128 ? rows : 128), 256, 0, c->stream>>>(all, rows);
+    else k_oz_residue<false><<<dim3((maxq + 255) / 256, rows), 256, 0, c->stream>>>(all, rows);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -1077,9 +1086,14 @@ int oz_slice_operands(acse_ctx* c, int prep_D, int sW) {
         oz_job(b, rows, pl->B[1], 0, P2, w.Mm, P2, nullptr, nullptr, 1);
         oz_job(b, rows, pl->B[2], 0, R2, w.Mf1, R2, nullptr, nullptr, 1);
         const OzOp* gB = root->gen->B;
-        oz_job(b, rows, gB[0], 0, P2, w.Mp + (size_t)S2 * S2, S2, nullptr, nullptr, 1, w.asym);
-        oz_job(b, rows, gB[1], 0, S2, w.Mm + (size_t)P2 * P2, P2, nullptr, nullptr, 1, w.asym);
-        oz_job(b, rows, gB[2], 0, R2, w.Mf2, R2, nullptr, nullptr, 1, w.asym);
+        OzSliceBatch gb;
+        oz_slice_batch_init(gb, pl->host->mods);
+        gb.gate = w.asym;
+        int grows = 0;
+        oz_job(gb, grows, gB[0], 0, P2, w.Mp + (size_t)S2 * S2, S2, nullptr, nullptr, 1);
+        oz_job(gb, grows, gB[1], 0, S2, w.Mm + (size_t)P2 * P2, P2, nullptr, nullptr, 1);
+        oz_job(gb, grows, gB[2], 0, R2, w.Mf2, R2, nullptr, nullptr, 1);
+        ACSE_TRY(oz_slice_launch(c, gb, grows));
     }
     oz_job(b, rows, pl->B[3], 0, R2, c->cur_W[1], R2, nullptr, nullptr, 1);
     oz_job(b, rows, pl->B[4], 0, P, c->cur_W[0], R2, pm, pm, 1);
