@@ -76,9 +76,10 @@ typedef enum {
  *                slices) and rebuilt exactly by the Chinese remainder theorem, with one rounding to FP64.
  *                With the default 8 (48 bits) the GEMM error is of the order of 2^-48 |A||B| K, below
  *                that of FP64 FMA.  The O(r^5) products (the transformation by 1D and the products of the pairs)
- *                run with 8 slices or fewer by the digit form of the scheme (error-free splitting, Ozaki, Ogita,
- *                Oishi and Rump, Numer. Algorithms 59, 2012) in ceil(6 oz_slices / 8) eight-bit digits, with
- *                more in double-float FP32.  The adjoint's O(r^6) GEMMs run by the modular form. */
+ *                run at r >= 16 with 8 slices or fewer by the digit form of the scheme (error-free splitting,
+ *                Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012) in ceil(6 oz_slices / 8) base-256
+ *                digits, with more in double-float FP32 (FP64 in the adjoint), and in FP64 below r = 16.  The
+ *                adjoint's O(r^6) GEMMs run by the modular form. */
 typedef enum { ACSE_FP64 = 0, ACSE_BF16X3 = 1, ACSE_TF32 = 2, ACSE_TF32X3 = 3, ACSE_OZAKI = 4 } acse_prec;
 /* 3-RDM reconstruction (Eq. 3rdm_recon / Eq. NY):
  *   ACSE_RECON_V   Valdemoro: the 3-cumulant is neglected;

@@ -276,8 +276,9 @@ int launch_gamma(acse_ctx* c, const double* const D[3]);
 int launch_gamma_M(acse_ctx* c, const double* const D[3]);
 int launch_w_sum(acse_ctx* c);
 // Ozaki contexts of more slices than the digit kernel takes run their O(r^5) products in double-float, but not those of
-// a reverse sweep: cotangents have any scale, and the pair has the range of FP32.
-static inline bool acse_use_dfl(const acse_ctx* c) { return c->oz && !c->in_adjoint; }
+// a reverse sweep: cotangents have any scale, and the pair has the range of FP32.  Below r = 16 all run in FP64.
+#define ACSE_OZ_RMIN 16
+static inline bool acse_use_dfl(const acse_ctx* c) { return c->oz && !c->in_adjoint && c->r >= ACSE_OZ_RMIN; }
 // particle-hole products on symmetrised pairs (acse_ph.cu)
 int launch_ph_pack_M(acse_ctx* c);
 int launch_ph_pack_W(acse_ctx* c, const double* const W[3], int sW);

@@ -7,16 +7,19 @@
 // (the x1 and x2 of the B kernel, and the adjoint's: rows (ij, k) of r^4 arrays, eight classes).
 //
 // Every row of A and of G gets a power-of-two scale 2^e (|x| 2^-e < 1/2 over the row) and each element the
-// fixed-point value X = round(x 2^(8D - e)), cut into D balanced base-256 digits (most significant first; -128 ..
-// 128, exact in bf16).  D = ceil(6 S / 8) digits hold at least the 6 S bits of oz_slices = S.  The products of one
-// level L = s + t <= D + 2 are accumulated in FP32 in their own TMEM accumulator: a level holds at most D <= 6
-// products of K <= 64 terms of magnitude <= 2^14, below 2^23, so every level sum is an exact integer.  The
-// epilogue adds the levels in int64 (sum_L v_L 2^(8 (D + 1 - L)), below 2^61, the last level rounded to that unit) and
-// rounds once to FP64, scaled by 2^(e_m + e_n - 8 (D + 1)).  What is left is the fixed-point rounding, 2^-8D of the
-// row scales: with the levels up to D + 1 only, the dropped level D + 2 (D - 1 products a term) was the larger
-// error (r = 30 residual 7.5e-14 against 3.4e-14 of double-float products).  Against eight base-64 digits: 26 digit
-// products in place of 36, seven levels in place of eight, and a digit is a byte of X + 128 (1 + 256 + ...): a
-// permute and half a packed FADD.
+// fixed-point value X = round(x 2^(8D + 1 - e)), |X| < 2^8D, cut into D base-256 digits (most significant first): the
+// leading one within -256 .. 256, the others balanced, -128 .. 127 (exact in bf16).  D = ceil(6 S / 8) digits hold at
+// least the 6 S bits of oz_slices = S below the row's leading one.  The products of one level L = s + t <= D + 2 are
+// accumulated in FP32 in their own TMEM accumulator: a level holds at most D <= 6 products of K <= 64 terms of
+// magnitude <= 2^14, twice that in the two with one leading digit and 2^16 in that of two, so it stays within 2^23
+// and every level sum is an exact integer.  The epilogue adds the levels in int64 (sum_L v_L 2^(8 (D + 1 - L)), below
+// 2^63, the last level rounded to that unit) and rounds once to FP64, scaled by 2^(e_m + e_n - 8 (D + 1) - 2).  What is
+// left is the fixed-point rounding, 2^-(8D + 1) of the row scales: with one bit less (the leading digit balanced like
+// the others) that was the larger part of the error at ragged r, U of a step at r = 20 1.39e-14 rms against 64 bits,
+// where double-float products gave 1.2e-14 and this gives 9.3e-15.  With the levels up to D + 1 only, the dropped level
+// D + 2 (D - 1 products a term) was the larger error (r = 30 residual 7.5e-14 against 3.4e-14 of double-float products).
+// Against eight base-64 digits: 26 digit products in place of 36, seven levels in place of eight, and a digit is a byte
+// of X + 128 (1 + 256 + ...): a permute and half a packed FADD.
 //
 // One block per SM, warp-specialised (the phases of a tile of 128 rows one after another behind block barriers
 // took 20 us a tile): eight producer warps load the rows of the next tile and write its digits into one of two
@@ -31,7 +34,9 @@
 // digits and the int64 normalisation, about half busy) and the chain TMEM read - MMA - TMEM read; HBM at 2 TB/s.
 // Every wait is bounded, and on expiry the kernel raises the device flag and stops.
 //
-// Used for S <= 8; more slices take the double-float kernels of acse_ph.cu.
+// Used for S <= 8 and r >= 16; more slices take the double-float kernels of acse_ph.cu, smaller r the FP64 ones, which
+// leave the rounding of the GEMMs alone in the error (U at r = 12: 7.2e-15 rms, digits of eight bits 1.28e-14,
+// double-float 7.7e-15; a residual at r = 15 takes 12 us longer).
 #include <cuda_bf16.h>
 
 #include "acse_internal.h"
@@ -68,16 +73,16 @@ struct RowsArgs {
 static __device__ __forceinline__ int rz_row_exp(unsigned int mh) {
     if (mh >= 0x7FF00000u) return RZ_BAD;
     if (mh == 0) return 0;
-    return min(1000, max(-960, (int)(mh >> 20) - 1023 + 2));   // 2^(8D - e) is a normal double
+    return min(1000, max(-960, (int)(mh >> 20) - 1023 + 2));   // 2^(8D + 1 - e) is a normal double
 }
 
-// 2^(8D - e) of a row; 0 for a bad one (whose digits are then whatever they are: its results are set to NaN).
+// 2^(8D + 1 - e) of a row; 0 for a bad one (whose digits are then whatever they are: its results are set to NaN).
 static __device__ __forceinline__ double rz_scale(int e, int D) {
-    return e == RZ_BAD ? 0.0 : oz_pow2(8 * D - e);
+    return e == RZ_BAD ? 0.0 : oz_pow2(8 * D + 1 - e);
 }
 
 // The D digits of the eight elements x (scale e) as bf16, one 16-byte chunk per digit tile: digit tile s - 1
-// (base + (s - 1) stride) holds digit s, most significant first.  Fixed point X = round(x 2^(8D - e)) plus the bias
+// (base + (s - 1) stride) holds digit s, most significant first.  Fixed point X = round(x 2^(8D + 1 - e)) plus the bias
 // 128 in every byte below the leading one: byte i of the sum minus 128 is the balanced digit of weight 256^i and
 // the rest is the leading digit.  One FP64 FMA with 1.5 2^52 + bias leaves that sum in the low bits of its
 // result: the FP64 pipe is otherwise idle here (42.5 M of them at r = 48 take it 73 us) while the ALU pipe bounds
@@ -103,7 +108,7 @@ static __device__ __forceinline__ void rz_digits8(const double (&x)[8], double s
                 f.x = __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7540u | (unsigned)(i & 3)));
                 f.y = __uint_as_float(__byte_perm(q, 0x4B000000u, 0x7540u | (unsigned)(i & 3)));
                 f = __fadd2_rn(f, make_float2(-8388736.0f, -8388736.0f));
-            } else {   // the leading digit, signed (|d| <= 128): bits 8 i .. of the sum
+            } else {   // the leading digit, signed (|d| <= 256): bits 8 i .. of the sum
                 const int tp = i < 4 ? (int)__funnelshift_r(lo[u], hi[u], 8 * i) : (int)hi[u] >> (8 * (i & 3));
                 const int tq = i < 4 ? (int)__funnelshift_r(lo[u + 1], hi[u + 1], 8 * i) : (int)hi[u + 1] >> (8 * (i & 3));
                 f = __fadd2_rn(make_float2(__int_as_float(0x4B400000 + tp), __int_as_float(0x4B400000 + tq)),
@@ -123,7 +128,7 @@ static __device__ __forceinline__ double rz_scaled(long long acc, int ex) {
     const unsigned int uh = (unsigned int)(u >> 32);
     const int n = uh ? __clz(uh) : 32 + __clz((unsigned int)u);
     const int E = ex + 63 - n + 1022;   // exponent field less one: the significand's leading bit adds it
-    const unsigned long long b = ((u << ((n - 1) & 63)) + 512) >> 10;   // |acc| < 2^62: n >= 2, no carry out
+    const unsigned long long b = ((u << ((n - 1) & 63)) + 512) >> 10;   // |acc| < 2^63: n >= 1, no carry out
     if (acc == 0) return 0.0;
     if (E < 1 || E > 2044) return oz_ll_scaled(acc, ex);
     return __longlong_as_double((long long)((b + ((unsigned long long)(unsigned)E << 52)) | (sg << 63)));
@@ -397,10 +402,10 @@ __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant
                     unsigned int w[RZ_DMAX + 1][2];   // level sums as integers (modulo 2^32)
 #pragma unroll
                     for (int j = 0; j <= RZ_DMAX; ++j) {
-                        // level j holds at most min(j + 1, 5) (the last) or j + 1 products: |v| <= n RP 2^14, within the
-                        // 2^22 of the FADD conversion for n RP <= 256
+                        // level j holds at most j + 1 products (the last D - 1 <= 5), in units of RP 2^14: one of 4, or two
+                        // of 2 and the rest of 1 (the last: of 1 only); within the 2^22 of the FADD conversion for n RP <= 256
                         const float2 f = make_float2(__uint_as_float(v[j][c]), __uint_as_float(v[j][c + 1]));
-                        if ((j == RZ_DMAX ? RZ_DMAX - 1 : j + 1) * RP <= 256) {
+                        if ((j == RZ_DMAX ? RZ_DMAX - 1 : j == 0 ? 4 : j + 3) * RP <= 256) {
                             const float2 m = __fadd2_rn(f, make_float2(12582912.0f, 12582912.0f));
                             w[j][0] = __float_as_uint(m.x) - 0x4B400000u;
                             w[j][1] = __float_as_uint(m.y) - 0x4B400000u;
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant
                 for (int u = 0; u < 2; ++u) {
                     const int en = eb[n + u];
                     z[u] = (em == RZ_BAD || en == RZ_BAD) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                          : rz_scaled(acc[n + u], em + en - 8 * (D + 1));
+                                                          : rz_scaled(acc[n + u], em + en - 8 * (D + 1) - 2);
                 }
                 if (v2) {
                     *reinterpret_cast<double2*>(o + n) = make_double2(z[0], z[1]);
@@ -485,7 +490,7 @@ static int rows_dispatch(acse_ctx* c, RowsArgs& a) {
     return s;
 }
 
-static bool rows_oz_applies(const acse_ctx* c) { return c->oz && c->opt.oz_slices <= RZ_SMAX; }
+static bool rows_oz_applies(const acse_ctx* c) { return c->oz && c->opt.oz_slices <= RZ_SMAX && c->r >= ACSE_OZ_RMIN; }
 
 // The transformation by 1D (trans: by its transpose) of the three arrays; ACSE_ERR_UNSUPPORTED where the kernel
 // does not apply.
