@@ -202,7 +202,7 @@ int launch_gamma_M(acse_ctx* c, const double* const D[3]) {
     const int r = c->r;
     ACSE_TRY(launch_gamma(c, D));
     const size_t n = (size_t)r * r * r * r;
-    const int nT = (r * r + 31) / 32, ntri = 3 * (nT * (nT + 1) / 2), nasym = ntri < 152 * 2 ? ntri : 152 * 2;
+    const int nT = (r * r + 31) / 32, ntri = 3 * (nT * (nT + 1) / 2), nasym = ntri < 152 * 4 ? ntri : 152 * 4;
     k_build_M<<<nasym + grid_for(n), TPB, 0, c->stream>>>(r, nasym, c->w.gam, D[0], D[1], D[2], c->w.M[0], c->w.M[1],
                                                           c->w.M[2], c->w.dmax);
     ACSE_LAUNCHED(c);

@@ -78,6 +78,7 @@ struct OzProb {
     int nb;             // operand rows rounded to X = round(a 2^(nb - e))
     int ngroups;        // T nch, modulus-major
     int tiles_n, tile_start;
+    const int* gate;    // null, or the problem is skipped where *gate is zero
 };
 
 struct __align__(128) OzBatch {
@@ -88,12 +89,14 @@ struct __align__(128) OzBatch {
     int nprob;
     int total_tiles;
     int* err;
-    const int* gate;      // null, or the launch is skipped where *gate is zero
     unsigned long long wait_ns;
     int inject_stall;
     const int* order;     // tiles of CTA c: order[cta_start[c] .. cta_start[c+1]) (longest first)
     const int* cta_start;
 };
+
+// A gated problem whose gate is down: every role of the kernel passes over its tiles.
+__device__ __forceinline__ bool oz_skip(const OzProb& P) { return P.gate && !*P.gate; }
 
 __device__ __forceinline__ int oz_find_problem(const OzBatch& b, int t) {
     int lo = 0, hi = b.nprob - 1;
@@ -129,18 +132,25 @@ struct OzSliceJob {
 
 struct OzSliceBatch {
     OzSliceJob j[OZ_MAXJ];
-    const int* gate;        // null, or the launch is skipped where *gate is zero
     int njobs;
     int T;
     float p[OZ_NMOD], pinv[OZ_NMOD];
     float cA[OZ_NMOD][4], cB[OZ_NMOD][4];
 };
 
+// 2^e of a row whose largest magnitude has the pattern mx (non-negative doubles order like their bit patterns; an
+// all-ones exponent is Inf or NaN).
+__device__ __forceinline__ double oz_row_scale(unsigned long long mx) {
+    const bool bad = mx >= 0x7FF0000000000000ull;
+    const int e = (bad || mx == 0) ? 0 : min(1000, max(-1000, (int)(mx >> 52) - 1023 + 2));
+    return bad ? __longlong_as_double(0x7ff8000000000000ll) : oz_pow2(e);
+}
+
 // Row scales: one warp per operand row takes the largest magnitude over the row (through the maps), which
 // fixes e (|a| 2^-e < 1/2); scale = 2^e, NaN for a row with a non-finite entry.
 __global__ void __launch_bounds__(256) k_oz_rowscale(const __grid_constant__ OzSliceBatch b, int rows) {
     const int grow = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (grow >= rows || (b.gate && !*b.gate)) return;
+    if (grow >= rows) return;
     int ji = 0;
     while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
     const OzSliceJob& J = b.j[ji];
@@ -152,12 +162,7 @@ __global__ void __launch_bounds__(256) k_oz_rowscale(const __grid_constant__ OzS
     for (int k = lane; k < J.K; k += 32) mx = max(mx, src[cm ? cm[k] : k] & 0x7FFFFFFFFFFFFFFFull);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) {
-        // non-negative doubles order like their bit patterns; an all-ones exponent is Inf or NaN
-        const bool bad = mx >= 0x7FF0000000000000ull;
-        const int e = (bad || mx == 0) ? 0 : min(1000, max(-1000, (int)(mx >> 52) - 1023 + 2));
-        J.scale[row] = bad ? __longlong_as_double(0x7ff8000000000000ll) : oz_pow2(e);
-    }
+    if (lane == 0) J.scale[row] = oz_row_scale(mx);
 }
 
 // Residues: block (x, y) covers elements 1024 x .. 1024 x + 1023 of operand row y (rows of all jobs in
@@ -179,14 +184,8 @@ __device__ __forceinline__ void oz_limbs(unsigned long long bits, int nb, int e,
     L[3] = sg * (__uint_as_float(0x4B000000u | l3) - 8388608.0f);
 }
 
-__device__ __forceinline__ void oz_residue_row(const OzSliceBatch& b, int grow) {
-    int ji = 0;
-    while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
-    const OzSliceJob& J = b.j[ji];
-    const int K = J.K;
-    const int qi = (int)blockIdx.x * 256 + (int)threadIdx.x;
-    if (qi >= (K + 3) >> 2) return;
-    const int row = grow - J.row0, k = 4 * qi;
+__device__ __forceinline__ void oz_residue4(const OzSliceBatch& b, const OzSliceJob& J, int row, int qi) {
+    const int K = J.K, k = 4 * qi;
     const int srow = J.rowmap ? J.rowmap[row] : row;
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(J.src + (size_t)srow * J.lds);
     const int* cm = J.colmap;
@@ -220,16 +219,38 @@ __device__ __forceinline__ void oz_residue_row(const OzSliceBatch& b, int grow) 
     }
 }
 
-// A block row per operand row, or (gated) a few that take every gridDim.y-th: r = 48, 7000 gated rows left at once took
-// 20 us as block rows of their own.
-template <bool GATED>
-__global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSliceBatch b, int rows) {
-    if (!GATED) {
-        oz_residue_row(b, (int)blockIdx.y);
-        return;
+__global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSliceBatch b) {
+    const int grow = (int)blockIdx.y;
+    int ji = 0;
+    while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
+    const int qi = (int)blockIdx.x * 256 + (int)threadIdx.x;
+    if (qi < (b.j[ji].K + 3) >> 2) oz_residue4(b, b.j[ji], grow - b.j[ji].row0, qi);
+}
+
+// Scales and residues of gated operands, a block per row in turn: one launch that leaves at once (1.5 us) where *gate
+// is zero.  (As rows of the launches above, 7000 of them at r = 48 took 20 us to be passed over.)
+__global__ void __launch_bounds__(256) k_oz_slice_gated(const __grid_constant__ OzSliceBatch b, int rows, const int* gate) {
+    if (!*gate) return;
+    __shared__ unsigned long long sh[8];
+    for (int grow = (int)blockIdx.x; grow < rows; grow += (int)gridDim.x) {
+        int ji = 0;
+        while (ji + 1 < b.njobs && b.j[ji + 1].row0 <= grow) ++ji;
+        const OzSliceJob& J = b.j[ji];   // (no maps)
+        const int row = grow - J.row0;
+        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(J.src + (size_t)row * J.lds);
+        unsigned long long mx = 0;
+        for (int k = threadIdx.x; k < J.K; k += 256) mx = max(mx, src[k] & 0x7FFFFFFFFFFFFFFFull);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 0; w < 8; ++w) mx = max(mx, sh[w]);
+            J.scale[row] = oz_row_scale(mx);
+        }
+        __syncthreads();
+        for (int qi = threadIdx.x; qi < (J.K + 3) >> 2; qi += 256) oz_residue4(b, J, row, qi);
     }
-    if (!*b.gate) return;
-    for (int grow = (int)blockIdx.y; grow < rows; grow += (int)gridDim.y) oz_residue_row(b, grow);
 }
 
 // ------------------------------------------------------------------------------- GEMM
@@ -240,7 +261,6 @@ __global__ void __launch_bounds__(256) k_oz_residue(const __grid_constant__ OzSl
 template <int BN, int STAGES, bool PAIR>
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __restrict__ bp) {
     const OzBatch& b = *bp;
-    if (b.gate && !*b.gate) return;   // the whole grid, before any barrier or tensor memory
     constexpr int A_BYTES = TC_BM * 128;
     constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * 128;
     constexpr int BM = PAIR ? 2 * TC_BM : TC_BM;   // rows of an output tile
@@ -295,6 +315,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
                 const int t = b.order[qi];
                 const int pi = oz_find_problem(b, t);
                 const OzProb& P = b.p[pi];
+                if (oz_skip(P)) continue;
                 const int local = t - P.tile_start;
                 const int m0 = (local / P.tiles_n) * BM + (int)rank * TC_BM;
                 const int n0 = (local % P.tiles_n) * BN + (int)rank * (BN / 2);
@@ -341,6 +362,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
             int it = 0, lt = 0;
             for (int qi = q0; qi < q1 && !*abort_flag; ++qi) {
                 const OzProb& P = b.p[oz_find_problem(b, b.order[qi])];
+                if (oz_skip(P)) continue;
                 for (int gi = 0; gi < P.ngroups && !*abort_flag; ++gi, ++lt) {
                     const int c = gi % P.nch;
                     const int n = min(P.cb, P.kbs - c * P.cb);
@@ -391,6 +413,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_gemm_oz(const OzBatch* __rest
         for (int qi = q0; qi < q1 && run; ++qi) {
             const int t = b.order[qi];
             const OzProb& P = b.p[oz_find_problem(b, t)];
+            if (oz_skip(P)) continue;
             const int local = t - P.tile_start;
             const int m0 = (local / P.tiles_n) * BM + (int)rank * TC_BM, n0 = (local % P.tiles_n) * BN;
             const int row = m0 + q * 32 + lane;
@@ -581,8 +604,8 @@ __device__ __forceinline__ void oz_crt_rows(const OzProb& P, const OzCrtParams& 
 template <bool TWO>
 __global__ void __launch_bounds__(256, TWO ? 2 : 3) k_oz_crt(const OzBatch* __restrict__ bp,
                                                              const __grid_constant__ OzCrtParams cp) {
-    if (bp->gate && !*bp->gate) return;
     const OzProb& P = bp->p[blockIdx.y];
+    if (oz_skip(P)) return;
     if (!TWO || P.nch == 1) oz_crt_rows<1>(P, cp);
     else oz_crt_rows<2>(P, cp);
 }
@@ -624,9 +647,9 @@ static int oz_launch_crt(const OzBatch* host, const OzBatch* dev, int nsm, cudaS
 //      [M_aa; D_aa], [M_bb; D_bb] packed (2P x P);
 //   B: M+ (S2 x S2), M- (P2 x P2), Mf1, W_ab (r^2 x r^2), W_aa, W_bb packed (P x P).
 // The problem table of s = +1 is the plan itself; that of s = -1 (`alt`) has the same operands with the
-// other row counts and borrows every buffer.  `gen`: the three products of a D that is not pair-Hermitian, with the same
-// A and B operands of their own (the 2P odd rows of M+, the 2S even ones of M-, the second flip of M), skipped on the
-// device (Work::asym) for any other D: its launches leave at once, 2-3 us each.
+// other row counts and borrows every buffer.  The last three products are those of a D that is not pair-Hermitian: the
+// first three A with B operands of their own (the 2P odd rows of M+, the 2S even ones of M-, the second flip of M),
+// gated by Work::asym, their tiles behind all others in every list.
 struct OzOp {
     __nv_bfloat16* sl;
     double* scale;
@@ -650,9 +673,7 @@ struct OzPlan {
     int* sched;         // tile lists of the persistent kernel (OzBatch::order, cta_start)
     int* err;
     struct OzPlan* alt;       // the pass's table for s = -1
-    struct OzPlan* gen;       // the products of a D that is not pair-Hermitian
     int borrowed;             // operands and staging belong to another plan
-    int borrowedA;            // the A operands do
     struct OzPlan* lists[2];  // GEMM lists of the adjoint (oz_gemm_list): a plan per list slot
     int shareB[OZ_MAXP];      // lists: problem i reads the B operand of problem shareB[i] - 1 (0: its own)
 };
@@ -858,7 +879,7 @@ extern "C" int acse_ozaki_plan_info(int oz_slices, int kmax, int k, int* moduli_
     return st;
 }
 
-// The seven products of a pass in the order of acse_gemm_list_f64 (the same-spin X and Y as one problem).
+// The ten products of a pass in the order of acse_gemm_list_f64 (the same-spin X and Y as one problem).
 static int oz_pass_table(acse_ctx* c, OzPlan* pl, const OzPlan* root, int sW) {
     Work& w = c->w;
     const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1), P = P2 / 2;
@@ -873,36 +894,11 @@ static int oz_pass_table(acse_ctx* c, OzPlan* pl, const OzPlan* root, int sW) {
     ACSE_TRY(add(4, pl->A[1], pl->B[1], ph_V2(c, sW), 2 * R2, 1.0, S2));
     ACSE_TRY(add(5, pl->A[5], pl->B[4], w.Cp[0], P, 2.0, 2 * P));
     ACSE_TRY(add(6, pl->A[6], pl->B[5], w.Cp[1], P, 2.0, 2 * P));
+    ACSE_TRY(add(7, pl->A[0], pl->B[6], w.V1 + S2, 2 * R2, 1.0, S2));
+    ACSE_TRY(add(8, pl->A[1], pl->B[7], ph_V2(c, sW) + P2, 2 * R2, 1.0, S2));
+    ACSE_TRY(add(9, pl->A[2], pl->B[8], w.Vf2, R2, 1.0, R2));
+    for (int i = 7; i < 10; ++i) pl->host->p[i].gate = w.asym;
     return oz_plan_finish(pl);
-}
-
-// The gated products of table pl (the plan of s = +1, root, or alt): operands of their own in root's.
-static int oz_gen_table(acse_ctx* c, OzPlan* pl, const OzPlan* root, int sW) {
-    Work& w = c->w;
-    const int r = c->r, R2 = r * r, S2 = r * (r + 1), P2 = r * (r - 1);
-    OzPlan* g = (OzPlan*)calloc(1, sizeof(OzPlan));
-    if (!g) return ACSE_ERR_NOMEM;
-    pl->gen = g;
-    g->borrowed = pl != root;
-    g->borrowedA = 1;
-    ACSE_TRY(oz_plan_init(g, pl->S, pl->bn, pl->pair, S2));
-    g->host->err = root->err;
-    g->host->gate = w.asym;
-    memcpy(g->A, pl->A, 3 * sizeof(OzOp));
-    if (g->borrowed) {
-        memcpy(g->B, root->gen->B, 3 * sizeof(OzOp));
-    } else {
-        ACSE_TRY(oz_op_alloc(g, g->B[0], P2, S2));
-        ACSE_TRY(oz_op_alloc(g, g->B[1], S2, P2));
-        ACSE_TRY(oz_op_alloc(g, g->B[2], R2, R2));
-    }
-    auto add = [&](int i, double* C, int ldc, int stage_rows) {
-        return oz_add(g, g->A[i], g->B[i], C, ldc, 1.0, stage_rows, g->borrowed ? root->gen->host->p[i].stage : nullptr);
-    };
-    ACSE_TRY(add(0, w.V1 + S2, 2 * R2, S2));
-    ACSE_TRY(add(1, ph_V2(c, sW) + P2, 2 * R2, S2));
-    ACSE_TRY(add(2, w.Vf2, R2, R2));
-    return oz_plan_finish(g);
 }
 
 int oz_plan_create(acse_ctx* c) {
@@ -920,6 +916,9 @@ int oz_plan_create(acse_ctx* c) {
     ACSE_TRY(oz_op_alloc(pl, pl->B[1], P2, P2));
     for (int i = 2; i < 4; ++i) ACSE_TRY(oz_op_alloc(pl, pl->B[i], R2, R2));
     for (int i = 4; i < 6; ++i) ACSE_TRY(oz_op_alloc(pl, pl->B[i], P, P));
+    ACSE_TRY(oz_op_alloc(pl, pl->B[6], P2, S2));
+    ACSE_TRY(oz_op_alloc(pl, pl->B[7], S2, P2));
+    ACSE_TRY(oz_op_alloc(pl, pl->B[8], R2, R2));
     if (cudaMalloc((void**)&pl->err, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return ACSE_ERR_NOMEM;
@@ -929,7 +928,6 @@ int oz_plan_create(acse_ctx* c) {
     pl->host->err = pl->err;
     pl->A[1].rows = P2;   // s = +1: W+ over S2 rows, W- over P2
     ACSE_TRY(oz_pass_table(c, pl, pl, +1));
-    ACSE_TRY(oz_gen_table(c, pl, pl, +1));
     OzPlan* alt = (OzPlan*)calloc(1, sizeof(OzPlan));
     if (!alt) return ACSE_ERR_NOMEM;
     pl->alt = alt;
@@ -940,8 +938,7 @@ int oz_plan_create(acse_ctx* c) {
     memcpy(alt->B, pl->B, sizeof(pl->B));
     alt->A[0].rows = P2;   // s = -1: the other way round
     alt->A[1].rows = S2;
-    ACSE_TRY(oz_pass_table(c, alt, pl, -1));
-    return oz_gen_table(c, alt, pl, -1);
+    return oz_pass_table(c, alt, pl, -1);
 }
 
 // Longest-processing-time tile lists of the persistent kernel (tile cost: its K blocks over all groups)
@@ -962,7 +959,8 @@ static int oz_plan_finish(OzPlan* pl) {
         }
         for (int p = 0; p < B.nprob; ++p) {
             const int n = ((B.p[p].M + pl->bm - 1) / pl->bm) * B.p[p].tiles_n;
-            for (int k = 0; k < n; ++k) cost[B.p[p].tile_start + k] = (long long)nmod * B.p[p].kbs + 4 * B.p[p].ngroups;
+            for (int k = 0; k < n; ++k)   // gated tiles are mostly passed over: a cost that deals them out last
+                cost[B.p[p].tile_start + k] = B.p[p].gate ? 1 : (long long)nmod * B.p[p].kbs + 4 * B.p[p].ngroups;
         }
         tc_lpt_schedule(cost, T, G, hs, hs + T);
         const bool ok = cudaMalloc((void**)&pl->sched, (size_t)(T + G + 1) * sizeof(int)) == cudaSuccess &&
@@ -987,11 +985,10 @@ static int oz_plan_finish(OzPlan* pl) {
 static void oz_plan_free(OzPlan* pl) {
     if (!pl) return;
     oz_plan_free(pl->alt);
-    oz_plan_free(pl->gen);
     for (int s = 0; s < 2; ++s) oz_plan_free(pl->lists[s]);
     for (int i = 0; i < OZ_MAXP && !pl->borrowed; ++i) {
-        if (pl->A[i].sl && !pl->borrowedA) cudaFree(pl->A[i].sl);
-        if (pl->A[i].scale && !pl->borrowedA) cudaFree(pl->A[i].scale);
+        if (pl->A[i].sl) cudaFree(pl->A[i].sl);
+        if (pl->A[i].scale) cudaFree(pl->A[i].scale);
         if (pl->shareB[i]) continue;   // an earlier problem's operand
         if (pl->B[i].sl) cudaFree(pl->B[i].sl);
         if (pl->B[i].scale) cudaFree(pl->B[i].scale);
@@ -1058,8 +1055,7 @@ static int oz_slice_launch(acse_ctx* c, const OzSliceBatch& all, int rows) {
     ACSE_LAUNCHED(c);
     int maxq = 1;
     for (int i = 0; i < all.njobs; ++i) maxq = (all.j[i].K + 3) / 4 > maxq ? (all.j[i].K + 3) / 4 : maxq;
-    if (all.gate) k_oz_residue<true><<<dim3((maxq + 255) / 256, rows < 128 ? rows : 128), 256, 0, c->stream>>>(all, rows);
-    else k_oz_residue<false><<<dim3((maxq + 255) / 256, rows), 256, 0, c->stream>>>(all, rows);
+    k_oz_residue<<<dim3((maxq + 255) / 256, rows), 256, 0, c->stream>>>(all);
     ACSE_LAUNCHED(c);
     return ACSE_OK;
 }
@@ -1085,15 +1081,14 @@ int oz_slice_operands(acse_ctx* c, int prep_D, int sW) {
         oz_job(b, rows, pl->B[0], 0, S2, w.Mp, S2, nullptr, nullptr, 1);
         oz_job(b, rows, pl->B[1], 0, P2, w.Mm, P2, nullptr, nullptr, 1);
         oz_job(b, rows, pl->B[2], 0, R2, w.Mf1, R2, nullptr, nullptr, 1);
-        const OzOp* gB = root->gen->B;
         OzSliceBatch gb;
         oz_slice_batch_init(gb, pl->host->mods);
-        gb.gate = w.asym;
         int grows = 0;
-        oz_job(gb, grows, gB[0], 0, P2, w.Mp + (size_t)S2 * S2, S2, nullptr, nullptr, 1);
-        oz_job(gb, grows, gB[1], 0, S2, w.Mm + (size_t)P2 * P2, P2, nullptr, nullptr, 1);
-        oz_job(gb, grows, gB[2], 0, R2, w.Mf2, R2, nullptr, nullptr, 1);
-        ACSE_TRY(oz_slice_launch(c, gb, grows));
+        oz_job(gb, grows, pl->B[6], 0, P2, w.Mp + (size_t)S2 * S2, S2, nullptr, nullptr, 1);
+        oz_job(gb, grows, pl->B[7], 0, S2, w.Mm + (size_t)P2 * P2, P2, nullptr, nullptr, 1);
+        oz_job(gb, grows, pl->B[8], 0, R2, w.Mf2, R2, nullptr, nullptr, 1);
+        k_oz_slice_gated<<<4 * root->nsm, 256, 0, c->stream>>>(gb, grows, w.asym);
+        ACSE_LAUNCHED(c);
     }
     oz_job(b, rows, pl->B[3], 0, R2, c->cur_W[1], R2, nullptr, nullptr, 1);
     oz_job(b, rows, pl->B[4], 0, P, c->cur_W[0], R2, pm, pm, 1);
@@ -1114,19 +1109,14 @@ int oz_gemm_launch(acse_ctx* c, int sW) {
     ACSE_LAUNCHED(c);
     ACSE_TRY(oz_launch_crt(pl->host, pl->dev, pl->nsm, c->stream));
     ACSE_LAUNCHED(c);
-    ACSE_TRY(prof_end(c));
-    ACSE_TRY(oz_launch_gemm(pl->gen, c->stream));
-    ACSE_LAUNCHED(c);
-    ACSE_TRY(oz_launch_crt(pl->gen->host, pl->gen->dev, pl->gen->nsm, c->stream));
-    ACSE_LAUNCHED(c);
-    return ACSE_OK;
+    return prof_end(c);
 }
 
 int oz_set_wait_ns(acse_ctx* c, unsigned long long ns, int inject_stall) {
     OzPlan* pl = (OzPlan*)c->oz_plan;
     if (!pl) return ACSE_ERR_UNSUPPORTED;
     ACSE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    for (OzPlan* q : {pl, pl->alt, pl->gen, pl->alt->gen}) {
+    for (OzPlan* q : {pl, pl->alt}) {
         q->host->wait_ns = ns ? ns : OZ_WAIT_NS;
         q->host->inject_stall = inject_stall;
         ACSE_CUDA_TRY(cudaMemcpy(q->dev, q->host, sizeof(OzBatch), cudaMemcpyHostToDevice));
