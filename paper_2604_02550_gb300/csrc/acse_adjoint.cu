@@ -846,14 +846,14 @@ static int vjp_D(acse_ctx* c, const double* const W[3], int sW, double scale, co
     GemmF64 g[9];
     int n = 0;
     const int n1 = sW > 0 ? S2 : P2, n2 = sW > 0 ? P2 : S2;
-    g[n++] = GemmF64{a->v1, sW > 0 ? w.Wp : w.Wm, a->mp, S2, S2, n1, n1, n1, S2, 1.0, 0.0, nullptr, nullptr, nullptr};
-    g[n++] = GemmF64{a->vf, w.Wf1, a->mf, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr, nullptr};
-    g[n++] = GemmF64{a->Xp[1], W[1], a->mx[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
-    g[n++] = GemmF64{a->Yp[1], W[1], a->my[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
-    g[n++] = GemmF64{a->v2, sW > 0 ? w.Wm : w.Wp, a->mm, P2, P2, n2, n2, n2, P2, 1.0, 0.0, nullptr, nullptr, nullptr};
+    g[n++] = GemmF64{a->v1, sW > 0 ? w.Wp : w.Wm, a->mp, S2, S2, n1, n1, n1, S2, 1.0, nullptr, nullptr, nullptr};
+    g[n++] = GemmF64{a->vf, w.Wf1, a->mf, R2, R2, R2, R2, R2, R2, 1.0, nullptr, nullptr, nullptr};
+    g[n++] = GemmF64{a->Xp[1], W[1], a->mx[1], R2, R2, R2, R2, R2, R2, 2.0, nullptr, nullptr, nullptr};
+    g[n++] = GemmF64{a->Yp[1], W[1], a->my[1], R2, R2, R2, R2, R2, R2, 2.0, nullptr, nullptr, nullptr};
+    g[n++] = GemmF64{a->v2, sW > 0 ? w.Wm : w.Wp, a->mm, P2, P2, n2, n2, n2, P2, 1.0, nullptr, nullptr, nullptr};
     for (int s = 0; s < 3; s += 2) {
-        g[n++] = GemmF64{a->Xp[s], W[s], a->mx[s], P, P, P, P, R2, P, 1.0, 0.0, nullptr, w.pmap, nullptr};
-        g[n++] = GemmF64{a->Yp[s], W[s], a->my[s], P, P, P, P, R2, P, 1.0, 0.0, nullptr, w.pmap, nullptr};
+        g[n++] = GemmF64{a->Xp[s], W[s], a->mx[s], P, P, P, P, R2, P, 1.0, nullptr, w.pmap, nullptr};
+        g[n++] = GemmF64{a->Yp[s], W[s], a->my[s], P, P, P, P, R2, P, 1.0, nullptr, w.pmap, nullptr};
     }
     ACSE_TRY(c->oz ? oz_gemm_list(c, g, n, sW > 0 ? 0 : 1) : gemm_f64_grouped(c, g, n, c->stream));
     AdjM am;

@@ -299,19 +299,19 @@ int acse_gemm_list_f64(acse_ctx* c, int sW, GemmF64* g, int* n) {
     const int n1 = sW > 0 ? S2 : P2, n2 = sW > 0 ? P2 : S2;
     int k = 0;
     double* const V2 = ph_V2(c, sW);
-    g[k++] = GemmF64{w.Wp, w.Mp, w.V1, n1, S2, S2, S2, S2, 2 * R2, 1.0, 0.0, nullptr, nullptr, nullptr};
-    g[k++] = GemmF64{w.Wf1, w.Mf1, w.V5f1, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr, nullptr};
-    g[k++] = GemmF64{w.M[1], c->cur_W[1], w.X[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
-    g[k++] = GemmF64{c->cur_D[1], c->cur_W[1], w.Y[1], R2, R2, R2, R2, R2, R2, 2.0, 0.0, nullptr, nullptr, nullptr};
-    g[k++] = GemmF64{w.Wm, w.Mm, V2, n2, P2, P2, P2, P2, 2 * R2, 1.0, 0.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wp, w.Mp, w.V1, n1, S2, S2, S2, S2, 2 * R2, 1.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wf1, w.Mf1, w.V5f1, R2, R2, R2, R2, R2, R2, 1.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.M[1], c->cur_W[1], w.X[1], R2, R2, R2, R2, R2, R2, 2.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{c->cur_D[1], c->cur_W[1], w.Y[1], R2, R2, R2, R2, R2, R2, 2.0, nullptr, nullptr, nullptr};
+    g[k++] = GemmF64{w.Wm, w.Mm, V2, n2, P2, P2, P2, P2, 2 * R2, 1.0, nullptr, nullptr, nullptr};
     for (int s = 0; s < 3; s += 2) {
         double* C = w.Cp[s / 2];
-        g[k++] = GemmF64{w.M[s], c->cur_W[s], C, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap, nullptr};
-        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], C + (size_t)P * P, P, P, P, R2, R2, P, 2.0, 0.0, w.pmap, w.pmap, nullptr};
+        g[k++] = GemmF64{w.M[s], c->cur_W[s], C, P, P, P, R2, R2, P, 2.0, w.pmap, w.pmap, nullptr};
+        g[k++] = GemmF64{c->cur_D[s], c->cur_W[s], C + (size_t)P * P, P, P, P, R2, R2, P, 2.0, w.pmap, w.pmap, nullptr};
     }
-    g[k++] = GemmF64{w.Wp, w.Mp + (size_t)S2 * S2, w.V1 + S2, n1, P2, S2, S2, S2, 2 * R2, 1.0, 0.0, nullptr, nullptr, w.asym};
-    g[k++] = GemmF64{w.Wm, w.Mm + (size_t)P2 * P2, V2 + P2, n2, S2, P2, P2, P2, 2 * R2, 1.0, 0.0, nullptr, nullptr, w.asym};
-    g[k++] = GemmF64{w.Wf1, w.Mf2, w.Vf2, R2, R2, R2, R2, R2, R2, 1.0, 0.0, nullptr, nullptr, w.asym};
+    g[k++] = GemmF64{w.Wp, w.Mp + (size_t)S2 * S2, w.V1 + S2, n1, P2, S2, S2, S2, 2 * R2, 1.0, nullptr, nullptr, w.asym};
+    g[k++] = GemmF64{w.Wm, w.Mm + (size_t)P2 * P2, V2 + P2, n2, S2, P2, P2, P2, 2 * R2, 1.0, nullptr, nullptr, w.asym};
+    g[k++] = GemmF64{w.Wf1, w.Mf2, w.Vf2, R2, R2, R2, R2, R2, R2, 1.0, nullptr, nullptr, w.asym};
     *n = k;
     return ACSE_OK;
 }

@@ -32,7 +32,7 @@ __device__ __forceinline__ void pk_unpair(int r, int u, int& a, int& b) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Dense GEMM problem: C[m*ldc + n] = alpha * sum_k A(m,k) B(n,k) (+ beta*C), with
+// Dense GEMM problem: C[m*ldc + n] = alpha * sum_k A(m,k) B(n,k), with
 //   A(m,k) = A[mapA(m)*lda + mapA(k)],  B(n,k) = B[mapB(n)*ldb + mapB(k)]  (K-major).
 // ------------------------------------------------------------------------------------------
 struct GemmF64 {
@@ -41,7 +41,7 @@ struct GemmF64 {
     double* C;
     int M, N, K;
     int lda, ldb, ldc;
-    double alpha, beta;
+    double alpha;
     const int* mapA;   // null, or the source row of every row of A and source column of every K index (the
     const int* mapB;   // pair numbering of a packed same-spin operand); the same for B
     const int* gate;   // null, or the product is formed only where *gate (device memory) is not zero
@@ -327,7 +327,7 @@ void oz_plan_destroy(acse_ctx* c);
 int oz_slice_operands(acse_ctx* c, int prep_D, int sW);   // the pass's FP64 operands -> scaled bf16 slices
 int oz_gemm_launch(acse_ctx* c, int sW);                  // every GEMM of the pass, one persistent launch
 int oz_set_wait_ns(acse_ctx* c, unsigned long long ns, int inject_stall);
-// Any list of up to 12 FP64 GEMMs (alpha a power of two, beta 0, mapA null) by the Ozaki scheme; `slot` (0 or
+// Any list of up to 12 FP64 GEMMs (alpha a power of two, mapA null) by the Ozaki scheme; `slot` (0 or
 // 1) names the list's plan, built on its first use (the adjoint's lists)
 int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot);
 

@@ -566,7 +566,7 @@ int ny_pass(acse_ctx* c) {
                     const double* A = (const double*)y->opA[g % 3] + (size_t)rb * R2 * ld + (size_t)q0 * R2;
                     const double* B = (const double*)y->opB[g % 3] + (size_t)cb * R2 * ld + (size_t)q0 * R2;
                     double* C = (double*)y->out[g] + (size_t)rb * R2 * y->n2 + (size_t)cb * R2;
-                    gl[ng++] = GemmF64{A, B, C, R2, R2, cnt * R2, (int)ld, (int)ld, (int)y->n2, 1.0, 0.0, nullptr, nullptr, nullptr};
+                    gl[ng++] = GemmF64{A, B, C, R2, R2, cnt * R2, (int)ld, (int)ld, (int)y->n2, 1.0, nullptr, nullptr, nullptr};
                 }
             ACSE_TRY(gemm_f64_grouped(c, gl, ng, c->stream));
         } else {

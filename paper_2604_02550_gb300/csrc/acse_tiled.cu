@@ -285,26 +285,39 @@ __global__ void __launch_bounds__(256) k_w_from_diag(int r, const T* __restrict_
 }
 
 // ------------------------------------------------------------------------- B -> H
-template <typename T>
 struct BTiledArgs {
     int r;
-    const T* X[3];      // pair GEMM outputs X^{ij}_{kp}, row stride r^2
-    const T* Y[3];      // pair GEMM outputs Y^{ij}_{kl}
-    const T* X5d;       // (2r^2) x (2r^2), rows (sK,k,j), columns (sI,i,l)
-    const T* X5f1;      // r^2 x r^2
-    const T* X5f2;
-    const T* M[3];
-    const T* gam;
-    const T* w;
-    const T* Q;
-    T* H[3];
-    const T* ny[4];     // NY three-body term per spin type (acse_ny.cu), added to B; null for V
+    const float* X[3];      // pair GEMM outputs X^{ij}_{kp}, row stride r^2
+    const float* Y[3];      // pair GEMM outputs Y^{ij}_{kl}
+    const float* X5d;       // (2r^2) x (2r^2), rows (sK,k,j), columns (sI,i,l)
+    const float* X5f1;      // r^2 x r^2
+    const float* X5f2;
+    const float* M[3];
+    const float* gam;
+    const float* w;
+    const float* Q;
+    float* H[3];
+    const float* ny[4];     // NY three-body term per spin type (acse_ny.cu), added to B; null for V
     int flip;           // spin-flip specialisation: no bb items; the b-led particle-hole blocks and the
                         // second flip sector are read as their alpha-led flips
-    const T* bx[8];     // precomputed products (k_B_pre, k_B_pipe<.., true>): per type t, x1 rows at bx[2t] and
-                        // x2^T rows at bx[2t + 1], r^2 per item (pair ij; k_B_pipe: the type's item number, see
-                        // acse_btc.cu)
-    const int* pmap;    // k_B_pre: pair number -> i r + j (i < j)
+    const float* bx[8];   // precomputed products (k_B_pipe<.., true>): per type t, x1 rows at bx[2t] and x2^T rows at
+                          // bx[2t + 1], r^2 per item (the type's item number, see acse_btc.cu)
+};
+
+// Arguments of k_B_pre (FP64 and Ozaki paths): Y, the particle-hole product, 1D, Q, the NY term or null, and the
+// precomputed products, per type t x1 rows at bx[2t] and x2^T rows at bx[2t + 1] of every pair ij.
+struct BPreArgs {
+    int r;
+    const double* Y[3];
+    const double* X5d;
+    const double* X5f1;
+    const double* X5f2;
+    const double* gam;
+    const double* Q;
+    double* H[3];
+    const double* ny[4];
+    const double* bx[8];
+    const int* pmap;    // pair number -> i r + j (i < j)
 };
 
 // FP64 and Ozaki paths.  Spin types t = 0 (aaaa), 1 (bbbb), 2 (abab), 3 (abba); the products x1[k][l] and x2^T[l][k]
@@ -317,7 +330,7 @@ struct BTiledArgs {
 // Blocks: the pairs i < j of aa and of bb (row (j, i) of H is minus row (i, j), rows (i, i) are zero), every pair of
 // ab.  The FP64 pipe (two operations a clock and SM) bounds it at about 19 r^4 operations, HBM at 17 r^4 doubles:
 // r = 48: 217 us, against 628 us for the kernel that combined all r^2 pairs of each type entry by entry.
-__global__ void __launch_bounds__(256) k_B_pre(const __grid_constant__ BTiledArgs<double> a) {
+__global__ void __launch_bounds__(256) k_B_pre(const __grid_constant__ BPreArgs a) {
     extern __shared__ __align__(16) double bp_sm[];   // N [r][ld], N' [r][ld] (ab)
     const int r = a.r, R2 = r * r, ld = r | 1, P = r * (r - 1) / 2;
     const size_t R22 = 2 * (size_t)R2;
@@ -485,7 +498,7 @@ __device__ __forceinline__ int bp_l(int kind, int lb, int nt, int b) { return ki
 // 16): no operand staging, each thread reads its 4 x 4 tile of x1 and of x2^T with 16-byte loads; the
 // shared memory holds only the B rows.
 template <int MAXT, int MINB, int RP, bool PRE = false>
-__global__ void __launch_bounds__(MAXT, MINB) k_B_pipe(const __grid_constant__ BTiledArgs<float> a) {
+__global__ void __launch_bounds__(MAXT, MINB) k_B_pipe(const __grid_constant__ BTiledArgs a) {
     extern __shared__ __align__(16) unsigned char tl_smem[];
     const int r = a.r, rp = RP ? RP : pad4(r), ld = rp + 4, R2 = r * r, bpitch = r + 1;
     const int nt = rp / 4, nt2 = nt * nt, S = (nt2 + 31) & ~31;
@@ -892,19 +905,18 @@ int launch_B_tiled(acse_ctx* c) {
     const int R2 = r * r;
     Work& w = c->w;
     if (c->opt.prec == ACSE_FP64) {
-        BTiledArgs<double> a;
+        BPreArgs a;
         a.r = r;
-        for (int s = 0; s < 3; ++s) { a.X[s] = w.X[s]; a.Y[s] = w.Y[s]; a.M[s] = w.M[s]; a.H[s] = w.H[s]; }
+        for (int s = 0; s < 3; ++s) { a.Y[s] = w.Y[s]; a.H[s] = w.H[s]; }
         a.X5d = w.X5d; a.X5f1 = w.X5f1; a.X5f2 = w.X5f2;
-        a.flip = 0;
         for (int t = 0; t < 4; ++t) a.ny[t] = (const double*)ny_terms(c, t);
-        a.gam = w.gam; a.w = w.w; a.Q = w.Q;
+        a.gam = w.gam; a.Q = w.Q;
         a.pmap = w.pmap;
         ACSE_TRY(launch_Bx(c));
         for (int k = 0; k < 8; ++k) a.bx[k] = w.bx64[k];
         k_B_pre<<<r * (r - 1) + R2, 256, b_smem(r), c->stream>>>(a);
     } else {
-        BTiledArgs<float> a;
+        BTiledArgs a;
         a.r = r;
         for (int s = 0; s < 3; ++s) {
             a.X[s] = w.tc_pairC[s];

@@ -1,4 +1,4 @@
-// FP64 grouped "NT" GEMM on the DFMA pipe:  C = alpha * A . B^T (+ beta C), A and B K-major.
+// FP64 grouped "NT" GEMM on the DFMA pipe:  C = alpha * A . B^T, A and B K-major.
 //
 // One launch runs every tile of up to GEMM_F64_MAXP problems (the sector GEMMs of one contraction pass).
 // GB300 issues two DFMA per clock and SM, so the kernel is bound by that pipe at any tile size: a warp's
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(GF_TPB) k_gemm_f64(const __grid_constant__ Gem
         }
         __syncthreads();
     }
-    const double alpha = P.alpha, beta = P.beta;
+    const double alpha = P.alpha;
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
         const int m = m0 + ty + 16 * i;
@@ -100,10 +100,7 @@ __global__ void __launch_bounds__(GF_TPB) k_gemm_f64(const __grid_constant__ Gem
         for (int j = 0; j < RT; ++j) {
             const int n = n0 + tx + 16 * j;
             if (n >= N) continue;
-            const size_t dst = (size_t)m * P.ldc + n;
-            double v = alpha * acc[i][j];
-            if (beta != 0.0) v += beta * P.C[dst];
-            P.C[dst] = v;
+            P.C[(size_t)m * P.ldc + n] = alpha * acc[i][j];
         }
     }
 }

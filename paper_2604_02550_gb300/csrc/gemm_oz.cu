@@ -70,7 +70,6 @@ struct OzProb {
                             // 1.32 ms, 8 times its work)
     const double* sa;   // 2^ea per row of A
     const double* sb;   // 2^eb per row of B
-    double alpha;
     int ealpha;         // alpha = 2^ealpha
     int M, N, ldc;
     int kbs;            // 64-element K blocks per modulus segment
@@ -779,7 +778,6 @@ static int oz_add(OzPlan* pl, const OzOp& a, const OzOp& b, double* C, int ldc, 
     p.C = C;
     p.sa = a.scale;
     p.sb = b.scale;
-    p.alpha = alpha;
     int ex = 0;
     if (frexp(alpha, &ex) != 0.5) return ACSE_ERR_ARG;   // alpha must be a power of two
     p.ealpha = ex - 1;
@@ -1157,7 +1155,7 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
     if (!root || slot < 0 || slot > 1 || n < 1 || n > OZ_MAXP) return ACSE_ERR_UNSUPPORTED;
     for (int i = 0; i < n; ++i) {
         int ex = 0;
-        if (frexp(g[i].alpha, &ex) != 0.5 || g[i].beta != 0.0 || g[i].mapA) return ACSE_ERR_ARG;
+        if (frexp(g[i].alpha, &ex) != 0.5 || g[i].mapA) return ACSE_ERR_ARG;
     }
     if (!root->lists[slot]) {
         const int s = oz_list_create(root, g, n, &root->lists[slot]);
@@ -1200,7 +1198,6 @@ int oz_gemm_list(acse_ctx* c, const GemmF64* g, int n, int slot) {
         frexp(g[i].alpha, &ex);
         p.C = g[i].C;
         p.ldc = g[i].ldc;
-        p.alpha = g[i].alpha;
         p.ealpha = ex - 1;
     }
     B.wait_ns = root->host->wait_ns;

@@ -29,10 +29,6 @@ __device__ __forceinline__ long long oz_fixedb(unsigned long long bits, int nb, 
     return (bits >> 63) ? -X : X;
 }
 
-// The same for S six-bit slices: X = round(a 2^(6S - e)), |X| < 2^(6S-1).  The rounding drops bits below
-// 2^-6S of the row scale, as the remainder x_{S+1} of the digit recursion does.
-__device__ __forceinline__ long long oz_fixed(unsigned long long bits, int S, int e) { return oz_fixedb(bits, 6 * S, e); }
-
 // acc 2^ex rounded to the nearest double (ties to even), with integer operations only (FP64 is slow on
 // this GPU): the leading bit of |acc| fixes the exponent, the 53 bits below it the significand, the
 // rest decides the rounding.  Results outside the normal range take the FP64 route.
@@ -58,27 +54,4 @@ __device__ __forceinline__ double oz_ll_scaled(long long acc, int ex) {
     const int E = msb + ex + 1023;
     if (E < 1 || E > 2046) return __ll2double_rn(acc) * oz_pow2(min(1023, max(-1022, ex)));
     return __longlong_as_double((long long)(sign | ((unsigned long long)E << 52) | (mant & 0xFFFFFFFFFFFFFull)));
-}
-
-// (-1)^neg (hi 2^64 + lo) 2^ex rounded to the nearest double (ties to even) with integer operations: the
-// leading 64 bits of the 128-bit magnitude are shifted down by one to fit a signed int64, every bit below
-// them folded into the lowest bit (a sticky bit, below the rounding position), and that goes through the
-// 64-bit rounding above.
-__device__ __forceinline__ double oz_u128_scaled(unsigned long long hi, unsigned long long lo, bool neg, int ex) {
-    unsigned long long top, rest;
-    int e0;   // magnitude = top 2^e0 + (rest below it)
-    if (hi != 0) {
-        const int sh = __clzll((long long)hi);
-        top = sh ? (hi << sh) | (lo >> (64 - sh)) : hi;
-        rest = sh ? lo << sh : lo;
-        e0 = 64 - sh;
-    } else {
-        if (lo == 0) return 0.0;
-        const int sh = __clzll((long long)lo);
-        top = lo << sh;
-        rest = 0;
-        e0 = -sh;
-    }
-    const long long v = (long long)((top >> 1) | (top & 1ull) | (rest != 0 ? 1ull : 0ull));
-    return oz_ll_scaled(neg ? -v : v, ex + e0 + 1);
 }
