@@ -108,7 +108,7 @@ def gemm_traffic(prec):
 
 OZ_SLICES = 8   # default slices of ACSE_OZAKI
 # moduli of the modular Ozaki GEMM, largest first; a context uses the least T whose product covers
-# 4 Kmax 2^(2 min(6S, 53)), Kmax = 2 r^2 its longest contraction
+# 4 Kmax 2^(2 min(6S, 53)), Kmax = r (r + 1) its longest contraction
 OZ_MODULI = (127, 125, 123, 121, 119, 113, 109, 107, 103, 101, 97, 89, 83, 79, 73, 71, 67, 61, 59)
 
 
@@ -120,15 +120,21 @@ def oz_moduli_count(S, Kmax):
     return T
 
 
-def flops_per_pass(r, packed=False, singlet=False):
+def flops_per_pass(r, packed=False, singlet=False, symmetrised=False):
     """2 M N K over the O(r^6) GEMMs of one contraction pass G(W):
     pair-pair: 3 spin sectors x ([M; D] (2 r^2 rows) x r^2 x r^2); particle-hole: one
     (2r^2)^3 diagonal-sector GEMM and two (r^2)^3 spin-flip GEMMs  ->  32 r^6.
-    packed=True counts the plan the tensor-core path runs: the same-spin pair GEMMs on pairs i < j
+    symmetrised=True counts what the FP64 and Ozaki paths run for a pair-Hermitian D, the mean of a residual and an
+    update pass: the particle-hole product on pairs a <= b and a < b (S = r(r+1), A = r(r-1): S or A rows x S x S and
+    A or S rows x A x A), one spin flip, the mixed-spin pairs and the packed same-spin ones -> 11 r^6.
+    packed=True counts the plan of the split precisions: the same-spin pair GEMMs on pairs i < j
     only (P = r(r-1)/2: [M; D] 2P rows x P columns x P K each).  singlet=True (spin-flip
     specialisation) drops the bb pair GEMM, the beta-led rows of the diagonal particle-hole GEMM
     and the second spin-flip GEMM."""
     R2 = r * r
+    if symmetrised:
+        S, A = r * (r + 1), r * (r - 1)
+        return (S + A) * (S * S + A * A) + 2 * (3 * R2 ** 3 + 2 * A * (A // 2) ** 2)
     if not packed:
         return 2 * (3 * (2 * R2) * R2 * R2 + (2 * R2) ** 3 + 2 * R2 ** 3)
     P = r * (r - 1) // 2
@@ -315,7 +321,7 @@ def run_batch(args, rank, world):
     clocks = sampler.stop()
     tune, split, launches = _lib.acse_batch_info(b)
     _lib.acse_batch_destroy(b)
-    fl = sum(2 * flops_per_pass(p.r, packed=prec != "fp64") for p in probs)
+    fl = sum(2 * flops_per_pass(p.r, packed=True, symmetrised=prec == "fp64") for p in probs)
     line = {"metric": "acse_residual_evals_per_s", "value": world * EVALS_PER_STEP * len(probs) * args.steps / dt,
             "unit": "residual evals/s", "evals_per_step": EVALS_PER_STEP * len(probs),
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -555,11 +561,11 @@ def main():
     per_step = ms_max / args.steps
     value = whole_job_rate(EVALS_PER_STEP * args.steps, world, ms_max)
     fl_alg = flops_per_pass(p.r)                       # 32 r^6: the unpacked formulation
-    # what the GEMM launch executes (the same-spin pair GEMMs on packed pairs on every path but FP64 FMA)
-    fl = fl_alg if prec == "fp64" else flops_per_pass(p.r, packed=True, singlet=singlet)
+    # what the GEMM launch executes
+    fl = flops_per_pass(p.r, packed=True, singlet=singlet, symmetrised=prec in ("fp64", "ozaki"))
     split = 3 if prec in ("bf16x3", "tf32x3") else 1
     if prec == "ozaki":
-        split = oz_moduli_count(OZ_SLICES, 2 * p.r * p.r)   # bf16 residue products per FP64 GEMM
+        split = oz_moduli_count(OZ_SLICES, p.r * (p.r + 1))   # bf16 residue products per FP64 GEMM
     # dominant kernel: the grouped O(r^6) GEMM launch (one per contraction pass)
     gemm_avg_s = gemm_ms / max(gemm_n, 1) / 1e3
     peaks = {}
@@ -581,10 +587,10 @@ def main():
     roof.update({"achieved": ach, "frac": ach / roof["peak"], "traffic": gemm_traffic(prec) if p.r == 48 else None,
                  "kernel": "grouped O(r^6) GEMM",
                  "flops_per_launch": split * fl,
-                 "flops_note": {"fp64": "2MNK, 32 r^6 per pass",
+                 "flops_note": {"fp64": "2MNK of the products on symmetrised and packed pairs, 11 r^6 per pass",
                                 "ozaki": f"bf16 residue products of the modular Ozaki scheme: {split} per FP64 "
                                          f"GEMM ({OZ_SLICES} slices: {min(6 * OZ_SLICES, 53)}-bit integer rows, "
-                                         f"{split} moduli), 2MNK each, same-spin pair GEMMs on pairs i<j; the "
+                                         f"{split} moduli), 2MNK each, products on symmetrised and packed pairs (11 r^6); the "
                                          f"timed launch includes the reconstruction kernel"}.get(
                      prec, "2MNK of the GEMMs the launch executes (same-spin pair GEMMs on pairs i<j)"),
                  "launch_ms": 1e3 * gemm_avg_s,
