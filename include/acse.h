@@ -18,7 +18,7 @@
  *     contracted as given, at about 1.5 times the cost in ACSE_FP64 and ACSE_OZAKI (the commutator form of
  *     Appendix B has used the Hermiticity of K and D, so A is then that form's value, not a commutator's).
  *   * h: r x r one-electron integrals; V: r^4 two-electron integrals in chemist's notation
- *     (pq|rs) stored [p][q][r][s].
+ *     (pq|rs) stored [p][q][r][s]; over real orbitals, so h is symmetric and V has the eightfold symmetry.
  *   * Reduced Hamiltonian (Eq. 2):  K = 1/2(<pq|rs> - <pq|sr>)
  *         + (h_pr d_qs + h_qs d_pr - h_ps d_qr - h_qr d_ps) / (2(N-1)),  <pq|rs> = (pr|qs),
  *     so that E = sum K.2D = sum_aa + sum_bb + 4 sum_ab.
@@ -73,7 +73,9 @@ typedef enum {
  *                rounded to an integer of min(6 oz_slices, 53) bits below its leading bit; the integer
  *                product is computed modulo T pairwise coprime moduli <= 127 (residues exact in bf16,
  *                sums exact in FP32, T the least count that covers the product: 17 at r = 48 with 8
- *                slices) and rebuilt exactly by the Chinese remainder theorem, with one rounding to FP64.
+ *                slices) and rebuilt by the Chinese remainder theorem in fixed point, to 2^-77 of the product P of
+ *                the moduli (2^-10 of the operands' rounding or less; what is smaller than that becomes zero),
+ *                with one rounding to FP64.
  *                With the default 8 (48 bits) the GEMM error is of the order of 2^-48 |A||B| K, below
  *                that of FP64 FMA.  The O(r^5) products (the transformation by 1D and the products of the pairs)
  *                run at r >= 16 with 8 slices or fewer by the digit form of the scheme (error-free splitting,
@@ -135,11 +137,11 @@ typedef struct {
 /* Create a context for one problem.  h (r*r) and V (r^4, chemist's (pq|rs)) are read once to
  * build the spin-blocked reduced Hamiltonian K of Eq. (2); they may be freed afterwards.
  * `cuda_stream` is a cudaStream_t (NULL = legacy default stream) on which every call of this
- * context is ordered.  All device workspace of the forward calls is allocated here (about 40 r^4
- * doubles plus the split-precision operand copies, and the FP64-accurate context of a precision
- * schedule), so acse_energy, acse_residual and acse_step allocate nothing.  The one exception is
- * acse_residual_backward: its first call on a context allocates the adjoint workspace (about 75 r^4
- * doubles, 3.2 GB at r = 48) and, for a split precision, the ACSE_OZAKI companion context; both stay
+ * context is ordered.  All device workspace of the forward calls is allocated here (about 61 r^4
+ * doubles in ACSE_FP64 and ACSE_OZAKI, 20 r^4 in the split precisions, plus the operand copies of the
+ * tensor-core precisions, and the FP64-accurate context of a precision schedule), so acse_energy, acse_residual and acse_step allocate nothing.  The one exception is
+ * acse_residual_backward: its first call on a context allocates the adjoint workspace (about 66 r^4
+ * doubles, 2.8 GB at r = 48, and the residues of its products in ACSE_OZAKI) and, for a split precision, the ACSE_OZAKI companion context; both stay
  * until acse_destroy.  On any failure *ctx is set to NULL (when ctx itself is not NULL) and nothing stays
  * allocated. */
 int acse_create(acse_ctx** ctx, const acse_opts* opts, const double* h, const double* V,

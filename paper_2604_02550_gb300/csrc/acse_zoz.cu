@@ -29,8 +29,8 @@
 // stores only the RP used elements of a row -- with 128-byte rows two buffers of six digits would not fit -- and
 // takes a thread's 16-byte chunks without bank conflicts.  K is permuted so that two adjacent threads share a
 // row's loads in 32-byte sectors: element q = 16 (kc >> 1) + 4 (j >> 1) + 2 (kc & 1) + (j & 1) is element j of chunk kc.
-// r = 48: 355 us for the eight classes (906 us before), 279 us for the transformation (679 us); r = 30: 67 and 55 us
-// (the products took 400 us of the B kernel in double-float, the transformation 104 us).  Bound by the ALU pipe (the
+// r = 48: 283 us for the eight classes, 290 us for the transformation (a block's phases one after another, six-bit
+// digits: 906 and 679 us); r = 30: 56 and 55 us (in double-float 400 us of the B kernel and 104 us).  Bound by the ALU pipe (the
 // digits and the int64 normalisation, about half busy) and the chain TMEM read - MMA - TMEM read; HBM at 2 TB/s.
 // Every wait is bounded, and on expiry the kernel raises the device flag and stops.
 //
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(RZ_THREADS, 1) k_rows_oz(const __grid_constant
                 // The digit tiles of G lie one after another along N, and those of one A digit s go to consecutive
                 // levels, so that t = t0 .. are one MMA of N = nb RP columns from column (s + t0 - 2) RP (at most 256).
                 // Level D + 2 starts with s = 2, t = D, the others with s = 1.  (One MMA per pair of digits, N = RP,
-                // took about 200 cycles each whatever N; r = 48: 386 -> 355 us for the pair products, 288 -> 279 us.)
+                // took about 200 cycles each whatever N: 9 and 3 % more for the pair products and the transformation at r = 48.)
                 const uint64_t da0 = rz_desc(A, TC_BM * 16), db0 = rz_desc(sB, RZ_DMAX * RP * 16);
                 for (int s = 1; s <= D; ++s) {
                     const int t1 = min(D, D + 2 - s);

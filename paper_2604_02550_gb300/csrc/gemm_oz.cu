@@ -17,7 +17,7 @@
 //     of x (P / p_t)^-1) in fixed point, the wrap-around modulo 2^96 being the reduction modulo 1; |x| <= P / 4, so the
 //     signed fraction is x / P itself, and x = P (x / P) is rounded once to FP64 and scaled by alpha 2^(ea + eb - 2 nb).
 // The result is the FP64 product up to the rounding of the operands to nb - 1 bits below each row's
-// leading bit, the 2^-69 P of the fraction's constants (2^-10 of the operand rounding or less) and one final
+// leading bit, the 2^-77 P of the fraction's constants (2^-10 of the operand rounding or less) and one final
 // rounding: no product level is dropped.  Against the six-bit slice form of
 // the scheme (36 slice products at S = 8) this takes 17 residue products at S = 8 and r = 48.
 //
