@@ -15,7 +15,7 @@
  *     Each block is r^4 doubles.  The aa and bb blocks are antisymmetric in (i,j) and in (k,l): the library
  *     relies on it and reads entries that it relates once.  Every block of a (real) 2-RDM is also
  *     pair-Hermitian, X[ij][kl] = X[kl][ij].  A D that is not, by more than 2^-47 of its largest entry, is
- *     contracted as given, at about 1.5 times the cost in ACSE_FP64 and ACSE_OZAKI (the commutator form of
+ *     contracted as given, at up to 1.5 times the cost in ACSE_FP64 and ACSE_OZAKI (the commutator form of
  *     Appendix B has used the Hermiticity of K and D, so A is then that form's value, not a commutator's).
  *   * h: r x r one-electron integrals; V: r^4 two-electron integrals in chemist's notation
  *     (pq|rs) stored [p][q][r][s]; over real orbitals, so h is symmetric and V has the eightfold symmetry.
